@@ -39,7 +39,8 @@ def _stale(obj, deps):
 def build(verbose=False, extra=()):
     """Compile and link; returns the library path.  Raises on failure."""
     os.makedirs(OUT, exist_ok=True)
-    headers = [os.path.join(ROOT, "include", "hf.h"), os.path.join(CSRC, "hf_internal.h")]
+    headers = [os.path.join(ROOT, "include", "hf.h"), os.path.join(CSRC, "hf_internal.h"),
+               os.path.join(CSRC, "hf_cast.h")]
     jobs = []
     objs = []
     for src in SOURCES:

@@ -31,7 +31,7 @@ constexpr size_t kPrefetchBytes = 32u << 20;  // world levels warmed in L2 per r
 constexpr int32_t kDefaultSun[3] = {321060, -321060, 262144};
 
 struct GraphKey {
-    uint32_t bytes, shadows, stats, twl, thl, mip, steps;
+    uint32_t bytes, shadows, kind, twl, thl, mip, steps;
     int32_t sun[3];
     bool operator==(const GraphKey &o) const { return std::memcmp(this, &o, sizeof(*this)) == 0; }
 };
@@ -66,7 +66,7 @@ struct hf_ctx {
     uint32_t *d_status = nullptr;
     uint32_t *h_status = nullptr;
     unsigned long long *d_stats = nullptr;
-    int occ[2][2] = {{0, 0}, {0, 0}};
+    int occ[2][hf::kTraceKinds] = {};  // batched trace blocks per SM, [shadows][kind]
     int occ_march = 0;
     bool pair = false;  // level 0 holds paired 2-byte texels (hf_create_pairs)
     uint32_t *d_sun = nullptr;  // per-cell shadow bounds (hf_sun.cu), allocated on first use
@@ -208,8 +208,7 @@ int ctx_view(const hf_ctx *c, CtxView *out) {
     out->stream = c->stream;
     out->device = c->device;
     out->sm_count = c->sm_count;
-    out->occ_shadows[0] = c->occ[0][0];
-    out->occ_shadows[1] = c->occ[1][0];
+    std::memcpy(out->occ, c->occ, sizeof(out->occ));
     return 0;
 }
 
@@ -396,9 +395,8 @@ static int create_impl(const hf_desc *d, hf_ctx *c, const uint16_t *texels = nul
     CK(cudaEventRecord(c->edit_done, c->stream));
     for (auto &s : c->slots) CK(cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming));
     for (int sh = 0; sh < 2; ++sh)
-        for (int st = 0; st < 2; ++st)
-            if (hf::trace_batched_occupancy(sh, st, c->pair, &c->occ[sh][st]) ||
-                c->occ[sh][st] < 1)
+        for (int k = 0; k < hf::kTraceKinds; ++k)
+            if (hf::trace_batched_occupancy(sh, k, c->pair, &c->occ[sh][k]) || c->occ[sh][k] < 1)
                 return HF_E_CUDA;
     if (hf::march_occupancy(&c->occ_march) || c->occ_march < 1) return HF_E_CUDA;
     CK(cudaStreamSynchronize(c->stream));
@@ -715,7 +713,7 @@ static int ensure_slot_cap(Slot &s, size_t bytes) {
 }
 
 static int launch_graph(hf_ctx *c, Slot &s, const GraphKey &key, const hf::RenderParams &p,
-                        bool shadows, bool stats, cudaStream_t stream) {
+                        bool shadows, int kind, cudaStream_t stream) {
     cudaGraphExec_t exec = nullptr;
     for (auto &g : s.graphs)
         if (g.first == key) exec = g.second;
@@ -731,8 +729,8 @@ static int launch_graph(hf_ctx *c, Slot &s, const GraphKey &key, const hf::Rende
         hf::RenderParams pc = p;
         void *args[] = {&pc};
         cudaKernelNodeParams kp{};
-        kp.func = const_cast<void *>(hf::trace_batched_fn(shadows, stats, c->pair));
-        kp.gridDim = dim3((unsigned)(c->sm_count * c->occ[shadows][stats]));
+        kp.func = const_cast<void *>(hf::trace_batched_fn(shadows, kind, c->pair));
+        kp.gridDim = dim3((unsigned)(c->sm_count * c->occ[shadows][kind]));
         kp.blockDim = dim3(hf::kThreads);
         kp.sharedMemBytes = 0;
         kp.kernelParams = args;
@@ -1117,7 +1115,9 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
     for (int i = 0; i < 3; ++i)
         if (iabs64(sun[i]) >= kLimit21) return HF_E_INVALID_ARG;
     const bool shadows = (o.flags & HF_SHADOWS) != 0;
-    const bool stats = (o.flags & HF_STATS) != 0;
+    const int kind = (o.flags & HF_STATS) ? hf::kTraceStats
+                     : o.max_steps        ? hf::kTraceGeneral
+                                          : hf::kTraceBeams;
     const uint32_t mip = o.mip_start == HF_MIP_AUTO ? hf::kDefaultMipStart : o.mip_start;
     const uint32_t mip_c = mip > c->L ? c->L : mip;
     const uint64_t guard = 4ull * (c->W + c->H) + 64;
@@ -1152,24 +1152,24 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         // each launch takes its camera record as a parameter: no copy to the device
         const auto *cd = (const hf::CamDev *)((const char *)s.h_staging + sizeof(hf::BatchHeader));
         for (uint32_t i = 0; i < n; ++i)
-            if (hf::launch_trace_plain(p, shadows, stats, cd[i], b.tiles[i], b.stream))
+            if (hf::launch_trace_plain(p, shadows, kind, cd[i], b.tiles[i], b.stream))
                 return HF_E_CUDA;
     } else if (o.flags & HF_NOGRAPH) {
         CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));
-        if (hf::launch_trace_batched(p, shadows, stats, c->sm_count * c->occ[shadows][stats],
+        if (hf::launch_trace_batched(p, shadows, kind, c->sm_count * c->occ[shadows][kind],
                                      b.stream))
             return HF_E_CUDA;
     } else {
         GraphKey key{};
         key.bytes = (uint32_t)b.bucket;
         key.shadows = shadows;
-        key.stats = stats;
+        key.kind = (uint32_t)kind;
         key.twl = (uint32_t)p.tile_w_log2;
         key.thl = (uint32_t)p.tile_h_log2;
         key.mip = mip_c;
         key.steps = steps;
         for (int i = 0; i < 3; ++i) key.sun[i] = sun[i];
-        rc = launch_graph(c, s, key, p, shadows, stats, b.stream);
+        rc = launch_graph(c, s, key, p, shadows, kind, b.stream);
         if (rc != HF_OK) return rc;
     }
     return finish_batch(c, b, (o.flags & HF_SYNC) != 0);

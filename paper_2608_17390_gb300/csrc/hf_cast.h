@@ -1,0 +1,624 @@
+// hf_cast.h -- the traversal of rays through the cells and their pyramid.
+//
+// Two traversals give the same hit:
+//
+//   cast_general  one ray, hierarchical DDA, every decision on rationals
+//                 num/den with 64-bit products.  Counts fetches, obeys a step
+//                 limit of the caller's.
+//   beam_*        the parts of a warp's traversal (hf_trace.cu): the rays of a
+//                 warp that go the same way are bounded by one beam, whose 32
+//                 next stretches are tested by the 32 lanes at once; rays are
+//                 walked, column by column in float with error bounds, only
+//                 through stretches that the beam does not prove empty.  What
+//                 the bounds leave open is decided exactly: a column that may
+//                 hold a hit on rationals, a ray through a cell corner by
+//                 cast_general.
+//
+// The functions are host code too, so that the two can be compared on a CPU.
+#pragma once
+
+#include <cmath>
+#include <cstdint>
+
+#include "hf_internal.h"
+
+#ifdef __CUDACC__
+#define HF_HD __host__ __device__ __forceinline__
+#else
+#define HF_HD inline
+#endif
+
+namespace hf {
+
+struct Ray {
+    int32_t ox, oy, oz, dx, dy, dz;
+};
+
+// One pyramid level as the traversal reads it (a per-block shared table, so
+// lanes at different levels read it in one shared-memory access).
+struct LevelDev {
+    const uint32_t *base;
+    uint32_t stride, rows;
+};
+
+struct Hit {
+    int32_t cx, cy;
+    int32_t tnum, tden;  // hit time tnum / tden
+    uint32_t word;       // hit cell word
+    uint8_t layer, face;
+};
+
+struct Counters {
+    uint32_t nodes, cells;
+};
+
+HF_HD uint32_t cast_load(const uint32_t *p) {
+#ifdef __CUDA_ARCH__
+    return __ldg(p);
+#else
+    return *p;
+#endif
+}
+
+HF_HD float cast_rcp(float v) {
+#ifdef __CUDA_ARCH__
+    return __frcp_rn(v);
+#else
+    return 1.0f / v;
+#endif
+}
+
+// sign carrier of z(t) - h S for t = num / den (den > 0):  (oz - hS) den + num dz
+HF_HD int64_t zd(int32_t oz_minus_hs, int32_t dz, int32_t num, int32_t den) {
+    return (int64_t)oz_minus_hs * den + (int64_t)num * dz;
+}
+
+// Node-form word of node (x, y) of the level `lv` for the storage the kernel
+// was instantiated for (the choice is made at compile time; `level` matters
+// for paired texels only).
+template <bool PAIR>
+HF_HD uint32_t cast_word(const LevelDev &lv, int level, int32_t x, int32_t y) {
+    if (PAIR && level == 0)
+        return pair_node(cast_load(lv.base + (uint32_t)y * (lv.stride >> 1) + ((uint32_t)x >> 1)),
+                         (uint32_t)x & 1);
+    return cast_load(lv.base + (uint32_t)y * lv.stride + (uint32_t)x);
+}
+
+// The two-interval test of one cell over [tin, tout] (tout finite).
+// Returns true and fills h on a hit; false exactly when nothing is solid
+// along the segment.
+HF_HD bool leaf_test(int32_t oz, int32_t dz, uint32_t word, int32_t tin_num, int32_t tin_den,
+                     int32_t tout_num, int32_t tout_den, uint8_t entry_face, Hit &h) {
+    const int32_t h0 = word & 0xFF, h1 = (word >> 8) & 0xFF, h2 = (word >> 16) & 0xFF;
+    const bool slab = h2 > h0;  // level-0 words are in node form
+    const int32_t a0 = oz - (h0 << kShift);
+    const int64_t zin0 = zd(a0, dz, tin_num, tin_den);
+    if (zin0 <= 0) {
+        h.layer = 0;
+        h.face = entry_face;
+        h.tnum = tin_num;
+        h.tden = tin_den;
+        return true;
+    }
+    const int32_t a1 = oz - (h1 << kShift), a2 = oz - (h2 << kShift);
+    int64_t zin1 = 0, zin2 = 0;
+    if (slab) {
+        zin1 = zd(a1, dz, tin_num, tin_den);
+        zin2 = zd(a2, dz, tin_num, tin_den);
+        if (zin1 >= 0 && zin2 <= 0) {
+            h.layer = 1;
+            h.face = entry_face;
+            h.tnum = tin_num;
+            h.tden = tin_den;
+            return true;
+        }
+    }
+    if (dz < 0) {
+        if (slab && zin2 > 0 && zd(a2, dz, tout_num, tout_den) <= 0) {
+            h.layer = 1;
+            h.face = kFacePZ;
+            h.tnum = a2;
+            h.tden = -dz;
+            return true;
+        }
+        if (zd(a0, dz, tout_num, tout_den) <= 0) {
+            h.layer = 0;
+            h.face = kFacePZ;
+            h.tnum = a0;
+            h.tden = -dz;
+            return true;
+        }
+    } else if (dz > 0) {
+        if (slab && zin1 < 0 && zd(a1, dz, tout_num, tout_den) >= 0) {
+            h.layer = 1;
+            h.face = kFaceNZ;
+            h.tnum = -a1;
+            h.tden = dz;
+            return true;
+        }
+    }
+    return false;
+}
+
+// A vertical ray (dx = dy = 0) stays in its start column for all t >= 0.
+// Writes h only when the ray hits.
+HF_HD bool vertical_test(const Ray &r, uint32_t word, Hit &h) {
+    const int32_t h0 = word & 0xFF, h1 = (word >> 8) & 0xFF, h2 = (word >> 16) & 0xFF;
+    const bool slab = h2 > h0;  // level-0 words are in node form
+    const int32_t a0 = r.oz - (h0 << kShift), a1 = r.oz - (h1 << kShift),
+                  a2 = r.oz - (h2 << kShift);
+    uint8_t layer, face;
+    int32_t tnum = 0, tden = 1;
+    if (a0 <= 0) {
+        layer = 0;
+        face = kFaceInside;
+    } else if (slab && a1 >= 0 && a2 <= 0) {
+        layer = 1;
+        face = kFaceInside;
+    } else if (r.dz < 0) {
+        face = kFacePZ;
+        tden = -r.dz;
+        layer = (slab && a2 > 0) ? 1 : 0;
+        tnum = layer ? a2 : a0;
+    } else if (r.dz > 0 && slab && a1 < 0) {
+        layer = 1;
+        face = kFaceNZ;
+        tnum = -a1;
+        tden = r.dz;
+    } else {
+        return false;
+    }
+    h.layer = layer;
+    h.face = face;
+    h.tnum = tnum;
+    h.tden = tden;
+    return true;
+}
+
+// The cell a ray occupies just after t = 0.
+HF_HD void cast_cell(const Ray &r, int32_t &cx, int32_t &cy) {
+    cx = (r.ox >> kShift) - (r.dx < 0 && (r.ox & 0xFFFF) == 0 ? 1 : 0);
+    cy = (r.oy >> kShift) - (r.dy < 0 && (r.oy & 0xFFFF) == 0 ? 1 : 0);
+}
+
+template <bool PAIR>
+HF_HD void vertical_hit(const LevelDev *lvt, const Ray &r, int32_t cx, int32_t cy, Hit &h) {
+    const uint32_t word = cast_word<PAIR>(lvt[0], 0, cx, cy);
+    if (vertical_test(r, word, h)) {
+        h.cx = cx;
+        h.cy = cy;
+        h.word = word;
+    }
+}
+
+// Exact first hit of one ray.  h.face = kFaceMiss on a
+// miss, kFaceError when max_steps nodes did not finish the ray.
+//
+// Skipping an empty node changes only the node index on the exit axis; the
+// finer bits on the other axis are found when the traversal descends, by
+// asking whether the ray has crossed the child midline by t_in (exact
+// cross-multiplied time comparison).  Every interior cell boundary of a node
+// is the midline of exactly one sub-level, so a ray that enters a cell through
+// its Y side while also crossing an X cell boundary (a corner) is detected on
+// the way down and reported with the X face.
+template <bool STATS, bool PAIR>
+HF_HD void cast_general(const LevelDev *lvt, const Ray &r, int start_level, int mip_start,
+                        int max_steps, Hit &h, Counters &cnt) {
+    h.face = kFaceMiss;
+    h.layer = 255;
+    int32_t cx, cy;
+    cast_cell(r, cx, cy);
+    if ((uint32_t)cx >= lvt[0].stride || (uint32_t)cy >= lvt[0].rows) return;
+    if (r.dx == 0 && r.dy == 0) {
+        if (STATS) cnt.cells++;
+        vertical_hit<PAIR>(lvt, r, cx, cy, h);
+        return;
+    }
+    // Per-ray sign constants.  A zero direction component counts as positive:
+    // its exit distance is then positive and never the smaller one, so the
+    // ray never leaves through that axis.
+    const int32_t adx = r.dx < 0 ? -r.dx : r.dx, ady = r.dy < 0 ? -r.dy : r.dy;
+    const int32_t gx = r.dx < 0 ? -1 : 1, gy = r.dy < 0 ? -1 : 1;  // step per exit
+    const int32_t px = r.dx < 0 ? 0 : 1, py = r.dy < 0 ? 0 : 1;    // exit side offset
+    const int32_t qx = px ^ 1, qy = py ^ 1;
+    const int32_t kx = -gx * r.ox, ky = -gy * r.oy;
+    const uint8_t face_x = r.dx < 0 ? kFacePX : kFaceNX;  // entry face of an x crossing
+    const uint8_t face_y = r.dy < 0 ? kFacePY : kFaceNY;
+    int level = start_level;  // <= mip_start, the coarsest level the ray climbs to
+    int32_t nx = cx >> level, ny = cy >> level;
+    int32_t tin_num = 0, tin_den = 1;
+    uint8_t entry = kFaceInside;
+    for (int it = 0;; ++it) {
+        // one bounds check per iteration, after every advance, ascent or
+        // descent: an index past the level's end, or below 0, means the ray
+        // has left the grid.  An ascent keeps the crossed axis out of range
+        // (it follows a step onto an even index n >= ceil(E / 2^l), so
+        // n / 2 >= ceil(E / 2^(l+1)); or onto -1, and -1 >> 1 = -1).  At an
+        // exact corner the other axis may come back in range, in a partial
+        // node past the grid's edge; the ray only moves further out, and a
+        // descent there lands on an out-of-range child, so it still misses.
+        // A ray that leaves on its last allowed iteration is a miss, not a
+        // step-limit error.
+        const LevelDev lv = lvt[level];
+        if ((uint32_t)nx >= lv.stride || (uint32_t)ny >= lv.rows) return;
+        if (it == max_steps) break;
+        const int32_t bx = (nx + px) * (1 << level);  // exit boundary (cells)
+        const int32_t by = (ny + py) * (1 << level);
+        const int32_t numx = gx * (bx * (1 << kShift)) + kx;  // > 0
+        const int32_t numy = gy * (by * (1 << kShift)) + ky;
+        const int64_t cmp = (int64_t)numx * ady - (int64_t)numy * adx;  // < 0: x exits first
+        const bool xfirst = cmp <= 0;
+        const int32_t tout_num = xfirst ? numx : numy;
+        const int32_t tout_den = xfirst ? adx : ady;
+        // level 0 holds cells in node form, so one word layout serves every
+        // level; for a single cell the emptiness test below is exact (the
+        // segment's z range [zlo, zhi] misses (-inf, h0] and [h1, h2] exactly
+        // when zlo > top, or zlo > h0 and zhi < h1)
+        const uint32_t word = cast_word<PAIR>(lv, level, nx, ny);
+        if (STATS) {
+            if (level > 0) cnt.nodes++;
+            else cnt.cells++;
+        }
+        const int32_t maxh0 = word & 0xFF, minh1 = (word >> 8) & 0xFF,
+                      maxtop = (word >> 16) & 0xFF;
+        const bool down = r.dz < 0;
+        const int32_t lo_num = down ? tout_num : tin_num, lo_den = down ? tout_den : tin_den;
+        const int32_t hi_num = down ? tin_num : tout_num, hi_den = down ? tin_den : tout_den;
+        const bool empty = zd(r.oz - (maxtop << kShift), r.dz, lo_num, lo_den) > 0 ||
+                           (zd(r.oz - (maxh0 << kShift), r.dz, lo_num, lo_den) > 0 &&
+                            zd(r.oz - (minh1 << kShift), r.dz, hi_num, hi_den) < 0);
+        if (empty) {
+            // advance past the node (or cell) through its exit side; at an
+            // exact corner both indices change and the X face is reported
+            if (cmp <= 0) nx += gx;
+            if (cmp >= 0) ny += gy;
+            entry = cmp <= 0 ? face_x : face_y;
+            tin_num = tout_num;
+            tin_den = tout_den;
+            // ascend when the crossed boundary is a parent boundary: the new index
+            // on the crossed axis is then even (odd for a negative direction)
+            // (as arithmetic, not a branch: one control path for every lane)
+            const int32_t crossed = cmp <= 0 ? (nx ^ qx) : (ny ^ qy);
+            const int32_t up = (level < mip_start ? 1 : 0) & ~crossed & 1;
+            level += up;
+            nx >>= up;
+            ny >>= up;
+            continue;
+        }
+        if (level > 0) {
+            // descend into the child that holds the ray just after t_in:
+            // the upper child on an axis when the ray has passed that
+            // axis' midline by t_in (for a negative direction, when not)
+            --level;
+            const int32_t xm = (2 * nx + 1) * (1 << level), ym = (2 * ny + 1) * (1 << level);
+            const int32_t midx = gx * (xm * (1 << kShift)) + kx;
+            const int64_t lx = (int64_t)midx * tin_den;
+            const int64_t rx = (int64_t)tin_num * adx;
+            const int64_t ly = (int64_t)(gy * (ym * (1 << kShift)) + ky) * tin_den;
+            const int64_t ry = (int64_t)tin_num * ady;
+            nx = 2 * nx + ((lx <= rx) != (gx < 0) ? 1 : 0);
+            ny = 2 * ny + ((ly <= ry) != (gy < 0) ? 1 : 0);
+            // a corner: the ray enters the cell through its Y side and an
+            // X cell boundary at the same instant; report the X face, and the
+            // time as that boundary's
+            if (lx == rx && adx != 0 && entry == face_y) {
+                entry = face_x;
+                tin_num = midx;
+                tin_den = adx;
+            }
+            continue;
+        }
+        // a non-empty cell holds the hit (the cell test is exact: the
+        // segment's z range meets (-inf, h0] or [h1, h2], and z is
+        // continuous along it): find its layer, face and time.
+        if (!leaf_test(r.oz, r.dz, word, tin_num, tin_den, tout_num, tout_den, entry, h)) {
+            h.face = kFaceError;  // unreachable: reported, never silent
+            h.layer = 255;
+            return;
+        }
+        h.cx = nx;
+        h.cy = ny;
+        h.word = word;
+        return;
+    }
+    h.face = kFaceError;
+    h.layer = 255;
+}
+
+// One ray of a beam: a ray with a horizontal component, whose axis of the
+// larger one (x on a tie) is u and whose other axis is v.  On an axis that the
+// ray descends along, cell index n becomes ~n, so it always moves toward larger
+// indices: a column (the cells of one u) is entered through its boundary u and
+// left through u + 1, and on its way the ray crosses at most one boundary of v.
+//
+// The direction's part of it is the same for all rays toward one sun.
+struct BeamDir {
+    int32_t key;       // bit 2: u is x; bits 1, 0: u, v mirrored
+    int32_t du, dv;    // |du|, |dv|
+    float rho, sigma;  // rise of v and of the height per column, to a relative 2^-23
+};
+struct BeamRay {
+    int32_t fu, fv;  // the start cell, mirrored
+    int32_t ku, kv;  // minus the start's mirrored position, in 2^-16 units
+    float z0;        // start height
+};
+
+// (dx, dy not both 0)
+HF_HD BeamDir beam_dir(int32_t dx, int32_t dy, int32_t dz) {
+    BeamDir d;
+    const int32_t ax = dx < 0 ? -dx : dx, ay = dy < 0 ? -dy : dy;
+    const bool x_major = ax >= ay;
+    const int32_t eu = x_major ? dx : dy, ev = x_major ? dy : dx;
+    d.du = x_major ? ax : ay;
+    d.dv = x_major ? ay : ax;
+    d.key = (x_major ? 4 : 0) | (eu < 0 ? 2 : 0) | (ev < 0 ? 1 : 0);
+    const float ru = cast_rcp((float)d.du);
+    d.rho = (float)d.dv * ru;
+    d.sigma = (float)dz * ru;
+    return d;
+}
+
+HF_HD BeamRay beam_ray(const BeamDir &d, const Ray &r) {
+    BeamRay q;
+    const int32_t ou = d.key & 4 ? r.ox : r.oy, ov = d.key & 4 ? r.oy : r.ox;
+    q.ku = d.key & 2 ? ou : -ou;
+    q.kv = d.key & 1 ? ov : -ov;
+    q.fu = (-q.ku) >> kShift;
+    q.fv = (-q.kv) >> kShift;
+    q.z0 = (float)r.oz * (1.0f / 65536.0f);
+    return q;
+}
+
+// A beam's rays, relative to the mirrored cell (u0, v0): at u = u0 + x every
+// ray has v - v0 in [a0 + r0 x, a1 + r1 x] and a height between b0 + s0 x and
+// b1 + s1 x, for x >= 0 (up to rounding, see beam_open).
+struct Beam {
+    int32_t u0, v0;
+    float a0, a1, r0, r1, b0, b1, s0, s1;
+};
+
+// A ray's start relative to the beam's cell: exact up to 256 cells, else
+// rounded.  At u0 + x the ray is at v - v0 = pv + rho (x - pu), and at the
+// height z0 + sigma (x - pu); its terms of the beam are those at x = 0.
+HF_HD float beam_pu(const BeamRay &q, const Beam &m) {
+    return (float)(-q.ku - m.u0 * (1 << kShift)) * (1.0f / 65536.0f);
+}
+HF_HD float beam_pv(const BeamRay &q, const Beam &m) {
+    return (float)(-q.kv - m.v0 * (1 << kShift)) * (1.0f / 65536.0f);
+}
+
+// A bound of the error of a beam's heights up to x columns on: slopes have a
+// relative error of 2^-23, and heights up to 4096 matter.
+HF_HD float beam_slack(const Beam &m, float x) {
+    return 0.02f + fmaxf(fabsf(m.s0), fabsf(m.s1)) * (fabsf(x) + 2.0f) * (1.0f / 1048576.0f);
+}
+
+// Whether the beam may meet a solid in mirrored columns [j 2^l, (j + 1) 2^l).
+// The rows it covers there are read as nodes of level l.
+template <bool PAIR>
+HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int key) {
+    const LevelDev lv = lvt[l];
+    const bool x_major = key & 4;
+    const uint32_t nu = x_major ? lv.stride : lv.rows, nv = x_major ? lv.rows : lv.stride;
+    const uint32_t ju = (uint32_t)(key & 2 ? ~j : j);
+    if (ju >= nu) return false;
+    const float x0 = (float)(j * (1 << l) - m.u0), x1 = x0 + (float)(1 << l);
+    const float zm = beam_slack(m, x1);
+    const float zlo = m.b0 + fminf(m.s0 * x0, m.s0 * x1) - zm;
+    const float zhi = m.b1 + fmaxf(m.s1 * x0, m.s1 * x1) + zm;
+    // (rows are off by less than 2^-6 at the largest grid)
+    const float vlo = m.a0 + fminf(m.r0 * x0, m.r1 * x0) - 0.015625f;
+    const float vhi = m.a1 + m.r1 * x1 + 0.015625f;
+    int32_t qa = (m.v0 + (int32_t)floorf(vlo)) >> l;
+    int32_t qb = (m.v0 + (int32_t)floorf(vhi)) >> l;
+    if (key & 1) {
+        const int32_t c = ~qa;
+        qa = ~qb;
+        qb = c;
+    }
+    qa = qa < 0 ? 0 : qa;
+    qb = qb < (int32_t)nv ? qb : (int32_t)nv - 1;
+    uint32_t top = 0, h0 = 0, h1 = 0xFF00;
+    for (int32_t jv = qa; jv <= qb; ++jv) {
+        const uint32_t w = cast_word<PAIR>(lv, l, (int32_t)(x_major ? ju : jv),
+                                           (int32_t)(x_major ? jv : ju)) & 0xFFFFFFu;
+        top = top > w ? top : w;
+        h0 = h0 > (w & 0xFF) ? h0 : (w & 0xFF);
+        h1 = h1 < (w & 0xFF00) ? h1 : (w & 0xFF00);
+    }
+    return !(zlo > (float)(top >> 16) || (zlo > (float)h0 && zhi < (float)(h1 >> 8)));
+}
+
+// A ray on its way through columns up to x1 (relative to the beam's cell).
+//
+// Rows: v is off by less than ev = (x1 + |pu| + |pv| + 1) 1.5 2^-22: rho by
+// 2^-23 of itself, x - pu and the sum by 2^-24, and |rho| <= 1.  Where v is
+// nearer than that to a boundary, the two are compared exactly; a ray through
+// the corner itself is left to cast_general.
+// Heights: off by less than e2 / 2 = (|sigma| (x1 + |pu| + 2) + |z0|) 2^-21.
+struct BeamWalk {
+    float pu, pv;
+    float ev, e2;
+    float zl;        // lower bound of the height where the column is entered
+    int32_t x, row;  // the column, and the row it is entered in
+    uint32_t cell;   // real index y W + x of that cell
+};
+
+enum { kBeamGoing = 0, kBeamOpen = 1, kBeamLeft = 2, kBeamCorner = 3 };
+
+// The row (relative to m.v0) of a ray as it enters column x of the beam, from
+// its v there.  False if it enters through a corner.
+HF_HD bool beam_row(const BeamDir &d, const BeamRay &q, const Beam &m, int32_t x, float v,
+                    float ev, int32_t &row) {
+    const float f = floorf(v);
+    row = (int32_t)f;
+    if (fabsf(v - f - 0.5f) < 0.5f - ev) return true;
+    // which of the ray's crossings of boundary row (the nearest) and of column
+    // x comes first
+    row = (int32_t)floorf(v + 0.5f);
+    const int64_t side = (int64_t)((m.v0 + row) * (1 << kShift) + q.kv) * d.du;
+    const int64_t here = (int64_t)((m.u0 + x) * (1 << kShift) + q.ku) * d.dv;
+    if (side > here) row -= 1;
+    return side != here;
+}
+
+// Places a ray at the mirrored column b0, or at its start if that lies beyond.
+// False if it enters through a corner.
+HF_HD bool beam_enter(const BeamDir &d, const BeamRay &q, const Beam &m, int32_t b0, int32_t b1,
+                      uint32_t W, BeamWalk &w) {
+    w.pu = beam_pu(q, m);
+    w.pv = beam_pv(q, m);
+    const float x1 = (float)(b1 - m.u0);
+    w.ev = (x1 + fabsf(w.pu) + fabsf(w.pv) + 1.0f) * (1.5f / 4194304.0f);
+    const float e = (fabsf(d.sigma) * (x1 + fabsf(w.pu) + 2.0f) + fabsf(q.z0)) * (1.0f / 2097152.0f);
+    w.e2 = 2.0f * e;
+    bool sure = true;
+    if (q.fu >= b0) {
+        w.x = q.fu - m.u0;
+        w.row = q.fv - m.v0;
+        w.zl = fabsf(q.z0) < 256.0f ? q.z0 : q.z0 - e;  // (a start below 256 is exact)
+    } else {
+        w.x = b0 - m.u0;
+        const float dx = (float)w.x - w.pu;
+        sure = beam_row(d, q, m, w.x, fmaf(d.rho, dx, w.pv), w.ev, w.row);
+        w.zl = fmaf(d.sigma, dx, q.z0) - e;
+    }
+    const int32_t u = m.u0 + w.x, v = m.v0 + w.row;
+    const uint32_t ru = (uint32_t)(d.key & 2 ? ~u : u), rv = (uint32_t)(d.key & 1 ? ~v : v);
+    w.cell = d.key & 4 ? rv * W + ru : ru * W + rv;
+    return sure;
+}
+
+// Word of cell index y W + x (pairs lie in one word: W is even).
+template <bool PAIR>
+HF_HD uint32_t beam_word(const uint32_t *cells, uint32_t cell) {
+    return PAIR ? pair_node(cast_load(cells + (cell >> 1)), cell & 1) : cast_load(cells + cell);
+}
+
+// Where a walk's column is left: the row, and a lower bound of the height.
+HF_HD bool beam_exit(const BeamDir &d, const BeamRay &q, const Beam &m, const BeamWalk &w,
+                     int32_t &row, float &zl) {
+    const float dx = (float)(w.x + 1) - w.pu;
+    zl = fmaf(d.sigma, dx, q.z0) - 0.5f * w.e2;
+    return beam_row(d, q, m, w.x + 1, fmaf(d.rho, dx, w.pv), w.ev, row);
+}
+
+HF_HD void beam_pass(BeamWalk &w, int32_t row, float zl, int32_t cell_u, int32_t cell_v) {
+    w.cell += (uint32_t)(cell_u + (row > w.row ? cell_v : 0));
+    w.x += 1;
+    w.row = row;
+    w.zl = zl;
+}
+
+// One column of a walk, whose one or two cells are tested together: past it if
+// they are empty (kBeamGoing).  kBeamOpen: they may not be; kBeamLeft: the ray
+// has left the grid sideways; kBeamCorner: it leaves through a corner.  rows:
+// the row past the grid.  cell_u, cell_v: what a step along u, v adds to the
+// cell index.
+template <bool PAIR>
+HF_HD int beam_step(const uint32_t *cells, const BeamDir &d, const BeamRay &q, const Beam &m,
+                    BeamWalk &w, int32_t rows, int32_t cell_u, int32_t cell_v) {
+    if (w.row >= rows) return kBeamLeft;
+    int32_t row;
+    float zl;
+    const bool sure = beam_exit(d, q, m, w, row, zl);
+    const uint32_t wa = beam_word<PAIR>(cells, w.cell);
+    const uint32_t wb = beam_word<PAIR>(
+        cells, w.cell + (uint32_t)(row > w.row && row < rows ? cell_v : 0));
+    const uint32_t ta = wa & 0xFF0000, tb = wb & 0xFF0000;
+    const uint32_t fa = wa & 0xFF, fb = wb & 0xFF, ma = wa & 0xFF00, mb = wb & 0xFF00;
+    const float top = (float)((ta > tb ? ta : tb) >> 16), h0 = (float)(fa > fb ? fa : fb);
+    const float h1 = (float)((ma < mb ? ma : mb) >> 8);
+    const float zlo = fminf(w.zl, zl), zhi = fmaxf(w.zl, zl) + w.e2;
+    if (!sure) return kBeamCorner;
+    if (!((zlo > top) | ((zlo > h0) & (zhi < h1)))) return kBeamOpen;
+    beam_pass(w, row, zl, cell_u, cell_v);
+    return kBeamGoing;
+}
+
+// Decides the column that beam_step left open, on exact rationals: true and h
+// filled, or false and the ray past it.
+template <bool PAIR>
+HF_HD bool beam_settle(const uint32_t *cells, int32_t oz, int32_t dz, const BeamDir &d,
+                       const BeamRay &q, const Beam &m, BeamWalk &w, int32_t rows, int32_t cell_u,
+                       int32_t cell_v, Hit &h) {
+    int32_t row;
+    float zl;
+    beam_exit(d, q, m, w, row, zl);
+    const bool x_major = d.key & 4;
+    const int32_t u = m.u0 + w.x;
+    const bool start = u == q.fu;
+    const int32_t end = (u + 1) * (1 << kShift) + q.ku;               // over du: the column's exit
+    const int32_t side = (m.v0 + w.row + 1) * (1 << kShift) + q.kv;   // over dv: the row's
+    int32_t num = start ? 0 : end - (1 << kShift), den = start ? 1 : d.du;
+    uint8_t face = start ? kFaceInside
+                   : x_major ? (d.key & 2 ? kFacePX : kFaceNX)
+                             : (d.key & 2 ? kFacePY : kFaceNY);
+    uint32_t cell = w.cell;
+    int32_t v = m.v0 + w.row;
+    for (bool second = false;; second = true) {
+        const bool last = second || row == w.row;
+        const uint32_t word = beam_word<PAIR>(cells, cell);
+        if (leaf_test(oz, dz, word, num, den, last ? end : side, last ? d.du : d.dv, face, h)) {
+            const int32_t ru = d.key & 2 ? ~u : u, rv = d.key & 1 ? ~v : v;
+            h.cx = x_major ? ru : rv;
+            h.cy = x_major ? rv : ru;
+            h.word = word;
+            return true;
+        }
+        if (last || row >= rows) break;
+        num = side;
+        den = d.dv;
+        face = x_major ? (d.key & 1 ? kFacePY : kFaceNY) : (d.key & 1 ? kFacePX : kFaceNX);
+        cell += (uint32_t)cell_v;
+        v += 1;
+    }
+    beam_pass(w, row, zl, cell_u, cell_v);
+    return false;
+}
+
+// The order in which a beam's columns are tested: rounds of 32 stretches of
+// 2^level columns.  A round that finds nothing is followed by one of longer
+// stretches, a long stretch that is open by a round of short ones from it on.
+// kBeamLevel: 2-cell stretches; kBeamTop: what an empty beam climbs to.
+// Open stretches that follow each other are walked as one.
+// Rays that start more than kBeamSpread cells apart (along v, where they pass
+// one column) are beams of their own.
+constexpr int kBeamLevel = 1, kBeamTop = 5;
+constexpr float kBeamSpread = 12.0f;
+
+// How many stretches make the run at the lowest bit of open (not 0), bit i.
+HF_HD int beam_run(uint32_t open, int i) {
+    const uint32_t rest = ~(open >> i);
+#ifdef __CUDA_ARCH__
+    return rest ? __ffs((int)rest) - 1 : 32;
+#else
+    return rest ? __builtin_ctz(rest) : 32;
+#endif
+}
+
+// The shortest stretches worth testing from u on: at least an eighth as long
+// as the beam is wide there, so that one covers few nodes.
+HF_HD int beam_least(const Beam &m, int32_t u, int base, int top) {
+    const float wide = (m.a1 - m.a0) + (m.r1 - m.r0) * (float)(u - m.u0 + 64);
+    int l = base;
+    while (l < top && wide > (float)(8 << l)) ++l;
+    return l;
+}
+
+// The first column to test, from u on: a beam that starts above every top
+// is empty until its lowest ray comes down to them; one that rises above them
+// is done (the limit is returned).  limit: the mirrored column past the grid.
+HF_HD int32_t beam_skip(const Beam &m, int32_t u, int32_t limit, float top) {
+    const float x0 = (float)(u - m.u0);
+    if (!(m.b0 + m.s0 * x0 - beam_slack(m, x0) > top)) return u;
+    if (m.s0 >= 0.0f) return limit;
+    // where the lowest line is 0.04 above the top: it falls by at most 4096 up
+    // to there, so it is off by less (and two columns are kept for a steep one)
+    const float x = (top + 0.04f - m.b0) / m.s0;
+    const float at = floorf(fminf(x, 40000.0f)) - 2.0f;
+    const int32_t c = m.u0 + (int32_t)at;
+    return c > u ? (c < limit ? c : limit) : u;
+}
+
+}  // namespace hf

@@ -62,9 +62,9 @@ constexpr uint32_t kSkyColour = 0xFFEBB487u;  // r 135, g 180, b 235, a 255
 constexpr int kMaxLevels = 14;  // 2^14 = 16384 = largest grid side
 constexpr int kShift = 16;      // 2^16 fixed-point units per world unit
 #ifndef HF_TRACE_THREADS
-#define HF_TRACE_THREADS 256  // measured: 128 / 256 / 512 (256: 0.4 % faster than 128)
+#define HF_TRACE_THREADS 128  // finer steps of registers per thread than 256 (see hf_trace.cu)
 #endif
-constexpr int kThreads = HF_TRACE_THREADS;  // threads per trace block (8 warps)
+constexpr int kThreads = HF_TRACE_THREADS;  // threads per trace block
 constexpr uint32_t kMaxCams = 4096;
 constexpr uint32_t kDefaultMipStart = 6;  // coarsest level used when the caller asks for the default
 #ifndef HF_SHADOW_MIP_EXTRA
@@ -186,14 +186,16 @@ int launch_voxel_trace(const RenderParams &p, const VoxelDev &v, const VoxelPara
                        uint32_t n_cams, uint32_t max_pixels, void *stream);
 
 // Launch wrappers (hf_trace.cu)
+// How the trace kernels follow rays: warps of rays in beams; one ray at a time
+// (a step limit set by the caller: p.max_steps); the same with fetch counters.
+enum TraceKind { kTraceBeams = 0, kTraceGeneral = 1, kTraceStats = 2, kTraceKinds = 3 };
 // The trace kernels are instantiated per level-0 storage; p.world.pair picks one.
-int launch_trace_batched(const RenderParams &p, bool shadows, bool stats, int blocks,
-                         void *stream);
+int launch_trace_batched(const RenderParams &p, bool shadows, int kind, int blocks, void *stream);
 // (the plain kernel takes its camera record as a launch parameter)
-int launch_trace_plain(const RenderParams &p, bool shadows, bool stats, const CamDev &cam,
+int launch_trace_plain(const RenderParams &p, bool shadows, int kind, const CamDev &cam,
                        uint32_t n_tiles, void *stream);
-const void *trace_batched_fn(bool shadows, bool stats, bool pair);
-int trace_batched_occupancy(bool shadows, bool stats, bool pair, int *blocks_per_sm);
+const void *trace_batched_fn(bool shadows, int kind, bool pair);
+int trace_batched_occupancy(bool shadows, int kind, bool pair, int *blocks_per_sm);
 
 // What the allocation-free render needs to know about a context (hf_api.cpp).
 struct CtxView {
@@ -201,7 +203,7 @@ struct CtxView {
     void *stream;
     int device;
     int sm_count;
-    int occ_shadows[2];  // batched-kernel blocks per SM without / with shadow rays
+    int occ[2][kTraceKinds];  // batched-kernel blocks per SM, [with shadow rays][kind]
 };
 int ctx_view(const ::hf_ctx *ctx, CtxView *out);
 

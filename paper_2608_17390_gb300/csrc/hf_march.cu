@@ -18,6 +18,8 @@
 namespace hf {
 namespace {
 
+constexpr int kMarchThreads = 256;
+
 struct MarchPoint {
     bool solid;
     int32_t cx, cy;
@@ -112,10 +114,10 @@ __device__ __forceinline__ const CamDev &stage(CamDev *slot, const CamDev *cams,
 }
 
 // Persistent: warps pop (camera, tile) items from the batch's atomic counter.
-__global__ void __launch_bounds__(kThreads) k_march_batched(const RenderParams p,
+__global__ void __launch_bounds__(kMarchThreads) k_march_batched(const RenderParams p,
                                                             const MarchParams m) {
     __shared__ uint32_t s_base[kMaxCams + 1];
-    __shared__ CamDev s_cam[kThreads / 32];
+    __shared__ CamDev s_cam[kMarchThreads / 32];
     const uint32_t n = p.hdr->n_cams;
     const uint32_t total = p.hdr->total_tiles;
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) s_base[i] = p.cams[i].tile_base;
@@ -148,13 +150,13 @@ __global__ void __launch_bounds__(kThreads) k_march_batched(const RenderParams p
 }  // namespace
 
 int launch_march_batched(const RenderParams &p, const MarchParams &m, int blocks, void *stream) {
-    k_march_batched<<<blocks, kThreads, 0, (cudaStream_t)stream>>>(p, m);
+    k_march_batched<<<blocks, kMarchThreads, 0, (cudaStream_t)stream>>>(p, m);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int march_occupancy(int *blocks_per_sm) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-               blocks_per_sm, reinterpret_cast<const void *>(&k_march_batched), kThreads, 0) ==
+               blocks_per_sm, reinterpret_cast<const void *>(&k_march_batched), kMarchThreads, 0) ==
                    cudaSuccess
                ? 0
                : -1;

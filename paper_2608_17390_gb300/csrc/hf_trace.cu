@@ -1,22 +1,17 @@
 // hf_trace.cu -- per-pixel exact ray casting through a two-interval height field.
 //
-// One warp owns one tile of tile_w x tile_h pixels; each lane traces the
-// tile's pixels lane, lane+32, ...  Every branch of the traversal is decided
-// with exact integer arithmetic on 32-bit operands and 64-bit products, so hit
-// cell, layer and face equal the definition bit for bit:
+// One warp owns one tile of tile_w x tile_h pixels; lane l takes the tile's
+// pixels l, l + 32, ...  The hit cell, layer and face of every ray equal the
+// definition bit for bit:
 //
 //   * ray generation: d = F + (2px+1-w) R + (h-1-2py) U (int32, bounded < 2^21);
-//   * times are rationals num/den with 0 <= num <= 2^30 and 0 < den < 2^21;
-//   * "z(t) vs h S" is the sign of (oz - hS) den + num dz (|.| < 2^52);
-//   * hierarchical DDA over the min/max pyramid: a node whose ray segment lies
-//     above its highest top, or above every floor and below every slab
-//     underside, is skipped to its exit (the hierarchy may only skip
-//     known-empty space, Section 3.2 of the paper); otherwise the traversal
-//     descends; at level 0 the cell's two solid intervals are tested (the
-//     SOLID predicate of Section 3.1, closed ends, floor unbounded below);
-//   * a skip changes only the node index on the exit axis; the finer bits of
-//     the other axis are recovered on descent by exact midline tests (no
-//     division);
+//   * the 32 rays of a warp are cast together, in beams (cast_beams): floats
+//     with error bounds prove space empty (the hierarchy may only skip
+//     known-empty space, Section 3.2 of the paper), and what they leave open is
+//     decided in exact integer arithmetic (hf_cast.h): the SOLID predicate of
+//     Section 3.1, closed ends, floor unbounded below;
+//   * renders with a step limit of the caller's, or with fetch counters, follow
+//     each ray by itself (cast_general);
 //   * a shadow ray starts at the floor of the hit point (an exact floor
 //     division: a float estimate and one integer correction), one fixed-point
 //     unit outward along the face normal.
@@ -27,45 +22,19 @@
 #include <mutex>
 
 #include "hf.h"
+#include "hf_cast.h"
 #include "hf_internal.h"
 
 namespace hf {
 namespace {
 
 #ifndef HF_TRACE_MIN_BLOCKS
-#define HF_TRACE_MIN_BLOCKS 3  // resident 256-thread blocks per SM asked of the register allocator (<= 85 registers)
+#define HF_TRACE_MIN_BLOCKS 7  // resident 128-thread blocks per SM asked of the register allocator (72 registers)
 #endif
 
 __constant__ float c_albedo[8][3] = HF_ALBEDO_TABLE;
 constexpr float kKa = kAmbient, kKd = kDiffuse;
 constexpr uint32_t kSky = kSkyColour;
-
-struct Ray {
-    int32_t ox, oy, oz, dx, dy, dz;
-};
-
-// One pyramid level as the traversal reads it (a per-block shared table, so
-// lanes at different levels read it in one shared-memory access).
-struct LevelDev {
-    const uint32_t *base;
-    uint32_t stride, rows;
-};
-
-struct Hit {
-    int32_t cx, cy;
-    int32_t tnum, tden;  // hit time tnum / tden
-    uint32_t word;       // hit cell word
-    uint8_t layer, face;
-};
-
-struct Counters {
-    uint32_t nodes, cells;
-};
-
-// sign carrier of z(t) - h S for t = num / den (den > 0):  (oz - hS) den + num dz
-__device__ __forceinline__ int64_t zd(int32_t oz_minus_hs, int32_t dz, int32_t num, int32_t den) {
-    return (int64_t)oz_minus_hs * den + (int64_t)num * dz;
-}
 
 // int64 -> float through two 32-bit conversions (64-bit integer conversions
 // run on the FP64 pipe, which is narrow on this GPU).  |v| < 2^52.
@@ -99,252 +68,6 @@ __device__ __forceinline__ uint32_t level0_word(const WorldDev &w, int32_t x, in
     return load_word(w, 0, x, y);
 }
 
-// The two-interval test of one cell over [tin, tout] (tout finite).
-// Returns true and fills h on a hit.
-__device__ __forceinline__ bool leaf_test(const Ray &r, uint32_t word, int32_t tin_num,
-                                          int32_t tin_den, int32_t tout_num, int32_t tout_den,
-                                          uint8_t entry_face, Hit &h) {
-    const int32_t h0 = word & 0xFF, h1 = (word >> 8) & 0xFF, h2 = (word >> 16) & 0xFF;
-    const bool slab = h2 > h0;  // level-0 words are in node form
-    const int32_t a0 = r.oz - (h0 << kShift);
-    const int64_t zin0 = zd(a0, r.dz, tin_num, tin_den);
-    if (zin0 <= 0) {
-        h.layer = 0;
-        h.face = entry_face;
-        h.tnum = tin_num;
-        h.tden = tin_den;
-        return true;
-    }
-    const int32_t a1 = r.oz - (h1 << kShift), a2 = r.oz - (h2 << kShift);
-    int64_t zin1 = 0, zin2 = 0;
-    if (slab) {
-        zin1 = zd(a1, r.dz, tin_num, tin_den);
-        zin2 = zd(a2, r.dz, tin_num, tin_den);
-        if (zin1 >= 0 && zin2 <= 0) {
-            h.layer = 1;
-            h.face = entry_face;
-            h.tnum = tin_num;
-            h.tden = tin_den;
-            return true;
-        }
-    }
-    if (r.dz < 0) {
-        if (slab && zin2 > 0 && zd(a2, r.dz, tout_num, tout_den) <= 0) {
-            h.layer = 1;
-            h.face = kFacePZ;
-            h.tnum = a2;
-            h.tden = -r.dz;
-            return true;
-        }
-        if (zd(a0, r.dz, tout_num, tout_den) <= 0) {
-            h.layer = 0;
-            h.face = kFacePZ;
-            h.tnum = a0;
-            h.tden = -r.dz;
-            return true;
-        }
-    } else if (r.dz > 0) {
-        if (slab && zin1 < 0 && zd(a1, r.dz, tout_num, tout_den) >= 0) {
-            h.layer = 1;
-            h.face = kFaceNZ;
-            h.tnum = -a1;
-            h.tden = r.dz;
-            return true;
-        }
-    }
-    return false;
-}
-
-// A vertical ray (dx = dy = 0) stays in its start column for all t >= 0.
-// Writes h only when the ray hits.
-__device__ __forceinline__ bool vertical_test(const Ray &r, uint32_t word, Hit &h) {
-    const int32_t h0 = word & 0xFF, h1 = (word >> 8) & 0xFF, h2 = (word >> 16) & 0xFF;
-    const bool slab = h2 > h0;  // level-0 words are in node form
-    const int32_t a0 = r.oz - (h0 << kShift), a1 = r.oz - (h1 << kShift),
-                  a2 = r.oz - (h2 << kShift);
-    uint8_t layer, face;
-    int32_t tnum = 0, tden = 1;
-    if (a0 <= 0) {
-        layer = 0;
-        face = kFaceInside;
-    } else if (slab && a1 >= 0 && a2 <= 0) {
-        layer = 1;
-        face = kFaceInside;
-    } else if (r.dz < 0) {
-        face = kFacePZ;
-        tden = -r.dz;
-        layer = (slab && a2 > 0) ? 1 : 0;
-        tnum = layer ? a2 : a0;
-    } else if (r.dz > 0 && slab && a1 < 0) {
-        layer = 1;
-        face = kFaceNZ;
-        tnum = -a1;
-        tden = r.dz;
-    } else {
-        return false;
-    }
-    h.layer = layer;
-    h.face = face;
-    h.tnum = tnum;
-    h.tden = tden;
-    return true;
-}
-
-// Exact first hit of one ray.  h.face = kFaceMiss on a miss, kFaceError when
-// max_steps iterations did not finish the ray.
-//
-// State: the node (nx, ny) at `level` that holds the ray just after t_in.
-// Skipping an empty node changes only the node index on the exit axis; the
-// finer bits on the other axis are found when the traversal descends, by
-// asking whether the ray has crossed the child midline by t_in (exact
-// cross-multiplied time comparison).  Every interior cell boundary of a node
-// is the midline of exactly one sub-level, so a ray that enters a cell through
-// its Y side while also crossing an X cell boundary (a corner) is detected on
-// the way down and reported with the X face.
-// EMPTY_FIRST picks the order of the two outcomes of the node test in the
-// code (empty: advance; else descend or hit); which order runs faster depends
-// on the kernel (measured: empty first with shadow rays, the other without).
-template <bool STATS, bool PAIR, bool EMPTY_FIRST>
-__device__ __forceinline__ void trace_ray(const WorldDev &w, const LevelDev *lvt, const Ray &r,
-                                          int start_level, int mip_start, int max_steps, Hit &h,
-                                          Counters &cnt) {
-    h.face = kFaceMiss;
-    h.layer = 255;
-    const int32_t adx = abs(r.dx), ady = abs(r.dy);
-    int32_t cx = r.ox >> kShift, cy = r.oy >> kShift;
-    if (r.dx < 0 && (r.ox & 0xFFFF) == 0) cx -= 1;
-    if (r.dy < 0 && (r.oy & 0xFFFF) == 0) cy -= 1;
-    if ((uint32_t)cx >= (uint32_t)w.W || (uint32_t)cy >= (uint32_t)w.H) return;
-
-    if (adx == 0 && ady == 0) {
-        const uint32_t word = level0_word<PAIR>(w, cx, cy);
-        if (STATS) cnt.cells++;
-        if (vertical_test(r, word, h)) {
-            h.cx = cx;
-            h.cy = cy;
-            h.word = word;
-        }
-        return;
-    }
-
-    // Per-ray sign constants.  A zero direction component counts as positive:
-    // its exit distance is then positive and never the smaller one, so the
-    // ray never leaves through that axis.
-    const int32_t gx = r.dx < 0 ? -1 : 1, gy = r.dy < 0 ? -1 : 1;  // step per exit
-    const int32_t px = r.dx < 0 ? 0 : 1, py = r.dy < 0 ? 0 : 1;    // exit side offset
-    const int32_t qx = px ^ 1, qy = py ^ 1;
-    const int32_t kx = -gx * r.ox, ky = -gy * r.oy;
-    const uint8_t face_x = r.dx < 0 ? kFacePX : kFaceNX;  // entry face of an x crossing
-    const uint8_t face_y = r.dy < 0 ? kFacePY : kFaceNY;
-    int level = start_level;  // <= mip_start, the coarsest level the ray climbs to
-    int32_t nx = cx >> level, ny = cy >> level;
-    int32_t tin_num = 0, tin_den = 1;
-    uint8_t entry = kFaceInside;
-
-
-    for (int it = 0;; ++it) {
-        // one bounds check per iteration, after every advance, ascent or
-        // descent: an index past the level's end, or below 0, means the ray
-        // has left the grid.  An ascent keeps the crossed axis out of range
-        // (it follows a step onto an even index n >= ceil(E / 2^l), so
-        // n / 2 >= ceil(E / 2^(l+1)); or onto -1, and -1 >> 1 = -1).  At an
-        // exact corner the other axis may come back in range, in a partial
-        // node past the grid's edge; the ray only moves further out, and a
-        // descent there lands on an out-of-range child, so it still misses.
-        // A ray that leaves on its last allowed iteration is a miss, not a
-        // step-limit error.
-        const LevelDev lv = lvt[level];
-        if ((uint32_t)nx >= lv.stride || (uint32_t)ny >= lv.rows) return;
-        if (it == max_steps) break;
-        const int32_t bx = (nx + px) << level;  // exit boundary (cells)
-        const int32_t by = (ny + py) << level;
-        const int32_t numx = gx * (bx << kShift) + kx;  // > 0
-        const int32_t numy = gy * (by << kShift) + ky;
-        const int64_t cmp = (int64_t)numx * ady - (int64_t)numy * adx;  // < 0: x exits first
-        const bool xfirst = cmp <= 0;
-        const int32_t tout_num = xfirst ? numx : numy;
-        const int32_t tout_den = xfirst ? adx : ady;
-        // level 0 holds cells in node form, so one word layout serves every
-        // level; for a single cell the emptiness test below is exact (the
-        // segment's z range [zlo, zhi] misses (-inf, h0] and [h1, h2] exactly
-        // when zlo > top, or zlo > h0 and zhi < h1)
-        const uint32_t word =
-            PAIR && level == 0
-                ? pair_node(__ldg(lv.base + (uint32_t)ny * (lv.stride >> 1) + ((uint32_t)nx >> 1)),
-                            (uint32_t)nx & 1)
-                : __ldg(lv.base + (uint32_t)ny * lv.stride + (uint32_t)nx);
-        const uint32_t node = word;
-        if (STATS) {
-            if (level > 0) cnt.nodes++;
-            else cnt.cells++;
-        }
-        const int32_t maxh0 = node & 0xFF, minh1 = (node >> 8) & 0xFF,
-                      maxtop = (node >> 16) & 0xFF;
-        const bool down = r.dz < 0;
-        const int32_t lo_num = down ? tout_num : tin_num, lo_den = down ? tout_den : tin_den;
-        const int32_t hi_num = down ? tin_num : tout_num, hi_den = down ? tin_den : tout_den;
-        const bool empty = zd(r.oz - (maxtop << kShift), r.dz, lo_num, lo_den) > 0 ||
-                           (zd(r.oz - (maxh0 << kShift), r.dz, lo_num, lo_den) > 0 &&
-                            zd(r.oz - (minh1 << kShift), r.dz, hi_num, hi_den) < 0);
-        // advance past the node (or cell) through its exit side; at an exact
-        // corner both indices change and the X face is reported
-        auto advance = [&]() {
-            if (cmp <= 0) nx += gx;
-            if (cmp >= 0) ny += gy;
-            entry = cmp <= 0 ? face_x : face_y;
-            tin_num = tout_num;
-            tin_den = tout_den;
-            // ascend when the crossed boundary is a parent boundary: the new index
-            // on the crossed axis is then even (odd for a negative direction)
-            // (as arithmetic, not a branch: one control path for every lane)
-            const int32_t crossed = cmp <= 0 ? (nx ^ qx) : (ny ^ qy);
-            const int32_t up = (level < mip_start ? 1 : 0) & ~crossed & 1;
-            level += up;
-            nx >>= up;
-            ny >>= up;
-        };
-        if (EMPTY_FIRST && empty) {
-            advance();
-            continue;
-        }
-        if (EMPTY_FIRST || !empty) {
-            if (level > 0) {
-                // descend into the child that holds the ray just after t_in:
-                // the upper child on an axis when the ray has passed that
-                // axis' midline by t_in (for a negative direction, when not)
-                --level;
-                const int32_t xm = (2 * nx + 1) << level, ym = (2 * ny + 1) << level;
-                const int64_t lx = (int64_t)(gx * (xm << kShift) + kx) * tin_den;
-                const int64_t rx = (int64_t)tin_num * adx;
-                const int64_t ly = (int64_t)(gy * (ym << kShift) + ky) * tin_den;
-                const int64_t ry = (int64_t)tin_num * ady;
-                nx = 2 * nx + ((lx <= rx) != (gx < 0) ? 1 : 0);
-                ny = 2 * ny + ((ly <= ry) != (gy < 0) ? 1 : 0);
-                // a corner: the ray enters the cell through its Y side and an
-                // X cell boundary at the same instant; report the X face
-                if (lx == rx && adx != 0 && entry == face_y) entry = face_x;
-                continue;
-            }
-            // a non-empty cell holds the hit (the cell test is exact: the
-            // segment's z range meets (-inf, h0] or [h1, h2], and z is
-            // continuous along it): find its layer, face and time.  The
-            // advance is reached from empty nodes and cells only.
-            if (!leaf_test(r, word, tin_num, tin_den, tout_num, tout_den, entry, h)) {
-                h.face = kFaceError;  // unreachable: reported, never silent
-                h.layer = 255;
-                return;
-            }
-            h.cx = nx;
-            h.cy = ny;
-            h.word = word;
-            return;
-        }
-        advance();
-    }
-    h.face = kFaceError;
-    h.layer = 255;
-}
-
 __device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visible,
                                           const float *ln) {
     float ndl;
@@ -368,30 +91,149 @@ __device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visi
     return out;
 }
 
-// Writes one pixel's outputs.
-__device__ __forceinline__ void store_pixel(const RenderParams &p, const CamDev &c, uint32_t pix,
-                                            const Hit &ph, float depth, bool visible,
-                                            bool shadows) {
-    const bool hit = ph.face < kFaceError;
-    if (shadows && c.shadow) __stcs(c.shadow + pix, (uint8_t)(visible ? 0 : 1));
-    if (c.hit_cell)
-        __stcs(c.hit_cell + pix,
-               hit ? (uint32_t)ph.cy * (uint32_t)p.world.W + (uint32_t)ph.cx : 0xFFFFFFFFu);
-    if (c.layer) __stcs(c.layer + pix, hit ? ph.layer : (uint8_t)255);
-    if (c.face) __stcs(c.face + pix, ph.face);
-    if (c.depth) __stcs(c.depth + pix, depth);
-    if (c.rgba) __stcs(c.rgba + pix, hit ? shade(ph.word, ph.face, visible, p.sun_n) : kSky);
+constexpr uint32_t kFull = 0xFFFFFFFFu;
+
+__device__ __forceinline__ float warp_min(float v) {
+    float r;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float warp_max(float v) {
+    float r;
+    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
-// One pixel: its primary ray, then (with shadows) the shadow ray, which
-// reuses the same traversal loop and registers.
-template <bool SHADOWS, bool STATS, bool PAIR>
-__device__ __forceinline__ void trace_pixel(const RenderParams &p, const LevelDev *lvt,
-                                            const CamDev &c, int start,
-                                            int32_t px, int32_t py, Counters &cnt,
-                                            Counters &scnt, uint32_t &nshadow, bool &err) {
+// Casts one ray per active lane; every lane of the warp calls.
+//
+// The rays that go the same way (axis of the larger component and both signs)
+// and start side by side form a beam.  Its 32 next stretches of columns are
+// tested by the 32 lanes at once, each against the one to three nodes that the
+// beam covers there; then the rays are walked, all together, through the
+// stretches that are not proven empty until they have hit or left.  One ray at
+// a time, the same empty space costs every lane 15 to 25 dependent node visits;
+// here it costs the warp one or two rounds.
+//
+// Bound by instruction issue, as the traversal of single rays was: 2048 x 2048
+// grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 10.03
+// ms, a 1080p eye-level view with shadows 192 -> 134 us, a hundred 1080p frames
+// over 2048 x 16384 cells 17.3 -> 10.4 ms.
+template <bool PAIR>
+__device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev *lvt,
+                                           const Ray &r, const BeamDir &d, bool active, int mip,
+                                           Hit &h) {
+    h.face = kFaceMiss;
+    h.layer = 255;
+    const uint32_t W = (uint32_t)p.world.W, H = (uint32_t)p.world.H;
+    const uint32_t *cells = p.world.base;
+    const int lane = threadIdx.x & 31;
+    const BeamRay q = beam_ray(d, r);
+    // rays that no beam takes: vertical ones, and (below) through corners
+    bool alone = active && (r.dx | r.dy) == 0;
+    active = active && !alone && (uint32_t)(d.key & 2 ? ~q.fu : q.fu) < (d.key & 4 ? W : H) &&
+             (uint32_t)(d.key & 1 ? ~q.fv : q.fv) < (d.key & 4 ? H : W);
+    uint32_t todo = __ballot_sync(kFull, active);
+    const int base_level = min(kBeamLevel, mip), top_level = min(kBeamTop, mip);
+    while (todo) {
+        // the first ray left, and the rays that go its way beside it
+        const int lead = __ffs(todo) - 1;
+        const int key = __shfl_sync(kFull, d.key, lead);
+        Beam m;
+        m.u0 = __shfl_sync(kFull, q.fu, lead);
+        m.v0 = __shfl_sync(kFull, q.fv, lead);
+        bool alive = (todo >> lane & 1) && d.key == key &&
+                     fabsf(beam_pv(q, m) - d.rho * beam_pu(q, m)) <= kBeamSpread;
+        todo &= ~__ballot_sync(kFull, alive);
+        m.u0 = __reduce_min_sync(kFull, alive ? q.fu : 0x7FFFFFFF);
+        const int32_t limit = key & 2 ? 0 : (int32_t)(key & 4 ? W : H);
+        const int32_t rows = (key & 1 ? 0 : (int32_t)(key & 4 ? H : W)) - m.v0;
+        const int32_t cell_u = (key & 2 ? -1 : 1) * (key & 4 ? 1 : (int32_t)W);
+        const int32_t cell_v = (key & 1 ? -1 : 1) * (key & 4 ? (int32_t)W : 1);
+        const float top = (float)((cast_load(lvt[p.world.L].base) >> 16) & 0xFF);
+        int32_t u = m.u0;
+        int level = base_level;
+        while (u < limit) {
+            {  // the beam of the rays that are left
+                const float big = 3.0e38f, pu = beam_pu(q, m);
+                const float a = beam_pv(q, m) - d.rho * pu, b = q.z0 - d.sigma * pu;
+                m.a0 = warp_min(alive ? a : big);
+                m.a1 = warp_max(alive ? a : -big);
+                m.r0 = warp_min(alive ? d.rho : big);
+                m.r1 = warp_max(alive ? d.rho : -big);
+                m.b0 = warp_min(alive ? b : big);
+                m.b1 = warp_max(alive ? b : -big);
+                m.s0 = warp_min(alive ? d.sigma : big);
+                m.s1 = warp_max(alive ? d.sigma : -big);
+            }
+            u = beam_skip(m, u, limit, top);
+            if (u >= limit) break;
+            const int least = beam_least(m, u, base_level, top_level);
+            level = max(level, least);
+            const int32_t j = u >> level;
+            uint32_t open = __ballot_sync(kFull, beam_open<PAIR>(lvt, m, level, j + lane, key));
+            if (level > least && open) {
+                u = max(u, (j + __ffs(open) - 1) * (1 << level));
+                level = least;
+                continue;
+            }
+            const int32_t next = (j + 32) * (1 << level);
+            if (!open) {
+                u = next;
+                level = min(level + 2, top_level);
+                continue;
+            }
+            do {
+                const int i = __ffs(open) - 1, run = beam_run(open, i);
+                open &= i + run < 32 ? 0xFFFFFFFFu << (i + run) : 0u;
+                const int32_t b0 = max(u, (j + i) * (1 << level));
+                const int32_t b1 = min((j + i + run) * (1 << level), limit);
+                bool go = alive && q.fu < b1;
+                BeamWalk w;
+                if (go && !beam_enter(d, q, m, b0, b1, W, w)) {
+                    alone = true;
+                    go = alive = false;
+                }
+                while (__any_sync(kFull, go)) {
+                    int at = kBeamGoing;
+                    do {
+                        if (go) {
+                            at = beam_step<PAIR>(cells, d, q, m, w, rows, cell_u, cell_v);
+                            go = at == kBeamGoing && w.x < b1 - m.u0;
+                        }
+                    } while (__any_sync(kFull, go));
+                    if (at == kBeamOpen) {
+                        alive = !beam_settle<PAIR>(cells, r.oz, r.dz, d, q, m, w, rows, cell_u,
+                                                   cell_v, h);
+                        go = alive && w.x < b1 - m.u0;
+                    } else if (at != kBeamGoing) {
+                        alive = false;
+                        alone = at == kBeamCorner;
+                    }
+                }
+            } while (open && __any_sync(kFull, alive));
+            if (!__any_sync(kFull, alive)) break;
+            u = next;
+        }
+    }
+    if (alone) {
+        Counters none{0, 0};
+        const int level = min(kBeamLevel, mip);
+        cast_general<false, PAIR>(lvt, r, level, mip, 0x7FFFFFFF, h, none);
+    }
+}
+
+// One pixel per lane: its primary ray, then (with shadows) the shadow ray, in
+// a second pass of the same traversal code.  Every lane of the warp calls;
+// `inside` says whether the lane has a pixel.
+template <bool SHADOWS, int KIND, bool PAIR>
+__device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelDev *lvt,
+                                             const CamDev &c, int start, int32_t px, int32_t py,
+                                             bool inside, const BeamDir &sun, Counters &cnt,
+                                             Counters &scnt, uint32_t &nshadow, bool &err) {
+    constexpr bool STATS = KIND == kTraceStats;
     const int32_t a = 2 * px + 1 - (int32_t)c.w;
     const int32_t b = (int32_t)c.h - 1 - 2 * py;
+    const uint32_t pix = (uint32_t)py * c.w + (uint32_t)px;
     Ray r;
     r.ox = c.o[0];
     r.oy = c.o[1];
@@ -399,79 +241,104 @@ __device__ __forceinline__ void trace_pixel(const RenderParams &p, const LevelDe
     r.dx = c.F[0] + a * c.R[0] + b * c.U[0];
     r.dy = c.F[1] + a * c.R[1] + b * c.U[1];
     r.dz = c.F[2] + a * c.R[2] + b * c.U[2];
-    Hit ph;  // primary hit, kept while the shadow ray runs
-    float depth = __int_as_float(0x7f800000);
+    uint32_t word = 0;  // of the primary hit, with its face: for the shading
+    uint8_t face = kFaceMiss;
     bool visible = true;
-    bool shadow_pass = false;
-    for (;;) {
+    bool cast = inside;  // this lane's ray of the pass
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+        const bool sp = SHADOWS && pass;
         Hit h;
-        // one call site: lanes in the primary and in the shadow pass run the
-        // same traversal code together
-        const bool sp = SHADOWS && shadow_pass;
         Counters pc{0, 0};
-        trace_ray<STATS, PAIR, SHADOWS>(p.world, lvt, r, sp ? min(kShadowStart, p.shadow_mip) : start,
-                               sp ? p.shadow_mip : p.mip_start, p.max_steps, h, pc);
+        if (KIND == kTraceBeams) {
+            const BeamDir d = sp ? sun : beam_dir(r.dx, r.dy, r.dz);
+            cast_beams<PAIR>(p, lvt, r, d, cast, sp ? p.shadow_mip : p.mip_start, h);
+        } else {
+            h.face = kFaceMiss;
+            h.layer = 255;
+            if (cast)
+                cast_general<STATS, PAIR>(lvt, r, sp ? min(kShadowStart, p.shadow_mip) : start,
+                                          sp ? p.shadow_mip : p.mip_start, p.max_steps, h, pc);
+        }
         if (STATS) {
             Counters &dst = sp ? scnt : cnt;
             dst.nodes += pc.nodes;
             dst.cells += pc.cells;
         }
-        if (h.face == kFaceError) err = true;
-        if (SHADOWS && shadow_pass) {
-            visible = h.face == kFaceMiss;
+        if (KIND != kTraceBeams && cast && h.face == kFaceError) err = true;
+        if (sp) {
+            if (cast) visible = h.face == kFaceMiss;
             break;
         }
-        ph = h;
+        cast = false;
         const bool hit = h.face < kFaceError;
-        if (hit) {
-            const float fx = (float)r.dx, fy = (float)r.dy, fz = (float)r.dz;
-            depth = ((float)h.tnum / (float)h.tden) * sqrtf(fx * fx + fy * fy + fz * fz) *
-                    (1.0f / 65536.0f);
-        }
-        if (!SHADOWS || !hit) break;
-        if (h.face == kFaceInside) {
-            visible = false;
-            break;
-        }
-        // shadow ray: floor of the hit point, one unit outward along the face normal
-        const float rcp_t = 1.0f / (float)h.tden;
-        int32_t sxp = r.ox + floor_div_small((int64_t)h.tnum * r.dx, h.tden, rcp_t);
-        int32_t syp = r.oy + floor_div_small((int64_t)h.tnum * r.dy, h.tden, rcp_t);
-        int32_t szp = r.oz + floor_div_small((int64_t)h.tnum * r.dz, h.tden, rcp_t);
-        switch (h.face) {
-            case kFaceNX: sxp -= 1; break;
-            case kFacePX: sxp += 1; break;
-            case kFaceNY: syp -= 1; break;
-            case kFacePY: syp += 1; break;
-            case kFaceNZ: szp -= 1; break;
-            default: szp += 1; break;
-        }
-        if (STATS) nshadow++;
-        if (p.sun_bounds) {
-            // the start cell's proven bounds decide most shadow rays at once:
-            // at or below F occluded, at or above G lit (hf_sun.cu)
-            int32_t bx = sxp >> kShift, by = syp >> kShift;
-            if (p.sun[0] < 0 && (sxp & 0xFFFF) == 0) bx -= 1;
-            if (p.sun[1] < 0 && (syp & 0xFFFF) == 0) by -= 1;
-            if ((uint32_t)bx < (uint32_t)p.world.W && (uint32_t)by < (uint32_t)p.world.H) {
-                const uint32_t fg = __ldg(p.sun_bounds + (uint32_t)by * (uint32_t)p.world.W + (uint32_t)bx);
-                if (STATS) scnt.cells++;
-                if (szp <= (int32_t)((fg & 0xFFFFu) << 8)) {
-                    visible = false;
-                    break;
-                }
-                if (szp >= (int32_t)((fg >> 16) << 8)) break;
+        if (inside) {
+            word = h.word;
+            face = h.face;
+            float depth = __int_as_float(0x7f800000);
+            if (hit) {
+                const float fx = (float)r.dx, fy = (float)r.dy, fz = (float)r.dz;
+                depth = ((float)h.tnum / (float)h.tden) * sqrtf(fx * fx + fy * fy + fz * fz) *
+                        (1.0f / 65536.0f);
             }
+            if (c.hit_cell)
+                __stcs(c.hit_cell + pix, hit ? (uint32_t)h.cy * (uint32_t)p.world.W + (uint32_t)h.cx
+                                             : 0xFFFFFFFFu);
+            if (c.layer) __stcs(c.layer + pix, hit ? h.layer : (uint8_t)255);
+            if (c.face) __stcs(c.face + pix, face);
+            if (c.depth) __stcs(c.depth + pix, depth);
         }
-        r.ox = sxp;
-        r.oy = syp;
-        r.oz = szp;
-        r.dx = p.sun[0];
-        r.dy = p.sun[1];
-        r.dz = p.sun[2];
-        shadow_pass = true;
+        if (!SHADOWS) break;
+        if (inside && h.face == kFaceInside) {
+            visible = false;
+        } else if (inside && hit) {
+            // shadow ray: floor of the hit point, one unit outward along the
+            // face normal.  The coordinate along the normal is exact: the ray
+            // crosses that axis by tnum (its |d| is tden); the other two are
+            // floored quotients.
+            const bool on_x = face <= kFacePX, on_z = face >= kFaceNZ;
+            const int32_t dn = on_x ? r.dx : on_z ? r.dz : r.dy;
+            const int32_t da = on_x ? r.dy : r.dx, db = on_z ? r.dy : r.dz;
+            const int32_t qn = dn < 0 ? 1 - h.tnum : h.tnum - 1;  // one unit back
+            const float rcp_t = 1.0f / (float)h.tden;
+            const int32_t qa = floor_div_small((int64_t)h.tnum * da, h.tden, rcp_t);
+            const int32_t qb = floor_div_small((int64_t)h.tnum * db, h.tden, rcp_t);
+            const int32_t sxp = r.ox + (on_x ? qn : qa);
+            const int32_t syp = r.oy + (on_x ? qa : on_z ? qb : qn);
+            const int32_t szp = r.oz + (on_z ? qn : qb);
+            if (STATS) nshadow++;
+            cast = true;
+            if (p.sun_bounds) {
+                // the start cell's proven bounds decide most shadow rays at once:
+                // at or below F occluded, at or above G lit (hf_sun.cu)
+                int32_t bx = sxp >> kShift, by = syp >> kShift;
+                if (p.sun[0] < 0 && (sxp & 0xFFFF) == 0) bx -= 1;
+                if (p.sun[1] < 0 && (syp & 0xFFFF) == 0) by -= 1;
+                if ((uint32_t)bx < (uint32_t)p.world.W && (uint32_t)by < (uint32_t)p.world.H) {
+                    const uint32_t fg =
+                        __ldg(p.sun_bounds + (uint32_t)by * (uint32_t)p.world.W + (uint32_t)bx);
+                    if (STATS) scnt.cells++;
+                    if (szp <= (int32_t)((fg & 0xFFFFu) << 8)) {
+                        visible = false;
+                        cast = false;
+                    } else if (szp >= (int32_t)((fg >> 16) << 8)) {
+                        cast = false;
+                    }
+                }
+            }
+            r.ox = sxp;
+            r.oy = syp;
+            r.oz = szp;
+            r.dx = p.sun[0];
+            r.dy = p.sun[1];
+            r.dz = p.sun[2];
+        }
+        if (!__any_sync(kFull, cast)) break;
     }
-    store_pixel(p, c, (uint32_t)py * c.w + (uint32_t)px, ph, depth, visible, SHADOWS);
+    if (!inside) return;
+    if (SHADOWS && c.shadow) __stcs(c.shadow + pix, (uint8_t)(visible ? 0 : 1));
+    if (c.rgba)
+        __stcs(c.rgba + pix, face < kFaceError ? shade(word, face, visible, p.sun_n) : kSky);
 }
 
 // Start level of a camera's primary rays: the largest level l <= mip_start
@@ -495,14 +362,15 @@ __device__ __forceinline__ int primary_start(const RenderParams &p, const CamDev
         const int32_t top = (word >> 16) & 0xFF;  // every level in node form
         above = c.o[2] > (top << kShift);
     }
-    const uint32_t mask = __ballot_sync(0xFFFFFFFFu, above);
+    const uint32_t mask = __ballot_sync(kFull, above);
     return max(min(2, p.mip_start), __ffs(~mask) - 2);
 }
 
 // One warp renders one tile: lane l traces the tile's pixels l, l+32, ...
-template <bool SHADOWS, bool STATS, bool PAIR>
+template <bool SHADOWS, int KIND, bool PAIR>
 __device__ __forceinline__ void trace_tile(const RenderParams &p, const LevelDev *lvt,
-                                           const CamDev &c, uint32_t local_tile, int lane) {
+                                           const BeamDir &sun, const CamDev &c,
+                                           uint32_t local_tile, int lane) {
     const uint32_t tx = local_tile % c.tiles_x, ty = local_tile / c.tiles_x;
     const int32_t tw_log2 = p.tile_w_log2;
     const int32_t x0 = (int32_t)tx << tw_log2, y0 = (int32_t)ty << p.tile_h_log2;
@@ -510,22 +378,23 @@ __device__ __forceinline__ void trace_tile(const RenderParams &p, const LevelDev
     Counters cnt{0, 0}, scnt{0, 0};
     uint32_t nshadow = 0, nrays = 0;
     bool err = false;
-    const int start = primary_start<PAIR>(p, c, lane);
+    constexpr bool STATS = KIND == kTraceStats;
+    const int start = KIND == kTraceBeams ? 0 : primary_start<PAIR>(p, c, lane);
     for (int i = lane; i < npix; i += 32) {
         const int32_t px = x0 + (i & ((1 << tw_log2) - 1));
         const int32_t py = y0 + (i >> tw_log2);
-        if (px < (int32_t)c.w && py < (int32_t)c.h) {
-            trace_pixel<SHADOWS, STATS, PAIR>(p, lvt, c, start, px, py, cnt, scnt, nshadow, err);
-            if (STATS) nrays++;
-        }
+        const bool inside = px < (int32_t)c.w && py < (int32_t)c.h;
+        trace_pixels<SHADOWS, KIND, PAIR>(p, lvt, c, start, px, py, inside, sun, cnt, scnt,
+                                          nshadow, err);
+        if (STATS && inside) nrays++;
     }
-    if (__any_sync(0xFFFFFFFFu, err) && lane == 0) atomicOr(p.status, 1u);
+    if (KIND != kTraceBeams && __any_sync(kFull, err) && lane == 0) atomicOr(p.status, 1u);
     if (STATS) {
-        const uint32_t vn = __reduce_add_sync(0xFFFFFFFFu, cnt.nodes);
-        const uint32_t vc = __reduce_add_sync(0xFFFFFFFFu, cnt.cells);
-        const uint32_t vr = __reduce_add_sync(0xFFFFFFFFu, nrays);
-        const uint32_t vs = __reduce_add_sync(0xFFFFFFFFu, nshadow);
-        const uint32_t vf = __reduce_add_sync(0xFFFFFFFFu, scnt.nodes + scnt.cells);
+        const uint32_t vn = __reduce_add_sync(kFull, cnt.nodes);
+        const uint32_t vc = __reduce_add_sync(kFull, cnt.cells);
+        const uint32_t vr = __reduce_add_sync(kFull, nrays);
+        const uint32_t vs = __reduce_add_sync(kFull, nshadow);
+        const uint32_t vf = __reduce_add_sync(kFull, scnt.nodes + scnt.cells);
         if (lane == 0) {
             atomicAdd(p.stats + 0, (unsigned long long)vn);
             atomicAdd(p.stats + 1, (unsigned long long)vc);
@@ -568,14 +437,16 @@ __device__ __forceinline__ const CamDev &stage_cam(CamDev *slot, const CamDev *c
 
 // Persistent batched kernel: warps pop (camera, tile) items from one atomic
 // counter until the batch is drained.  One launch renders every camera.
-template <bool SHADOWS, bool STATS, bool PAIR>
+template <bool SHADOWS, int KIND, bool PAIR>
 __global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS) k_trace_batched(const RenderParams p) {
     __shared__ uint32_t s_base[kMaxCams + 1];
     __shared__ CamDev s_cam[kThreads / 32];
     __shared__ LevelDev s_lv[kMaxLevels + 1];
     const uint32_t n = p.hdr->n_cams;
     const uint32_t total = p.hdr->total_tiles;
+    __shared__ BeamDir s_sun;
     prefetch_world(p);
+    if (SHADOWS && threadIdx.x == 32) s_sun = beam_dir(p.sun[0], p.sun[1], p.sun[2]);
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) s_base[i] = p.cams[i].tile_base;
     fill_levels(s_lv, p.world);
     __syncthreads();
@@ -583,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS) k_trace_batched
     for (;;) {
         uint32_t t = 0;
         if (lane == 0) t = atomicAdd(&p.hdr->counter, 1u);
-        t = __shfl_sync(0xFFFFFFFFu, t, 0);
+        t = __shfl_sync(kFull, t, 0);
         if (t >= total) break;
         // last camera whose first tile is <= t
         uint32_t lo = 0, hi = n;
@@ -593,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS) k_trace_batched
             else hi = mid;
         }
         const CamDev &c = stage_cam(&s_cam[threadIdx.x >> 5], p.cams, lo, lane);
-        trace_tile<SHADOWS, STATS, PAIR>(p, s_lv, c, t - s_base[lo], lane);
+        trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, c, t - s_base[lo], lane);
     }
 }
 
@@ -602,73 +473,78 @@ __global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS) k_trace_batched
 // it to the device; each warp stages it in shared memory like the batched
 // kernel (reading the fields from parameter space instead changes the
 // traversal's register allocation, measured 3-8 % slower on large images).
-template <bool SHADOWS, bool STATS, bool PAIR>
+template <bool SHADOWS, int KIND, bool PAIR>
 __global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS)
     k_trace_plain(const __grid_constant__ RenderParams p, const __grid_constant__ CamDev cam,
                   uint32_t n_tiles) {
     __shared__ LevelDev s_lv[kMaxLevels + 1];
     __shared__ CamDev s_cam[kThreads / 32];
+    __shared__ BeamDir s_sun;
     prefetch_world(p);
+    if (SHADOWS && threadIdx.x == 32) s_sun = beam_dir(p.sun[0], p.sun[1], p.sun[2]);
     fill_levels(s_lv, p.world);
     __syncthreads();
     const uint32_t t = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     if (t >= n_tiles) return;
     const int lane = threadIdx.x & 31;
     const CamDev &c = stage_cam(&s_cam[threadIdx.x >> 5], &cam, 0, lane);
-    trace_tile<SHADOWS, STATS, PAIR>(p, s_lv, c, t, lane);
+    trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, c, t, lane);
 }
 
-template <bool SH, bool ST, bool PA>
+template <bool SH, int KIND, bool PA>
 const void *batched_ptr() {
-    return reinterpret_cast<const void *>(&k_trace_batched<SH, ST, PA>);
+    return reinterpret_cast<const void *>(&k_trace_batched<SH, KIND, PA>);
 }
 
-template <bool PA>
-const void *batched_fn(bool shadows, bool stats) {
-    if (shadows) return stats ? batched_ptr<true, true, PA>() : batched_ptr<true, false, PA>();
-    return stats ? batched_ptr<false, true, PA>() : batched_ptr<false, false, PA>();
+template <bool SH, bool PA>
+const void *batched_fn(int kind) {
+    return kind == kTraceBeams     ? batched_ptr<SH, kTraceBeams, PA>()
+           : kind == kTraceGeneral ? batched_ptr<SH, kTraceGeneral, PA>()
+                                   : batched_ptr<SH, kTraceStats, PA>();
 }
 
-template <bool SH, bool ST, bool PA>
+template <bool SH, int KIND, bool PA>
 void plain_launch(const RenderParams &p, uint32_t blocks, cudaStream_t s, const CamDev &cam,
                   uint32_t n_tiles) {
-    k_trace_plain<SH, ST, PA><<<blocks, kThreads, 0, s>>>(p, cam, n_tiles);
+    k_trace_plain<SH, KIND, PA><<<blocks, kThreads, 0, s>>>(p, cam, n_tiles);
 }
 
 }  // namespace
 
-const void *trace_batched_fn(bool shadows, bool stats, bool pair) {
-    return pair ? batched_fn<true>(shadows, stats) : batched_fn<false>(shadows, stats);
+const void *trace_batched_fn(bool shadows, int kind, bool pair) {
+    if (shadows) return pair ? batched_fn<true, true>(kind) : batched_fn<true, false>(kind);
+    return pair ? batched_fn<false, true>(kind) : batched_fn<false, false>(kind);
 }
 
-int trace_batched_occupancy(bool shadows, bool stats, bool pair, int *blocks_per_sm) {
+int trace_batched_occupancy(bool shadows, int kind, bool pair, int *blocks_per_sm) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        blocks_per_sm, trace_batched_fn(shadows, stats, pair), kThreads, 0);
+        blocks_per_sm, trace_batched_fn(shadows, kind, pair), kThreads, 0);
     return e == cudaSuccess ? 0 : -1;
 }
 
-int launch_trace_batched(const RenderParams &p, bool shadows, bool stats, int blocks,
-                         void *stream) {
+int launch_trace_batched(const RenderParams &p, bool shadows, int kind, int blocks, void *stream) {
     void *args[] = {const_cast<RenderParams *>(&p)};
     const cudaError_t e =
-        cudaLaunchKernel(trace_batched_fn(shadows, stats, p.world.pair != 0), dim3(blocks),
+        cudaLaunchKernel(trace_batched_fn(shadows, kind, p.world.pair != 0), dim3(blocks),
                          dim3(kThreads), args, 0, (cudaStream_t)stream);
     return e == cudaSuccess ? 0 : -1;
 }
 
-int launch_trace_plain(const RenderParams &p, bool shadows, bool stats, const CamDev &cam,
+int launch_trace_plain(const RenderParams &p, bool shadows, int kind, const CamDev &cam,
                        uint32_t n_tiles, void *stream) {
     if (n_tiles == 0) return 0;
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t warps = kThreads / 32;
     const uint32_t blocks = (n_tiles + warps - 1) / warps;
     using Fn = void (*)(const RenderParams &, uint32_t, cudaStream_t, const CamDev &, uint32_t);
-    static const Fn table[8] = {
-        plain_launch<false, false, false>, plain_launch<false, false, true>,
-        plain_launch<false, true, false>,  plain_launch<false, true, true>,
-        plain_launch<true, false, false>,  plain_launch<true, false, true>,
-        plain_launch<true, true, false>,   plain_launch<true, true, true>};
-    table[(shadows ? 4 : 0) + (stats ? 2 : 0) + (p.world.pair ? 1 : 0)](p, blocks, s, cam, n_tiles);
+    static const Fn table[12] = {
+        plain_launch<false, kTraceBeams, false>,   plain_launch<false, kTraceBeams, true>,
+        plain_launch<false, kTraceGeneral, false>, plain_launch<false, kTraceGeneral, true>,
+        plain_launch<false, kTraceStats, false>,   plain_launch<false, kTraceStats, true>,
+        plain_launch<true, kTraceBeams, false>,    plain_launch<true, kTraceBeams, true>,
+        plain_launch<true, kTraceGeneral, false>,  plain_launch<true, kTraceGeneral, true>,
+        plain_launch<true, kTraceStats, false>,    plain_launch<true, kTraceStats, true>};
+    table[(shadows ? 6 : 0) + 2 * kind + (p.world.pair ? 1 : 0)](p, blocks, s, cam, n_tiles);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -833,8 +709,9 @@ extern "C" int hf_render_noalloc(hf_ctx *ctx, const hf_camera *cams, uint32_t n,
         p.sun[i] = sun[i];
         p.sun_n[i] = (float)(sun[i] / sn);
     }
-    const int blocks = v.sm_count * v.occ_shadows[shadows ? 1 : 0];
-    if (launch_trace_batched(p, shadows, false, blocks, stream)) return HF_E_CUDA;
+    const int kind = o.max_steps ? kTraceGeneral : kTraceBeams;
+    const int blocks = v.sm_count * v.occ[shadows ? 1 : 0][kind];
+    if (launch_trace_batched(p, shadows, kind, blocks, stream)) return HF_E_CUDA;
     if (o.flags & HF_SYNC) {
         uint32_t status = 0;
         if (cudaMemcpyAsync(&status, p.status, sizeof(status), cudaMemcpyDeviceToHost, stream) !=
