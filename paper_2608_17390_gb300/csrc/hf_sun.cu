@@ -41,7 +41,7 @@
 // cells whose bands reach the edited rectangle (a parallelogram along L).
 // The band rows and the rise depend on the column of travel only, not on the
 // cell: a full build first tabulates them (k_sun_rows) after the bounds words,
-// and the build and later repairs read the tables instead of dividing.
+// and the build and later repairs read the table instead of dividing.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -52,18 +52,33 @@
 namespace hf {
 namespace {
 
-// Tables after the bounds words, one entry per column of major travel j =
-// -1 .. kRowTable - 2 (entry j + 1), all set by one pass per sun:
-//   rows:  floor(lmin j / lmaj), the minor-axis rows a ray has crossed;
-//   rise:  floor and ceil of 256 j lz / lmaj, its rise in the bounds' units
-//          (2^-8 world units), saturated at kRiseSat (every quantity it is
-//          compared with is below 2^17, so saturation changes no outcome).
-// A bound reads columns up to K + 63 (K <= kSunMaxReach), so every lookup is
-// in range; one outside it would fall back to the float-estimated division.
+// A table after the bounds words, one entry per column of major travel, set by
+// one pass per sun.  Entry i = k + 2, k = -2 .. kRowTable - 3:
+//   x:  q(k + 1), where q(j) = floor(lmin j / lmaj), the minor-axis rows a ray
+//       has crossed after j columns;
+//   y:  ceil of 256 k lz / lmaj, and z: floor of 256 (k - 1) lz / lmaj, its
+//       rise in the bounds' units (2^-8 world units), saturated at kRiseSat
+//       (every quantity it is compared with is below 2^17, so saturation
+//       changes no outcome).
+// A bound reads columns up to K + 63 (K <= kSunMaxReach): always in range.
 constexpr int kRowTable = (int)kSunMaxReach + 128;
 constexpr int32_t kRiseSat = 1 << 21;
 
-__global__ void k_sun_rows(int32_t *q, int64_t lmin, int64_t lmaj, int64_t lz) {
+constexpr int kSunThreads = 128;
+// Cells of a thread along the minor axis.  Their bands overlap, so V cells read
+// V + 3 words a column instead of 4 V.  x major: the lanes of a warp lie along
+// the major axis and every load is one row of words (4; 2 cost 12 % more, 8 the
+// same); y major: along the minor axis, where V also spreads a warp's loads (2).
+constexpr int kSunCellsX = 4, kSunCellsY = 2;
+// Up to this many groups of 32 threads, 8 warps share a group's columns: a
+// repair after a crater, or a small world, leaves too few groups to hide the
+// latency of a thread's up to 1056 columns one after the other (a repair toward
+// (400000, 100000, 100000) 0.143 -> 0.086 ms with its edit; a 2048^2 build, 32768
+// groups, 0.55 -> 0.91 ms if split, as each warp then stops later).
+constexpr int kSunSplit = 8;
+constexpr uint32_t kSunSplitBelow = 16384;
+
+__global__ void k_sun_rows(int4 *tab, int64_t lmin, int64_t lmaj, int64_t lz) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kRowTable) return;
     // once per sun: exact divisions are affordable here
@@ -72,16 +87,15 @@ __global__ void k_sun_rows(int32_t *q, int64_t lmin, int64_t lmaj, int64_t lz) {
         if (n % d != 0 && n < 0) f -= 1;
         return f;
     };
-    const int64_t j = i - 1, rise = 256 * j * lz;
-    const int64_t fl = floor_div(rise, lmaj), ce = fl + (fl * lmaj != rise ? 1 : 0);
-    q[i] = (int32_t)floor_div(lmin * j, lmaj);
-    q[kRowTable + i] = (int32_t)min(fl, (int64_t)kRiseSat);
-    q[2 * kRowTable + i] = (int32_t)min(ce, (int64_t)kRiseSat);
+    const int64_t k = i - 2;
+    const int64_t up = -floor_div(-256 * k * lz, lmaj), down = floor_div(256 * (k - 1) * lz, lmaj);
+    tab[i] = make_int4((int32_t)floor_div(lmin * (k + 1), lmaj), (int32_t)min(up, (int64_t)kRiseSat),
+                       (int32_t)min(down, (int64_t)kRiseSat), 0);
 }
 
-// Node-form word of level-0 cell (x, y), either storage (top = byte 2, floor = byte 0).
-__device__ __forceinline__ uint32_t cell_node(const WorldDev &w, int32_t x, int32_t y) {
-    return level0_node(w, x, y);
+// Words of the bounds, rounded up to whole table entries.
+__host__ __device__ __forceinline__ size_t sun_words(int32_t W, int32_t H) {
+    return ((size_t)W * (size_t)H + 3) & ~(size_t)3;
 }
 
 struct SunAxes {
@@ -92,151 +106,196 @@ struct SunAxes {
     bool x_major;   // the major axis is x
 };
 
-__device__ __forceinline__ uint32_t word_at(const WorldDev &w, const SunAxes &a, int32_t cu,
-                                            int32_t cv) {
-    return a.x_major ? cell_node(w, cu, cv) : cell_node(w, cv, cu);
+// q(j) = floor(lmin j / lmaj), j >= -1
+__device__ __forceinline__ int32_t rows_after(const int4 *tab, int32_t j) {
+    return __ldg(&tab[j + 1].x);
 }
 
-// floor(a / b) for b > 0 and |a / b| < 2^22: a float estimate, then one
-// exact correction (the estimate's relative error is a few 2^-24, so it is
-// off by at most one).  Integer division by a run-time 64-bit divisor is a
-// long software routine on the GPU; this is a handful of instructions.
-__device__ __forceinline__ int64_t floor_div_est(int64_t a, int64_t b, float rcp_b) {
-    int64_t q = (int64_t)floorf((float)a * rcp_b);
-    const int64_t r = a - q * b;
-    if (r < 0) q -= 1;
-    else if (r >= b) q += 1;
-    return q;
+// A level-0 cell as the bounds use it: 255 - floor in the low half, top in the
+// high half, so that one 16-bit pairwise maximum over a band's cells gives its
+// lowest floor and its highest top.
+template <bool PAIR>
+__device__ __forceinline__ uint32_t sun_cell(const WorldDev &w, int32_t x, int32_t y) {
+    uint32_t n;
+    if (PAIR)
+        n = pair_node(__ldg(w.base + (uint32_t)y * ((uint32_t)w.W >> 1) + ((uint32_t)x >> 1)),
+                      (uint32_t)x & 1);
+    else
+        n = __ldg(w.base + (uint32_t)y * (uint32_t)w.W + (uint32_t)x);
+    return (n ^ 0xFFu) & 0x00FF00FFu;
 }
 
-// Level-5 node (32 x 32 cells) at major / minor node coordinates.
-__device__ __forceinline__ uint32_t node5_at(const WorldDev &w, const SunAxes &a, int32_t nu,
-                                             int32_t nv) {
-    const int32_t x = a.x_major ? nu : nv, y = a.x_major ? nv : nu;
-    return __ldg(w.base + w.off[5] + (uint32_t)y * w.stride[5] + (uint32_t)x);
-}
+// V cells of one thread, next to each other along the minor axis in the
+// direction of the sun's minor component: cell i lies at minor coordinate
+// cv + sv i.
+//
+// Column k of a cell reads the band of rows j = 0 .. 1 + B from row(k) =
+// cv + sv i + (sv > 0 ? q(k - 1) : 1 + q(k - 1)) on, in direction sv: the rows
+// 0 .. 1 + A for F, all of them for G, A = |q(k) - q(k - 1)| <= 1 and
+// B = |q(k + 1) - q(k - 1)| <= A + 1.  So the V cells share V + 1 + B rows.
+template <int V>
+struct SunCells {
+    int32_t F[V], G[V];
+};
 
-// floor(lmin * j / lmaj) from the rows table.
-__device__ __forceinline__ int64_t rows_after(const SunAxes &a, const int32_t *rq, int32_t j,
-                                              float rcp_maj) {
-    if ((uint32_t)(j + 1) < (uint32_t)kRowTable) return __ldg(rq + j + 1);
-    return floor_div_est((int64_t)a.lmin * j, a.lmaj, rcp_maj);
-}
-
-// floor (up = false) or ceil (up = true) of 256 j lz / lmaj, j >= 0,
-// saturated at kRiseSat, from the rise tables.
-__device__ __forceinline__ int32_t rise_after(const SunAxes &a, const int32_t *rq, int32_t j,
-                                              bool up, float rcp_maj) {
-    if ((uint32_t)(j + 1) < (uint32_t)kRowTable) return __ldg(rq + (up ? 2 : 1) * kRowTable + j + 1);
-    const int64_t num = (int64_t)j * 256 * a.lz;
-    if (num >= (int64_t)kRiseSat * a.lmaj) return kRiseSat;
-    const int64_t f = floor_div_est(num, a.lmaj, rcp_maj);
-    return (int32_t)(up && f * a.lmaj != num ? f + 1 : f);
-}
-
-// F and G of the cell at major / minor coordinates (cu, cv), rounded to the
-// stored units (F down, G up, 2^-8 world units), computed by the 32 lanes of a
-// warp: lane l takes column k = k0 + l of each round of 32 (its band's lowest
-// floor for F, its widest band's highest top for G), and the warp keeps the
-// largest term.  Rounding is monotone, so the largest rounded term is the
-// rounded largest term: lanes round first and reduce in 32 bits.  A bound
-// stops at the first column it cannot use any more (the grid's end, or for F
-// a band that leaves the grid -- monotone in k, so every lane past it is out
-// too) or once no later column can raise it.  Where the pyramid has a level
-// 5, a round whose region's highest floor (F) or top (G) cannot raise the
-// bound loads no cells; the result is the same.
-__device__ void bounds_of_warp(const WorldDev &w, const SunAxes &a, const int32_t *rq, int32_t cu,
-                               int32_t cv, int32_t NU, int32_t NV, int lane, int32_t &F16,
-                               int32_t &G16) {
-    const unsigned full = 0xFFFFFFFFu;
-    const float rcp_maj = 1.0f / (float)a.lmaj;
-    // In the stored units a term is a height h (a floor for F, a top for G)
-    // times 256, less the rise 256 (k or k - 1) lz / lmaj: exactly, the F term
-    // of column k rounded down is 256 h - ceil(256 k lz / lmaj), and the G term
-    // rounded up is 256 h - floor(256 (k - 1) lz / lmaj).  Negative F terms
-    // and non-positive G terms never win (F, G >= 0 from k = 0).
-    const uint32_t c0 = word_at(w, a, cu, cv);
-    F16 = (int32_t)(c0 & 0xFF) << 8;  // k = 0: the start cell's floor
-    {  // G, k = 0: the rows the ray can cross in its start column (it moves at
-       // most one row there, |lmin| <= lmaj), strictly above: top + 2^-16,
-       // rounded up
-        const int32_t r0 = cv + (a.lmin < 0 ? -1 : 0), r1 = cv + 1;
-        int32_t t = -1;
-        if (lane <= r1 - r0) {
-            const int32_t r = r0 + lane;
-            if (r >= 0 && r < NV) t = (int32_t)((word_at(w, a, cu, r) >> 16) & 0xFF);
-        }
-        t = __reduce_max_sync(full, t);
-        G16 = t < 0 ? 0 : (t << 8) + 1;
+// One column: col, row: its major coordinate and the first cell's row(k).
+// EDGE: some of it may lie outside the grid (a cell there is neutral); f_on:
+// cells whose F still counts.
+template <bool XM, bool PAIR, int V, int A, int B, bool EDGE>
+__device__ __forceinline__ void sun_column(const WorldDev &w, int32_t col, int32_t row, int32_t sv,
+                                           int32_t up, int32_t down, uint32_t f_on,
+                                           SunCells<V> &c) {
+    const int32_t NU = XM ? w.W : w.H, NV = XM ? w.H : w.W;
+    const bool in_col = !EDGE || (uint32_t)col < (uint32_t)NU;
+    uint32_t p[V + 1 + B];
+#pragma unroll
+    for (int j = 0; j < V + 1 + B; ++j) {
+        const int32_t r = row + sv * j;
+        p[j] = 0;
+        if (!EDGE || (in_col && (uint32_t)r < (uint32_t)NV))
+            p[j] = XM ? sun_cell<PAIR>(w, col, r) : sun_cell<PAIR>(w, r, col);
     }
-    constexpr int32_t top_all = 255 << 8;
-    const bool skip = w.L >= 5;
-    bool f_on = true, g_on = true;
-    for (int32_t k0 = 1;; k0 += 32) {
-        // no column from k0 on can raise a bound already this high
-        if (f_on && top_all - (F16 + 1) < rise_after(a, rq, k0, true, rcp_maj)) f_on = false;
-        if (g_on && top_all - G16 <= rise_after(a, rq, k0 - 1, false, rcp_maj)) g_on = false;
-        if (!f_on && !g_on) break;
-        const int32_t k = k0 + lane;
+    const int32_t cf = (255 << 8) - up;
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        uint32_t f = __vmaxu2(p[i], p[i + 1]);
+        if (A) f = __vmaxu2(f, p[i + 1 + A]);
+        uint32_t g = f;
+        if (B > A) g = __vmaxu2(g, p[i + 1 + B]);
+        // the whole F band in the grid
+        const bool f_ok = !EDGE || (in_col && (f_on >> i & 1) &&
+                                    (uint32_t)(row + sv * i) < (uint32_t)NV &&
+                                    (uint32_t)(row + sv * (i + 1 + A)) < (uint32_t)NV);
+        if (f_ok) c.F[i] = max(c.F[i], cf - (int32_t)((f & 0xFFu) << 8));
+        c.G[i] = max(c.G[i], (int32_t)((g >> 16) << 8) - down);  // (never raised by neutral cells)
+    }
+}
+
+template <bool XM, bool PAIR, int V, bool EDGE>
+__device__ __forceinline__ void sun_round(const WorldDev &w, const SunAxes &a, const int4 *tab,
+                                          int32_t k0, int32_t cu, int32_t cv, int32_t sv,
+                                          uint32_t f_on, SunCells<V> &c) {
+    int32_t qm = rows_after(tab, k0 - 1), qk = rows_after(tab, k0);
+#pragma unroll 1
+    for (int32_t k = k0; k < k0 + 32; ++k) {
+        const int4 e = __ldg(&tab[k + 2]);
+        const int32_t col = cu + a.smaj * k, row = cv + (sv > 0 ? qm : 1 + qm);
+        if (qk != qm) {
+            if (abs(e.x - qm) > 1)
+                sun_column<XM, PAIR, V, 1, 2, EDGE>(w, col, row, sv, e.y, e.z, f_on, c);
+            else
+                sun_column<XM, PAIR, V, 1, 1, EDGE>(w, col, row, sv, e.y, e.z, f_on, c);
+        } else {
+            if (e.x != qm)
+                sun_column<XM, PAIR, V, 0, 1, EDGE>(w, col, row, sv, e.y, e.z, f_on, c);
+            else
+                sun_column<XM, PAIR, V, 0, 0, EDGE>(w, col, row, sv, e.y, e.z, f_on, c);
+        }
+        qm = qk;
+        qk = e.x;
+    }
+}
+
+// Bounds of the V cells of each thread of a warp, rounded to the stored units
+// (F down, G up, 2^-8 world units).  In these units a term is a height h times
+// 256, less the rise: exactly, the F term of column k rounded down is 256 h -
+// ceil(256 k lz / lmaj), and the G term rounded up is 256 h - floor(256 (k - 1)
+// lz / lmaj).
+//
+// Columns go in rounds of 32, of which this warp takes every step-th from
+// `first` on.  F stops with the first round that holds a column it cannot use
+// (the grid's end, or a band that leaves the grid: once one does, all later
+// ones do too, but for column 1 of a cell on the grid's last row).  The rounds
+// end once none can raise any of the warp's bounds (maxh0, maxtop: the world's
+// highest floor and top), and where the pyramid has a level 5, a round over a
+// region whose highest floor and top cannot raise any is skipped; neither
+// changes a bound.
+// cu, cv: the first cell; on: which cells are real.
+template <bool XM, bool PAIR, int V>
+__device__ __forceinline__ void sun_bounds_of(const WorldDev &w, const SunAxes &a, const int4 *tab,
+                                              int32_t cu, int32_t cv, int32_t sv, uint32_t on,
+                                              int32_t first, int32_t step, SunCells<V> &c) {
+    constexpr unsigned full = 0xFFFFFFFFu;
+    const int32_t NU = XM ? w.W : w.H, NV = XM ? w.H : w.W;
+    const int lane = threadIdx.x & 31;
+    auto cell = [&](int32_t u, int32_t v) {
+        return XM ? sun_cell<PAIR>(w, u, v) : sun_cell<PAIR>(w, v, u);
+    };
+    // k = 0: for F the start cell's floor; for G the rows the ray can cross in
+    // its start column (it moves at most one row there), strictly above: top +
+    // 2^-16, rounded up
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        c.F[i] = c.G[i] = 0;
+        if (!(on >> i & 1)) continue;
+        const int32_t v = cv + sv * i;
+        const uint32_t p = cell(cu, v);
+        uint32_t top = p >> 16;
+        if (v + 1 < NV) top = max(top, cell(cu, v + 1) >> 16);
+        if (a.lmin < 0 && v > 0) top = max(top, cell(cu, v - 1) >> 16);
+        c.F[i] = (int32_t)(255 - (p & 0xFF)) << 8;
+        c.G[i] = (int32_t)(top << 8) + 1;
+    }
+    const uint32_t root = __ldg(w.base + w.off[w.L]);
+    const int32_t maxh0 = w.L ? (int32_t)(root & 0xFF) << 8 : 255 << 8;
+    const int32_t maxtop = w.L ? (int32_t)((root >> 16) & 0xFF) << 8 : 255 << 8;
+    // cells whose F band leaves the grid in column k
+    auto f_out = [&](int32_t k) {
+        const int32_t qa = rows_after(tab, k - 1), qb = rows_after(tab, k);
         const int32_t col = cu + a.smaj * k;
-        const bool in_col = col >= 0 && col < NU;
-        // rows floor(lmin * j / lmaj) of travel j = k - 1, k, k + 1
-        const int64_t qm = rows_after(a, rq, k - 1, rcp_maj);
-        const int64_t qk = rows_after(a, rq, k, rcp_maj);
-        const int64_t qp = rows_after(a, rq, k + 1, rcp_maj);
-        const int32_t f0 = cv + (int32_t)min(qm, qk), f1 = cv + 1 + (int32_t)max(qm, qk);
-        const int32_t g0 = cv + (int32_t)min(qm, qp), g1 = cv + 1 + (int32_t)max(qm, qp);
-        const bool f_ok = in_col && f0 >= 0 && f1 < NV;  // the whole F band in the grid
-        const bool g_ok = in_col && g1 >= 0 && g0 < NV;  // some of the G band in the grid
-        bool f_need = f_on, g_need = g_on;
-        if (skip && (f_need || g_need)) {
-            // the round's region: its columns and the rows of all its G bands
-            const int32_t rlo = max(__reduce_min_sync(full, g_ok ? g0 : 0x7FFFFFFF), 0);
-            const int32_t rhi = min(__reduce_max_sync(full, g_ok ? g1 : -1), NV - 1);
-            const int32_t ca = cu + a.smaj * k0, cb = cu + a.smaj * (k0 + 31);
-            const int32_t clo = max(min(ca, cb), 0), chi = min(max(ca, cb), NU - 1);
-            int32_t mh = -1, mt = -1;
-            if (rlo <= rhi && clo <= chi) {
-                const int32_t nu0 = clo >> 5, nv0 = rlo >> 5;
-                const int32_t nnu = (chi >> 5) - nu0 + 1, nnv = (rhi >> 5) - nv0 + 1;
-                if (lane < nnu * nnv) {
-                    const uint32_t n = node5_at(w, a, nu0 + lane % nnu, nv0 + lane / nnu);
-                    mh = (int32_t)(n & 0xFF);
-                    mt = (int32_t)((n >> 16) & 0xFF);
-                }
-                mh = __reduce_max_sync(full, mh);
-                mt = __reduce_max_sync(full, mt);
-            }
-            f_need = f_need && mh >= 0 && (mh << 8) - (F16 + 1) >= rise_after(a, rq, k0, true, rcp_maj);
-            g_need = g_need && mt >= 0 && (mt << 8) - G16 > rise_after(a, rq, k0 - 1, false, rcp_maj);
+        uint32_t out = 0;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            const int32_t v = cv + sv * i;
+            if (col < 0 || col >= NU || v + min(qa, qb) < 0 || v + 1 + max(qa, qb) >= NV)
+                out |= 1u << i;
         }
-        if (f_need || g_need) {
-            int32_t m = 255, t = -1;
-            if (g_ok || f_ok)
-                for (int32_t r = max(g0, 0); r <= min(g1, NV - 1); ++r) {
-                    const uint32_t c = word_at(w, a, col, r);
-                    if (r >= f0 && r <= f1) m = min(m, (int32_t)(c & 0xFF));
-                    t = max(t, (int32_t)((c >> 16) & 0xFF));
-                }
-            if (f_need) {
-                int32_t v = -1;
-                if (f_ok) {
-                    const int32_t q = (m << 8) - rise_after(a, rq, k, true, rcp_maj);
-                    v = q < 0 ? -1 : q;
-                }
-                F16 = max(F16, __reduce_max_sync(full, v));
-            }
-            if (g_need) {
-                int32_t v = 0;
-                if (g_ok) {
-                    const int32_t q = (t << 8) - rise_after(a, rq, k - 1, false, rcp_maj);
-                    v = q <= 0 ? 0 : q;
-                }
-                G16 = max(G16, __reduce_max_sync(full, v));
-            }
+        return out;
+    };
+    const uint32_t out1 = f_out(1);
+    for (int32_t k0 = 1 + 32 * first;; k0 += 32 * step) {
+        const uint32_t f_on = k0 == 1 ? on : on & ~(out1 | f_out(k0 - 1));
+        int32_t lo_f = 1 << 20, lo_g = 1 << 20;  // the lowest bounds that may still rise
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            if (f_on >> i & 1) lo_f = min(lo_f, c.F[i]);
+            if (on >> i & 1) lo_g = min(lo_g, c.G[i]);
         }
-        if (f_on && !__all_sync(full, f_ok)) f_on = false;
-        if (g_on && !__all_sync(full, g_ok)) g_on = false;
+        lo_f = __reduce_min_sync(full, lo_f);
+        lo_g = __reduce_min_sync(full, lo_g);
+        const int4 rise = __ldg(&tab[k0 + 2]);
+        if (maxh0 - (lo_f + 1) < rise.y && maxtop - lo_g <= rise.z) break;
+        const int32_t ca = cu + a.smaj * k0, cb = cu + a.smaj * (k0 + 31);
+        // the rows the round reads, first and last in direction sv
+        const int32_t qm = rows_after(tab, k0 - 1), qe = rows_after(tab, k0 + 32);
+        const int32_t ra = cv + (sv > 0 ? qm : 1 + qm);
+        const int32_t rb = cv + sv * (V - 1) + (sv > 0 ? 1 + qe : qe);
+        const int32_t rlo = min(ra, rb), rhi = max(ra, rb);
+        // the region of the whole warp
+        const int32_t u0 = __reduce_min_sync(full, min(ca, cb));
+        const int32_t u1 = __reduce_max_sync(full, max(ca, cb));
+        const int32_t v0 = __reduce_min_sync(full, rlo), v1 = __reduce_max_sync(full, rhi);
+        if (u1 < 0 || u0 >= NU || v1 < 0 || v0 >= NV) break;  // and so are all later rounds
+        if (w.L >= 5) {
+            const int32_t a0 = max(u0, 0) >> 5, a1 = min(u1, NU - 1) >> 5;
+            const int32_t b0 = max(v0, 0) >> 5, b1 = min(v1, NV - 1) >> 5;
+            const int32_t nu = a1 - a0 + 1, n_nodes = nu * (b1 - b0 + 1);
+            int32_t mh = 0, mt = 0;
+            for (int32_t n = lane; n < n_nodes; n += 32) {
+                const int32_t u = a0 + n % nu, v = b0 + n / nu;
+                const uint32_t node = __ldg(w.base + w.off[5] + (uint32_t)(XM ? v : u) * w.stride[5] +
+                                            (uint32_t)(XM ? u : v));
+                mh = max(mh, (int32_t)(node & 0xFF));
+                mt = max(mt, (int32_t)((node >> 16) & 0xFF));
+            }
+            mh = __reduce_max_sync(full, mh) << 8;
+            mt = __reduce_max_sync(full, mt) << 8;
+            if (mh - (lo_f + 1) < rise.y && mt - lo_g <= rise.z) continue;
+        }
+        if (u0 >= 0 && u1 < NU && v0 >= 0 && v1 < NV && __all_sync(full, f_on == on))
+            sun_round<XM, PAIR, V, false>(w, a, tab, k0, cu, cv, sv, f_on, c);
+        else
+            sun_round<XM, PAIR, V, true>(w, a, tab, k0, cu, cv, sv, f_on, c);
     }
 }
 
@@ -244,7 +303,7 @@ __device__ void bounds_of_warp(const WorldDev &w, const SunAxes &a, const int32_
 // [eu0, eu1) x [ev0, ev1) (major / minor coordinates): some column of the
 // rectangle within `reach` columns downstream, with the cell's widest band
 // over those columns meeting the rectangle's rows.
-__device__ bool depends_on(const SunAxes &a, const int32_t *rq, int32_t cu, int32_t cv,
+__device__ bool depends_on(const SunAxes &a, const int4 *tab, int32_t cu, int32_t cv,
                            int32_t eu0, int32_t ev0, int32_t eu1, int32_t ev1, int32_t reach) {
     int32_t ka = a.smaj > 0 ? eu0 - cu : cu - (eu1 - 1);
     int32_t kb = a.smaj > 0 ? eu1 - 1 - cu : cu - eu0;
@@ -253,38 +312,96 @@ __device__ bool depends_on(const SunAxes &a, const int32_t *rq, int32_t cu, int3
     if (ka > kb) return false;
     // floor is monotone, so the band's lowest and highest rows over the
     // columns ka..kb come from travel ka - 1 and kb + 1
-    const float rcp_maj = 1.0f / (float)a.lmaj;
-    const int64_t qa = rows_after(a, rq, ka - 1, rcp_maj), qb = rows_after(a, rq, kb + 1, rcp_maj);
-    const int32_t r0 = cv + (int32_t)min(qa, qb);
-    const int32_t r1 = cv + 1 + (int32_t)max(qa, qb);
-    return r1 >= ev0 && r0 < ev1;
+    const int32_t qa = rows_after(tab, ka - 1), qb = rows_after(tab, kb + 1);
+    return cv + 1 + max(qa, qb) >= ev0 && cv + min(qa, qb) < ev1;
 }
 
-// One warp per cell of the rectangle [x0, x1) x [y0, y1).  With edit.z >
-// edit.x, only the cells whose bounds depend on the edited rectangle
-// [edit.x, edit.z) x [edit.y, edit.w) are recomputed (the others keep theirs).
-__global__ void k_sun_bounds(const WorldDev w, uint32_t *fg, SunAxes a, int32_t x0, int32_t y0,
-                             int32_t nx, uint32_t n, int4 edit, int32_t reach) {
-    // the thread index in 64 bits: a warp per cell of a grid of up to 2^28
-    // cells is up to 2^33 threads
-    const uint32_t i = (uint32_t)(((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (i >= n) return;  // warp-uniform
-    const int32_t x = x0 + (int32_t)(i % (uint32_t)nx), y = y0 + (int32_t)(i / (uint32_t)nx);
-    const int32_t *rq = reinterpret_cast<const int32_t *>(fg + (size_t)w.W * (size_t)w.H);
-    if (edit.z > edit.x) {
-        const bool dep = a.x_major ? depends_on(a, rq, x, y, edit.x, edit.y, edit.z, edit.w, reach)
-                                   : depends_on(a, rq, y, x, edit.y, edit.x, edit.w, edit.z, reach);
-        if (!dep) return;  // warp-uniform
+// Bound by instruction issue (about 15 instructions per cell and column).  One
+// warp per cell, its lanes taking 32 columns each round, cost about 1700 warp
+// instructions a cell in loads of bands no other cell shared, reductions and
+// per-lane table reads: 2048^2 world, default sun, 6.4 -> 0.55 ms.
+// The cells of the rectangle [x0, x1) x [y0, y1), V per thread along the minor
+// axis, a warp's threads next to each other along x (nwx warps a row).  SPLIT:
+// the warps of a block share the rounds of the same cells.  With edit.z >
+// edit.x, only the cells whose bounds depend on the edited rectangle [edit.x,
+// edit.z) x [edit.y, edit.w) are recomputed (the others keep theirs).
+template <bool XM, bool PAIR, int V, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? kSunSplit * 32 : kSunThreads)
+    k_sun_bounds(const WorldDev w, uint32_t *fg, const SunAxes a, int32_t x0, int32_t y0, int32_t x1,
+                 int32_t y1, uint32_t nwx, uint32_t n_groups, int4 edit, int32_t reach) {
+    __shared__ int32_t s_part[SPLIT ? 2 * V * kSunSplit * 32 : 1];
+    const uint32_t group = SPLIT ? blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (group >= n_groups) return;
+    const int lane = threadIdx.x & 31, sub = SPLIT ? threadIdx.x >> 5 : 0;
+    const int4 *tab = reinterpret_cast<const int4 *>(fg + sun_words(w.W, w.H));
+    const int32_t sv = a.lmin < 0 ? -1 : 1;
+    const int32_t wx = (int32_t)(group % nwx), wy = (int32_t)(group / nwx);
+    // the thread's first cell along the minor axis, and its major coordinate
+    const int32_t v0 = XM ? y0 + wy * V : x0 + (wx * 32 + lane) * V, v1 = XM ? y1 : x1;
+    const int32_t u = XM ? x0 + wx * 32 + lane : y0 + wy;
+    const int32_t cu = XM ? min(u, x1 - 1) : u;
+    const int32_t cv = min(v0, v1 - 1) + (sv < 0 ? V - 1 : 0);
+    uint32_t on = 0;
+    if (v0 < v1 && (!XM || u < x1))
+        for (int i = 0; i < V; ++i) {
+            const int32_t v = cv + sv * i;
+            if (v >= v1) continue;
+            if (edit.z > edit.x &&
+                !(XM ? depends_on(a, tab, cu, v, edit.x, edit.y, edit.z, edit.w, reach)
+                     : depends_on(a, tab, cu, v, edit.y, edit.x, edit.w, edit.z, reach)))
+                continue;
+            on |= 1u << i;
+        }
+    if (!__any_sync(0xFFFFFFFFu, on != 0)) return;  // (all warps of a split group alike)
+    SunCells<V> c;
+    sun_bounds_of<XM, PAIR, V>(w, a, tab, cu, cv, sv, on, sub, SPLIT ? kSunSplit : 1, c);
+    if (SPLIT) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            s_part[(2 * i * kSunSplit + sub) * 32 + lane] = c.F[i];
+            s_part[((2 * i + 1) * kSunSplit + sub) * 32 + lane] = c.G[i];
+        }
+        __syncthreads();
+        if (sub) return;
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            for (int t = 1; t < kSunSplit; ++t) {
+                c.F[i] = max(c.F[i], s_part[(2 * i * kSunSplit + t) * 32 + lane]);
+                c.G[i] = max(c.G[i], s_part[((2 * i + 1) * kSunSplit + t) * 32 + lane]);
+            }
     }
-    int32_t F16, G16;
-    if (a.x_major)
-        bounds_of_warp(w, a, rq, x, y, w.W, w.H, lane, F16, G16);
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        if (!(on >> i & 1)) continue;
+        const int32_t v = cv + sv * i;
+        fg[(uint32_t)(XM ? v : cu) * (uint32_t)w.W + (uint32_t)(XM ? cu : v)] =
+            (uint32_t)c.F[i] | ((uint32_t)c.G[i] << 16);
+    }
+}
+
+template <bool XM, bool PAIR, int V>
+int sun_launch(const WorldDev &w, uint32_t *fg, const SunAxes &a, const int32_t r[4], int4 edit,
+               int32_t reach, cudaStream_t s) {
+    const uint32_t nx = (uint32_t)(r[2] - r[0]), ny = (uint32_t)(r[3] - r[1]);
+    const uint32_t per = XM ? 32 : 32 * V, nwx = (nx + per - 1) / per;
+    const uint32_t n = nwx * (XM ? (ny + V - 1) / V : ny);
+    if (n <= kSunSplitBelow)
+        k_sun_bounds<XM, PAIR, V, true><<<n, kSunSplit * 32, 0, s>>>(w, fg, a, r[0], r[1], r[2], r[3],
+                                                                     nwx, n, edit, reach);
     else
-        bounds_of_warp(w, a, rq, y, x, w.H, w.W, lane, F16, G16);
-    if (lane == 0)
-        fg[(uint32_t)y * (uint32_t)w.W + (uint32_t)x] =
-            (uint32_t)max(F16, 0) | ((uint32_t)max(G16, 0) << 16);
+        k_sun_bounds<XM, PAIR, V, false>
+            <<<(n * 32 + kSunThreads - 1) / kSunThreads, kSunThreads, 0, s>>>(
+                w, fg, a, r[0], r[1], r[2], r[3], nwx, n, edit, reach);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int sun_launch(const WorldDev &w, uint32_t *fg, const SunAxes &a, const int32_t r[4], int4 edit,
+               int32_t reach, cudaStream_t s) {
+    if (a.x_major)
+        return w.pair ? sun_launch<true, true, kSunCellsX>(w, fg, a, r, edit, reach, s)
+                      : sun_launch<true, false, kSunCellsX>(w, fg, a, r, edit, reach, s);
+    return w.pair ? sun_launch<false, true, kSunCellsY>(w, fg, a, r, edit, reach, s)
+                  : sun_launch<false, false, kSunCellsY>(w, fg, a, r, edit, reach, s);
 }
 
 SunAxes axes_of(const int32_t sun[3]) {
@@ -332,25 +449,20 @@ void sun_bounds_region(const WorldDev &w, const int32_t sun[3], int32_t x0, int3
 }
 
 size_t sun_bounds_bytes(int32_t W, int32_t H) {
-    return ((size_t)W * (size_t)H + 3 * (size_t)kRowTable) * sizeof(uint32_t);
+    return sun_words(W, H) * sizeof(uint32_t) + kRowTable * sizeof(int4);
 }
 
 int sun_bounds(const WorldDev &w, uint32_t *fg, const int32_t sun[3], int32_t x0, int32_t y0,
                int32_t x1, int32_t y1, void *stream) {
     if (!sun_bounds_eligible(sun)) return -1;
-    {  // this sun's row and rise tables, which the bounds and later repairs read
-        const SunAxes a = axes_of(sun);
-        k_sun_rows<<<(kRowTable + 255) / 256, 256, 0, (cudaStream_t)stream>>>(
-            reinterpret_cast<int32_t *>(fg + (size_t)w.W * (size_t)w.H), a.lmin, a.lmaj, a.lz);
-        if (cudaGetLastError() != cudaSuccess) return -1;
-    }
+    const SunAxes a = axes_of(sun);
+    // this sun's table, which the bounds and later repairs read
+    k_sun_rows<<<(kRowTable + 127) / 128, 128, 0, (cudaStream_t)stream>>>(
+        reinterpret_cast<int4 *>(fg + sun_words(w.W, w.H)), a.lmin, a.lmaj, a.lz);
+    if (cudaGetLastError() != cudaSuccess) return -1;
     if (x1 <= x0 || y1 <= y0) return 0;
-    const uint32_t nx = (uint32_t)(x1 - x0), n = nx * (uint32_t)(y1 - y0);
-    const uint32_t threads = 128, blocks = (n + threads / 32 - 1) / (threads / 32);
-    k_sun_bounds<<<blocks, threads, 0, (cudaStream_t)stream>>>(w, fg, axes_of(sun), x0, y0,
-                                                                (int32_t)nx, n,
-                                                                make_int4(0, 0, 0, 0), 0);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    const int32_t r[4] = {x0, y0, x1, y1};
+    return sun_launch(w, fg, a, r, make_int4(0, 0, 0, 0), 0, (cudaStream_t)stream);
 }
 
 int sun_bounds_repair(const WorldDev &w, uint32_t *fg, const int32_t sun[3], int32_t x0,
@@ -362,12 +474,7 @@ int sun_bounds_repair(const WorldDev &w, uint32_t *fg, const int32_t sun[3], int
     if (r[2] <= r[0] || r[3] <= r[1]) return 0;
     const SunAxes a = axes_of(sun);
     const int32_t reach = (int32_t)(255 * (int64_t)a.lmaj / a.lz + 2);
-    const uint32_t nx = (uint32_t)(r[2] - r[0]), n = nx * (uint32_t)(r[3] - r[1]);
-    const uint32_t threads = 128, blocks = (n + threads / 32 - 1) / (threads / 32);
-    k_sun_bounds<<<blocks, threads, 0, (cudaStream_t)stream>>>(w, fg, a, r[0], r[1], (int32_t)nx,
-                                                                n, make_int4(x0, y0, x1, y1),
-                                                                reach);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return sun_launch(w, fg, a, r, make_int4(x0, y0, x1, y1), reach, (cudaStream_t)stream);
 }
 
 }  // namespace hf
