@@ -522,7 +522,7 @@ int hf_edit(hf_ctx *c, uint32_t x0, uint32_t y0, uint32_t w, uint32_t h, const u
                            (int32_t)(y0 + h), c->stream))
         return HF_E_CUDA;
     if (c->d_vox && hf::voxel_repair(c->wd, c->vd, (int32_t)x0, (int32_t)y0, (int32_t)(x0 + w),
-                                     (int32_t)(y0 + h), false, c->stream))
+                                     (int32_t)(y0 + h), c->stream))
         return HF_E_CUDA;
     if (c->sun_valid) {  // the shadow bounds of the cells upstream of the rectangle
         if (hf::sun_bounds_repair(c->wd, c->d_sun, c->sun_dir, (int32_t)x0, (int32_t)y0,
@@ -541,11 +541,9 @@ int hf_rebuild(hf_ctx *c) {
     for (auto &s : c->slots)
         if (s.pending) CK(cudaStreamWaitEvent(c->stream, s.done, 0));
     if (hf::pyramid_build(c->d_world, c->wd, c->stream)) return HF_E_CUDA;
-    if (c->d_vox) {
-        CK(cudaMemsetAsync(c->d_vox, 0, c->vox_words * 4, c->stream));
-        if (hf::voxel_repair(c->wd, c->vd, 0, 0, (int32_t)c->W, (int32_t)c->H, true, c->stream))
-            return HF_E_CUDA;
-    }
+    if (c->d_vox &&
+        hf::voxel_repair(c->wd, c->vd, 0, 0, (int32_t)c->W, (int32_t)c->H, c->stream))
+        return HF_E_CUDA;
     if (c->sun_valid &&
         hf::sun_bounds(c->wd, c->d_sun, c->sun_dir, 0, 0, (int32_t)c->W, (int32_t)c->H, c->stream)) {
         c->sun_valid = false;
@@ -1337,21 +1335,22 @@ int hf_voxel_build(hf_ctx *c, const hf_voxel_desc *d) {
     CK(cudaSetDevice(c->device));
     for (auto &s : c->slots)
         if (s.pending) CK(cudaStreamWaitEvent(c->stream, s.done, 0));
-    CK(cudaStreamSynchronize(c->stream));
-    if (c->d_vox) {
-        cudaFree(c->d_vox);
-        c->d_vox = nullptr;
-    }
-    if (cudaMalloc(&c->d_vox, off * 4) != cudaSuccess) {
-        (void)cudaGetLastError();
-        c->d_vox = nullptr;
-        return HF_E_OOM;
+    if (!c->d_vox || c->vox_words != off) {  // (a rebuild of the same size keeps its words)
+        CK(cudaStreamSynchronize(c->stream));
+        if (c->d_vox) {
+            cudaFree(c->d_vox);
+            c->d_vox = nullptr;
+        }
+        if (cudaMalloc(&c->d_vox, off * 4) != cudaSuccess) {
+            (void)cudaGetLastError();
+            c->d_vox = nullptr;
+            return HF_E_OOM;
+        }
     }
     v.words = c->d_vox;
     c->vd = v;
     c->vox_words = off;
-    CK(cudaMemsetAsync(c->d_vox, 0, off * 4, c->stream));
-    if (hf::voxel_repair(c->wd, c->vd, 0, 0, (int32_t)c->W, (int32_t)c->H, true, c->stream))
+    if (hf::voxel_repair(c->wd, c->vd, 0, 0, (int32_t)c->W, (int32_t)c->H, c->stream))
         return HF_E_CUDA;
     CK(cudaEventRecord(c->edit_done, c->stream));
     CK(cudaStreamSynchronize(c->stream));

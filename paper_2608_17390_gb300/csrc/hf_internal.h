@@ -178,10 +178,10 @@ struct VoxelParams {
     int32_t inner;    // samples per occupied leaf voxel
     float far_dist;   // world units
 };
-// Recompute the voxels over cell rectangle [x0, x1) x [y0, y1), every level
-// (fresh: the words are zero, as after allocation).
+// Recompute the voxels over cell rectangle [x0, x1) x [y0, y1), every level.
+// Words are written whole; over the whole grid, every word of the pyramid is.
 int voxel_repair(const WorldDev &w, const VoxelDev &v, int32_t x0, int32_t y0, int32_t x1,
-                 int32_t y1, bool fresh, void *stream);
+                 int32_t y1, void *stream);
 int launch_voxel_trace(const RenderParams &p, const VoxelDev &v, const VoxelParams &q,
                        uint32_t n_cams, uint32_t max_pixels, void *stream);
 

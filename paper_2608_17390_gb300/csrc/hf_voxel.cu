@@ -27,21 +27,14 @@ namespace hf {
 namespace {
 
 constexpr int kVoxThreads = 128;
+constexpr int kVoxTailThreads = 1024;
+constexpr int32_t kVoxTailWords = 16384;  // levels of up to this many words share one block
 
 __host__ __device__ __forceinline__ uint32_t spread3(uint32_t v) {
     return (v & 1u) | ((v & 2u) << 2) | ((v & 4u) << 4);
 }
 __host__ __device__ __forceinline__ uint32_t morton3(uint32_t x, uint32_t y, uint32_t z) {
     return spread3(x) | (spread3(y) << 1) | (spread3(z) << 2);
-}
-
-// word index and bit of voxel (x, y, z) of level l
-__device__ __forceinline__ void vox_addr(const VoxelDev &v, int l, uint32_t x, uint32_t y,
-                                         uint32_t z, uint32_t &word, uint32_t &bit) {
-    const uint32_t tile = ((z >> 3) * v.ty[l] + (y >> 3)) * v.tx[l] + (x >> 3);
-    const uint32_t m = morton3(x & 7, y & 7, z & 7);
-    word = v.off[l] + tile * 16 + (m >> 5);
-    bit = m & 31;
 }
 
 // One level of the pyramid as the traversal reads it: a per-block shared
@@ -79,87 +72,171 @@ __device__ __forceinline__ float vox_quot(float pk, int32_t vs, int32_t vs_log2,
     return __fdiv_rn(pk, (float)(vs << l));
 }
 
-__device__ __forceinline__ bool vox_occupied(const VoxelDev &v, int l, uint32_t x, uint32_t y,
-                                             uint32_t z) {
-    uint32_t w, b;
-    vox_addr(v, l, x, y, z, w, b);
-    return (__ldg(v.words + w) >> b) & 1u;
+// h / vz for h < 512, vz <= 256, by a multiplication with recip = 2^20 / vz + 1
+// (the product's excess, h (recip vz - 2^20) <= 2^17, stays below 2^20).
+__device__ __forceinline__ int32_t vox_div(int32_t h, uint32_t recip) {
+    return (int32_t)(((uint32_t)h * recip) >> 20);
 }
 
+// Bits [lo, hi] of word q of a mask.
+__device__ __forceinline__ uint32_t vox_bits(int32_t lo, int32_t hi, int q) {
+    lo = max(lo - 32 * q, 0);
+    hi = min(hi - 32 * q, 31);
+    return lo > hi ? 0u : (0xFFFFFFFFu << lo) & (0xFFFFFFFFu >> (31 - hi));
+}
 
-// Level-0 voxel columns [i0, i0+ni) x [j0, j0+nj): the layers each column's
-// cells occupy, gathered as a bit mask, then written into the column's bits.
-// In an 8^3 tile the layers 2q and 2q+1 of one column share a word (the bits
-// morton and morton + 4), so one atomic pair per word updates them; a fresh
-// build (zeroed words) needs only the OR.
-__global__ void k_vox_level0(const WorldDev w, const VoxelDev v, int32_t i0, int32_t j0,
-                             int32_t ni, int32_t nj, int fresh) {
-    const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ni * nj) return;
-    const int32_t i = i0 + t % ni, j = j0 + t / ni;
-    uint32_t mask[kVoxMaxLayers / 32];
+// The 32 x 32 bit matrix of the lanes' words, transposed.
+__device__ __forceinline__ uint32_t vox_transpose(uint32_t x, int lane) {
+    const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
 #pragma unroll
-    for (int q = 0; q < kVoxMaxLayers / 32; ++q) mask[q] = 0;
+    for (int i = 0; i < 5; ++i) {
+        const int s = 16 >> i;
+        const uint32_t m = masks[i], y = __shfl_xor_sync(0xFFFFFFFFu, x, s);
+        x = lane & s ? (x & ~m) | ((y >> s) & m) : (x & m) | ((y & m) << s);
+    }
+    return x;
+}
+
+// Level 0.  In an 8^3 tile a word holds 4 x 4 columns of 2 layers (voxel bits
+// x0 y0 z0 x1 y1), so a warp takes two blocks of 4 x 4 columns beside each
+// other in x, a column per lane in bit order (x0 y0 x1 y1, then the block).
+// Each lane gathers its column's layers as a mask of NQ words; a transposition
+// across the warp then gives lane k the 32 columns' bits of layer 32 q + k, and
+// a pair of lanes two layers, of which the even one writes the first block's
+// word and the odd one the second's.  Words are written whole: no atomics, and
+// no clearing first.  Warps (pi, bj): tile column pi0 + .., block row bj0 + ...
+//
+// Bound by instruction issue (about 35 a cell and warp, for slabs mostly).  One
+// thread per column with a loop over layers and an atomic per word took 920 us
+// on 2048 x 16384 cells at (4, 8, 2), against 20 us to read the cells; now 100.
+template <int NQ>
+__global__ void __launch_bounds__(128)
+    k_vox_level0(const WorldDev w, const VoxelDev v, int32_t pi0, int32_t bj0, int32_t npi,
+                 int32_t n_warps) {
+    const int32_t warp = (int32_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (warp >= n_warps) return;
+    const int lane = threadIdx.x & 31;
+    const int32_t pi = pi0 + warp % npi, bj = bj0 + warp / npi;
+    const int32_t i = pi * 8 + (lane >> 4) * 4 + (lane & 1) + ((lane >> 1) & 2);
+    const int32_t j = bj * 4 + ((lane >> 1) & 1) + ((lane >> 2) & 2);
     const int32_t nz = v.nz[0];
-    for (int32_t y = j * v.vy; y < min((j + 1) * v.vy, w.H); ++y)
-        for (int32_t x = i * v.vx; x < min((i + 1) * v.vx, w.W); ++x) {
-            const uint32_t node = level0_node(w, x, y);
+    const uint32_t recip = (1u << 20) / (uint32_t)v.vz + 1;
+    uint32_t mask[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) mask[q] = 0;
+    if (i < v.nx[0] && j < v.ny[0]) {
+        int32_t floor_max = 0;
+        auto add = [&](uint32_t node) {
             const int32_t h0 = node & 0xFF, h1 = (node >> 8) & 0xFF, h2 = (node >> 16) & 0xFF;
-            // floor: layers k with k vz <= h0; slab: h1 <= (k+1) vz and k vz <= h2
-            int32_t ka = 0, kb = min(h0 / v.vz, nz - 1);
-            for (int pass = 0; pass < 2; ++pass) {
-                for (int32_t k = ka; k <= kb; ++k) mask[k >> 5] |= 1u << (k & 31);
-                if (pass == 0) {
-                    if (h2 <= h0) break;  // no slab (node form: slab iff top > floor)
-                    ka = max(0, (h1 + v.vz - 1) / v.vz - 1);
-                    kb = min(h2 / v.vz, nz - 1);
-                }
+            // floor: layers k with k vz <= h0 (the highest floor's hold all);
+            // slab: h1 <= (k+1) vz and k vz <= h2
+            floor_max = max(floor_max, h0);
+            if (h2 > h0) {  // node form: slab iff top > floor
+                const int32_t ka = max(vox_div(h1 + v.vz - 1, recip) - 1, 0);
+                const int32_t kb = min(vox_div(h2, recip), nz - 1);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) mask[q] |= vox_bits(ka, kb, q);
             }
+        };
+        const int32_t x0 = i * v.vx, x1 = min(x0 + v.vx, w.W);
+        const int32_t y1 = min((j + 1) * v.vy, w.H);
+        if (v.vx == 4 && (w.W & 3) == 0 && !w.pair) {  // one 16-byte load a row
+            for (int32_t y = j * v.vy; y < y1; ++y) {
+                const uint4 c = __ldg(reinterpret_cast<const uint4 *>(
+                    w.base + (uint32_t)y * (uint32_t)w.W + (uint32_t)x0));
+                add(c.x);
+                add(c.y);
+                add(c.z);
+                add(c.w);
+            }
+        } else {
+            for (int32_t y = j * v.vy; y < y1; ++y)
+                for (int32_t x = x0; x < x1; ++x) add(level0_node(w, x, y));
         }
-    const uint32_t xl = (uint32_t)i & 7, yl = (uint32_t)j & 7;
-    const uint32_t base_bit = (xl & 1) | ((yl & 1) << 1) | ((xl & 2) << 2) | ((yl & 2) << 3);
-    const uint32_t word_xy = ((xl >> 2) << 1) | ((yl >> 2) << 2);
-    for (int32_t k = 0; k < nz; k += 2) {  // layers k, k+1: z bit 0 = 0, 1
-        const uint32_t zl = (uint32_t)k & 7;
-        const uint32_t tile = ((uint32_t)(k >> 3) * v.ty[0] + ((uint32_t)j >> 3)) * v.tx[0] + ((uint32_t)i >> 3);
-        const uint32_t wi = word_xy | ((zl >> 1) & 1) | ((zl >> 2) << 3);
-        uint32_t *wp = v.words + v.off[0] + tile * 16 + wi;
-        const uint32_t b0 = (mask[k >> 5] >> (k & 31)) & 1u;
-        const uint32_t b1 = k + 1 < nz ? (mask[(k + 1) >> 5] >> ((k + 1) & 31)) & 1u : 0u;
-        const uint32_t set = (b0 << base_bit) | (b1 << (base_bit + 4));
-        if (!fresh) atomicAnd(wp, ~((1u << base_bit) | (1u << (base_bit + 4))));
-        if (set) atomicOr(wp, set);
+        const int32_t kb = min(vox_div(floor_max, recip), nz - 1);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) mask[q] |= vox_bits(0, kb, q);
+    }
+    auto spread = [](uint32_t b) {  // nibble g of 16 bits to the low half of byte g
+        b = (b | (b << 8)) & 0x00FF00FFu;
+        return (b | (b << 4)) & 0x0F0F0F0Fu;
+    };
+    const int32_t tz = (nz + 7) >> 3, tj = bj >> 1;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const uint32_t own = vox_transpose(mask[q], lane);
+        const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, own, 1);
+        const uint32_t word = lane & 1 ? spread(other >> 16) | (spread(own >> 16) << 4)
+                                       : spread(own & 0xFFFFu) | (spread(other & 0xFFFFu) << 4);
+        const int32_t z = 32 * q + (lane & ~1);
+        if ((z >> 3) < tz)
+            v.words[v.off[0] + (uint32_t)(((z >> 3) * v.ty[0] + tj) * v.tx[0] + pi) * 16 +
+                    (((z >> 1) & 1) | ((lane & 1) << 1) | ((bj & 1) << 2) | (((z >> 2) & 1) << 3))] =
+                word;
     }
 }
 
-// Level-l words over the tiles that hold columns [i0, i0+ni) x [j0, j0+nj)
-// (every layer): each word's 32 voxels, each the OR of its eight level-(l-1)
-// children, stored whole.
-__global__ void k_vox_up(const VoxelDev v, int l, int32_t ti0, int32_t tj0, int32_t nti,
-                         int32_t ntj) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int32_t ntz = (v.nz[l] + 7) >> 3;
-    if (t >= (int64_t)nti * ntj * ntz * 16) return;
-    const uint32_t wi = (uint32_t)(t & 15);
-    const int64_t tt = t >> 4;
-    const int32_t tx = ti0 + (int32_t)(tt % nti), ty = tj0 + (int32_t)((tt / nti) % ntj),
-                  tz = (int32_t)(tt / ((int64_t)nti * ntj));
+// One word of level l >= 1, tile (tx, ty, tz) and word wi = Z1 X2 Y2 Z2 (lowest
+// first): its voxels' children fill the eight consecutive words Z1 * 8 .. of
+// child tile 2 t + (X2, Y2, Z2), child word c = Z0 X1 Y1, in whose byte X0 Y0
+// lie the eight children of one voxel.  So nibble c of the word says which
+// bytes of child word c are not zero.
+__device__ __forceinline__ void vox_up_word(const VoxelDev &v, int l, int32_t tx, int32_t ty,
+                                            int32_t tz, uint32_t wi) {
+    const int32_t cx = 2 * tx + ((wi >> 1) & 1), cy = 2 * ty + ((wi >> 2) & 1),
+                  cz = 2 * tz + (wi >> 3);
     uint32_t word = 0;
-    for (uint32_t bit = 0; bit < 32; ++bit) {
-        const uint32_t m = (wi << 5) | bit;
-        const int32_t x = tx * 8 + (int32_t)((m & 1) | ((m >> 2) & 2) | ((m >> 4) & 4));
-        const int32_t y = ty * 8 + (int32_t)(((m >> 1) & 1) | ((m >> 3) & 2) | ((m >> 5) & 4));
-        const int32_t z = tz * 8 + (int32_t)(((m >> 2) & 1) | ((m >> 4) & 2) | ((m >> 6) & 4));
-        if (x >= v.nx[l] || y >= v.ny[l] || z >= v.nz[l]) continue;
-        bool occ = false;
-        for (int c = 0; c < 8 && !occ; ++c) {
-            const int32_t cx = 2 * x + (c & 1), cy = 2 * y + ((c >> 1) & 1), cz = 2 * z + (c >> 2);
-            if (cx < v.nx[l - 1] && cy < v.ny[l - 1] && cz < v.nz[l - 1])
-                occ = vox_occupied(v, l - 1, cx, cy, cz);
+    if (cx < v.tx[l - 1] && cy < v.ty[l - 1] && cz < ((v.nz[l - 1] + 7) >> 3)) {
+        // (not the read-only path: the words may be this kernel's own)
+        const uint4 *p = reinterpret_cast<const uint4 *>(
+            v.words + v.off[l - 1] + (uint32_t)((cz * v.ty[l - 1] + cy) * v.tx[l - 1] + cx) * 16 +
+            (wi & 1) * 8);
+        const uint4 a = __ldcg(p), b = __ldcg(p + 1);
+        const uint32_t c[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t any = (((c[k] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | c[k]) >> 7 & 0x01010101u;
+            word |= ((any * 0x01020408u) >> 24 & 0xFu) << (4 * k);
         }
-        word |= (occ ? 1u : 0u) << bit;
     }
-    v.words[v.off[l] + (((uint32_t)tz * v.ty[l] + (uint32_t)ty) * v.tx[l] + (uint32_t)tx) * 16 + wi] = word;
+    v.words[v.off[l] + (uint32_t)((tz * v.ty[l] + ty) * v.tx[l] + tx) * 16 + wi] = word;
+}
+
+// The tiles of a level over level-0 columns [i0, i1) x [j0, j1).
+struct VoxTiles {
+    int32_t x, y, nx, ny, n_words;
+};
+__host__ __device__ __forceinline__ VoxTiles vox_tiles(const VoxelDev &v, int l, int32_t i0,
+                                                       int32_t j0, int32_t i1, int32_t j1) {
+    VoxTiles t;
+    t.x = i0 >> (l + 3);
+    t.y = j0 >> (l + 3);
+    t.nx = ((i1 - 1) >> (l + 3)) - t.x + 1;
+    t.ny = ((j1 - 1) >> (l + 3)) - t.y + 1;
+    t.n_words = t.nx * t.ny * ((v.nz[l] + 7) >> 3) * 16;
+    return t;
+}
+
+__device__ __forceinline__ void vox_up_index(const VoxelDev &v, int l, const VoxTiles &t, int32_t n) {
+    const int32_t tile = n >> 4;
+    vox_up_word(v, l, t.x + tile % t.nx, t.y + (tile / t.nx) % t.ny, tile / (t.nx * t.ny),
+                (uint32_t)n & 15);
+}
+
+__global__ void __launch_bounds__(256) k_vox_up(const VoxelDev v, int l, const VoxTiles t) {
+    const int32_t n = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (n < t.n_words) vox_up_index(v, l, t, n);
+}
+
+// Levels l_from.. of a small region in one block (its own writes are visible to
+// it after a barrier).
+__global__ void __launch_bounds__(kVoxTailThreads)
+    k_vox_tail(const VoxelDev v, int l_from, int32_t i0, int32_t j0, int32_t i1, int32_t j1) {
+    for (int l = l_from; l < v.levels; ++l) {
+        const VoxTiles t = vox_tiles(v, l, i0, j0, i1, j1);
+        for (int32_t n = threadIdx.x; n < t.n_words; n += blockDim.x) vox_up_index(v, l, t, n);
+        __syncthreads();
+    }
 }
 
 __global__ void __launch_bounds__(kVoxThreads) k_vox_trace(const RenderParams p, const VoxelDev v,
@@ -304,23 +381,27 @@ __global__ void __launch_bounds__(kVoxThreads) k_vox_trace(const RenderParams p,
 }  // namespace
 
 int voxel_repair(const WorldDev &w, const VoxelDev &v, int32_t x0, int32_t y0, int32_t x1,
-                 int32_t y1, bool fresh, void *stream) {
+                 int32_t y1, void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
     if (x1 <= x0 || y1 <= y0) return 0;
-    int32_t i0 = x0 / v.vx, i1 = (x1 - 1) / v.vx + 1, j0 = y0 / v.vy, j1 = (y1 - 1) / v.vy + 1;
+    const int32_t i0 = x0 / v.vx, i1 = (x1 - 1) / v.vx + 1, j0 = y0 / v.vy, j1 = (y1 - 1) / v.vy + 1;
     {
-        const int32_t n = (i1 - i0) * (j1 - j0);
-        k_vox_level0<<<(n + 127) / 128, 128, 0, s>>>(w, v, i0, j0, i1 - i0, j1 - j0, fresh ? 1 : 0);
+        const int32_t pi0 = i0 >> 3, npi = ((i1 - 1) >> 3) - pi0 + 1;
+        // block rows in pairs at the grid's end: a tile's rows past it are written too
+        const int32_t bj0 = j0 >> 2, bj1 = j1 == v.ny[0] ? 2 * v.ty[0] : ((j1 - 1) >> 2) + 1;
+        const int32_t n = npi * (bj1 - bj0), blocks = (n + 3) / 4;
+        const int nq = (v.nz[0] + 31) / 32;
+        if (nq > 4) k_vox_level0<8><<<blocks, 128, 0, s>>>(w, v, pi0, bj0, npi, n);
+        else if (nq > 2) k_vox_level0<4><<<blocks, 128, 0, s>>>(w, v, pi0, bj0, npi, n);
+        else k_vox_level0<2><<<blocks, 128, 0, s>>>(w, v, pi0, bj0, npi, n);
     }
-    for (int l = 1; l < v.levels; ++l) {
-        i0 >>= 1;
-        j0 >>= 1;
-        i1 = (i1 + 1) >> 1;
-        j1 = (j1 + 1) >> 1;
-        const int32_t ti0 = i0 >> 3, tj0 = j0 >> 3, ti1 = (i1 + 7) >> 3, tj1 = (j1 + 7) >> 3;
-        const int64_t n = (int64_t)(ti1 - ti0) * (tj1 - tj0) * ((v.nz[l] + 7) >> 3) * 16;
-        k_vox_up<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(v, l, ti0, tj0, ti1 - ti0, tj1 - tj0);
+    int l = 1;
+    for (; l < v.levels; ++l) {
+        const VoxTiles t = vox_tiles(v, l, i0, j0, i1, j1);
+        if (t.n_words <= kVoxTailWords) break;
+        k_vox_up<<<(t.n_words + 255) / 256, 256, 0, s>>>(v, l, t);
     }
+    if (l < v.levels) k_vox_tail<<<1, kVoxTailThreads, 0, s>>>(v, l, i0, j0, i1, j1);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
