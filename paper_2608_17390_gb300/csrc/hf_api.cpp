@@ -1384,14 +1384,13 @@ int hf_render_voxel(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outpu
     q.inner = (int32_t)(o.inner ? o.inner : 4);
     q.far_dist = o.far_dist != 0.0f ? o.far_dist : 600.0f;
     if (o.outer > 1u << 20 || o.inner > 4096 || !(q.far_dist > 0.0f)) return HF_E_INVALID_ARG;
-    uint32_t maxpix = 0;
-    for (uint32_t i = 0; i < n; ++i) maxpix = std::max(maxpix, cams[i].w * cams[i].h);
     Batch b;
     int rc = prepare_batch(c, cams, n, outs, 8, 4, false, o.cuda_stream, b);
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
     CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));
-    if (hf::launch_voxel_trace(b.p, c->vd, q, n, maxpix, b.stream)) return HF_E_CUDA;
+    const uint32_t most = *std::max_element(b.tiles.begin(), b.tiles.end());
+    if (hf::launch_voxel_trace(b.p, c->vd, q, n, most, b.stream)) return HF_E_CUDA;
     return finish_batch(c, b, (o.flags & HF_SYNC) != 0);
 }
 

@@ -183,7 +183,7 @@ struct VoxelParams {
 int voxel_repair(const WorldDev &w, const VoxelDev &v, int32_t x0, int32_t y0, int32_t x1,
                  int32_t y1, void *stream);
 int launch_voxel_trace(const RenderParams &p, const VoxelDev &v, const VoxelParams &q,
-                       uint32_t n_cams, uint32_t max_pixels, void *stream);
+                       uint32_t n_cams, uint32_t max_tiles, void *stream);  // tiles of 8 x 4 pixels
 
 // Launch wrappers (hf_trace.cu)
 // How the trace kernels follow rays: warps of rays in beams; one ray at a time
