@@ -1255,9 +1255,11 @@ int hf_render_scatter(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_foo
     sp.nu = o.nu ? o.nu : 1024;
     sp.nv = o.nv ? o.nv : 1024;
     sp.nz = o.nz ? o.nz : 16;
-    sp.depth_max = o.depth_max != 0.0f ? o.depth_max : 1024.0f;
+    const float depth_max = o.depth_max != 0.0f ? o.depth_max : 1024.0f;
+    sp.qscale = 16777215.0f / depth_max;  // 2^24 - 1 steps
+    sp.per_step = depth_max / 16777215.0f;
     sp.raw = (o.flags & HF_SCATTER_RAW) ? 1 : 0;
-    if (sp.nu > 8192 || sp.nv > 8192 || sp.nz < 2 || sp.nz > 4096 || !(sp.depth_max > 0.0f))
+    if (sp.nu > 8192 || sp.nv > 8192 || sp.nz < 2 || sp.nz > 4096 || !(depth_max > 0.0f))
         return HF_E_INVALID_ARG;
     int32_t sun[3] = {o.sun[0], o.sun[1], o.sun[2]};
     if (sun[0] == 0 && sun[1] == 0 && sun[2] == 0)

@@ -155,7 +155,7 @@ int march_occupancy(int *blocks_per_sm);
 struct ScatterParams {
     uint32_t nu, nv, nz;     // footprint samples across and along; points per column interval
     uint32_t max_pixels;     // largest w * h of the batch
-    float depth_max;         // depth quantisation range (world units)
+    float qscale, per_step;  // depth steps per world unit, world units per step (rounded quotients)
     uint32_t colour[8];      // resolved colour per material (an up-facing, lit surface)
     int32_t raw;             // 1: leave the packed words in hit_cell, no resolve
 };
