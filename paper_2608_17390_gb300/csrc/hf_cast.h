@@ -394,9 +394,11 @@ HF_HD float beam_slack(const Beam &m, float x) {
 }
 
 // Whether the beam may meet a solid in mirrored columns [j 2^l, (j + 1) 2^l).
-// The rows it covers there are read as nodes of level l.
+// The rows it covers there are read as nodes of level l.  high: their highest top.
 template <bool PAIR>
-HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int key) {
+HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int key,
+                     uint32_t &high) {
+    high = 0;
     const LevelDev lv = lvt[l];
     const bool x_major = key & 4;
     const uint32_t nu = x_major ? lv.stride : lv.rows, nv = x_major ? lv.rows : lv.stride;
@@ -426,10 +428,12 @@ HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int k
         h0 = h0 > (w & 0xFF) ? h0 : (w & 0xFF);
         h1 = h1 < (w & 0xFF00) ? h1 : (w & 0xFF00);
     }
-    return !(zlo > (float)(top >> 16) || (zlo > (float)h0 && zhi < (float)(h1 >> 8)));
+    high = top >> 16;
+    return !(zlo > (float)high || (zlo > (float)h0 && zhi < (float)(h1 >> 8)));
 }
 
-// A ray on its way through columns up to x1 (relative to the beam's cell).
+// A ray on its way through the columns of a run, up to x1 (columns x, rows and
+// heights are relative to the beam's cell).
 //
 // Rows: v is off by less than ev = (x1 + |pu| + |pv| + 1) 1.5 2^-22: rho by
 // 2^-23 of itself, x - pu and the sum by 2^-24, and |rho| <= 1.  Where v is
@@ -439,22 +443,22 @@ HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int k
 struct BeamWalk {
     float pu, pv;
     float ev, e2;
+    float zbase;     // z0 - e2 / 2
     float zl;        // lower bound of the height where the column is entered
-    int32_t x, row;  // the column, and the row it is entered in
-    uint32_t cell;   // real index y W + x of that cell
+    int32_t row;     // the row it is entered in
 };
 
 enum { kBeamGoing = 0, kBeamOpen = 1, kBeamLeft = 2, kBeamCorner = 3 };
 
-// The row (relative to m.v0) of a ray as it enters column x of the beam, from
-// its v there.  False if it enters through a corner.
-HF_HD bool beam_row(const BeamDir &d, const BeamRay &q, const Beam &m, int32_t x, float v,
-                    float ev, int32_t &row) {
-    const float f = floorf(v);
+// The row (relative to m.v0) in which a ray enters column x of the beam.  False
+// if it enters through a corner.
+HF_HD bool beam_row(const BeamDir &d, const BeamRay &q, const Beam &m, const BeamWalk &w,
+                    int32_t x, float dx, int32_t &row) {
+    const float v = fmaf(d.rho, dx, w.pv), f = floorf(v);
     row = (int32_t)f;
-    if (fabsf(v - f - 0.5f) < 0.5f - ev) return true;
-    // which of the ray's crossings of boundary row (the nearest) and of column
-    // x comes first
+    if (fabsf(v - f - 0.5f) < 0.5f - w.ev) return true;
+    // which of the ray's crossings of the nearest row boundary and of column x
+    // comes first
     row = (int32_t)floorf(v + 0.5f);
     const int64_t side = (int64_t)((m.v0 + row) * (1 << kShift) + q.kv) * d.du;
     const int64_t here = (int64_t)((m.u0 + x) * (1 << kShift) + q.ku) * d.dv;
@@ -462,31 +466,23 @@ HF_HD bool beam_row(const BeamDir &d, const BeamRay &q, const Beam &m, int32_t x
     return side != here;
 }
 
-// Places a ray at the mirrored column b0, or at its start if that lies beyond.
-// False if it enters through a corner.
-HF_HD bool beam_enter(const BeamDir &d, const BeamRay &q, const Beam &m, int32_t b0, int32_t b1,
-                      uint32_t W, BeamWalk &w) {
+// Places a ray at column x0 of the run [x0, x1), or at its start if that lies
+// beyond.  False if it enters through a corner.
+HF_HD bool beam_enter(const BeamDir &d, const BeamRay &q, const Beam &m, int32_t x0, int32_t x1,
+                      BeamWalk &w) {
     w.pu = beam_pu(q, m);
     w.pv = beam_pv(q, m);
-    const float x1 = (float)(b1 - m.u0);
-    w.ev = (x1 + fabsf(w.pu) + fabsf(w.pv) + 1.0f) * (1.5f / 4194304.0f);
-    const float e = (fabsf(d.sigma) * (x1 + fabsf(w.pu) + 2.0f) + fabsf(q.z0)) * (1.0f / 2097152.0f);
+    const float apu = fabsf(w.pu), far = (float)x1 + apu;
+    w.ev = (far + fabsf(w.pv) + 1.0f) * (1.5f / 4194304.0f);
+    const float e = (fabsf(d.sigma) * (far + 2.0f) + fabsf(q.z0)) * (1.0f / 2097152.0f);
     w.e2 = 2.0f * e;
-    bool sure = true;
-    if (q.fu >= b0) {
-        w.x = q.fu - m.u0;
-        w.row = q.fv - m.v0;
-        w.zl = fabsf(q.z0) < 256.0f ? q.z0 : q.z0 - e;  // (a start below 256 is exact)
-    } else {
-        w.x = b0 - m.u0;
-        const float dx = (float)w.x - w.pu;
-        sure = beam_row(d, q, m, w.x, fmaf(d.rho, dx, w.pv), w.ev, w.row);
-        w.zl = fmaf(d.sigma, dx, q.z0) - e;
-    }
-    const int32_t u = m.u0 + w.x, v = m.v0 + w.row;
-    const uint32_t ru = (uint32_t)(d.key & 2 ? ~u : u), rv = (uint32_t)(d.key & 1 ? ~v : v);
-    w.cell = d.key & 4 ? rv * W + ru : ru * W + rv;
-    return sure;
+    w.zbase = q.z0 - e;
+    w.row = q.fv - m.v0;
+    w.zl = fabsf(q.z0) < 256.0f ? q.z0 : w.zbase;  // (a start below 256 is exact)
+    if (q.fu - m.u0 >= x0) return true;
+    const float dx = (float)x0 - w.pu;
+    w.zl = fmaf(d.sigma, dx, w.zbase);
+    return beam_row(d, q, m, w, x0, dx, w.row);
 }
 
 // Word of cell index y W + x (pairs lie in one word: W is even).
@@ -495,58 +491,57 @@ HF_HD uint32_t beam_word(const uint32_t *cells, uint32_t cell) {
     return PAIR ? pair_node(cast_load(cells + (cell >> 1)), cell & 1) : cast_load(cells + cell);
 }
 
-// Where a walk's column is left: the row, and a lower bound of the height.
-HF_HD bool beam_exit(const BeamDir &d, const BeamRay &q, const Beam &m, const BeamWalk &w,
-                     int32_t &row, float &zl) {
-    const float dx = (float)(w.x + 1) - w.pu;
-    zl = fmaf(d.sigma, dx, q.z0) - 0.5f * w.e2;
-    return beam_row(d, q, m, w.x + 1, fmaf(d.rho, dx, w.pv), w.ev, row);
+// How mirrored rows and columns relative to the beam's cell lie in the grid:
+// cell (x, row) has index at + x step_u + row step_v, and rows from `rows` on
+// lie past the grid.
+struct BeamGrid {
+    const uint32_t *cells;
+    uint32_t at;
+    int32_t step_u, step_v, rows;
+};
+HF_HD BeamGrid beam_grid(const uint32_t *cells, const Beam &m, int key, uint32_t W, uint32_t H) {
+    BeamGrid g;
+    const bool x_major = key & 4;
+    const uint32_t ru = (uint32_t)(key & 2 ? ~m.u0 : m.u0), rv = (uint32_t)(key & 1 ? ~m.v0 : m.v0);
+    g.cells = cells;
+    g.at = x_major ? rv * W + ru : ru * W + rv;
+    g.step_u = (key & 2 ? -1 : 1) * (x_major ? 1 : (int32_t)W);
+    g.step_v = (key & 1 ? -1 : 1) * (x_major ? (int32_t)W : 1);
+    g.rows = (key & 1 ? 0 : (int32_t)(x_major ? H : W)) - m.v0;
+    return g;
 }
 
-HF_HD void beam_pass(BeamWalk &w, int32_t row, float zl, int32_t cell_u, int32_t cell_v) {
-    w.cell += (uint32_t)(cell_u + (row > w.row ? cell_v : 0));
-    w.x += 1;
-    w.row = row;
-    w.zl = zl;
-}
-
-// One column of a walk, whose one or two cells are tested together: past it if
-// they are empty (kBeamGoing).  kBeamOpen: they may not be; kBeamLeft: the ray
-// has left the grid sideways; kBeamCorner: it leaves through a corner.  rows:
-// the row past the grid.  cell_u, cell_v: what a step along u, v adds to the
-// cell index.
+// Column x of a walk, whose one or two cells are tested together.  row, zl:
+// where it is left (in and out of the walk: the caller moves on with them).
+// kBeamGoing: the cells are empty; kBeamOpen: they may not be; kBeamLeft: the
+// ray has left the grid sideways; kBeamCorner: it leaves through a corner.
 template <bool PAIR>
-HF_HD int beam_step(const uint32_t *cells, const BeamDir &d, const BeamRay &q, const Beam &m,
-                    BeamWalk &w, int32_t rows, int32_t cell_u, int32_t cell_v) {
-    if (w.row >= rows) return kBeamLeft;
-    int32_t row;
-    float zl;
-    const bool sure = beam_exit(d, q, m, w, row, zl);
-    const uint32_t wa = beam_word<PAIR>(cells, w.cell);
-    const uint32_t wb = beam_word<PAIR>(
-        cells, w.cell + (uint32_t)(row > w.row && row < rows ? cell_v : 0));
+HF_HD int beam_step(const BeamGrid &g, const BeamDir &d, const BeamRay &q, const Beam &m,
+                    const BeamWalk &w, int32_t x, int32_t &row, float &zl) {
+    if (w.row >= g.rows) return kBeamLeft;
+    const float dx = (float)(x + 1) - w.pu;
+    zl = fmaf(d.sigma, dx, w.zbase);
+    const bool sure = beam_row(d, q, m, w, x + 1, dx, row);
+    const uint32_t ca = g.at + (uint32_t)(x * g.step_u + w.row * g.step_v);
+    const uint32_t cb = ca + (uint32_t)(row > w.row && row < g.rows ? g.step_v : 0);
+    const uint32_t wa = beam_word<PAIR>(g.cells, ca), wb = beam_word<PAIR>(g.cells, cb);
     const uint32_t ta = wa & 0xFF0000, tb = wb & 0xFF0000;
     const uint32_t fa = wa & 0xFF, fb = wb & 0xFF, ma = wa & 0xFF00, mb = wb & 0xFF00;
     const float top = (float)((ta > tb ? ta : tb) >> 16), h0 = (float)(fa > fb ? fa : fb);
     const float h1 = (float)((ma < mb ? ma : mb) >> 8);
     const float zlo = fminf(w.zl, zl), zhi = fmaxf(w.zl, zl) + w.e2;
     if (!sure) return kBeamCorner;
-    if (!((zlo > top) | ((zlo > h0) & (zhi < h1)))) return kBeamOpen;
-    beam_pass(w, row, zl, cell_u, cell_v);
-    return kBeamGoing;
+    return (zlo > top) | ((zlo > h0) & (zhi < h1)) ? kBeamGoing : kBeamOpen;
 }
 
-// Decides the column that beam_step left open, on exact rationals: true and h
-// filled, or false and the ray past it.
+// Decides a column that beam_step left open, on exact rationals: true and h
+// filled, or false.  row: where the ray leaves it.
 template <bool PAIR>
-HF_HD bool beam_settle(const uint32_t *cells, int32_t oz, int32_t dz, const BeamDir &d,
-                       const BeamRay &q, const Beam &m, BeamWalk &w, int32_t rows, int32_t cell_u,
-                       int32_t cell_v, Hit &h) {
-    int32_t row;
-    float zl;
-    beam_exit(d, q, m, w, row, zl);
+HF_HD bool beam_settle(const BeamGrid &g, int32_t oz, int32_t dz, const BeamDir &d,
+                       const BeamRay &q, const Beam &m, const BeamWalk &w, int32_t x, int32_t row,
+                       Hit &h) {
     const bool x_major = d.key & 4;
-    const int32_t u = m.u0 + w.x;
+    const int32_t u = m.u0 + x;
     const bool start = u == q.fu;
     const int32_t end = (u + 1) * (1 << kShift) + q.ku;               // over du: the column's exit
     const int32_t side = (m.v0 + w.row + 1) * (1 << kShift) + q.kv;   // over dv: the row's
@@ -554,11 +549,11 @@ HF_HD bool beam_settle(const uint32_t *cells, int32_t oz, int32_t dz, const Beam
     uint8_t face = start ? kFaceInside
                    : x_major ? (d.key & 2 ? kFacePX : kFaceNX)
                              : (d.key & 2 ? kFacePY : kFaceNY);
-    uint32_t cell = w.cell;
+    uint32_t cell = g.at + (uint32_t)(x * g.step_u + w.row * g.step_v);
     int32_t v = m.v0 + w.row;
     for (bool second = false;; second = true) {
         const bool last = second || row == w.row;
-        const uint32_t word = beam_word<PAIR>(cells, cell);
+        const uint32_t word = beam_word<PAIR>(g.cells, cell);
         if (leaf_test(oz, dz, word, num, den, last ? end : side, last ? d.du : d.dv, face, h)) {
             const int32_t ru = d.key & 2 ? ~u : u, rv = d.key & 1 ? ~v : v;
             h.cx = x_major ? ru : rv;
@@ -566,15 +561,13 @@ HF_HD bool beam_settle(const uint32_t *cells, int32_t oz, int32_t dz, const Beam
             h.word = word;
             return true;
         }
-        if (last || row >= rows) break;
+        if (last || row >= g.rows) return false;
         num = side;
         den = d.dv;
         face = x_major ? (d.key & 1 ? kFacePY : kFaceNY) : (d.key & 1 ? kFacePX : kFaceNX);
-        cell += (uint32_t)cell_v;
+        cell += (uint32_t)g.step_v;
         v += 1;
     }
-    beam_pass(w, row, zl, cell_u, cell_v);
-    return false;
 }
 
 // The order in which a beam's columns are tested: rounds of 32 stretches of

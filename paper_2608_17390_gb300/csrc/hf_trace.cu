@@ -22,15 +22,17 @@
 #include <mutex>
 
 #include "hf.h"
-#include "hf_cast.h"
+#include "hf_beam.h"
 #include "hf_internal.h"
 
 namespace hf {
 namespace {
 
-#ifndef HF_TRACE_MIN_BLOCKS
-#define HF_TRACE_MIN_BLOCKS 7  // resident 128-thread blocks per SM asked of the register allocator (72 registers)
-#endif
+// Resident 128-thread blocks per SM asked of the register allocator: six leave
+// each thread 80 registers.  64 views with shadows / a 1080p eye-level view:
+// five blocks 9.77 ms / 138 us, six 9.63 / 132, seven (72 registers, more
+// address arithmetic) 10.22 / 136, eight 10.25 / 140.
+constexpr int kTraceMinBlocks = 6;
 
 __constant__ float c_albedo[8][3] = HF_ALBEDO_TABLE;
 constexpr float kKa = kAmbient, kKd = kDiffuse;
@@ -91,33 +93,18 @@ __device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visi
     return out;
 }
 
-constexpr uint32_t kFull = 0xFFFFFFFFu;
-
-__device__ __forceinline__ float warp_min(float v) {
-    float r;
-    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-__device__ __forceinline__ float warp_max(float v) {
-    float r;
-    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
-
 // Casts one ray per active lane; every lane of the warp calls.
 //
-// The rays that go the same way (axis of the larger component and both signs)
-// and start side by side form a beam.  Its 32 next stretches of columns are
-// tested by the 32 lanes at once, each against the one to three nodes that the
-// beam covers there; then the rays are walked, all together, through the
-// stretches that are not proven empty until they have hit or left.  One ray at
-// a time, the same empty space costs every lane 15 to 25 dependent node visits;
-// here it costs the warp one or two rounds.
+// The rays that go the same way and start side by side form a beam (hf_beam.h);
+// they are walked, all together, through the runs of columns that it does not
+// prove empty, until they have hit or left.  One ray at a time, the same empty
+// space costs every lane 15 to 25 dependent node visits; here it costs the warp
+// one or two rounds.
 //
 // Bound by instruction issue, as the traversal of single rays was: 2048 x 2048
-// grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 10.03
-// ms, a 1080p eye-level view with shadows 192 -> 134 us, a hundred 1080p frames
-// over 2048 x 16384 cells 17.3 -> 10.4 ms.
+// grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 9.63
+// ms, a 1080p eye-level view with shadows 192 -> 132 us, a hundred 1080p frames
+// over 2048 x 16384 cells 17.3 -> 10.2 ms.
 template <bool PAIR>
 __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev *lvt,
                                            const Ray &r, const BeamDir &d, bool active, int mip,
@@ -133,86 +120,45 @@ __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev
     active = active && !alone && (uint32_t)(d.key & 2 ? ~q.fu : q.fu) < (d.key & 4 ? W : H) &&
              (uint32_t)(d.key & 1 ? ~q.fv : q.fv) < (d.key & 4 ? H : W);
     uint32_t todo = __ballot_sync(kFull, active);
-    const int base_level = min(kBeamLevel, mip), top_level = min(kBeamTop, mip);
     while (todo) {
         // the first ray left, and the rays that go its way beside it
         const int lead = __ffs(todo) - 1;
-        const int key = __shfl_sync(kFull, d.key, lead);
-        Beam m;
-        m.u0 = __shfl_sync(kFull, q.fu, lead);
-        m.v0 = __shfl_sync(kFull, q.fv, lead);
-        bool alive = (todo >> lane & 1) && d.key == key &&
-                     fabsf(beam_pv(q, m) - d.rho * beam_pu(q, m)) <= kBeamSpread;
+        BeamScan s;
+        s.key = __shfl_sync(kFull, d.key, lead);
+        s.m.u0 = __shfl_sync(kFull, q.fu, lead);
+        s.m.v0 = __shfl_sync(kFull, q.fv, lead);
+        bool alive = (todo >> lane & 1) && d.key == s.key &&
+                     fabsf(beam_pv(q, s.m) - d.rho * beam_pu(q, s.m)) <= kBeamSpread;
         todo &= ~__ballot_sync(kFull, alive);
-        m.u0 = __reduce_min_sync(kFull, alive ? q.fu : 0x7FFFFFFF);
-        const int32_t limit = key & 2 ? 0 : (int32_t)(key & 4 ? W : H);
-        const int32_t rows = (key & 1 ? 0 : (int32_t)(key & 4 ? H : W)) - m.v0;
-        const int32_t cell_u = (key & 2 ? -1 : 1) * (key & 4 ? 1 : (int32_t)W);
-        const int32_t cell_v = (key & 1 ? -1 : 1) * (key & 4 ? (int32_t)W : 1);
-        const float top = (float)((cast_load(lvt[p.world.L].base) >> 16) & 0xFF);
-        int32_t u = m.u0;
-        int level = base_level;
-        while (u < limit) {
-            {  // the beam of the rays that are left
-                const float big = 3.0e38f, pu = beam_pu(q, m);
-                const float a = beam_pv(q, m) - d.rho * pu, b = q.z0 - d.sigma * pu;
-                m.a0 = warp_min(alive ? a : big);
-                m.a1 = warp_max(alive ? a : -big);
-                m.r0 = warp_min(alive ? d.rho : big);
-                m.r1 = warp_max(alive ? d.rho : -big);
-                m.b0 = warp_min(alive ? b : big);
-                m.b1 = warp_max(alive ? b : -big);
-                m.s0 = warp_min(alive ? d.sigma : big);
-                m.s1 = warp_max(alive ? d.sigma : -big);
+        s.m.u0 = __reduce_min_sync(kFull, alive ? q.fu : 0x7FFFFFFF);
+        beam_scan(s, p.world, lvt, mip);
+        const BeamGrid g = beam_grid(cells, s.m, s.key, W, H);
+        int32_t b0, b1;
+        while (beam_next<PAIR>(s, lvt, d, q, alive, b0, b1)) {
+            const int32_t x1 = b1 - s.m.u0;
+            int32_t x = b0 - s.m.u0;
+            BeamWalk w;
+            if (!beam_enter(d, q, s.m, x, x1, w) && alive) {
+                alone = true;
+                alive = false;
             }
-            u = beam_skip(m, u, limit, top);
-            if (u >= limit) break;
-            const int least = beam_least(m, u, base_level, top_level);
-            level = max(level, least);
-            const int32_t j = u >> level;
-            uint32_t open = __ballot_sync(kFull, beam_open<PAIR>(lvt, m, level, j + lane, key));
-            if (level > least && open) {
-                u = max(u, (j + __ffs(open) - 1) * (1 << level));
-                level = least;
-                continue;
-            }
-            const int32_t next = (j + 32) * (1 << level);
-            if (!open) {
-                u = next;
-                level = min(level + 2, top_level);
-                continue;
-            }
+            // column by column, all rays together
             do {
-                const int i = __ffs(open) - 1, run = beam_run(open, i);
-                open &= i + run < 32 ? 0xFFFFFFFFu << (i + run) : 0u;
-                const int32_t b0 = max(u, (j + i) * (1 << level));
-                const int32_t b1 = min((j + i + run) * (1 << level), limit);
-                bool go = alive && q.fu < b1;
-                BeamWalk w;
-                if (go && !beam_enter(d, q, m, b0, b1, W, w)) {
-                    alone = true;
-                    go = alive = false;
-                }
-                while (__any_sync(kFull, go)) {
-                    int at = kBeamGoing;
-                    do {
-                        if (go) {
-                            at = beam_step<PAIR>(cells, d, q, m, w, rows, cell_u, cell_v);
-                            go = at == kBeamGoing && w.x < b1 - m.u0;
-                        }
-                    } while (__any_sync(kFull, go));
+                if (alive && s.m.u0 + x >= q.fu) {
+                    int32_t row;
+                    float zl;
+                    const int at = beam_step<PAIR>(g, d, q, s.m, w, x, row, zl);
                     if (at == kBeamOpen) {
-                        alive = !beam_settle<PAIR>(cells, r.oz, r.dz, d, q, m, w, rows, cell_u,
-                                                   cell_v, h);
-                        go = alive && w.x < b1 - m.u0;
+                        alive = !beam_settle<PAIR>(g, r.oz, r.dz, d, q, s.m, w, x, row, h);
                     } else if (at != kBeamGoing) {
                         alive = false;
                         alone = at == kBeamCorner;
                     }
+                    w.row = row;
+                    w.zl = zl;
                 }
-            } while (open && __any_sync(kFull, alive));
+            } while (__any_sync(kFull, alive) && ++x < x1);
             if (!__any_sync(kFull, alive)) break;
-            u = next;
         }
     }
     if (alone) {
@@ -438,7 +384,7 @@ __device__ __forceinline__ const CamDev &stage_cam(CamDev *slot, const CamDev *c
 // Persistent batched kernel: warps pop (camera, tile) items from one atomic
 // counter until the batch is drained.  One launch renders every camera.
 template <bool SHADOWS, int KIND, bool PAIR>
-__global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS) k_trace_batched(const RenderParams p) {
+__global__ void __launch_bounds__(kThreads, kTraceMinBlocks) k_trace_batched(const RenderParams p) {
     __shared__ uint32_t s_base[kMaxCams + 1];
     __shared__ CamDev s_cam[kThreads / 32];
     __shared__ LevelDev s_lv[kMaxLevels + 1];
@@ -474,7 +420,7 @@ __global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS) k_trace_batched
 // kernel (reading the fields from parameter space instead changes the
 // traversal's register allocation, measured 3-8 % slower on large images).
 template <bool SHADOWS, int KIND, bool PAIR>
-__global__ void __launch_bounds__(kThreads, HF_TRACE_MIN_BLOCKS)
+__global__ void __launch_bounds__(kThreads, kTraceMinBlocks)
     k_trace_plain(const __grid_constant__ RenderParams p, const __grid_constant__ CamDev cam,
                   uint32_t n_tiles) {
     __shared__ LevelDev s_lv[kMaxLevels + 1];

@@ -4,7 +4,7 @@ can be compared without a GPU -- corners, boundaries and grazes on a lattice,
 directions from one unit to the limit on either axis, rays across the largest
 grids, heights to the top of the range, every start level and climb limit,
 and warps of rays from scattered to narrow.  The kernel's loop over a warp
-(cast_beams in csrc/hf_trace.cu) is written out here lane by lane.
+(cast_beams in csrc/hf_trace.cu, beam_next in csrc/hf_beam.h) is written out here lane by lane.
 """
 
 import ctypes
@@ -25,7 +25,7 @@ SHIM = r"""
 #include <algorithm>
 using namespace hf;
 static long beamed = 0;  // rays that a beam decided
-// cast_beams of hf_trace.cu with the lanes of a warp in turn
+// cast_beams of hf_trace.cu and beam_next of hf_beam.h, with the lanes of a warp in turn
 template <bool PAIR>
 static void beams(const LevelDev *lv, int top_level_of_world, const Ray *r, int n, int mip, Hit *h) {
     const uint32_t W = lv[0].stride, H = lv[0].rows, *cells = lv[0].base;
@@ -65,9 +65,7 @@ static void beams(const LevelDev *lv, int top_level_of_world, const Ray *r, int 
                 b[k] = q[k].z0 - d[k].sigma * beam_pu(q[k], m);
             }
         const int32_t limit = key & 2 ? 0 : (int32_t)(key & 4 ? W : H);
-        const int32_t edge = (key & 1 ? 0 : (int32_t)(key & 4 ? H : W)) - m.v0;
-        const int32_t cell_u = (key & 2 ? -1 : 1) * (key & 4 ? 1 : (int32_t)W);
-        const int32_t cell_v = (key & 1 ? -1 : 1) * (key & 4 ? (int32_t)W : 1);
+        const BeamGrid g = beam_grid(cells, m, key, W, H);
         int32_t u = m.u0;
         int level = base_level;
         while (u < limit) {
@@ -89,8 +87,9 @@ static void beams(const LevelDev *lv, int top_level_of_world, const Ray *r, int 
             level = std::max(level, least);
             const int32_t j = u >> level;
             uint32_t open = 0;
+            uint32_t high;
             for (int i = 0; i < 32; ++i)
-                open |= (uint32_t)beam_open<PAIR>(lv, m, level, j + i, key) << i;
+                open |= (uint32_t)beam_open<PAIR>(lv, m, level, j + i, key, high) << i;
             if (level > least && open) {
                 u = std::max(u, (j + __builtin_ctz(open)) * (1 << level));
                 level = least;
@@ -105,18 +104,21 @@ static void beams(const LevelDev *lv, int top_level_of_world, const Ray *r, int 
                 for (int k = 0; k < n; ++k) {
                     if (!alive[k] || q[k].fu >= b1) continue;
                     BeamWalk w;
-                    if (!beam_enter(d[k], q[k], m, b0, b1, W, w)) {
+                    if (!beam_enter(d[k], q[k], m, b0 - m.u0, b1 - m.u0, w)) {
                         alive[k] = false;
                         alone[k] = true;
                     }
-                    while (alive[k] && w.x < b1 - m.u0) {
-                        const int at = beam_step<PAIR>(cells, d[k], q[k], m, w, edge, cell_u,
-                                                       cell_v);
+                    for (int32_t x = std::max(b0, q[k].fu) - m.u0; alive[k] && x < b1 - m.u0; ++x) {
+                        int32_t row = 0;
+                        float zl = 0;
+                        const int at = beam_step<PAIR>(g, d[k], q[k], m, w, x, row, zl);
                         if (at == kBeamOpen)
-                            alive[k] = !beam_settle<PAIR>(cells, r[k].oz, r[k].dz, d[k], q[k], m, w,
-                                                          edge, cell_u, cell_v, h[k]);
+                            alive[k] = !beam_settle<PAIR>(g, r[k].oz, r[k].dz, d[k], q[k], m, w, x, row,
+                                                          h[k]);
                         else if (at != kBeamGoing)
                             alive[k] = false, alone[k] = at == kBeamCorner;
+                        w.row = row;
+                        w.zl = zl;
                     }
                 }
             }
