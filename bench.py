@@ -350,7 +350,8 @@ def run_hf(args):
     else:
         opts = hf.make_opts(flags=flags, mip_start=args.mip, tile_w=args.tile_w,
                             tile_h=args.tile_h)
-    tile_w, tile_h, mip_start = opts.tile_w or 8, opts.tile_h or 4, opts.mip_start
+    opts.tile_w, opts.tile_h = opts.tile_w or 8, opts.tile_h or 4  # (what the line reports)
+    tile_w, tile_h, mip_start = opts.tile_w, opts.tile_h, opts.mip_start
     rng = np.random.default_rng(1234)
     H, W = cells.shape
 

@@ -152,7 +152,8 @@ typedef struct {
 
 typedef struct {
     uint32_t tile_w, tile_h; /* pixels per warp tile (powers of two, product 32..256);
-                                0,0 = default 8 x 4 */
+                                0,0 = default: 8 x 4, or 4 x 8 to 4 x 32 where the
+                                batch fills the GPU several times over */
     uint32_t mip_start;      /* coarsest pyramid level the traversal uses and starts at;
                                 0 = flat cell-by-cell DDA; HF_MIP_AUTO = library default;
                                 larger values are clamped to the pyramid's top level */
@@ -271,7 +272,7 @@ typedef struct {
     uint32_t steps;          /* forward samples over the clipped segment; 0 = 128 */
     uint32_t bisections;     /* bisection iterations after the first solid sample; 0 = 4 */
     float far_dist;          /* far plane distance in world units; 0 = 600 */
-    uint32_t tile_w, tile_h; /* warp tile as in hf_render_opts; 0,0 = 8 x 4 */
+    uint32_t tile_w, tile_h; /* pixels per warp tile as in hf_render_opts; 0,0 = 8 x 4 */
     uint32_t flags;          /* HF_SYNC */
     void *cuda_stream;       /* NULL = the context's stream */
 } hf_march_opts;

@@ -1094,6 +1094,32 @@ static int render_host_staged(hf_ctx *c, const hf_camera *cams, uint32_t n, cons
     return HF_OK;
 }
 
+// The warp tile of a render that leaves its sides at 0.  8 x 4 is one pixel per
+// lane, the most warps: right while a render fills the GPU but a few times over,
+// as its slowest warps decide its end.  Beyond that narrow and tall tiles win:
+// 32 pixels of 4 x 8 go through nearly the same columns of the grid, and longer
+// tiles share one fetch of the tile and of its camera.  Measured over 2048 x 2048
+// and 2048 x 16384 cells (us, 8 x 4 against the choice):
+//   groups of 32 pixels per resident warp   8 x 4    choice
+//   1280 x 720 with shadows       8           81      76  (4 x 8;  4 x 16: 77)
+//   960 x 540 with shadows        4           59      61  (4 x 8, so still 8 x 4)
+//   1920 x 1080 with shadows     18          149     140  (4 x 16; 4 x 32: 142)
+//   4K with shadows              71          517     477  (4 x 32; 4 x 16: 487)
+//   20 views of 1920 x 1080     355         2142    1952  (4 x 32; 4 x 16: 1997)
+// Stores to host memory want wide rows, and the traversal of single rays was
+// tuned on 8 x 4: both keep it.
+static void default_tile(const hf_camera *cams, uint32_t n, bool beams, uint64_t warps,
+                         uint32_t flags, uint32_t &tw, uint32_t &th) {
+    tw = 8;
+    th = 4;
+    if (!beams || (flags & HF_HOST_OUTPUTS)) return;
+    uint64_t groups = 0;
+    for (uint32_t i = 0; i < n; ++i) groups += ((uint64_t)cams[i].w * cams[i].h + 31) / 32;
+    if (groups < 6 * warps) return;
+    tw = 4;
+    th = groups < 16 * warps ? 8 : groups < 64 * warps ? 16 : 32;
+}
+
 int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *outs,
               const hf_render_opts *opts) {
     if (!c) return HF_E_INVALID_ARG;
@@ -1106,7 +1132,7 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         if (o.flags & (HF_HOST_OUTPUTS | HF_PLAIN | HF_NOWAIT)) return HF_E_INVALID_ARG;
         return render_host_staged(c, cams, n, outs, o);
     }
-    const uint32_t tw = o.tile_w ? o.tile_w : 8, th = o.tile_h ? o.tile_h : 4;
+    uint32_t tw = o.tile_w ? o.tile_w : 8, th = o.tile_h ? o.tile_h : 4;
     int32_t sun[3] = {o.sun[0], o.sun[1], o.sun[2]};
     if (sun[0] == 0 && sun[1] == 0 && sun[2] == 0)
         for (int i = 0; i < 3; ++i) sun[i] = kDefaultSun[i];
@@ -1123,6 +1149,10 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
     if (steps > 0x7FFFFFFFu) return HF_E_INVALID_ARG;
     for (uint32_t i = 0; i < n; ++i)  // before anything is built or enqueued
         if (hf_validate_camera(c->W, c->H, &cams[i]) != HF_OK) return HF_E_INVALID_ARG;
+    if (!o.tile_w && !o.tile_h)
+        default_tile(cams, n, kind == hf::kTraceBeams,
+                     (uint64_t)c->sm_count * c->occ[shadows][kind] * (hf::kThreads / 32), o.flags, tw,
+                     th);
     const uint32_t *bounds = nullptr;
     if (shadows) {
         const int brc = ensure_sun_bounds(c, sun, &bounds);
