@@ -1103,6 +1103,7 @@ static int render_host_staged(hf_ctx *c, const hf_camera *cams, uint32_t n, cons
 //   groups of 32 pixels per resident warp   8 x 4    choice
 //   1280 x 720 with shadows       8           81      76  (4 x 8;  4 x 16: 77)
 //   960 x 540 with shadows        4           59      61  (4 x 8, so still 8 x 4)
+//   1920 x 1080                  15          119     113  (4 x 16; 4 x 8: 118)
 //   1920 x 1080 with shadows     18          149     140  (4 x 16; 4 x 32: 142)
 //   4K with shadows              71          517     477  (4 x 32; 4 x 16: 487)
 //   20 views of 1920 x 1080     355         2142    1952  (4 x 32; 4 x 16: 1997)
@@ -1117,7 +1118,7 @@ static void default_tile(const hf_camera *cams, uint32_t n, bool beams, uint64_t
     for (uint32_t i = 0; i < n; ++i) groups += ((uint64_t)cams[i].w * cams[i].h + 31) / 32;
     if (groups < 6 * warps) return;
     tw = 4;
-    th = groups < 16 * warps ? 8 : groups < 64 * warps ? 16 : 32;
+    th = groups < 12 * warps ? 8 : groups < 64 * warps ? 16 : 32;
 }
 
 int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *outs,

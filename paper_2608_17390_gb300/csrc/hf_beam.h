@@ -58,8 +58,8 @@ __device__ __forceinline__ bool beam_next(BeamScan &s, const LevelDev *lvt, cons
     while (!s.open) {
         if (s.u >= s.limit) return false;
         {  // the beam of the rays that are left
-            const float big = 3.0e38f, pu = beam_pu(q, s.m);
-            const float a = beam_pv(q, s.m) - d.rho * pu, b = q.z0 - d.sigma * pu;
+            const float big = 3.0e38f;
+            const float a = q.pv - d.rho * q.pu, b = q.z0 - d.sigma * q.pu;
             s.m.a0 = warp_min(alive ? a : big);
             s.m.a1 = warp_max(alive ? a : -big);
             s.m.r0 = warp_min(alive ? d.rho : big);

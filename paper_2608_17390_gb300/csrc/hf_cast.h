@@ -10,9 +10,8 @@
 //                 next stretches are tested by the 32 lanes at once; rays are
 //                 walked, column by column in float with error bounds, only
 //                 through stretches that the beam does not prove empty.  What
-//                 the bounds leave open is decided exactly: a column that may
-//                 hold a hit on rationals, a ray through a cell corner by
-//                 cast_general.
+//                 the bounds leave open is decided exactly, on rationals, and
+//                 a ray through a cell corner is left to cast_general.
 //
 // The functions are host code too, so that the two can be compared on a CPU.
 #pragma once
@@ -63,6 +62,15 @@ HF_HD uint32_t cast_load(const uint32_t *p) {
 HF_HD float cast_rcp(float v) {
 #ifdef __CUDA_ARCH__
     return __frcp_rn(v);
+#else
+    return 1.0f / v;
+#endif
+}
+
+// 1 / v to a relative 2^-22.
+HF_HD float cast_rcp_fast(float v) {
+#ifdef __CUDA_ARCH__
+    return __fdividef(1.0f, v);
 #else
     return 1.0f / v;
 #endif
@@ -341,6 +349,7 @@ struct BeamRay {
     int32_t fu, fv;  // the start cell, mirrored
     int32_t ku, kv;  // minus the start's mirrored position, in 2^-16 units
     float z0;        // start height
+    float pu, pv;    // the start relative to the beam's cell (beam_place)
 };
 
 // (dx, dy not both 0)
@@ -369,6 +378,12 @@ HF_HD BeamRay beam_ray(const BeamDir &d, const Ray &r) {
     return q;
 }
 
+HF_HD Ray beam_unray(const BeamDir &d, const BeamRay &q, int32_t oz, int32_t dz) {
+    const int32_t ou = d.key & 2 ? q.ku : -q.ku, ov = d.key & 1 ? q.kv : -q.kv;
+    const int32_t eu = d.key & 2 ? -d.du : d.du, ev = d.key & 1 ? -d.dv : d.dv;
+    return d.key & 4 ? Ray{ou, ov, oz, eu, ev, dz} : Ray{ov, ou, oz, ev, eu, dz};
+}
+
 // A beam's rays, relative to the mirrored cell (u0, v0): at u = u0 + x every
 // ray has v - v0 in [a0 + r0 x, a1 + r1 x] and a height between b0 + s0 x and
 // b1 + s1 x, for x >= 0 (up to rounding, see beam_open).
@@ -377,14 +392,12 @@ struct Beam {
     float a0, a1, r0, r1, b0, b1, s0, s1;
 };
 
-// A ray's start relative to the beam's cell: exact up to 256 cells, else
+// Takes a ray's start relative to the beam's cell: exact up to 256 cells, else
 // rounded.  At u0 + x the ray is at v - v0 = pv + rho (x - pu), and at the
 // height z0 + sigma (x - pu); its terms of the beam are those at x = 0.
-HF_HD float beam_pu(const BeamRay &q, const Beam &m) {
-    return (float)(-q.ku - m.u0 * (1 << kShift)) * (1.0f / 65536.0f);
-}
-HF_HD float beam_pv(const BeamRay &q, const Beam &m) {
-    return (float)(-q.kv - m.v0 * (1 << kShift)) * (1.0f / 65536.0f);
+HF_HD void beam_place(BeamRay &q, const Beam &m) {
+    q.pu = (float)(-q.ku - m.u0 * (1 << kShift)) * (1.0f / 65536.0f);
+    q.pv = (float)(-q.kv - m.v0 * (1 << kShift)) * (1.0f / 65536.0f);
 }
 
 // A bound of the error of a beam's heights up to x columns on: slopes have a
@@ -441,7 +454,6 @@ HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int k
 // the corner itself is left to cast_general.
 // Heights: off by less than e2 / 2 = (|sigma| (x1 + |pu| + 2) + |z0|) 2^-21.
 struct BeamWalk {
-    float pu, pv;
     float ev, e2;
     float zbase;     // z0 - e2 / 2
     float zl;        // lower bound of the height where the column is entered
@@ -454,7 +466,7 @@ enum { kBeamGoing = 0, kBeamOpen = 1, kBeamLeft = 2, kBeamCorner = 3 };
 // if it enters through a corner.
 HF_HD bool beam_row(const BeamDir &d, const BeamRay &q, const Beam &m, const BeamWalk &w,
                     int32_t x, float dx, int32_t &row) {
-    const float v = fmaf(d.rho, dx, w.pv), f = floorf(v);
+    const float v = fmaf(d.rho, dx, q.pv), f = floorf(v);
     row = (int32_t)f;
     if (fabsf(v - f - 0.5f) < 0.5f - w.ev) return true;
     // which of the ray's crossings of the nearest row boundary and of column x
@@ -470,17 +482,15 @@ HF_HD bool beam_row(const BeamDir &d, const BeamRay &q, const Beam &m, const Bea
 // beyond.  False if it enters through a corner.
 HF_HD bool beam_enter(const BeamDir &d, const BeamRay &q, const Beam &m, int32_t x0, int32_t x1,
                       BeamWalk &w) {
-    w.pu = beam_pu(q, m);
-    w.pv = beam_pv(q, m);
-    const float apu = fabsf(w.pu), far = (float)x1 + apu;
-    w.ev = (far + fabsf(w.pv) + 1.0f) * (1.5f / 4194304.0f);
+    const float apu = fabsf(q.pu), far = (float)x1 + apu;
+    w.ev = (far + fabsf(q.pv) + 1.0f) * (1.5f / 4194304.0f);
     const float e = (fabsf(d.sigma) * (far + 2.0f) + fabsf(q.z0)) * (1.0f / 2097152.0f);
     w.e2 = 2.0f * e;
     w.zbase = q.z0 - e;
     w.row = q.fv - m.v0;
     w.zl = fabsf(q.z0) < 256.0f ? q.z0 : w.zbase;  // (a start below 256 is exact)
     if (q.fu - m.u0 >= x0) return true;
-    const float dx = (float)x0 - w.pu;
+    const float dx = (float)x0 - q.pu;
     w.zl = fmaf(d.sigma, dx, w.zbase);
     return beam_row(d, q, m, w, x0, dx, w.row);
 }
@@ -511,63 +521,146 @@ HF_HD BeamGrid beam_grid(const uint32_t *cells, const Beam &m, int key, uint32_t
     return g;
 }
 
-// Column x of a walk, whose one or two cells are tested together.  row, zl:
-// where it is left (in and out of the walk: the caller moves on with them).
-// kBeamGoing: the cells are empty; kBeamOpen: they may not be; kBeamLeft: the
-// ray has left the grid sideways; kBeamCorner: it leaves through a corner.
+// A column of a walk: where it is left, and its one or two cells.
+struct BeamColumn {
+    int32_t row;      // the row it is left in
+    float zl;         // lower bound of the height where it is left
+    uint32_t wa, wb;  // words of the cells of the row it is entered in, and left in
+};
+
+// Column x of a walk, whose cells are tested together.  kBeamGoing: they are
+// empty; kBeamOpen: they may not be; kBeamLeft: the ray has left the grid
+// sideways; kBeamCorner: it leaves through a corner.
 template <bool PAIR>
 HF_HD int beam_step(const BeamGrid &g, const BeamDir &d, const BeamRay &q, const Beam &m,
-                    const BeamWalk &w, int32_t x, int32_t &row, float &zl) {
+                    const BeamWalk &w, int32_t x, BeamColumn &c) {
     if (w.row >= g.rows) return kBeamLeft;
-    const float dx = (float)(x + 1) - w.pu;
-    zl = fmaf(d.sigma, dx, w.zbase);
-    const bool sure = beam_row(d, q, m, w, x + 1, dx, row);
+    const float dx = (float)(x + 1) - q.pu;
+    c.zl = fmaf(d.sigma, dx, w.zbase);
+    const bool sure = beam_row(d, q, m, w, x + 1, dx, c.row);
     const uint32_t ca = g.at + (uint32_t)(x * g.step_u + w.row * g.step_v);
-    const uint32_t cb = ca + (uint32_t)(row > w.row && row < g.rows ? g.step_v : 0);
+    const uint32_t cb = ca + (uint32_t)(c.row > w.row && c.row < g.rows ? g.step_v : 0);
     const uint32_t wa = beam_word<PAIR>(g.cells, ca), wb = beam_word<PAIR>(g.cells, cb);
+    c.wa = wa;
+    c.wb = wb;
     const uint32_t ta = wa & 0xFF0000, tb = wb & 0xFF0000;
     const uint32_t fa = wa & 0xFF, fb = wb & 0xFF, ma = wa & 0xFF00, mb = wb & 0xFF00;
     const float top = (float)((ta > tb ? ta : tb) >> 16), h0 = (float)(fa > fb ? fa : fb);
     const float h1 = (float)((ma < mb ? ma : mb) >> 8);
-    const float zlo = fminf(w.zl, zl), zhi = fmaxf(w.zl, zl) + w.e2;
+    const float zlo = fminf(w.zl, c.zl), zhi = fmaxf(w.zl, c.zl) + w.e2;
     if (!sure) return kBeamCorner;
     return (zlo > top) | ((zlo > h0) & (zhi < h1)) ? kBeamGoing : kBeamOpen;
 }
 
-// Decides a column that beam_step left open, on exact rationals: true and h
-// filled, or false.  row: where the ray leaves it.
-template <bool PAIR>
-HF_HD bool beam_settle(const BeamGrid &g, int32_t oz, int32_t dz, const BeamDir &d,
-                       const BeamRay &q, const Beam &m, const BeamWalk &w, int32_t x, int32_t row,
-                       Hit &h) {
-    const bool x_major = d.key & 4;
-    const int32_t u = m.u0 + x;
-    const bool start = u == q.fu;
-    const int32_t end = (u + 1) * (1 << kShift) + q.ku;               // over du: the column's exit
+// A hit as the walk finds it: mirrored cell (u, v), its word, and how it was hit.
+enum { kBeamWallU = 0, kBeamWallV = 1, kBeamAbove = 2, kBeamBottom = 3, kBeamLayer1 = 4 };
+struct BeamHit {
+    int32_t u, v;
+    uint32_t word;
+    int32_t kind;  // the side it was entered through, with its layer; -1: no hit
+};
+
+// Decides a column that beam_step left open from the bounds of the heights where
+// the ray enters it, changes row and leaves it.  The hit's kind, -1 if there is
+// none, -2 if it is too close to tell.  second: it is in the row of the exit.
+//
+// The row changes where v = row + 1, at x - pu = (row + 1 - pv) / rho, off by
+// less than 2 ev / rho.
+HF_HD int beam_decide(const BeamGrid &g, const BeamDir &d, const BeamRay &q, const BeamWalk &w,
+                      const BeamColumn &c, bool &second) {
+    float il = w.zl, iu = w.zl + w.e2, ol = c.zl, ou = c.zl + w.e2;
+    uint32_t word = c.wa;
+    second = false;
+    if (c.row > w.row) {
+        const float inv = cast_rcp_fast(d.rho), es = fabsf(d.sigma) * (2.0f * w.ev) * inv;
+        const float zs = fmaf(d.sigma, ((float)(w.row + 1) - q.pv) * inv, w.zbase);
+        const float sl = zs - es, su = zs + w.e2 + es;
+        const float lo = fminf(il, sl), hi = fmaxf(iu, su);
+        second = (lo > (float)(word >> 16 & 0xFF)) |
+                 ((lo > (float)(word & 0xFF)) & (hi < (float)(word >> 8 & 0xFF)));
+        if (second) {
+            if (c.row >= g.rows) return -1;
+            word = c.wb;
+            il = sl;
+            iu = su;
+        } else {
+            ol = sl;
+            ou = su;
+        }
+    }
+    const float h0 = (float)(word & 0xFF), h1 = (float)(word >> 8 & 0xFF),
+                h2 = (float)(word >> 16 & 0xFF);
+    const bool slab = h2 > h0;
+    const bool gap = slab & (il > h0) & (iu < h1);
+    if (iu <= h0) return second;
+    if (slab & (il >= h1) & (iu <= h2)) return second + kBeamLayer1;
+    if ((il > h2) & (ou <= h2)) return slab ? kBeamAbove + kBeamLayer1 : kBeamAbove;
+    if (gap & (ou <= h0)) return kBeamAbove;
+    if (gap & (ol >= h1)) return kBeamBottom + kBeamLayer1;
+    const float lo = fminf(il, ol), hi = fmaxf(iu, ou);
+    return (lo > h2) | ((lo > h0) & (hi < h1)) ? -1 : -2;
+}
+
+// The same on exact rationals: the hit's kind, or -1.  One column in two hundred
+// comes here (beam_decide needs half of its instructions).
+HF_HD int beam_exact(const BeamGrid &g, int32_t oz, int32_t dz, const BeamDir &d,
+                     const BeamRay &q, const Beam &m, const BeamWalk &w, int32_t x,
+                     const BeamColumn &c, bool &second) {
+    const bool start = m.u0 + x == q.fu;
+    const int32_t end = (m.u0 + x + 1) * (1 << kShift) + q.ku;        // over du: the column's exit
     const int32_t side = (m.v0 + w.row + 1) * (1 << kShift) + q.kv;   // over dv: the row's
     int32_t num = start ? 0 : end - (1 << kShift), den = start ? 1 : d.du;
-    uint8_t face = start ? kFaceInside
-                   : x_major ? (d.key & 2 ? kFacePX : kFaceNX)
-                             : (d.key & 2 ? kFacePY : kFaceNY);
-    uint32_t cell = g.at + (uint32_t)(x * g.step_u + w.row * g.step_v);
-    int32_t v = m.v0 + w.row;
-    for (bool second = false;; second = true) {
-        const bool last = second || row == w.row;
-        const uint32_t word = beam_word<PAIR>(g.cells, cell);
-        if (leaf_test(oz, dz, word, num, den, last ? end : side, last ? d.du : d.dv, face, h)) {
-            const int32_t ru = d.key & 2 ? ~u : u, rv = d.key & 1 ? ~v : v;
-            h.cx = x_major ? ru : rv;
-            h.cy = x_major ? rv : ru;
-            h.word = word;
-            return true;
-        }
-        if (last || row >= g.rows) return false;
+    Hit h;
+    for (second = false;; second = true) {
+        const bool last = second || c.row == w.row;
+        if (leaf_test(oz, dz, second ? c.wb : c.wa, num, den, last ? end : side,
+                      last ? d.du : d.dv, kFaceInside, h))
+            return (h.face == kFacePZ ? kBeamAbove : h.face == kFaceNZ ? kBeamBottom : second) +
+                   (h.layer ? kBeamLayer1 : 0);
+        if (last || c.row >= g.rows) return -1;
         num = side;
         den = d.dv;
-        face = x_major ? (d.key & 1 ? kFacePY : kFaceNY) : (d.key & 1 ? kFacePX : kFaceNX);
-        cell += (uint32_t)g.step_v;
-        v += 1;
     }
+}
+
+// Decides a column that beam_step left open: whether there is a hit, and h.
+HF_HD bool beam_settle(const BeamGrid &g, int32_t oz, int32_t dz, const BeamDir &d,
+                       const BeamRay &q, const Beam &m, const BeamWalk &w, int32_t x,
+                       const BeamColumn &c, BeamHit &h) {
+    bool second;
+    int kind = beam_decide(g, d, q, w, c, second);
+    if (kind < -1) kind = beam_exact(g, oz, dz, d, q, m, w, x, c, second);
+    if (kind < 0) return false;
+    h.u = m.u0 + x;
+    h.v = m.v0 + w.row + second;
+    h.word = second ? c.wb : c.wa;
+    h.kind = kind;
+    return true;
+}
+
+// The hit of a ray that has one.
+HF_HD Hit beam_hit(const BeamHit &b, int32_t oz, int32_t dz, const BeamDir &d, const BeamRay &q) {
+    Hit h;
+    const bool x_major = d.key & 4;
+    const int what = b.kind & 3;
+    const bool top = what == kBeamAbove, level = what >= kBeamAbove;
+    const bool on_v = what == kBeamWallV, start = what == kBeamWallU && b.u == q.fu;
+    const int32_t ru = d.key & 2 ? ~b.u : b.u, rv = d.key & 1 ? ~b.v : b.v;
+    h.cx = x_major ? ru : rv;
+    h.cy = x_major ? rv : ru;
+    h.word = b.word;
+    h.layer = b.kind >> 2;
+    // a face of x or y: the one that a mirrored ray enters through is the positive one
+    const bool pos = d.key & (on_v ? 1 : 2);
+    h.face = level ? (top ? kFacePZ : kFaceNZ)
+             : start ? kFaceInside
+                     : (x_major != on_v ? kFaceNX : kFaceNY) + (pos ? 1 : 0);
+    const int32_t n = (top ? (h.layer ? b.word >> 16 : b.word) : b.word >> 8) & 0xFF;
+    const int32_t fall = oz - (n << kShift);
+    const int32_t at = (on_v ? b.v : b.u) * (1 << kShift) + (on_v ? q.kv : q.ku);
+    h.tnum = level ? (top ? fall : -fall) : start ? 0 : at;
+    h.tden = level ? (top ? -dz : dz) : start ? 1 : on_v ? d.dv : d.du;
+    return h;
 }
 
 // The order in which a beam's columns are tested: rounds of 32 stretches of

@@ -112,7 +112,7 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
     int32_t found = 0;
     const int lane = threadIdx.x & 31;
     const BeamDir d = beam_dir(r.dx, r.dy, r.dz);
-    const BeamRay q = beam_ray(d, r);
+    BeamRay q = beam_ray(d, r);
     // samples per column and per unit of height
     const float per_u = __fdividef(65536.0f, (float)d.du * m.dt);
     const float per_z = __fdividef(1.0f, fabsf(m.dz) * m.dt);
@@ -129,14 +129,14 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
         bool alive = (todo >> lane & 1) && d.key == s.key;
         todo &= ~__ballot_sync(kFull, alive);
         beam_scan(s, p.world, lvt, p.world.L);
-        const float pu = beam_pu(q, s.m);
+        beam_place(q, s.m);
         int32_t next = 1, b0, b1;
         uint32_t peak;
         while (beam_next<false>(s, lvt, d, q, alive, b0, b1, &peak)) {
             // the samples in these columns, at heights up to the highest top
             // there: a little more either side than rounding can move them
-            float lo = ((float)(b0 - s.m.u0) - 0.02f - pu) * per_u;
-            float hi = ((float)(b1 - s.m.u0) + 0.02f - pu) * per_u;
+            float lo = ((float)(b0 - s.m.u0) - 0.02f - q.pu) * per_u;
+            float hi = ((float)(b1 - s.m.u0) + 0.02f - q.pu) * per_u;
             if (lo * 0.999998f - 0.02f > steps) alive = false;  // past its last sample
             const float rise = (float)peak + 0.02f - m.oz;
             if (m.dz < 0.0f) lo = fmaxf(lo, -rise * per_z);
@@ -147,7 +147,7 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
             found = max(found, march_samples(p.world, m, alive, first, last));
             // samples that rounding may have moved into the columns beyond stay
             // to be taken again with those, which may be higher
-            const float done = ((float)(b1 - s.m.u0) - 0.02f - pu) * per_u * 0.999998f - 0.02f;
+            const float done = ((float)(b1 - s.m.u0) - 0.02f - q.pu) * per_u * 0.999998f - 0.02f;
             next = max(next, (int32_t)fminf(fmaxf(done, 0.0f), steps + 1.0f));
             alive = alive && !found;
             if (!__any_sync(kFull, alive)) break;

@@ -29,9 +29,9 @@ namespace hf {
 namespace {
 
 // Resident 128-thread blocks per SM asked of the register allocator: six leave
-// each thread 80 registers.  64 views with shadows / a 1080p eye-level view:
-// five blocks 9.77 ms / 138 us, six 9.63 / 132, seven (72 registers, more
-// address arithmetic) 10.22 / 136, eight 10.25 / 140.
+// each thread 80 registers (without shadows 72 are used, so seven blocks fit).
+// 64 views with shadows / a 1080p eye-level view: four blocks 10.62 ms / 141 us,
+// five 9.66 / 129, six 9.39 / 126, seven (11 % more instructions) 9.75 / 127.
 constexpr int kTraceMinBlocks = 6;
 
 __constant__ float c_albedo[8][3] = HF_ALBEDO_TABLE;
@@ -72,16 +72,9 @@ __device__ __forceinline__ uint32_t level0_word(const WorldDev &w, int32_t x, in
 
 __device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visible,
                                           const float *ln) {
-    float ndl;
-    switch (face) {
-        case kFaceNX: ndl = -ln[0]; break;
-        case kFacePX: ndl = ln[0]; break;
-        case kFaceNY: ndl = -ln[1]; break;
-        case kFacePY: ndl = ln[1]; break;
-        case kFaceNZ: ndl = -ln[2]; break;
-        case kFacePZ: ndl = ln[2]; break;
-        default: ndl = 0.0f;
-    }
+    // the normal's axis is face / 2, its sign face's lowest bit
+    const float n = face < kFaceNY ? ln[0] : face < kFaceNZ ? ln[1] : ln[2];
+    const float ndl = face == kFaceInside ? 0.0f : face & 1 ? n : -n;
     const float k = kKa + kKd * fmaxf(ndl, 0.0f) * (visible ? 1.0f : 0.0f);
     const uint32_t m = (word >> 24) & 7;
     uint32_t out = 0xFF000000u;
@@ -93,7 +86,8 @@ __device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visi
     return out;
 }
 
-// Casts one ray per active lane; every lane of the warp calls.
+// Casts one ray per active lane; every lane of the warp calls.  only: of a hit
+// nothing matters but that there is one.
 //
 // The rays that go the same way and start side by side form a beam (hf_beam.h);
 // they are walked, all together, through the runs of columns that it does not
@@ -102,21 +96,20 @@ __device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visi
 // one or two rounds.
 //
 // Bound by instruction issue, as the traversal of single rays was: 2048 x 2048
-// grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 9.63
-// ms, a 1080p eye-level view with shadows 192 -> 132 us, a hundred 1080p frames
-// over 2048 x 16384 cells 17.3 -> 10.2 ms.
+// grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 9.39
+// ms, a 1080p eye-level view with shadows 192 -> 126 us, a hundred 1080p frames
+// over 2048 x 16384 cells 17.3 -> 8.1 ms.
 template <bool PAIR>
 __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev *lvt,
-                                           const Ray &r, const BeamDir &d, bool active, int mip,
-                                           Hit &h) {
-    h.face = kFaceMiss;
-    h.layer = 255;
+                                           const BeamDir &d, BeamRay q, int32_t oz, int32_t dz,
+                                           bool active, int mip, bool only, Hit &h) {
+    BeamHit b;
+    b.kind = -1;
     const uint32_t W = (uint32_t)p.world.W, H = (uint32_t)p.world.H;
     const uint32_t *cells = p.world.base;
     const int lane = threadIdx.x & 31;
-    const BeamRay q = beam_ray(d, r);
     // rays that no beam takes: vertical ones, and (below) through corners
-    bool alone = active && (r.dx | r.dy) == 0;
+    bool alone = active && d.du == 0;
     active = active && !alone && (uint32_t)(d.key & 2 ? ~q.fu : q.fu) < (d.key & 4 ? W : H) &&
              (uint32_t)(d.key & 1 ? ~q.fv : q.fv) < (d.key & 4 ? H : W);
     uint32_t todo = __ballot_sync(kFull, active);
@@ -124,13 +117,15 @@ __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev
         // the first ray left, and the rays that go its way beside it
         const int lead = __ffs(todo) - 1;
         BeamScan s;
-        s.key = __shfl_sync(kFull, d.key, lead);
-        s.m.u0 = __shfl_sync(kFull, q.fu, lead);
-        s.m.v0 = __shfl_sync(kFull, q.fv, lead);
+        s.key = __reduce_max_sync(kFull, lane == lead ? d.key : -1);
+        s.m.u0 = __reduce_max_sync(kFull, lane == lead ? q.fu : (int)0x80000000);
+        s.m.v0 = __reduce_max_sync(kFull, lane == lead ? q.fv : (int)0x80000000);
+        beam_place(q, s.m);
         bool alive = (todo >> lane & 1) && d.key == s.key &&
-                     fabsf(beam_pv(q, s.m) - d.rho * beam_pu(q, s.m)) <= kBeamSpread;
+                     fabsf(q.pv - d.rho * q.pu) <= kBeamSpread;
         todo &= ~__ballot_sync(kFull, alive);
         s.m.u0 = __reduce_min_sync(kFull, alive ? q.fu : 0x7FFFFFFF);
+        beam_place(q, s.m);
         beam_scan(s, p.world, lvt, mip);
         const BeamGrid g = beam_grid(cells, s.m, s.key, W, H);
         int32_t b0, b1;
@@ -145,27 +140,40 @@ __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev
             // column by column, all rays together
             do {
                 if (alive && s.m.u0 + x >= q.fu) {
-                    int32_t row;
-                    float zl;
-                    const int at = beam_step<PAIR>(g, d, q, s.m, w, x, row, zl);
+                    BeamColumn c;
+                    const int at = beam_step<PAIR>(g, d, q, s.m, w, x, c);
                     if (at == kBeamOpen) {
-                        alive = !beam_settle<PAIR>(g, r.oz, r.dz, d, q, s.m, w, x, row, h);
+                        alive = !beam_settle(g, oz, dz, d, q, s.m, w, x, c, b);
                     } else if (at != kBeamGoing) {
                         alive = false;
                         alone = at == kBeamCorner;
                     }
-                    w.row = row;
-                    w.zl = zl;
+                    w.row = c.row;
+                    w.zl = c.zl;
                 }
             } while (__any_sync(kFull, alive) && ++x < x1);
             if (!__any_sync(kFull, alive)) break;
         }
     }
+    h.face = kFaceMiss;
+    h.layer = 255;
     if (alone) {
         Counters none{0, 0};
         const int level = min(kBeamLevel, mip);
-        cast_general<false, PAIR>(lvt, r, level, mip, 0x7FFFFFFF, h, none);
+        cast_general<false, PAIR>(lvt, beam_unray(d, q, oz, dz), level, mip, 0x7FFFFFFF, h, none);
+    } else if (only) {
+        h.face = b.kind < 0 ? kFaceMiss : kFaceInside;
+    } else if (b.kind >= 0) {
+        h = beam_hit(b, oz, dz, d, q);
     }
+}
+
+// The ray of a camera's pixel.
+__device__ __forceinline__ Ray primary_ray(const CamDev &c, int32_t px, int32_t py) {
+    const int32_t a = 2 * px + 1 - (int32_t)c.w;
+    const int32_t b = (int32_t)c.h - 1 - 2 * py;
+    return Ray{c.o[0], c.o[1], c.o[2], c.F[0] + a * c.R[0] + b * c.U[0],
+               c.F[1] + a * c.R[1] + b * c.U[1], c.F[2] + a * c.R[2] + b * c.U[2]};
 }
 
 // One pixel per lane: its primary ray, then (with shadows) the shadow ray, in
@@ -177,16 +185,7 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
                                              bool inside, const BeamDir &sun, Counters &cnt,
                                              Counters &scnt, uint32_t &nshadow, bool &err) {
     constexpr bool STATS = KIND == kTraceStats;
-    const int32_t a = 2 * px + 1 - (int32_t)c.w;
-    const int32_t b = (int32_t)c.h - 1 - 2 * py;
-    const uint32_t pix = (uint32_t)py * c.w + (uint32_t)px;
-    Ray r;
-    r.ox = c.o[0];
-    r.oy = c.o[1];
-    r.oz = c.o[2];
-    r.dx = c.F[0] + a * c.R[0] + b * c.U[0];
-    r.dy = c.F[1] + a * c.R[1] + b * c.U[1];
-    r.dz = c.F[2] + a * c.R[2] + b * c.U[2];
+    Ray r = primary_ray(c, px, py);
     uint32_t word = 0;  // of the primary hit, with its face: for the shading
     uint8_t face = kFaceMiss;
     bool visible = true;
@@ -198,7 +197,8 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
         Counters pc{0, 0};
         if (KIND == kTraceBeams) {
             const BeamDir d = sp ? sun : beam_dir(r.dx, r.dy, r.dz);
-            cast_beams<PAIR>(p, lvt, r, d, cast, sp ? p.shadow_mip : p.mip_start, h);
+            cast_beams<PAIR>(p, lvt, d, beam_ray(d, r), r.oz, r.dz, cast,
+                             sp ? p.shadow_mip : p.mip_start, sp, h);
         } else {
             h.face = kFaceMiss;
             h.layer = 255;
@@ -218,6 +218,10 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
         }
         cast = false;
         const bool hit = h.face < kFaceError;
+        // the ray again, from the camera: it need not be held through the cast
+        asm volatile("" : "+r"(px), "+r"(py)::"memory");
+        r = primary_ray(c, px, py);
+        const uint32_t pix = (uint32_t)py * c.w + (uint32_t)px;
         if (inside) {
             word = h.word;
             face = h.face;
@@ -246,7 +250,7 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
             const int32_t dn = on_x ? r.dx : on_z ? r.dz : r.dy;
             const int32_t da = on_x ? r.dy : r.dx, db = on_z ? r.dy : r.dz;
             const int32_t qn = dn < 0 ? 1 - h.tnum : h.tnum - 1;  // one unit back
-            const float rcp_t = 1.0f / (float)h.tden;
+            const float rcp_t = __fdividef(1.0f, (float)h.tden);
             const int32_t qa = floor_div_small((int64_t)h.tnum * da, h.tden, rcp_t);
             const int32_t qb = floor_div_small((int64_t)h.tnum * db, h.tden, rcp_t);
             const int32_t sxp = r.ox + (on_x ? qn : qa);
@@ -282,6 +286,7 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
         if (!__any_sync(kFull, cast)) break;
     }
     if (!inside) return;
+    const uint32_t pix = (uint32_t)py * c.w + (uint32_t)px;
     if (SHADOWS && c.shadow) __stcs(c.shadow + pix, (uint8_t)(visible ? 0 : 1));
     if (c.rgba)
         __stcs(c.rgba + pix, face < kFaceError ? shade(word, face, visible, p.sun_n) : kSky);

@@ -54,15 +54,17 @@ static void beams(const LevelDev *lv, int top_level_of_world, const Ray *r, int 
         m.v0 = q[lead].fv;
         int32_t u0 = 0x7FFFFFFF;
         for (int k = 0; k < n; ++k) {
+            beam_place(q[k], m);
             alive[k] = todo[k] && d[k].key == key &&
-                       std::fabs(beam_pv(q[k], m) - d[k].rho * beam_pu(q[k], m)) <= kBeamSpread;
+                       std::fabs(q[k].pv - d[k].rho * q[k].pu) <= kBeamSpread;
             if (alive[k]) todo[k] = false, u0 = std::min(u0, q[k].fu);
         }
         m.u0 = u0;
         for (int k = 0; k < n; ++k)
             if (alive[k]) {
-                a[k] = beam_pv(q[k], m) - d[k].rho * beam_pu(q[k], m);
-                b[k] = q[k].z0 - d[k].sigma * beam_pu(q[k], m);
+                beam_place(q[k], m);
+                a[k] = q[k].pv - d[k].rho * q[k].pu;
+                b[k] = q[k].z0 - d[k].sigma * q[k].pu;
             }
         const int32_t limit = key & 2 ? 0 : (int32_t)(key & 4 ? W : H);
         const BeamGrid g = beam_grid(cells, m, key, W, H);
@@ -104,21 +106,22 @@ static void beams(const LevelDev *lv, int top_level_of_world, const Ray *r, int 
                 for (int k = 0; k < n; ++k) {
                     if (!alive[k] || q[k].fu >= b1) continue;
                     BeamWalk w;
+                    BeamHit b;
                     if (!beam_enter(d[k], q[k], m, b0 - m.u0, b1 - m.u0, w)) {
                         alive[k] = false;
                         alone[k] = true;
                     }
                     for (int32_t x = std::max(b0, q[k].fu) - m.u0; alive[k] && x < b1 - m.u0; ++x) {
-                        int32_t row = 0;
-                        float zl = 0;
-                        const int at = beam_step<PAIR>(g, d[k], q[k], m, w, x, row, zl);
+                        BeamColumn c = {};
+                        const int at = beam_step<PAIR>(g, d[k], q[k], m, w, x, c);
                         if (at == kBeamOpen)
-                            alive[k] = !beam_settle<PAIR>(g, r[k].oz, r[k].dz, d[k], q[k], m, w, x, row,
-                                                          h[k]);
+                            alive[k] = !beam_settle(g, r[k].oz, r[k].dz, d[k], q[k], m, w, x, c, b);
                         else if (at != kBeamGoing)
                             alive[k] = false, alone[k] = at == kBeamCorner;
-                        w.row = row;
-                        w.zl = zl;
+                        if (at == kBeamOpen && !alive[k])
+                            h[k] = beam_hit(b, r[k].oz, r[k].dz, d[k], q[k]);
+                        w.row = c.row;
+                        w.zl = c.zl;
                     }
                 }
             }
