@@ -73,9 +73,13 @@ constexpr int kSunCellsX = 4, kSunCellsY = 2;
 // Up to this many groups of 32 threads, 8 warps share a group's columns: a
 // repair after a crater, or a small world, leaves too few groups to hide the
 // latency of a thread's up to 1056 columns one after the other (a repair toward
-// (400000, 100000, 100000) 0.143 -> 0.086 ms with its edit; a 2048^2 build, 32768
-// groups, 0.55 -> 0.91 ms if split, as each warp then stops later).
+// (400000, 100000, 100000) 0.143 -> 0.084 ms with its edit; a 2048^2 build, 32768
+// groups, took two thirds longer if split, as each warp then stops later).
 constexpr int kSunSplit = 8;
+// Columns of a round are read in parts of 16, and a part over a region whose
+// nodes of 8 x 8 cells show nothing high enough is left out: two 2048^2 builds and
+// 1080p views 1331 -> 1254 us (parts of 8: 1282; of 16 over 16 x 16 nodes: 1.5 % more).
+constexpr int kSunPart = 16, kSunPartLevel = 3;
 constexpr uint32_t kSunSplitBelow = 16384;
 
 __global__ void k_sun_rows(int4 *tab, int64_t lmin, int64_t lmaj, int64_t lz) {
@@ -114,15 +118,16 @@ __device__ __forceinline__ int32_t rows_after(const int4 *tab, int32_t j) {
 // A level-0 cell as the bounds use it: 255 - floor in the low half, top in the
 // high half, so that one 16-bit pairwise maximum over a band's cells gives its
 // lowest floor and its highest top.
+//
+// `at` is 4 (y W + x), the byte at which the cell's word starts: a 32-bit offset
+// from one pointer (a world has at most 2^28 cells) that the load adds itself.
+// With a 64-bit address per load a 2048^2 build with the default sun took 0.47
+// ms instead of 0.41.
 template <bool PAIR>
-__device__ __forceinline__ uint32_t sun_cell(const WorldDev &w, int32_t x, int32_t y) {
-    uint32_t n;
-    if (PAIR)
-        n = pair_node(__ldg(w.base + (uint32_t)y * ((uint32_t)w.W >> 1) + ((uint32_t)x >> 1)),
-                      (uint32_t)x & 1);
-    else
-        n = __ldg(w.base + (uint32_t)y * (uint32_t)w.W + (uint32_t)x);
-    return (n ^ 0xFFu) & 0x00FF00FFu;
+__device__ __forceinline__ uint32_t sun_cell(const WorldDev &w, uint32_t at) {
+    const char *base = reinterpret_cast<const char *>(w.base);
+    const uint32_t word = __ldg(reinterpret_cast<const uint32_t *>(base + (PAIR ? at >> 1 & ~3u : at)));
+    return ((PAIR ? pair_node(word, at >> 2 & 1) : word) ^ 0xFFu) & 0x00FF00FFu;
 }
 
 // V cells of one thread, next to each other along the minor axis in the
@@ -133,6 +138,10 @@ __device__ __forceinline__ uint32_t sun_cell(const WorldDev &w, int32_t x, int32
 // cv + sv i + (sv > 0 ? q(k - 1) : 1 + q(k - 1)) on, in direction sv: the rows
 // 0 .. 1 + A for F, all of them for G, A = |q(k) - q(k - 1)| <= 1 and
 // B = |q(k + 1) - q(k - 1)| <= A + 1.  So the V cells share V + 1 + B rows.
+// F and G are kept times 256, so that a term is a cell's byte, shifted, plus the
+// column's rise: one add with maximum (and for F one multiplication that takes
+// the low half of the band's maximum; for G the low half only adds less than a
+// unit, which the final shift drops).
 template <int V>
 struct SunCells {
     int32_t F[V], G[V];
@@ -148,26 +157,25 @@ __device__ __forceinline__ void sun_column(const WorldDev &w, int32_t col, int32
     const int32_t NU = XM ? w.W : w.H, NV = XM ? w.H : w.W;
     const bool in_col = !EDGE || (uint32_t)col < (uint32_t)NU;
     uint32_t p[V + 1 + B];
+    const uint32_t at = 4u * (uint32_t)(XM ? row * w.W + col : col * w.W + row);
+    const uint32_t per_row = 4u * (uint32_t)(XM ? sv * w.W : sv);
 #pragma unroll
     for (int j = 0; j < V + 1 + B; ++j) {
-        const int32_t r = row + sv * j;
         p[j] = 0;
-        if (!EDGE || (in_col && (uint32_t)r < (uint32_t)NV))
-            p[j] = XM ? sun_cell<PAIR>(w, col, r) : sun_cell<PAIR>(w, r, col);
+        if (!EDGE || (in_col && (uint32_t)(row + sv * j) < (uint32_t)NV))
+            p[j] = sun_cell<PAIR>(w, at + (uint32_t)j * per_row);
     }
-    const int32_t cf = (255 << 8) - up;
+    const int32_t cf = ((255 << 8) - up) * 256, cg = -down * 256;
 #pragma unroll
     for (int i = 0; i < V; ++i) {
-        uint32_t f = __vmaxu2(p[i], p[i + 1]);
-        if (A) f = __vmaxu2(f, p[i + 1 + A]);
-        uint32_t g = f;
-        if (B > A) g = __vmaxu2(g, p[i + 1 + B]);
+        const uint32_t f = A ? __vimax3_u16x2(p[i], p[i + 1], p[i + 1 + A]) : __vmaxu2(p[i], p[i + 1]);
+        const uint32_t g = B > A ? __vmaxu2(f, p[i + 1 + B]) : f;
         // the whole F band in the grid
         const bool f_ok = !EDGE || (in_col && (f_on >> i & 1) &&
                                     (uint32_t)(row + sv * i) < (uint32_t)NV &&
                                     (uint32_t)(row + sv * (i + 1 + A)) < (uint32_t)NV);
-        if (f_ok) c.F[i] = max(c.F[i], cf - (int32_t)((f & 0xFFu) << 8));
-        c.G[i] = max(c.G[i], (int32_t)((g >> 16) << 8) - down);  // (never raised by neutral cells)
+        if (f_ok) c.F[i] = __viaddmax_s32((int32_t)(f * 0xFFFF0000u), cf, c.F[i]);
+        c.G[i] = __viaddmax_s32((int32_t)g, cg, c.G[i]);  // (never raised by neutral cells)
     }
 }
 
@@ -177,7 +185,7 @@ __device__ __forceinline__ void sun_round(const WorldDev &w, const SunAxes &a, c
                                           uint32_t f_on, SunCells<V> &c) {
     int32_t qm = rows_after(tab, k0 - 1), qk = rows_after(tab, k0);
 #pragma unroll 1
-    for (int32_t k = k0; k < k0 + 32; ++k) {
+    for (int32_t k = k0; k < k0 + kSunPart; ++k) {
         const int4 e = __ldg(&tab[k + 2]);
         const int32_t col = cu + a.smaj * k, row = cv + (sv > 0 ? qm : 1 + qm);
         if (qk != qm) {
@@ -194,6 +202,32 @@ __device__ __forceinline__ void sun_round(const WorldDev &w, const SunAxes &a, c
         qm = qk;
         qk = e.x;
     }
+}
+
+// Whether a floor or top in region [u0, u1] x [v0, v1] (it meets the grid) can
+// raise a bound: the highest there, from the nodes of a level, against the
+// lowest bounds and the rise in the region's first column.
+template <bool XM>
+__device__ __forceinline__ bool sun_may_rise(const WorldDev &w, int level, int32_t u0, int32_t u1,
+                                             int32_t v0, int32_t v1, int32_t lo_f, int32_t lo_g,
+                                             int32_t up, int32_t down) {
+    // lanes side by side along the region's longer axis
+    constexpr int kU = XM ? 8 : 2, kV = 32 / kU;
+    const int32_t NU = XM ? w.W : w.H, NV = XM ? w.H : w.W;
+    const int lane = threadIdx.x & 31;
+    const int32_t a1 = min(u1, NU - 1) >> level, b1 = min(v1, NV - 1) >> level;
+    const uint32_t *nodes = w.base + w.off[level];
+    const uint32_t stride = w.stride[level];
+    uint32_t top = 0, h0 = 0;
+    for (int32_t u = (max(u0, 0) >> level) + lane % kU; u <= a1; u += kU)
+        for (int32_t v = (max(v0, 0) >> level) + lane / kU; v <= b1; v += kV) {
+            const uint32_t n = __ldg(nodes + (uint32_t)(XM ? v : u) * stride + (uint32_t)(XM ? u : v));
+            top = max(top, n & 0xFF0000u);
+            h0 = max(h0, n & 0xFFu);
+        }
+    const int32_t mt = (int32_t)(__reduce_max_sync(0xFFFFFFFFu, top) >> 8);
+    const int32_t mh = (int32_t)(__reduce_max_sync(0xFFFFFFFFu, h0) << 8);
+    return mh - (lo_f + 1) >= up || mt - lo_g > down;
 }
 
 // Bounds of the V cells of each thread of a warp, rounded to the stored units
@@ -217,9 +251,8 @@ __device__ __forceinline__ void sun_bounds_of(const WorldDev &w, const SunAxes &
                                               int32_t first, int32_t step, SunCells<V> &c) {
     constexpr unsigned full = 0xFFFFFFFFu;
     const int32_t NU = XM ? w.W : w.H, NV = XM ? w.H : w.W;
-    const int lane = threadIdx.x & 31;
     auto cell = [&](int32_t u, int32_t v) {
-        return XM ? sun_cell<PAIR>(w, u, v) : sun_cell<PAIR>(w, v, u);
+        return sun_cell<PAIR>(w, 4u * (uint32_t)(XM ? v * w.W + u : u * w.W + v));
     };
     // k = 0: for F the start cell's floor; for G the rows the ray can cross in
     // its start column (it moves at most one row there), strictly above: top +
@@ -233,8 +266,8 @@ __device__ __forceinline__ void sun_bounds_of(const WorldDev &w, const SunAxes &
         uint32_t top = p >> 16;
         if (v + 1 < NV) top = max(top, cell(cu, v + 1) >> 16);
         if (a.lmin < 0 && v > 0) top = max(top, cell(cu, v - 1) >> 16);
-        c.F[i] = (int32_t)(255 - (p & 0xFF)) << 8;
-        c.G[i] = (int32_t)(top << 8) + 1;
+        c.F[i] = (int32_t)(255 - (p & 0xFF)) << 16;
+        c.G[i] = ((int32_t)(top << 8) + 1) << 8;
     }
     const uint32_t root = __ldg(w.base + w.off[w.L]);
     const int32_t maxh0 = w.L ? (int32_t)(root & 0xFF) << 8 : 255 << 8;
@@ -255,47 +288,49 @@ __device__ __forceinline__ void sun_bounds_of(const WorldDev &w, const SunAxes &
     const uint32_t out1 = f_out(1);
     for (int32_t k0 = 1 + 32 * first;; k0 += 32 * step) {
         const uint32_t f_on = k0 == 1 ? on : on & ~(out1 | f_out(k0 - 1));
-        int32_t lo_f = 1 << 20, lo_g = 1 << 20;  // the lowest bounds that may still rise
+        int32_t lo_f, lo_g;  // the lowest bounds that may still rise
+        auto lowest = [&] {
+            lo_f = lo_g = 1 << 28;
 #pragma unroll
-        for (int i = 0; i < V; ++i) {
-            if (f_on >> i & 1) lo_f = min(lo_f, c.F[i]);
-            if (on >> i & 1) lo_g = min(lo_g, c.G[i]);
-        }
-        lo_f = __reduce_min_sync(full, lo_f);
-        lo_g = __reduce_min_sync(full, lo_g);
+            for (int i = 0; i < V; ++i) {
+                if (f_on >> i & 1) lo_f = min(lo_f, c.F[i]);
+                if (on >> i & 1) lo_g = min(lo_g, c.G[i]);
+            }
+            lo_f = __reduce_min_sync(full, lo_f) >> 8;
+            lo_g = __reduce_min_sync(full, lo_g) >> 8;
+        };
+        lowest();
         const int4 rise = __ldg(&tab[k0 + 2]);
         if (maxh0 - (lo_f + 1) < rise.y && maxtop - lo_g <= rise.z) break;
-        const int32_t ca = cu + a.smaj * k0, cb = cu + a.smaj * (k0 + 31);
-        // the rows the round reads, first and last in direction sv
-        const int32_t qm = rows_after(tab, k0 - 1), qe = rows_after(tab, k0 + 32);
-        const int32_t ra = cv + (sv > 0 ? qm : 1 + qm);
-        const int32_t rb = cv + sv * (V - 1) + (sv > 0 ? 1 + qe : qe);
-        const int32_t rlo = min(ra, rb), rhi = max(ra, rb);
-        // the region of the whole warp
-        const int32_t u0 = __reduce_min_sync(full, min(ca, cb));
-        const int32_t u1 = __reduce_max_sync(full, max(ca, cb));
-        const int32_t v0 = __reduce_min_sync(full, rlo), v1 = __reduce_max_sync(full, rhi);
-        if (u1 < 0 || u0 >= NU || v1 < 0 || v0 >= NV) break;  // and so are all later rounds
-        if (w.L >= 5) {
-            const int32_t a0 = max(u0, 0) >> 5, a1 = min(u1, NU - 1) >> 5;
-            const int32_t b0 = max(v0, 0) >> 5, b1 = min(v1, NV - 1) >> 5;
-            const int32_t nu = a1 - a0 + 1, n_nodes = nu * (b1 - b0 + 1);
-            int32_t mh = 0, mt = 0;
-            for (int32_t n = lane; n < n_nodes; n += 32) {
-                const int32_t u = a0 + n % nu, v = b0 + n / nu;
-                const uint32_t node = __ldg(w.base + w.off[5] + (uint32_t)(XM ? v : u) * w.stride[5] +
-                                            (uint32_t)(XM ? u : v));
-                mh = max(mh, (int32_t)(node & 0xFF));
-                mt = max(mt, (int32_t)((node >> 16) & 0xFF));
+        // what the warp reads in columns [k, k + n): first and last of each axis
+        int32_t u0, u1, v0, v1;
+        auto region = [&](int32_t k, int32_t n) {
+            const int32_t ca = cu + a.smaj * k, cb = cu + a.smaj * (k + n - 1);
+            // the first and the last row in direction sv
+            const int32_t qm = rows_after(tab, k - 1), qe = rows_after(tab, k + n);
+            const int32_t ra = cv + (sv > 0 ? qm : 1 + qm);
+            const int32_t rb = cv + sv * (V - 1) + (sv > 0 ? 1 + qe : qe);
+            u0 = __reduce_min_sync(full, min(ca, cb));
+            u1 = __reduce_max_sync(full, max(ca, cb));
+            v0 = __reduce_min_sync(full, min(ra, rb));
+            v1 = __reduce_max_sync(full, max(ra, rb));
+            return u1 >= 0 && u0 < NU && v1 >= 0 && v0 < NV;  // it meets the grid
+        };
+        if (!region(k0, 32)) break;  // and so do all later rounds
+        if (w.L >= 5 && !sun_may_rise<XM>(w, 5, u0, u1, v0, v1, lo_f, lo_g, rise.y, rise.z)) continue;
+#pragma unroll 1
+        for (int32_t k = k0; k < k0 + 32; k += kSunPart) {
+            if (!region(k, kSunPart)) break;
+            if (w.L >= kSunPartLevel) {
+                if (k > k0) lowest();
+                const int4 e = __ldg(&tab[k + 2]);
+                if (!sun_may_rise<XM>(w, kSunPartLevel, u0, u1, v0, v1, lo_f, lo_g, e.y, e.z)) continue;
             }
-            mh = __reduce_max_sync(full, mh) << 8;
-            mt = __reduce_max_sync(full, mt) << 8;
-            if (mh - (lo_f + 1) < rise.y && mt - lo_g <= rise.z) continue;
+            if (u0 >= 0 && u1 < NU && v0 >= 0 && v1 < NV && __all_sync(full, f_on == on))
+                sun_round<XM, PAIR, V, false>(w, a, tab, k, cu, cv, sv, f_on, c);
+            else
+                sun_round<XM, PAIR, V, true>(w, a, tab, k, cu, cv, sv, f_on, c);
         }
-        if (u0 >= 0 && u1 < NU && v0 >= 0 && v1 < NV && __all_sync(full, f_on == on))
-            sun_round<XM, PAIR, V, false>(w, a, tab, k0, cu, cv, sv, f_on, c);
-        else
-            sun_round<XM, PAIR, V, true>(w, a, tab, k0, cu, cv, sv, f_on, c);
     }
 }
 
@@ -316,10 +351,10 @@ __device__ bool depends_on(const SunAxes &a, const int4 *tab, int32_t cu, int32_
     return cv + 1 + max(qa, qb) >= ev0 && cv + min(qa, qb) < ev1;
 }
 
-// Bound by instruction issue (about 15 instructions per cell and column).  One
+// Bound by instruction issue (about 10 instructions per cell and column).  One
 // warp per cell, its lanes taking 32 columns each round, cost about 1700 warp
 // instructions a cell in loads of bands no other cell shared, reductions and
-// per-lane table reads: 2048^2 world, default sun, 6.4 -> 0.55 ms.
+// per-lane table reads: 2048^2 world, default sun, 6.4 -> 0.40 ms.
 // The cells of the rectangle [x0, x1) x [y0, y1), V per thread along the minor
 // axis, a warp's threads next to each other along x (nwx warps a row).  SPLIT:
 // the warps of a block share the rounds of the same cells.  With edit.z >
@@ -375,7 +410,7 @@ __global__ void __launch_bounds__(SPLIT ? kSunSplit * 32 : kSunThreads)
         if (!(on >> i & 1)) continue;
         const int32_t v = cv + sv * i;
         fg[(uint32_t)(XM ? v : cu) * (uint32_t)w.W + (uint32_t)(XM ? cu : v)] =
-            (uint32_t)c.F[i] | ((uint32_t)c.G[i] << 16);
+            (uint32_t)(c.F[i] >> 8) | ((uint32_t)(c.G[i] >> 8) << 16);
     }
 }
 
