@@ -180,7 +180,7 @@ __device__ __forceinline__ void sun_column(const WorldDev &w, int32_t col, int32
 }
 
 template <bool XM, bool PAIR, int V, bool EDGE>
-__device__ __forceinline__ void sun_round(const WorldDev &w, const SunAxes &a, const int4 *tab,
+__device__ __forceinline__ void sun_part(const WorldDev &w, const SunAxes &a, const int4 *tab,
                                           int32_t k0, int32_t cu, int32_t cv, int32_t sv,
                                           uint32_t f_on, SunCells<V> &c) {
     int32_t qm = rows_after(tab, k0 - 1), qk = rows_after(tab, k0);
@@ -236,19 +236,20 @@ __device__ __forceinline__ bool sun_may_rise(const WorldDev &w, int level, int32
 // ceil(256 k lz / lmaj), and the G term rounded up is 256 h - floor(256 (k - 1)
 // lz / lmaj).
 //
-// Columns go in rounds of 32, of which this warp takes every step-th from
-// `first` on.  F stops with the first round that holds a column it cannot use
-// (the grid's end, or a band that leaves the grid: once one does, all later
-// ones do too, but for column 1 of a cell on the grid's last row).  The rounds
-// end once none can raise any of the warp's bounds (maxh0, maxtop: the world's
-// highest floor and top), and where the pyramid has a level 5, a round over a
-// region whose highest floor and top cannot raise any is skipped; neither
-// changes a bound.
+// Columns go in rounds of 32, each in parts of kSunPart.  F stops with the first
+// round that holds a column it cannot use (the grid's end, or a band that leaves
+// the grid: once one does, all later ones do too, but for column 1 of a cell on
+// the grid's last row).  The parts end once none can raise any of the warp's
+// bounds (maxh0, maxtop: the world's highest floor and top), and a round or part
+// over a region whose highest floor and top (of its level-5 nodes, of its nodes
+// of kSunPartLevel) cannot raise any is skipped; neither changes a bound.  SPLIT:
+// this warp takes every kSunSplit-th part from `first` on (and not whole rounds:
+// with 10 rounds for 8 warps, two of them would have twice the work).
 // cu, cv: the first cell; on: which cells are real.
-template <bool XM, bool PAIR, int V>
+template <bool XM, bool PAIR, int V, bool SPLIT>
 __device__ __forceinline__ void sun_bounds_of(const WorldDev &w, const SunAxes &a, const int4 *tab,
                                               int32_t cu, int32_t cv, int32_t sv, uint32_t on,
-                                              int32_t first, int32_t step, SunCells<V> &c) {
+                                              int32_t first, SunCells<V> &c) {
     constexpr unsigned full = 0xFFFFFFFFu;
     const int32_t NU = XM ? w.W : w.H, NV = XM ? w.H : w.W;
     auto cell = [&](int32_t u, int32_t v) {
@@ -286,51 +287,59 @@ __device__ __forceinline__ void sun_bounds_of(const WorldDev &w, const SunAxes &
         return out;
     };
     const uint32_t out1 = f_out(1);
-    for (int32_t k0 = 1 + 32 * first;; k0 += 32 * step) {
-        const uint32_t f_on = k0 == 1 ? on : on & ~(out1 | f_out(k0 - 1));
-        int32_t lo_f, lo_g;  // the lowest bounds that may still rise
-        auto lowest = [&] {
-            lo_f = lo_g = 1 << 28;
+    int32_t lo_f, lo_g;  // the lowest bounds that may still rise
+    auto lowest = [&](uint32_t f_on) {
+        lo_f = lo_g = 1 << 28;
 #pragma unroll
-            for (int i = 0; i < V; ++i) {
-                if (f_on >> i & 1) lo_f = min(lo_f, c.F[i]);
-                if (on >> i & 1) lo_g = min(lo_g, c.G[i]);
-            }
-            lo_f = __reduce_min_sync(full, lo_f) >> 8;
-            lo_g = __reduce_min_sync(full, lo_g) >> 8;
-        };
-        lowest();
-        const int4 rise = __ldg(&tab[k0 + 2]);
-        if (maxh0 - (lo_f + 1) < rise.y && maxtop - lo_g <= rise.z) break;
-        // what the warp reads in columns [k, k + n): first and last of each axis
-        int32_t u0, u1, v0, v1;
-        auto region = [&](int32_t k, int32_t n) {
-            const int32_t ca = cu + a.smaj * k, cb = cu + a.smaj * (k + n - 1);
-            // the first and the last row in direction sv
-            const int32_t qm = rows_after(tab, k - 1), qe = rows_after(tab, k + n);
-            const int32_t ra = cv + (sv > 0 ? qm : 1 + qm);
-            const int32_t rb = cv + sv * (V - 1) + (sv > 0 ? 1 + qe : qe);
-            u0 = __reduce_min_sync(full, min(ca, cb));
-            u1 = __reduce_max_sync(full, max(ca, cb));
-            v0 = __reduce_min_sync(full, min(ra, rb));
-            v1 = __reduce_max_sync(full, max(ra, rb));
-            return u1 >= 0 && u0 < NU && v1 >= 0 && v0 < NV;  // it meets the grid
-        };
-        if (!region(k0, 32)) break;  // and so do all later rounds
-        if (w.L >= 5 && !sun_may_rise<XM>(w, 5, u0, u1, v0, v1, lo_f, lo_g, rise.y, rise.z)) continue;
-#pragma unroll 1
-        for (int32_t k = k0; k < k0 + 32; k += kSunPart) {
-            if (!region(k, kSunPart)) break;
-            if (w.L >= kSunPartLevel) {
-                if (k > k0) lowest();
-                const int4 e = __ldg(&tab[k + 2]);
-                if (!sun_may_rise<XM>(w, kSunPartLevel, u0, u1, v0, v1, lo_f, lo_g, e.y, e.z)) continue;
-            }
-            if (u0 >= 0 && u1 < NU && v0 >= 0 && v1 < NV && __all_sync(full, f_on == on))
-                sun_round<XM, PAIR, V, false>(w, a, tab, k, cu, cv, sv, f_on, c);
-            else
-                sun_round<XM, PAIR, V, true>(w, a, tab, k, cu, cv, sv, f_on, c);
+        for (int i = 0; i < V; ++i) {
+            if (f_on >> i & 1) lo_f = min(lo_f, c.F[i]);
+            if (on >> i & 1) lo_g = min(lo_g, c.G[i]);
         }
+        lo_f = __reduce_min_sync(full, lo_f) >> 8;
+        lo_g = __reduce_min_sync(full, lo_g) >> 8;
+    };
+    // what the warp reads in columns [k, k + n): first and last of each axis
+    int32_t u0, u1, v0, v1;
+    auto region = [&](int32_t k, int32_t n) {
+        const int32_t ca = cu + a.smaj * k, cb = cu + a.smaj * (k + n - 1);
+        // the first and the last row in direction sv
+        const int32_t qm = rows_after(tab, k - 1), qe = rows_after(tab, k + n);
+        const int32_t ra = cv + (sv > 0 ? qm : 1 + qm);
+        const int32_t rb = cv + sv * (V - 1) + (sv > 0 ? 1 + qe : qe);
+        u0 = __reduce_min_sync(full, min(ca, cb));
+        u1 = __reduce_max_sync(full, max(ca, cb));
+        v0 = __reduce_min_sync(full, min(ra, rb));
+        v1 = __reduce_max_sync(full, max(ra, rb));
+        return u1 >= 0 && u0 < NU && v1 >= 0 && v0 < NV;  // it meets the grid
+    };
+    // f_on: cells whose F band was in the grid up to the round of column k
+    uint32_t f_on = on;
+#pragma unroll 1
+    for (int32_t k = 1 + (SPLIT ? kSunPart * first : 0);;
+         k += SPLIT ? kSunPart * kSunSplit : kSunPart) {
+        const bool round = (k - 1) % 32 == 0;
+        if (SPLIT || round) {
+            const int32_t k0 = (k - 1) / 32 * 32 + 1;
+            f_on = k0 == 1 ? on : on & ~(out1 | f_out(k0 - 1));
+        }
+        lowest(f_on);
+        const int4 rise = __ldg(&tab[k + 2]);
+        if (maxh0 - (lo_f + 1) < rise.y && maxtop - lo_g <= rise.z) break;
+        if (!SPLIT && round && w.L >= 5) {
+            if (!region(k, 32)) break;  // and so do all later rounds
+            if (!sun_may_rise<XM>(w, 5, u0, u1, v0, v1, lo_f, lo_g, rise.y, rise.z)) {
+                k += 32 - kSunPart;
+                continue;
+            }
+        }
+        if (!region(k, kSunPart)) break;
+        if (w.L >= kSunPartLevel &&
+            !sun_may_rise<XM>(w, kSunPartLevel, u0, u1, v0, v1, lo_f, lo_g, rise.y, rise.z))
+            continue;
+        if (u0 >= 0 && u1 < NU && v0 >= 0 && v1 < NV && __all_sync(full, f_on == on))
+            sun_part<XM, PAIR, V, false>(w, a, tab, k, cu, cv, sv, f_on, c);
+        else
+            sun_part<XM, PAIR, V, true>(w, a, tab, k, cu, cv, sv, f_on, c);
     }
 }
 
@@ -389,7 +398,7 @@ __global__ void __launch_bounds__(SPLIT ? kSunSplit * 32 : kSunThreads)
         }
     if (!__any_sync(0xFFFFFFFFu, on != 0)) return;  // (all warps of a split group alike)
     SunCells<V> c;
-    sun_bounds_of<XM, PAIR, V>(w, a, tab, cu, cv, sv, on, sub, SPLIT ? kSunSplit : 1, c);
+    sun_bounds_of<XM, PAIR, V, SPLIT>(w, a, tab, cu, cv, sv, on, sub, c);
     if (SPLIT) {
 #pragma unroll
         for (int i = 0; i < V; ++i) {
