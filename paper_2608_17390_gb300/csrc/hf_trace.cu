@@ -29,9 +29,10 @@ namespace hf {
 namespace {
 
 // Resident 128-thread blocks per SM asked of the register allocator: six leave
-// each thread 80 registers (without shadows 72 are used, so seven blocks fit).
-// 64 views with shadows / a 1080p eye-level view: four blocks 10.62 ms / 141 us,
-// five 9.66 / 129, six 9.39 / 126, seven (11 % more instructions) 9.75 / 127.
+// each thread 80 registers (the batched kernel with shadows uses 78, the others
+// 72 at most, so that seven fit).  64 views with shadows / 100 frames of 1080p
+// without: four blocks 10.62 ms / -, five 9.66 / -, six 9.39 / 8.15, seven (up to
+// 4 % more instructions) 9.43 / 8.57.
 constexpr int kTraceMinBlocks = 6;
 
 __constant__ float c_albedo[8][3] = HF_ALBEDO_TABLE;
@@ -70,13 +71,12 @@ __device__ __forceinline__ uint32_t level0_word(const WorldDev &w, int32_t x, in
     return load_word(w, 0, x, y);
 }
 
-__device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visible,
+__device__ __forceinline__ uint32_t shade(uint32_t m, uint8_t face, bool visible,
                                           const float *ln) {
     // the normal's axis is face / 2, its sign face's lowest bit
     const float n = face < kFaceNY ? ln[0] : face < kFaceNZ ? ln[1] : ln[2];
     const float ndl = face == kFaceInside ? 0.0f : face & 1 ? n : -n;
     const float k = kKa + kKd * fmaxf(ndl, 0.0f) * (visible ? 1.0f : 0.0f);
-    const uint32_t m = (word >> 24) & 7;
     uint32_t out = 0xFF000000u;
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) {
@@ -97,7 +97,7 @@ __device__ __forceinline__ uint32_t shade(uint32_t word, uint8_t face, bool visi
 //
 // Bound by instruction issue, as the traversal of single rays was: 2048 x 2048
 // grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 9.39
-// ms, a 1080p eye-level view with shadows 192 -> 126 us, a hundred 1080p frames
+// ms, a 1080p eye-level view with shadows 192 -> 122 us, a hundred 1080p frames
 // over 2048 x 16384 cells 17.3 -> 8.1 ms.
 template <bool PAIR>
 __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev *lvt,
@@ -168,6 +168,21 @@ __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev
     }
 }
 
+// What a warp works on, in shared memory: its camera's record and its tile's
+// first pixel.  Fields are read when they are needed instead of being held in
+// registers through a cast, where registers decide how many warps fit.
+struct TileDev {
+    CamDev cam;
+    int32_t x0, y0;
+};
+
+// Pixel i of the warp's tile.
+__device__ __forceinline__ void tile_pixel(const RenderParams &p, const TileDev &t, int i,
+                                           int32_t &px, int32_t &py) {
+    px = t.x0 + (i & ((1 << p.tile_w_log2) - 1));
+    py = t.y0 + (i >> p.tile_w_log2);
+}
+
 // The ray of a camera's pixel.
 __device__ __forceinline__ Ray primary_ray(const CamDev &c, int32_t px, int32_t py) {
     const int32_t a = 2 * px + 1 - (int32_t)c.w;
@@ -181,13 +196,16 @@ __device__ __forceinline__ Ray primary_ray(const CamDev &c, int32_t px, int32_t 
 // `inside` says whether the lane has a pixel.
 template <bool SHADOWS, int KIND, bool PAIR>
 __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelDev *lvt,
-                                             const CamDev &c, int start, int32_t px, int32_t py,
-                                             bool inside, const BeamDir &sun, Counters &cnt,
-                                             Counters &scnt, uint32_t &nshadow, bool &err) {
+                                             const TileDev &t, int start, int i, bool &inside,
+                                             const BeamDir &sun, Counters &cnt, Counters &scnt,
+                                             uint32_t &nshadow, bool &err) {
     constexpr bool STATS = KIND == kTraceStats;
+    const CamDev &c = t.cam;
+    int32_t px, py;
+    tile_pixel(p, t, i, px, py);
+    inside = px < (int32_t)c.w && py < (int32_t)c.h;
     Ray r = primary_ray(c, px, py);
-    uint32_t word = 0;  // of the primary hit, with its face: for the shading
-    uint8_t face = kFaceMiss;
+    uint32_t tag = kFaceMiss;  // of the primary hit: face and material (bits 8..10)
     bool visible = true;
     bool cast = inside;  // this lane's ray of the pass
 #pragma unroll 1
@@ -219,12 +237,18 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
         cast = false;
         const bool hit = h.face < kFaceError;
         // the ray again, from the camera: it need not be held through the cast
-        asm volatile("" : "+r"(px), "+r"(py)::"memory");
+        if (SHADOWS) {
+            asm volatile("" : "+r"(i)::"memory");
+            tile_pixel(p, t, i, px, py);
+            inside = px < (int32_t)c.w && py < (int32_t)c.h;
+        } else {
+            asm volatile("" : "+r"(px), "+r"(py)::"memory");
+        }
         r = primary_ray(c, px, py);
         const uint32_t pix = (uint32_t)py * c.w + (uint32_t)px;
         if (inside) {
-            word = h.word;
-            face = h.face;
+            const uint8_t face = h.face;
+            tag = face | (h.word >> 16 & 0x700);
             float depth = __int_as_float(0x7f800000);
             if (hit) {
                 const float fx = (float)r.dx, fy = (float)r.dy, fz = (float)r.dz;
@@ -246,7 +270,7 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
             // face normal.  The coordinate along the normal is exact: the ray
             // crosses that axis by tnum (its |d| is tden); the other two are
             // floored quotients.
-            const bool on_x = face <= kFacePX, on_z = face >= kFaceNZ;
+            const bool on_x = h.face <= kFacePX, on_z = h.face >= kFaceNZ;
             const int32_t dn = on_x ? r.dx : on_z ? r.dz : r.dy;
             const int32_t da = on_x ? r.dy : r.dx, db = on_z ? r.dy : r.dz;
             const int32_t qn = dn < 0 ? 1 - h.tnum : h.tnum - 1;  // one unit back
@@ -285,11 +309,11 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
         }
         if (!__any_sync(kFull, cast)) break;
     }
-    if (!inside) return;
+    if (px >= (int32_t)c.w || py >= (int32_t)c.h) return;
     const uint32_t pix = (uint32_t)py * c.w + (uint32_t)px;
+    const uint8_t face = tag & 0xFF;
     if (SHADOWS && c.shadow) __stcs(c.shadow + pix, (uint8_t)(visible ? 0 : 1));
-    if (c.rgba)
-        __stcs(c.rgba + pix, face < kFaceError ? shade(word, face, visible, p.sun_n) : kSky);
+    if (c.rgba) __stcs(c.rgba + pix, face < kFaceError ? shade(tag >> 8, face, visible, p.sun_n) : kSky);
 }
 
 // Start level of a camera's primary rays: the largest level l <= mip_start
@@ -320,23 +344,22 @@ __device__ __forceinline__ int primary_start(const RenderParams &p, const CamDev
 // One warp renders one tile: lane l traces the tile's pixels l, l+32, ...
 template <bool SHADOWS, int KIND, bool PAIR>
 __device__ __forceinline__ void trace_tile(const RenderParams &p, const LevelDev *lvt,
-                                           const BeamDir &sun, const CamDev &c,
-                                           uint32_t local_tile, int lane) {
-    const uint32_t tx = local_tile % c.tiles_x, ty = local_tile / c.tiles_x;
-    const int32_t tw_log2 = p.tile_w_log2;
-    const int32_t x0 = (int32_t)tx << tw_log2, y0 = (int32_t)ty << p.tile_h_log2;
-    const int32_t npix = 1 << (tw_log2 + p.tile_h_log2);
+                                           const BeamDir &sun, TileDev &t, uint32_t local_tile,
+                                           int lane) {
+    const CamDev &c = t.cam;
+    if (lane == 0) {
+        t.x0 = (int32_t)(local_tile % c.tiles_x) << p.tile_w_log2;
+        t.y0 = (int32_t)(local_tile / c.tiles_x) << p.tile_h_log2;
+    }
+    __syncwarp();
     Counters cnt{0, 0}, scnt{0, 0};
     uint32_t nshadow = 0, nrays = 0;
     bool err = false;
     constexpr bool STATS = KIND == kTraceStats;
     const int start = KIND == kTraceBeams ? 0 : primary_start<PAIR>(p, c, lane);
-    for (int i = lane; i < npix; i += 32) {
-        const int32_t px = x0 + (i & ((1 << tw_log2) - 1));
-        const int32_t py = y0 + (i >> tw_log2);
-        const bool inside = px < (int32_t)c.w && py < (int32_t)c.h;
-        trace_pixels<SHADOWS, KIND, PAIR>(p, lvt, c, start, px, py, inside, sun, cnt, scnt,
-                                          nshadow, err);
+    for (int i = lane; i < 1 << (p.tile_w_log2 + p.tile_h_log2); i += 32) {
+        bool inside;
+        trace_pixels<SHADOWS, KIND, PAIR>(p, lvt, t, start, i, inside, sun, cnt, scnt, nshadow, err);
         if (STATS && inside) nrays++;
     }
     if (KIND != kTraceBeams && __any_sync(kFull, err) && lane == 0) atomicOr(p.status, 1u);
@@ -373,13 +396,12 @@ __device__ __forceinline__ void fill_levels(LevelDev *s_lv, const WorldDev &w) {
     if (k <= w.L) s_lv[k] = LevelDev{w.base + w.off[k], (uint32_t)w.stride[k], (uint32_t)w.rows[k]};
 }
 
-// Copy camera i into this warp's shared slot (fields are then read on demand
-// instead of being held in registers for the whole tile).
-__device__ __forceinline__ const CamDev &stage_cam(CamDev *slot, const CamDev *cams, uint32_t i,
-                                                   int lane) {
+// Copy camera i into this warp's shared slot.
+__device__ __forceinline__ TileDev &stage_cam(TileDev *slot, const CamDev *cams, uint32_t i,
+                                              int lane) {
     static_assert(sizeof(CamDev) % 4 == 0 && sizeof(CamDev) / 4 <= 32, "one word per lane");
     const uint32_t *src = reinterpret_cast<const uint32_t *>(cams + i);
-    uint32_t *dst = reinterpret_cast<uint32_t *>(slot);
+    uint32_t *dst = reinterpret_cast<uint32_t *>(&slot->cam);
     __syncwarp();
     if (lane < (int)(sizeof(CamDev) / 4)) dst[lane] = src[lane];
     __syncwarp();
@@ -391,7 +413,7 @@ __device__ __forceinline__ const CamDev &stage_cam(CamDev *slot, const CamDev *c
 template <bool SHADOWS, int KIND, bool PAIR>
 __global__ void __launch_bounds__(kThreads, kTraceMinBlocks) k_trace_batched(const RenderParams p) {
     __shared__ uint32_t s_base[kMaxCams + 1];
-    __shared__ CamDev s_cam[kThreads / 32];
+    __shared__ TileDev s_tile[kThreads / 32];
     __shared__ LevelDev s_lv[kMaxLevels + 1];
     const uint32_t n = p.hdr->n_cams;
     const uint32_t total = p.hdr->total_tiles;
@@ -414,8 +436,8 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks) k_trace_batched(con
             if (s_base[mid] <= t) lo = mid;
             else hi = mid;
         }
-        const CamDev &c = stage_cam(&s_cam[threadIdx.x >> 5], p.cams, lo, lane);
-        trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, c, t - s_base[lo], lane);
+        TileDev &tile = stage_cam(&s_tile[threadIdx.x >> 5], p.cams, lo, lane);
+        trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, tile, t - s_base[lo], lane);
     }
 }
 
@@ -429,7 +451,7 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks)
     k_trace_plain(const __grid_constant__ RenderParams p, const __grid_constant__ CamDev cam,
                   uint32_t n_tiles) {
     __shared__ LevelDev s_lv[kMaxLevels + 1];
-    __shared__ CamDev s_cam[kThreads / 32];
+    __shared__ TileDev s_tile[kThreads / 32];
     __shared__ BeamDir s_sun;
     prefetch_world(p);
     if (SHADOWS && threadIdx.x == 32) s_sun = beam_dir(p.sun[0], p.sun[1], p.sun[2]);
@@ -438,8 +460,8 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks)
     const uint32_t t = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     if (t >= n_tiles) return;
     const int lane = threadIdx.x & 31;
-    const CamDev &c = stage_cam(&s_cam[threadIdx.x >> 5], &cam, 0, lane);
-    trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, c, t, lane);
+    TileDev &tile = stage_cam(&s_tile[threadIdx.x >> 5], &cam, 0, lane);
+    trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, tile, t, lane);
 }
 
 template <bool SH, int KIND, bool PA>
