@@ -18,6 +18,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #include "hf_internal.h"
 
@@ -73,6 +74,26 @@ HF_HD float cast_rcp_fast(float v) {
     return __fdividef(1.0f, v);
 #else
     return 1.0f / v;
+#endif
+}
+
+// Maximum of each 16-bit half.
+HF_HD uint32_t max_halves(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __vmaxu2(a, b);
+#else
+    const uint32_t al = a & 0xFFFF, bl = b & 0xFFFF, ah = a >> 16, bh = b >> 16;
+    return (al > bl ? al : bl) | (ah > bh ? ah : bh) << 16;
+#endif
+}
+
+HF_HD int32_t float_bits(float v) {
+#ifdef __CUDA_ARCH__
+    return __float_as_int(v);
+#else
+    int32_t i;
+    memcpy(&i, &v, sizeof i);
+    return i;
 #endif
 }
 
@@ -349,7 +370,7 @@ struct BeamRay {
     int32_t fu, fv;  // the start cell, mirrored
     int32_t ku, kv;  // minus the start's mirrored position, in 2^-16 units
     float z0;        // start height
-    float pu, pv;    // the start relative to the beam's cell (beam_place)
+    float pu, pv;    // the start relative to the beam's cell, v less a half (beam_place)
 };
 
 // (dx, dy not both 0)
@@ -385,7 +406,7 @@ HF_HD Ray beam_unray(const BeamDir &d, const BeamRay &q, int32_t oz, int32_t dz)
 }
 
 // A beam's rays, relative to the mirrored cell (u0, v0): at u = u0 + x every
-// ray has v - v0 in [a0 + r0 x, a1 + r1 x] and a height between b0 + s0 x and
+// ray has v - v0 - 1/2 in [a0 + r0 x, a1 + r1 x] and a height between b0 + s0 x and
 // b1 + s1 x, for x >= 0 (up to rounding, see beam_open).
 struct Beam {
     int32_t u0, v0;
@@ -393,11 +414,12 @@ struct Beam {
 };
 
 // Takes a ray's start relative to the beam's cell: exact up to 256 cells, else
-// rounded.  At u0 + x the ray is at v - v0 = pv + rho (x - pu), and at the
-// height z0 + sigma (x - pu); its terms of the beam are those at x = 0.
+// rounded.  At u0 + x the ray is at v - v0 = 1/2 + pv + rho (x - pu) (so that the
+// nearest integer to v - v0 - 1/2 is the row), and at the height z0 + sigma
+// (x - pu); its terms of the beam are those at x = 0.
 HF_HD void beam_place(BeamRay &q, const Beam &m) {
     q.pu = (float)(-q.ku - m.u0 * (1 << kShift)) * (1.0f / 65536.0f);
-    q.pv = (float)(-q.kv - m.v0 * (1 << kShift)) * (1.0f / 65536.0f);
+    q.pv = (float)(-q.kv - m.v0 * (1 << kShift) - (1 << (kShift - 1))) * (1.0f / 65536.0f);
 }
 
 // A bound of the error of a beam's heights up to x columns on: slopes have a
@@ -422,8 +444,8 @@ HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int k
     const float zlo = m.b0 + fminf(m.s0 * x0, m.s0 * x1) - zm;
     const float zhi = m.b1 + fmaxf(m.s1 * x0, m.s1 * x1) + zm;
     // (rows are off by less than 2^-6 at the largest grid)
-    const float vlo = m.a0 + fminf(m.r0 * x0, m.r1 * x0) - 0.015625f;
-    const float vhi = m.a1 + m.r1 * x1 + 0.015625f;
+    const float vlo = m.a0 + fminf(m.r0 * x0, m.r1 * x0) + (0.5f - 0.015625f);
+    const float vhi = m.a1 + m.r1 * x1 + (0.5f + 0.015625f);
     int32_t qa = (m.v0 + (int32_t)floorf(vlo)) >> l;
     int32_t qb = (m.v0 + (int32_t)floorf(vhi)) >> l;
     if (key & 1) {
@@ -433,24 +455,24 @@ HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int k
     }
     qa = qa < 0 ? 0 : qa;
     qb = qb < (int32_t)nv ? qb : (int32_t)nv - 1;
-    uint32_t top = 0, h0 = 0, h1 = 0xFF00;
+    uint32_t tops = 0, h1 = 0xFF00;  // highest top and floor, lowest slab
     for (int32_t jv = qa; jv <= qb; ++jv) {
         const uint32_t w = cast_word<PAIR>(lv, l, (int32_t)(x_major ? ju : jv),
-                                           (int32_t)(x_major ? jv : ju)) & 0xFFFFFFu;
-        top = top > w ? top : w;
-        h0 = h0 > (w & 0xFF) ? h0 : (w & 0xFF);
+                                           (int32_t)(x_major ? jv : ju));
+        tops = max_halves(tops, w & 0xFF00FF);
         h1 = h1 < (w & 0xFF00) ? h1 : (w & 0xFF00);
     }
-    high = top >> 16;
-    return !(zlo > (float)high || (zlo > (float)h0 && zhi < (float)(h1 >> 8)));
+    high = tops >> 16;
+    const float h0 = (float)(tops & 0xFF);
+    return !(zlo > (float)high || (zlo > h0 && zhi < (float)(h1 >> 8)));
 }
 
 // A ray on its way through the columns of a run, up to x1 (columns x, rows and
 // heights are relative to the beam's cell).
 //
 // Rows: v is off by less than ev = (x1 + |pu| + |pv| + 1) 1.5 2^-22: rho by
-// 2^-23 of itself, x - pu and the sum by 2^-24, and |rho| <= 1.  Where v is
-// nearer than that to a boundary, the two are compared exactly; a ray through
+// 2^-23 of itself, x - pu, the start and the sum by 2^-24, and |rho| <= 1.  Where
+// v is nearer than that to a boundary, the two are compared exactly; a ray through
 // the corner itself is left to cast_general.
 // Heights: off by less than e2 / 2 = (|sigma| (x1 + |pu| + 2) + |z0|) 2^-21.
 struct BeamWalk {
@@ -466,12 +488,13 @@ enum { kBeamGoing = 0, kBeamOpen = 1, kBeamLeft = 2, kBeamCorner = 3 };
 // if it enters through a corner.
 HF_HD bool beam_row(const BeamDir &d, const BeamRay &q, const Beam &m, const BeamWalk &w,
                     int32_t x, float dx, int32_t &row) {
-    const float v = fmaf(d.rho, dx, q.pv), f = floorf(v);
-    row = (int32_t)f;
-    if (fabsf(v - f - 0.5f) < 0.5f - w.ev) return true;
+    // rounding to the nearest integer by an addition: 3 2^22 has units of 1
+    const float v = fmaf(d.rho, dx, q.pv), t = v + 12582912.0f, f = t - 12582912.0f;
+    row = float_bits(t) - 0x4B400000;
+    if (fabsf(v - f) < 0.5f - w.ev) return true;
     // which of the ray's crossings of the nearest row boundary and of column x
     // comes first
-    row = (int32_t)floorf(v + 0.5f);
+    row = (int32_t)floorf(v + 1.0f);
     const int64_t side = (int64_t)((m.v0 + row) * (1 << kShift) + q.kv) * d.du;
     const int64_t here = (int64_t)((m.u0 + x) * (1 << kShift) + q.ku) * d.dv;
     if (side > here) row -= 1;
@@ -543,9 +566,9 @@ HF_HD int beam_step(const BeamGrid &g, const BeamDir &d, const BeamRay &q, const
     const uint32_t wa = beam_word<PAIR>(g.cells, ca), wb = beam_word<PAIR>(g.cells, cb);
     c.wa = wa;
     c.wb = wb;
-    const uint32_t ta = wa & 0xFF0000, tb = wb & 0xFF0000;
-    const uint32_t fa = wa & 0xFF, fb = wb & 0xFF, ma = wa & 0xFF00, mb = wb & 0xFF00;
-    const float top = (float)((ta > tb ? ta : tb) >> 16), h0 = (float)(fa > fb ? fa : fb);
+    const uint32_t high = max_halves(wa & 0xFF00FF, wb & 0xFF00FF);  // top and floor
+    const uint32_t ma = wa & 0xFF00, mb = wb & 0xFF00;
+    const float top = (float)(high >> 16), h0 = (float)(high & 0xFF);
     const float h1 = (float)((ma < mb ? ma : mb) >> 8);
     const float zlo = fminf(w.zl, c.zl), zhi = fmaxf(w.zl, c.zl) + w.e2;
     if (!sure) return kBeamCorner;
@@ -564,7 +587,7 @@ struct BeamHit {
 // the ray enters it, changes row and leaves it.  The hit's kind, -1 if there is
 // none, -2 if it is too close to tell.  second: it is in the row of the exit.
 //
-// The row changes where v = row + 1, at x - pu = (row + 1 - pv) / rho, off by
+// The row changes where v = row + 1, at x - pu = (row + 1/2 - pv) / rho, off by
 // less than 2 ev / rho.
 HF_HD int beam_decide(const BeamGrid &g, const BeamDir &d, const BeamRay &q, const BeamWalk &w,
                       const BeamColumn &c, bool &second) {
@@ -573,7 +596,7 @@ HF_HD int beam_decide(const BeamGrid &g, const BeamDir &d, const BeamRay &q, con
     second = false;
     if (c.row > w.row) {
         const float inv = cast_rcp_fast(d.rho), es = fabsf(d.sigma) * (2.0f * w.ev) * inv;
-        const float zs = fmaf(d.sigma, ((float)(w.row + 1) - q.pv) * inv, w.zbase);
+        const float zs = fmaf(d.sigma, ((float)w.row + 0.5f - q.pv) * inv, w.zbase);
         const float sl = zs - es, su = zs + w.e2 + es;
         const float lo = fminf(il, sl), hi = fmaxf(iu, su);
         second = (lo > (float)(word >> 16 & 0xFF)) |

@@ -96,9 +96,9 @@ __device__ __forceinline__ uint32_t shade(uint32_t m, uint8_t face, bool visible
 // one or two rounds.
 //
 // Bound by instruction issue, as the traversal of single rays was: 2048 x 2048
-// grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 9.39
-// ms, a 1080p eye-level view with shadows 192 -> 122 us, a hundred 1080p frames
-// over 2048 x 16384 cells 17.3 -> 8.1 ms.
+// grid with caves and walls, 64 views of 188 M rays with shadows 13.47 -> 9.27
+// ms, a 1080p eye-level view with shadows 192 -> 120 us, a hundred 1080p frames
+// over 2048 x 16384 cells 17.3 -> 8.0 ms.
 template <bool PAIR>
 __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev *lvt,
                                            const BeamDir &d, BeamRay q, int32_t oz, int32_t dz,
