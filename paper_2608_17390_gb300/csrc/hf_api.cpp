@@ -214,6 +214,38 @@ int ctx_view(const hf_ctx *c, CtxView *out) {
 
 }  // namespace hf
 
+// A beam pays where the rays of a warp go through the same cells.  The angle that
+// the warp's group of 32 pixels spans (8 x 4, or a row of a wide tile), times the
+// length of the world, says how far they fall apart.  Rays each by itself over
+// beams, single views and batches of 16, with and without shadows, 8 x 4 tiles:
+//   span (rad)   0.017        0.025       0.033       0.05        0.067       0.1
+//   256^2        1.29 - 1.85  1.28 - 1.8  1.07 - 1.7  1.01 - 1.65 0.91 - 1.43 0.77 - 1.48
+//   2048^2       1.47 - 1.80  1.28 - 1.8  1.11 - 1.4  0.90 - 1.73 0.78 - 1.60 0.66 - 1.73
+//   2048 x 8192  1.49 - 2.03  1.16 - 1.9  0.73 - 2.0  0.21 - 1.54 0.17 - 1.48 0.12 - 1.39
+// So spans up to 0.04 get beams, up to 0.06 in worlds of up to 512 cells, and up to
+// 0.028 in worlds of more than 4096.  In a batch the pixels of cameras beyond that
+// may make up one in 32: they cost up to ten times as much.
+namespace hf {
+bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw) {
+    const int32_t size = W > H ? W : H;
+    const double most = size <= 512 ? 0.06 : size <= 4096 ? 0.04 : 0.028;
+    const double gw = tw < 32 ? tw : 32, gh = 32 / gw;
+    uint64_t all = 0, wide = 0;
+    for (uint32_t i = 0; i < n; ++i) {
+        const hf_camera &k = cams[i];
+        auto norm2 = [](const int32_t *v) {
+            return (double)v[0] * v[0] + (double)v[1] * v[1] + (double)v[2] * v[2];
+        };
+        // neighbouring pixels are 2 |right|, 2 |up| apart at distance |fwd|
+        const double across = 4.0 * gw * gw * norm2(k.right), along = 4.0 * gh * gh * norm2(k.up);
+        const uint64_t px = (uint64_t)k.w * k.h;
+        all += px;
+        if ((across > along ? across : along) > most * most * norm2(k.fwd)) wide += px;
+    }
+    return wide * 32 <= all;
+}
+}  // namespace hf
+
 extern "C" {
 
 const char *hf_strerror(int code) {
@@ -1141,8 +1173,9 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         if (iabs64(sun[i]) >= kLimit21) return HF_E_INVALID_ARG;
     const bool shadows = (o.flags & HF_SHADOWS) != 0;
     const int kind = (o.flags & HF_STATS) ? hf::kTraceStats
-                     : o.max_steps        ? hf::kTraceGeneral
-                                          : hf::kTraceBeams;
+                     : o.max_steps || !hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw)
+                         ? hf::kTraceGeneral
+                         : hf::kTraceBeams;
     const uint32_t mip = o.mip_start == HF_MIP_AUTO ? hf::kDefaultMipStart : o.mip_start;
     const uint32_t mip_c = mip > c->L ? c->L : mip;
     const uint64_t guard = 4ull * (c->W + c->H) + 64;
@@ -1223,7 +1256,8 @@ int hf_render_march(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outpu
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
     CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));
-    if (hf::launch_march_batched(b.p, m, c->sm_count * c->occ_march, b.stream)) return HF_E_CUDA;
+    const bool beams = hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw);
+    if (hf::launch_march_batched(b.p, m, beams, c->sm_count * c->occ_march, b.stream)) return HF_E_CUDA;
     return finish_batch(c, b, (o.flags & HF_SYNC) != 0);
 }
 

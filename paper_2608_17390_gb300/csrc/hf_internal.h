@@ -10,6 +10,7 @@
 //   BatchHeader (tile counter, camera count, tile count), then CamDev[n].
 #pragma once
 
+#include "hf.h"
 #include <cuda_runtime.h>
 #include <cstdint>
 
@@ -146,7 +147,8 @@ struct MarchParams {
     int32_t bisections;  // halvings of the bracketing interval
     float far_dist;      // world units
 };
-int launch_march_batched(const RenderParams &p, const MarchParams &m, int blocks, void *stream);
+int launch_march_batched(const RenderParams &p, const MarchParams &m, bool beams, int blocks,
+                         void *stream);
 int march_occupancy(int *blocks_per_sm);
 
 // Parameters of the scattered comparison renderer (hf_scatter.cu).  The
@@ -188,6 +190,8 @@ int launch_voxel_trace(const RenderParams &p, const VoxelDev &v, const VoxelPara
 // Launch wrappers (hf_trace.cu)
 // How the trace kernels follow rays: warps of rays in beams; one ray at a time
 // (a step limit set by the caller: p.max_steps); the same with fetch counters.
+// Whether the rays of a warp's 32 pixels stay close enough for beams (hf_api.cpp).
+bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw);
 enum TraceKind { kTraceBeams = 0, kTraceGeneral = 1, kTraceStats = 2, kTraceKinds = 3 };
 // The trace kernels are instantiated per level-0 storage; p.world.pair picks one.
 int launch_trace_batched(const RenderParams &p, bool shadows, int kind, int blocks, void *stream);

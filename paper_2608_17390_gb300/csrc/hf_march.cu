@@ -32,6 +32,14 @@ constexpr int kMarchThreads = 128;
 // Nine blocks leave each thread 56 registers.  12 views of 1280 x 800 with 128
 // samples a ray: seven blocks 638 us, nine 622, eleven (46 registers) 692.
 constexpr int kMarchMinBlocks = 9;
+// From this many samples a ray on, and where the rays of a warp stay close (as
+// for the exact cast), beams are cheaper than taking every sample.  Every sample
+// / beams: 12 views of 1280 x 800 over 2048 x 16384 cells, 32 samples 630 / 609
+// us, 128 1517 / 596; but 16 views of 640 x 360 near the ground of a 2048 x 2048
+// world, 48 samples 0.70, 96 1.03, 128 1.26 times as fast with beams.  The kernel
+// without beams needs 36 registers, and 12 blocks fit.
+constexpr int kMarchBeamSteps = 96;
+constexpr int kMarchAllMinBlocks = 12;
 
 struct MarchPoint {
     bool solid;
@@ -82,33 +90,10 @@ __device__ __forceinline__ int32_t march_samples(const WorldDev &w, const MarchR
     return found;
 }
 
-// One pixel per lane; every lane of the warp calls.
-__device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchParams &mp,
-                                             const LevelDev *lvt, const CamDev &c, int32_t px,
-                                             int32_t py, bool inside) {
-    const int32_t a = 2 * px + 1 - (int32_t)c.w;
-    const int32_t b = (int32_t)c.h - 1 - 2 * py;
-    const float inv_s = 1.0f / 65536.0f;
-    const Ray r{c.o[0], c.o[1], c.o[2], c.F[0] + a * c.R[0] + b * c.U[0],
-                c.F[1] + a * c.R[1] + b * c.U[1], c.F[2] + a * c.R[2] + b * c.U[2]};
-    MarchRay m;
-    m.ox = __fmul_rn(__int2float_rn(r.ox), inv_s);
-    m.oy = __fmul_rn(__int2float_rn(r.oy), inv_s);
-    m.oz = __fmul_rn(__int2float_rn(r.oz), inv_s);
-    m.dx = __fmul_rn(__int2float_rn(r.dx), inv_s);
-    m.dy = __fmul_rn(__int2float_rn(r.dy), inv_s);
-    m.dz = __fmul_rn(__int2float_rn(r.dz), inv_s);
-    float sq = __fmul_rn(m.dx, m.dx);
-    sq = __fadd_rn(sq, __fmul_rn(m.dy, m.dy));
-    sq = __fadd_rn(sq, __fmul_rn(m.dz, m.dz));
-    const float len = __fsqrt_rn(sq);
-    float t_end = __fdiv_rn(mp.far_dist, len);
-    if (m.dz < 0.0f) {
-        const float tz = __fdiv_rn(-m.oz, m.dz);
-        if (tz < t_end) t_end = tz;
-    }
-    m.dt = __fdiv_rn(t_end, (float)(mp.steps + 1));
-
+// The first solid sample of each lane's ray, or 0; every lane of the warp calls.
+__device__ __forceinline__ int32_t march_beams(const RenderParams &p, const MarchParams &mp,
+                                               const LevelDev *lvt, const Ray &r, const MarchRay &m,
+                                               bool inside) {
     int32_t found = 0;
     const int lane = threadIdx.x & 31;
     const BeamDir d = beam_dir(r.dx, r.dy, r.dz);
@@ -155,6 +140,45 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
     }
     if (__any_sync(kFull, inside && plain))
         found = max(found, march_samples(p.world, m, inside && plain, 1, mp.steps));
+    return found;
+}
+
+// One pixel per lane; every lane of the warp calls.
+template <bool BEAMS>
+__device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchParams &mp,
+                                             const LevelDev *lvt, const CamDev &c, int32_t px,
+                                             int32_t py, bool inside) {
+    const int32_t a = 2 * px + 1 - (int32_t)c.w;
+    const int32_t b = (int32_t)c.h - 1 - 2 * py;
+    const float inv_s = 1.0f / 65536.0f;
+    const Ray r{c.o[0], c.o[1], c.o[2], c.F[0] + a * c.R[0] + b * c.U[0],
+                c.F[1] + a * c.R[1] + b * c.U[1], c.F[2] + a * c.R[2] + b * c.U[2]};
+    MarchRay m;
+    m.ox = __fmul_rn(__int2float_rn(r.ox), inv_s);
+    m.oy = __fmul_rn(__int2float_rn(r.oy), inv_s);
+    m.oz = __fmul_rn(__int2float_rn(r.oz), inv_s);
+    m.dx = __fmul_rn(__int2float_rn(r.dx), inv_s);
+    m.dy = __fmul_rn(__int2float_rn(r.dy), inv_s);
+    m.dz = __fmul_rn(__int2float_rn(r.dz), inv_s);
+    float sq = __fmul_rn(m.dx, m.dx);
+    sq = __fadd_rn(sq, __fmul_rn(m.dy, m.dy));
+    sq = __fadd_rn(sq, __fmul_rn(m.dz, m.dz));
+    const float len = __fsqrt_rn(sq);
+    float t_end = __fdiv_rn(mp.far_dist, len);
+    if (m.dz < 0.0f) {
+        const float tz = __fdiv_rn(-m.oz, m.dz);
+        if (tz < t_end) t_end = tz;
+    }
+    m.dt = __fdiv_rn(t_end, (float)(mp.steps + 1));
+
+    int32_t found = 0;
+    if (!BEAMS && inside)
+        for (int32_t i = 1; i <= mp.steps; ++i)
+            if (march_at(p.world, m, __fmul_rn((float)i, m.dt)).solid) {
+                found = i;
+                break;
+            }
+    if (BEAMS) found = march_beams(p, mp, lvt, r, m, inside);
 
     if (!inside) return;
     uint32_t cell = 0xFFFFFFFFu;
@@ -189,7 +213,8 @@ __device__ __forceinline__ const CamDev &stage(CamDev *slot, const CamDev *cams,
 }
 
 // Persistent: warps pop (camera, tile) items from the batch's atomic counter.
-__global__ void __launch_bounds__(kMarchThreads, kMarchMinBlocks)
+template <bool BEAMS>
+__global__ void __launch_bounds__(kMarchThreads, BEAMS ? kMarchMinBlocks : kMarchAllMinBlocks)
     k_march_batched(const RenderParams p, const MarchParams m) {
     __shared__ LevelDev s_lv[kMaxLevels + 1];
     __shared__ uint32_t s_base[kMaxCams + 1];
@@ -222,21 +247,29 @@ __global__ void __launch_bounds__(kMarchThreads, kMarchMinBlocks)
         for (int i = lane; i < npix; i += 32) {
             const int32_t px = x0 + (i & ((1 << p.tile_w_log2) - 1));
             const int32_t py = y0 + (i >> p.tile_w_log2);
-            march_pixels(p, m, s_lv, c, px, py, px < (int32_t)c.w && py < (int32_t)c.h);
+            march_pixels<BEAMS>(p, m, s_lv, c, px, py, px < (int32_t)c.w && py < (int32_t)c.h);
         }
     }
 }
 
 }  // namespace
 
-int launch_march_batched(const RenderParams &p, const MarchParams &m, int blocks, void *stream) {
-    k_march_batched<<<blocks, kMarchThreads, 0, (cudaStream_t)stream>>>(p, m);
+// blocks: as many as are resident of the kernel with beams (march_occupancy).
+int launch_march_batched(const RenderParams &p, const MarchParams &m, bool beams, int blocks,
+                         void *stream) {
+    cudaStream_t s = (cudaStream_t)stream;
+    if (beams && m.steps >= kMarchBeamSteps) {
+        k_march_batched<true><<<blocks, kMarchThreads, 0, s>>>(p, m);
+    } else {
+        const int all = (blocks * kMarchAllMinBlocks + kMarchMinBlocks - 1) / kMarchMinBlocks;
+        k_march_batched<false><<<all, kMarchThreads, 0, s>>>(p, m);
+    }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int march_occupancy(int *blocks_per_sm) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-               blocks_per_sm, reinterpret_cast<const void *>(&k_march_batched), kMarchThreads, 0) ==
+               blocks_per_sm, reinterpret_cast<const void *>(&k_march_batched<true>), kMarchThreads, 0) ==
                    cudaSuccess
                ? 0
                : -1;

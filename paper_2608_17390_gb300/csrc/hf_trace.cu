@@ -682,7 +682,9 @@ extern "C" int hf_render_noalloc(hf_ctx *ctx, const hf_camera *cams, uint32_t n,
         p.sun[i] = sun[i];
         p.sun_n[i] = (float)(sun[i] / sn);
     }
-    const int kind = o.max_steps ? kTraceGeneral : kTraceBeams;
+    const int kind = o.max_steps || !beams_fit(v.world.W, v.world.H, cams, n, tw)
+                         ? kTraceGeneral
+                         : kTraceBeams;
     const int blocks = v.sm_count * v.occ[shadows ? 1 : 0][kind];
     if (launch_trace_batched(p, shadows, kind, blocks, stream)) return HF_E_CUDA;
     if (o.flags & HF_SYNC) {

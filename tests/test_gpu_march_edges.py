@@ -21,10 +21,11 @@ def _check(got, ref, what):
     assert np.array_equal(got["depth"].view(np.uint32), ref["depth"].view(np.uint32)), what
 
 
+@pytest.mark.parametrize("wide", [True, False])
 @pytest.mark.parametrize("W,H,pairs", [(1, 1, False), (37, 53, False), (300, 9, False), (130, 97, True)])
 @pytest.mark.parametrize("steps,far,tile", [(128, 600.0, (8, 4)), (1000, 90.0, (4, 32)), (7, 5000.0, (32, 1)),
                                             (64, 0.05, (16, 8))])
-def test_samples_around_the_beams(hf, W, H, pairs, steps, far, tile):
+def test_samples_around_the_beams(hf, W, H, pairs, steps, far, tile, wide):
     rng = np.random.default_rng(W * H + steps)
     cells, _ = synth.make_grid(W, H, seed=W + H, slab_frac=0.4, n_walls=max(1, W // 10))
     if pairs:
@@ -34,6 +35,8 @@ def test_samples_around_the_beams(hf, W, H, pairs, steps, far, tile):
         x, y = rng.uniform(0.1, W - 0.1), rng.uniform(0.1, H - 0.1)
         z = [0.0, 60.0, 125.0, 210.0, 400.0, 90.0, 3000.0][k]
         hfov = 60 if max(w, h) < 30 or w >= h else 10
+        if not wide:  # (rays close enough for beams)
+            hfov = min(0.09 * w / max(min(tile[0], 32), 32 // min(tile[0], 32)) * 45, 60)
         cams.append(synth.pose_to_camera(x, y, z, 51.0 * k, [-90, -45, -10, 0, -30, 20, -70][k], hfov, w, h))
     for g in range(60):
         o = [int(rng.integers(0, W * S)), int(rng.integers(0, H * S)), int(rng.integers(0, 250 * S))]
