@@ -37,9 +37,10 @@ constexpr int kMarchMinBlocks = 9;
 // / beams: 12 views of 1280 x 800 over 2048 x 16384 cells, 32 samples 630 / 609
 // us, 128 1517 / 596; but 16 views of 640 x 360 near the ground of a 2048 x 2048
 // world, 48 samples 0.70, 96 1.03, 128 1.26 times as fast with beams.  The kernel
-// without beams needs 36 registers, and 12 blocks fit.
+// without beams needs 40 registers, so that 48 warps fit an SM; in blocks of 128
+// threads it is 3 % slower.
 constexpr int kMarchBeamSteps = 96;
-constexpr int kMarchAllMinBlocks = 12;
+constexpr int kMarchAllMinBlocks = 6, kMarchAllThreads = 256;
 
 struct MarchPoint {
     bool solid;
@@ -214,15 +215,16 @@ __device__ __forceinline__ const CamDev &stage(CamDev *slot, const CamDev *cams,
 
 // Persistent: warps pop (camera, tile) items from the batch's atomic counter.
 template <bool BEAMS>
-__global__ void __launch_bounds__(kMarchThreads, BEAMS ? kMarchMinBlocks : kMarchAllMinBlocks)
+__global__ void __launch_bounds__(BEAMS ? kMarchThreads : kMarchAllThreads,
+                                  BEAMS ? kMarchMinBlocks : kMarchAllMinBlocks)
     k_march_batched(const RenderParams p, const MarchParams m) {
     __shared__ LevelDev s_lv[kMaxLevels + 1];
     __shared__ uint32_t s_base[kMaxCams + 1];
-    __shared__ CamDev s_cam[kMarchThreads / 32];
+    __shared__ CamDev s_cam[(BEAMS ? kMarchThreads : kMarchAllThreads) / 32];
     const uint32_t n = p.hdr->n_cams;
     const uint32_t total = p.hdr->total_tiles;
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) s_base[i] = p.cams[i].tile_base;
-    if (threadIdx.x <= (unsigned)p.world.L) {
+    if (BEAMS && threadIdx.x <= (unsigned)p.world.L) {
         const int l = threadIdx.x;
         s_lv[l] = LevelDev{p.world.base + p.world.off[l], p.world.stride[l], p.world.rows[l]};
     }
@@ -262,7 +264,7 @@ int launch_march_batched(const RenderParams &p, const MarchParams &m, bool beams
         k_march_batched<true><<<blocks, kMarchThreads, 0, s>>>(p, m);
     } else {
         const int all = (blocks * kMarchAllMinBlocks + kMarchMinBlocks - 1) / kMarchMinBlocks;
-        k_march_batched<false><<<all, kMarchThreads, 0, s>>>(p, m);
+        k_march_batched<false><<<all, kMarchAllThreads, 0, s>>>(p, m);
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
