@@ -58,7 +58,8 @@ def _dist():
 
 # ------------------------------------------------------------- ncu traffic
 
-TRACE_SOURCES = ("paper_2608_17390_gb300/csrc/hf_trace.cu", "paper_2608_17390_gb300/csrc/hf_internal.h")
+TRACE_SOURCES = tuple("paper_2608_17390_gb300/csrc/" + f
+                      for f in ("hf_trace.cu", "hf_beam.h", "hf_cast.h", "hf_internal.h"))
 
 
 def trace_source_hash():
@@ -583,8 +584,10 @@ def run_hf(args):
                      "peak_source": src,
                      "bytes_per_ray": alg_bytes / max(rays, 1),
                      "note": "algorithmic bytes = 4 B x (pyramid nodes + cells + shadow-ray "
-                             "fetches, counted in-kernel) + %d B output per ray; most fetches "
-                             "are L2/L1 hits" % (14 + (1 if wl["shadows"] else 0))},
+                             "fetches of the traversal ray by ray, counted in-kernel by a render "
+                             "with HF_STATS) + %d B output per ray; the timed kernels test nodes "
+                             "for 32 rays at a time and fetch fewer, mostly from L1 and L2"
+                             % (14 + (1 if wl["shadows"] else 0))},
         "alu_roofline": _alu_roofline(args.workload, rays, r_ms, "%dx%d" % (tile_w, tile_h),
                                       mip_start, info["sm_count"],
                                       (ck or {}).get("sm_mhz") or _peak_sm_mhz()),
