@@ -8,14 +8,16 @@ namespace hf {
 
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 
+// (volatile: every lane must execute them together, so they stay where they are
+// called, also where only some lanes go on to use the result)
 __device__ __forceinline__ float warp_min(float v) {
     float r;
-    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
 __device__ __forceinline__ float warp_max(float v) {
     float r;
-    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
 
