@@ -40,7 +40,8 @@ def build(verbose=False, extra=()):
     """Compile and link; returns the library path.  Raises on failure."""
     os.makedirs(OUT, exist_ok=True)
     headers = [os.path.join(ROOT, "include", "hf.h"), os.path.join(CSRC, "hf_internal.h"),
-               os.path.join(CSRC, "hf_cast.h"), os.path.join(CSRC, "hf_beam.h")]
+               os.path.join(CSRC, "hf_cast.h"), os.path.join(CSRC, "hf_beam.h"),
+               os.path.join(CSRC, "hf_march.h")]
     jobs = []
     objs = []
     for src in SOURCES:

@@ -52,7 +52,8 @@ __device__ __forceinline__ void beam_scan(BeamScan &s, const WorldDev &w, const 
 
 // The next run, columns [b0, b1), for the rays still alive (at least one); false
 // when no more of the grid can hold a solid on their way.  All lanes call.
-template <bool PAIR>
+// SAMPLES: for the rounded samples on the rays (hf_march.h).
+template <bool PAIR, bool SAMPLES = false>
 __device__ __forceinline__ bool beam_next(BeamScan &s, const LevelDev *lvt, const BeamDir &d,
                                           const BeamRay &q, bool alive, int32_t &b0, int32_t &b1,
                                           uint32_t *peak = nullptr) {
@@ -71,13 +72,13 @@ __device__ __forceinline__ bool beam_next(BeamScan &s, const LevelDev *lvt, cons
             s.m.s0 = warp_min(alive ? d.sigma : big);
             s.m.s1 = warp_max(alive ? d.sigma : -big);
         }
-        s.u = beam_skip(s.m, s.u, s.limit, s.top);
+        s.u = beam_skip<SAMPLES>(s.m, s.u, s.limit, s.top);
         if (s.u >= s.limit) return false;
         const int least = beam_least(s.m, s.u, s.base_level, s.top_level);
         s.level = max(s.level, least);
         s.j = s.u >> s.level;
         const uint32_t open = __ballot_sync(
-            kFull, beam_open<PAIR>(lvt, s.m, s.level, s.j + lane, s.key, s.high));
+            kFull, beam_open<PAIR, SAMPLES>(lvt, s.m, s.level, s.j + lane, s.key, s.high));
         if (s.level > least && open) {
             s.u = max(s.u, (s.j + __ffs(open) - 1) * (1 << s.level));
             s.level = least;

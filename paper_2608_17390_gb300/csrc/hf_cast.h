@@ -423,14 +423,20 @@ HF_HD void beam_place(BeamRay &q, const Beam &m) {
 }
 
 // A bound of the error of a beam's heights up to x columns on: slopes have a
-// relative error of 2^-23, and heights up to 4096 matter.
+// relative error of 2^-23, and heights up to 4096 matter.  SAMPLES: of the heights of
+// rounded samples, which lie up to kSampleAlong / 2 columns off their rays along u,
+// and as far before the start (hf_march.h).
+constexpr float kSampleAlong = 1.0f / 256.0f;
+template <bool SAMPLES = false>
 HF_HD float beam_slack(const Beam &m, float x) {
-    return 0.02f + fmaxf(fabsf(m.s0), fabsf(m.s1)) * (fabsf(x) + 2.0f) * (1.0f / 1048576.0f);
+    float per = (fabsf(x) + 2.0f) * (1.0f / 1048576.0f);
+    if (SAMPLES) per += kSampleAlong;
+    return 0.02f + fmaxf(fabsf(m.s0), fabsf(m.s1)) * per;
 }
 
 // Whether the beam may meet a solid in mirrored columns [j 2^l, (j + 1) 2^l).
 // The rows it covers there are read as nodes of level l.  high: their highest top.
-template <bool PAIR>
+template <bool PAIR, bool SAMPLES = false>
 HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int key,
                      uint32_t &high) {
     high = 0;
@@ -440,10 +446,10 @@ HF_HD bool beam_open(const LevelDev *lvt, const Beam &m, int l, int32_t j, int k
     const uint32_t ju = (uint32_t)(key & 2 ? ~j : j);
     if (ju >= nu) return false;
     const float x0 = (float)(j * (1 << l) - m.u0), x1 = x0 + (float)(1 << l);
-    const float zm = beam_slack(m, x1);
+    const float zm = beam_slack<SAMPLES>(m, x1);
     const float zlo = m.b0 + fminf(m.s0 * x0, m.s0 * x1) - zm;
     const float zhi = m.b1 + fmaxf(m.s1 * x0, m.s1 * x1) + zm;
-    // (rows are off by less than 2^-6 at the largest grid)
+    // (rows, of samples too, are off by less than 2^-6 at the largest grid)
     const float vlo = m.a0 + fminf(m.r0 * x0, m.r1 * x0) + (0.5f - 0.015625f);
     const float vhi = m.a1 + m.r1 * x1 + (0.5f + 0.015625f);
     int32_t qa = (m.v0 + (int32_t)floorf(vlo)) >> l;
@@ -718,9 +724,10 @@ HF_HD int beam_least(const Beam &m, int32_t u, int base, int top) {
 // The first column to test, from u on: a beam that starts above every top
 // is empty until its lowest ray comes down to them; one that rises above them
 // is done (the limit is returned).  limit: the mirrored column past the grid.
+template <bool SAMPLES = false>
 HF_HD int32_t beam_skip(const Beam &m, int32_t u, int32_t limit, float top) {
     const float x0 = (float)(u - m.u0);
-    if (!(m.b0 + m.s0 * x0 - beam_slack(m, x0) > top)) return u;
+    if (!(m.b0 + m.s0 * x0 - beam_slack<SAMPLES>(m, x0) > top)) return u;
     if (m.s0 >= 0.0f) return limit;
     // where the lowest line is 0.04 above the top: it falls by at most 4096 up
     // to there, so it is off by less (and two columns are kept for a steep one)

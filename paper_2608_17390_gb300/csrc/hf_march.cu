@@ -15,15 +15,14 @@
 // Samples that cannot be solid are not taken: the 32 rays of a warp are bounded
 // by beams as in the exact cast (hf_beam.h), and only samples whose column lies
 // in a stretch that the beam does not prove empty, at a height that its cells
-// reach, are looked up.  A sample's rounded position is off its ray by less than
-// 2^-8 cells and 2^-10 height units (three roundings of values up to 16384 and
-// 4096), which the beams' slack of 2^-6 and 0.02 covers beside their own error.
+// reach, are looked up (hf_march.h: the bounds of their rounding).
 // Bound by instruction issue: 12 views of 1280 x 800 over 2048 x 16384 cells, 128
-// samples a ray, 1.229 -> 0.622 ms (1270 -> 612 M warp instructions).
+// samples a ray, 1.229 -> 0.627 ms.
 #include <cuda_runtime.h>
 
 #include "hf_beam.h"
 #include "hf_internal.h"
+#include "hf_march.h"
 
 namespace hf {
 namespace {
@@ -44,35 +43,21 @@ constexpr int kMarchAllMinBlocks = 6, kMarchAllThreads = 256;
 
 struct MarchPoint {
     bool solid;
-    int32_t cx, cy;
+    MarchSpot at;
     uint8_t layer;
 };
 
-__device__ __forceinline__ MarchPoint march_solid(const WorldDev &w, float x, float y, float z) {
+__device__ __forceinline__ MarchPoint march_at(const WorldDev &w, const MarchRay &m, float t) {
     MarchPoint r;
-    r.cx = (int32_t)floorf(x);
-    r.cy = (int32_t)floorf(y);
+    r.at = march_spot(m, t);
     r.solid = false;
     r.layer = 0;
-    if ((uint32_t)r.cx < (uint32_t)w.W && (uint32_t)r.cy < (uint32_t)w.H) {
-        const uint32_t c = level0_node(w, r.cx, r.cy);
-        const uint32_t h0 = c & 0xFF, h1 = (c >> 8) & 0xFF, h2 = (c >> 16) & 0xFF;
-        const bool floor_ = z <= (float)h0;
-        const bool upper = h2 > h0 && z >= (float)h1 && z <= (float)h2;  // node-form cell
-        r.solid = floor_ || upper;
+    if ((uint32_t)r.at.cx < (uint32_t)w.W && (uint32_t)r.at.cy < (uint32_t)w.H) {
+        bool floor_;
+        r.solid = march_solid(level0_node(w, r.at.cx, r.at.cy), r.at.z, floor_);
         r.layer = floor_ ? 0 : 1;
     }
     return r;
-}
-
-// A pixel ray in float; sample i lies at t = i dt, i = 1 .. steps.
-struct MarchRay {
-    float ox, oy, oz, dx, dy, dz, dt;
-};
-
-__device__ __forceinline__ MarchPoint march_at(const WorldDev &w, const MarchRay &m, float t) {
-    return march_solid(w, __fadd_rn(m.ox, __fmul_rn(t, m.dx)), __fadd_rn(m.oy, __fmul_rn(t, m.dy)),
-                       __fadd_rn(m.oz, __fmul_rn(t, m.dz)));
 }
 
 // The first solid sample of each active lane's ray among i .. last, or 0.
@@ -99,9 +84,7 @@ __device__ __forceinline__ int32_t march_beams(const RenderParams &p, const Marc
     const int lane = threadIdx.x & 31;
     const BeamDir d = beam_dir(r.dx, r.dy, r.dz);
     BeamRay q = beam_ray(d, r);
-    // samples per column and per unit of height
-    const float per_u = __fdividef(65536.0f, (float)d.du * m.dt);
-    const float per_z = __fdividef(1.0f, fabsf(m.dz) * m.dt);
+    const MarchRate rate = march_rate(m, d);
     const float steps = (float)mp.steps;
     // every sample of a ray that is vertical or whose spacing is no ordinary number
     const bool plain = d.du == 0 || !(m.dt > 1e-9f && m.dt < 1e9f);
@@ -115,26 +98,18 @@ __device__ __forceinline__ int32_t march_beams(const RenderParams &p, const Marc
         bool alive = (todo >> lane & 1) && d.key == s.key;
         todo &= ~__ballot_sync(kFull, alive);
         beam_scan(s, p.world, lvt, p.world.L);
+        s.u = s.m.u0 - 1;  // (rounding may put samples there)
         beam_place(q, s.m);
         int32_t next = 1, b0, b1;
         uint32_t peak;
-        while (beam_next<false>(s, lvt, d, q, alive, b0, b1, &peak)) {
-            // the samples in these columns, at heights up to the highest top
-            // there: a little more either side than rounding can move them
-            float lo = ((float)(b0 - s.m.u0) - 0.02f - q.pu) * per_u;
-            float hi = ((float)(b1 - s.m.u0) + 0.02f - q.pu) * per_u;
-            if (lo * 0.999998f - 0.02f > steps) alive = false;  // past its last sample
-            const float rise = (float)peak + 0.02f - m.oz;
-            if (m.dz < 0.0f) lo = fmaxf(lo, -rise * per_z);
-            else hi = fminf(hi, rise * per_z);
-            lo = fminf(fmaxf(lo * (lo > 0.0f ? 0.999998f : 1.0f) - 0.02f, 0.0f), steps + 1.0f);
-            hi = fminf(fmaxf(hi * 1.000002f + 0.02f, 0.0f), steps);
-            const int32_t first = max(next, (int32_t)lo), last = (int32_t)hi;
-            found = max(found, march_samples(p.world, m, alive, first, last));
-            // samples that rounding may have moved into the columns beyond stay
-            // to be taken again with those, which may be higher
-            const float done = ((float)(b1 - s.m.u0) - 0.02f - q.pu) * per_u * 0.999998f - 0.02f;
-            next = max(next, (int32_t)fminf(fmaxf(done, 0.0f), steps + 1.0f));
+        while (beam_next<false, true>(s, lvt, d, q, alive, b0, b1, &peak)) {
+            const MarchRun run = march_run(m, rate, q.pu, (float)(b0 - s.m.u0),
+                                           (float)(b1 - s.m.u0), (float)peak, steps);
+            alive = alive && !run.past;
+            const int32_t i = march_samples(p.world, m, alive, max(next, run.first), run.last);
+            // one in the column beyond, which may be higher, is met again there
+            if (i && march_column(march_spot(m, rn_mul((float)i, m.dt)), s.key) < b1) found = i;
+            next = max(next, run.done);
             alive = alive && !found;
             if (!__any_sync(kFull, alive)) break;
         }
@@ -193,7 +168,7 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
             else ta = tm;
         }
         const MarchPoint hit = march_at(p.world, m, tb);
-        cell = (uint32_t)hit.cy * (uint32_t)p.world.W + (uint32_t)hit.cx;
+        cell = (uint32_t)hit.at.cy * (uint32_t)p.world.W + (uint32_t)hit.at.cx;
         layer = hit.layer;
         depth = __fmul_rn(tb, len);
     }
