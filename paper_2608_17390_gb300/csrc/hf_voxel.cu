@@ -245,8 +245,10 @@ __global__ void __launch_bounds__(kVoxTailThreads)
 // level (one step each level): the first one where the camera's voxel is empty,
 // else 0.  Lane k looks at level k.  A voxel's index on level k is the quotient's
 // floor there, provided that halving it gives the index of level k + 1 (rounding
-// may differ for an extent that is no power of two); a camera outside the grid
-// stays at the top.  Every lane of the warp calls.
+// may differ for an extent that is no power of two).  Rays start at o only if the
+// camera lies in the box of level 0: above it, it may still lie in the last
+// voxels of coarser levels, which reach past it, but its rays start where they
+// enter the box, and from the top.  Every lane of the warp calls.
 __device__ __forceinline__ int vox_start(const VoxelDev &v, const VoxLevel *lv, const float *o,
                                          const int32_t *vs, const int32_t *ve, int lane) {
     constexpr uint32_t full = 0xFFFFFFFFu;
@@ -263,6 +265,7 @@ __device__ __forceinline__ int vox_start(const VoxelDev &v, const VoxLevel *lv, 
     }
     const bool occ = good && vox_occupied(v, lv[k], (uint32_t)n[0], (uint32_t)n[1], (uint32_t)n[2]);
     const uint32_t goods = __ballot_sync(full, good), occs = __ballot_sync(full, occ);
+    if (!(goods & 1)) return top;
     // bit 31 is the top level: the run of occupied voxels from there on
     const int down = min(__clz(~(occs << (31 - top))), top);
     return goods >> (top - down) & 1 ? top - down : min(top - down + 1, top);
