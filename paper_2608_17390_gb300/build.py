@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhf.so")
-SOURCES = ["hf_api.cpp", "hf_trace.cu", "hf_pyramid.cu", "hf_march.cu", "hf_scatter.cu", "hf_voxel.cu",
+SOURCES = ["hf_api.cpp", "hf_trace.cu", "hf_single.cu", "hf_pyramid.cu", "hf_march.cu", "hf_scatter.cu", "hf_voxel.cu",
            "hf_serve.cpp", "hf_sun.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -41,7 +41,7 @@ def build(verbose=False, extra=()):
     os.makedirs(OUT, exist_ok=True)
     headers = [os.path.join(ROOT, "include", "hf.h"), os.path.join(CSRC, "hf_internal.h"),
                os.path.join(CSRC, "hf_cast.h"), os.path.join(CSRC, "hf_beam.h"),
-               os.path.join(CSRC, "hf_march.h")]
+               os.path.join(CSRC, "hf_march.h"), os.path.join(CSRC, "hf_trace.h")]
     jobs = []
     objs = []
     for src in SOURCES:

@@ -761,7 +761,7 @@ static int launch_graph(hf_ctx *c, Slot &s, const GraphKey &key, const hf::Rende
         cudaKernelNodeParams kp{};
         kp.func = const_cast<void *>(hf::trace_batched_fn(shadows, kind, c->pair));
         kp.gridDim = dim3((unsigned)(c->sm_count * c->occ[shadows][kind]));
-        kp.blockDim = dim3(hf::kThreads);
+        kp.blockDim = dim3((unsigned)hf::trace_threads(kind));
         kp.sharedMemBytes = 0;
         kp.kernelParams = args;
         if (cudaGraphAddKernelNode(&kern, graph, &copy, 1, &kp) != cudaSuccess ||
@@ -1185,7 +1185,7 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         if (hf_validate_camera(c->W, c->H, &cams[i]) != HF_OK) return HF_E_INVALID_ARG;
     if (!o.tile_w && !o.tile_h)
         default_tile(cams, n, kind == hf::kTraceBeams,
-                     (uint64_t)c->sm_count * c->occ[shadows][kind] * (hf::kThreads / 32), o.flags, tw,
+                     (uint64_t)c->sm_count * c->occ[shadows][kind] * (hf::trace_threads(kind) / 32), o.flags, tw,
                      th);
     const uint32_t *bounds = nullptr;
     if (shadows) {

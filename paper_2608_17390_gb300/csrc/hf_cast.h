@@ -2,22 +2,23 @@
 //
 // Two traversals give the same hit:
 //
-//   cast_general  one ray, hierarchical DDA, every decision on rationals
-//                 num/den with 64-bit products.  Counts fetches, obeys a step
-//                 limit of the caller's.
+//   cast_single   one ray, hierarchical DDA, every decision on rationals
+//                 num/den with 64-bit products (hf_single.cu).  Counts fetches,
+//                 obeys a step limit of the caller's.
 //   beam_*        the parts of a warp's traversal (hf_trace.cu): the rays of a
 //                 warp that go the same way are bounded by one beam, whose 32
 //                 next stretches are tested by the 32 lanes at once; rays are
 //                 walked, column by column in float with error bounds, only
 //                 through stretches that the beam does not prove empty.  What
 //                 the bounds leave open is decided exactly, on rationals, and
-//                 a ray through a cell corner is left to cast_general.
+//                 a ray through a cell corner is left to the other (cast_general).
 //
 // The functions are host code too, so that the two can be compared on a CPU.
 #pragma once
 
 #include <cmath>
 #include <cstdint>
+#include <cstdlib>
 #include <cstring>
 
 #include "hf_internal.h"
@@ -210,43 +211,49 @@ HF_HD void cast_cell(const Ray &r, int32_t &cx, int32_t &cy) {
     cy = (r.oy >> kShift) - (r.dy < 0 && (r.oy & 0xFFFF) == 0 ? 1 : 0);
 }
 
-template <bool PAIR>
-HF_HD void vertical_hit(const LevelDev *lvt, const Ray &r, int32_t cx, int32_t cy, Hit &h) {
-    const uint32_t word = cast_word<PAIR>(lvt[0], 0, cx, cy);
-    if (vertical_test(r, word, h)) {
-        h.cx = cx;
-        h.cy = cy;
-        h.word = word;
-    }
-}
-
-// Exact first hit of one ray.  h.face = kFaceMiss on a
-// miss, kFaceError when max_steps nodes did not finish the ray.
+// Exact first hit of one ray.  h.face = kFaceMiss on a miss, kFaceError when
+// max_steps iterations did not finish the ray.  lvt: the world's levels; W, H and
+// cells are those of level 0.
 //
+// State: the node (nx, ny) at `level` that holds the ray just after t_in.
 // Skipping an empty node changes only the node index on the exit axis; the
 // finer bits on the other axis are found when the traversal descends, by
 // asking whether the ray has crossed the child midline by t_in (exact
 // cross-multiplied time comparison).  Every interior cell boundary of a node
 // is the midline of exactly one sub-level, so a ray that enters a cell through
 // its Y side while also crossing an X cell boundary (a corner) is detected on
-// the way down and reported with the X face.
-template <bool STATS, bool PAIR>
-HF_HD void cast_general(const LevelDev *lvt, const Ray &r, int start_level, int mip_start,
-                        int max_steps, Hit &h, Counters &cnt) {
+// the way down and reported with the X face (X_TIME: and with the time as that
+// boundary's, over |dx|).
+// EMPTY_FIRST picks the order of the two outcomes of the node test in the
+// code (empty: advance; else descend or hit); which order runs faster depends
+// on the kernel (measured: empty first with shadow rays, the other without).
+template <bool STATS, bool PAIR, bool EMPTY_FIRST, bool X_TIME>
+HF_HD void cast_single(int32_t W, int32_t H, const uint32_t *cells, const LevelDev *lvt,
+                       const Ray &r, int start_level, int mip_start, int max_steps, Hit &h,
+                       Counters &cnt) {
     h.face = kFaceMiss;
     h.layer = 255;
+    // (abs, and not a choice of sign: the compiler then knows that both are
+    // positive; the products below cost 5 % of the kernel's time otherwise)
+    const int32_t adx = abs(r.dx), ady = abs(r.dy);
     int32_t cx, cy;
     cast_cell(r, cx, cy);
-    if ((uint32_t)cx >= lvt[0].stride || (uint32_t)cy >= lvt[0].rows) return;
-    if (r.dx == 0 && r.dy == 0) {
+    if ((uint32_t)cx >= (uint32_t)W || (uint32_t)cy >= (uint32_t)H) return;
+
+    if (adx == 0 && ady == 0) {
+        const uint32_t word = cast_word<PAIR>(LevelDev{cells, (uint32_t)W, (uint32_t)H}, 0, cx, cy);
         if (STATS) cnt.cells++;
-        vertical_hit<PAIR>(lvt, r, cx, cy, h);
+        if (vertical_test(r, word, h)) {
+            h.cx = cx;
+            h.cy = cy;
+            h.word = word;
+        }
         return;
     }
+
     // Per-ray sign constants.  A zero direction component counts as positive:
     // its exit distance is then positive and never the smaller one, so the
     // ray never leaves through that axis.
-    const int32_t adx = r.dx < 0 ? -r.dx : r.dx, ady = r.dy < 0 ? -r.dy : r.dy;
     const int32_t gx = r.dx < 0 ? -1 : 1, gy = r.dy < 0 ? -1 : 1;  // step per exit
     const int32_t px = r.dx < 0 ? 0 : 1, py = r.dy < 0 ? 0 : 1;    // exit side offset
     const int32_t qx = px ^ 1, qy = py ^ 1;
@@ -257,6 +264,7 @@ HF_HD void cast_general(const LevelDev *lvt, const Ray &r, int start_level, int 
     int32_t nx = cx >> level, ny = cy >> level;
     int32_t tin_num = 0, tin_den = 1;
     uint8_t entry = kFaceInside;
+
     for (int it = 0;; ++it) {
         // one bounds check per iteration, after every advance, ascent or
         // descent: an index past the level's end, or below 0, means the ray
@@ -296,9 +304,9 @@ HF_HD void cast_general(const LevelDev *lvt, const Ray &r, int start_level, int 
         const bool empty = zd(r.oz - (maxtop << kShift), r.dz, lo_num, lo_den) > 0 ||
                            (zd(r.oz - (maxh0 << kShift), r.dz, lo_num, lo_den) > 0 &&
                             zd(r.oz - (minh1 << kShift), r.dz, hi_num, hi_den) < 0);
-        if (empty) {
-            // advance past the node (or cell) through its exit side; at an
-            // exact corner both indices change and the X face is reported
+        // advance past the node (or cell) through its exit side; at an exact
+        // corner both indices change and the X face is reported
+        auto advance = [&]() {
             if (cmp <= 0) nx += gx;
             if (cmp >= 0) ny += gy;
             entry = cmp <= 0 ? face_x : face_y;
@@ -312,46 +320,62 @@ HF_HD void cast_general(const LevelDev *lvt, const Ray &r, int start_level, int 
             level += up;
             nx >>= up;
             ny >>= up;
+        };
+        if (EMPTY_FIRST && empty) {
+            advance();
             continue;
         }
-        if (level > 0) {
-            // descend into the child that holds the ray just after t_in:
-            // the upper child on an axis when the ray has passed that
-            // axis' midline by t_in (for a negative direction, when not)
-            --level;
-            const int32_t xm = (2 * nx + 1) * (1 << level), ym = (2 * ny + 1) * (1 << level);
-            const int32_t midx = gx * (xm * (1 << kShift)) + kx;
-            const int64_t lx = (int64_t)midx * tin_den;
-            const int64_t rx = (int64_t)tin_num * adx;
-            const int64_t ly = (int64_t)(gy * (ym * (1 << kShift)) + ky) * tin_den;
-            const int64_t ry = (int64_t)tin_num * ady;
-            nx = 2 * nx + ((lx <= rx) != (gx < 0) ? 1 : 0);
-            ny = 2 * ny + ((ly <= ry) != (gy < 0) ? 1 : 0);
-            // a corner: the ray enters the cell through its Y side and an
-            // X cell boundary at the same instant; report the X face, and the
-            // time as that boundary's
-            if (lx == rx && adx != 0 && entry == face_y) {
-                entry = face_x;
-                tin_num = midx;
-                tin_den = adx;
+        if (EMPTY_FIRST || !empty) {
+            if (level > 0) {
+                // descend into the child that holds the ray just after t_in:
+                // the upper child on an axis when the ray has passed that
+                // axis' midline by t_in (for a negative direction, when not)
+                --level;
+                const int32_t xm = (2 * nx + 1) * (1 << level), ym = (2 * ny + 1) * (1 << level);
+                const int32_t midx = gx * (xm * (1 << kShift)) + kx;
+                const int64_t lx = (int64_t)midx * tin_den;
+                const int64_t rx = (int64_t)tin_num * adx;
+                const int64_t ly = (int64_t)(gy * (ym * (1 << kShift)) + ky) * tin_den;
+                const int64_t ry = (int64_t)tin_num * ady;
+                nx = 2 * nx + ((lx <= rx) != (gx < 0) ? 1 : 0);
+                ny = 2 * ny + ((ly <= ry) != (gy < 0) ? 1 : 0);
+                // a corner: the ray enters the cell through its Y side and an
+                // X cell boundary at the same instant; report the X face
+                if (lx == rx && adx != 0 && entry == face_y) {
+                    entry = face_x;
+                    if (X_TIME) {
+                        tin_num = midx;
+                        tin_den = adx;
+                    }
+                }
+                continue;
             }
-            continue;
-        }
-        // a non-empty cell holds the hit (the cell test is exact: the
-        // segment's z range meets (-inf, h0] or [h1, h2], and z is
-        // continuous along it): find its layer, face and time.
-        if (!leaf_test(r.oz, r.dz, word, tin_num, tin_den, tout_num, tout_den, entry, h)) {
-            h.face = kFaceError;  // unreachable: reported, never silent
-            h.layer = 255;
+            // a non-empty cell holds the hit (the cell test is exact: the
+            // segment's z range meets (-inf, h0] or [h1, h2], and z is
+            // continuous along it): find its layer, face and time.  The
+            // advance is reached from empty nodes and cells only.
+            if (!leaf_test(r.oz, r.dz, word, tin_num, tin_den, tout_num, tout_den, entry, h)) {
+                h.face = kFaceError;  // unreachable: reported, never silent
+                h.layer = 255;
+                return;
+            }
+            h.cx = nx;
+            h.cy = ny;
+            h.word = word;
             return;
         }
-        h.cx = nx;
-        h.cy = ny;
-        h.word = word;
-        return;
+        advance();
     }
     h.face = kFaceError;
     h.layer = 255;
+}
+
+// The same as the warps of beams have it for a ray that no beam takes.
+template <bool STATS, bool PAIR>
+HF_HD void cast_general(const LevelDev *lvt, const Ray &r, int start_level, int mip_start,
+                        int max_steps, Hit &h, Counters &cnt) {
+    cast_single<STATS, PAIR, true, true>((int32_t)lvt[0].stride, (int32_t)lvt[0].rows, lvt[0].base,
+                                         lvt, r, start_level, mip_start, max_steps, h, cnt);
 }
 
 // One ray of a beam: a ray with a horizontal component, whose axis of the

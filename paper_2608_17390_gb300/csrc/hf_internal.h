@@ -62,10 +62,6 @@ constexpr uint32_t kSkyColour = 0xFFEBB487u;  // r 135, g 180, b 235, a 255
 
 constexpr int kMaxLevels = 14;  // 2^14 = 16384 = largest grid side
 constexpr int kShift = 16;      // 2^16 fixed-point units per world unit
-#ifndef HF_TRACE_THREADS
-#define HF_TRACE_THREADS 128  // finer steps of registers per thread than 256 (see hf_trace.cu)
-#endif
-constexpr int kThreads = HF_TRACE_THREADS;  // threads per trace block
 constexpr uint32_t kMaxCams = 4096;
 constexpr uint32_t kDefaultMipStart = 6;  // coarsest level used when the caller asks for the default
 #ifndef HF_SHADOW_MIP_EXTRA
@@ -187,18 +183,25 @@ int voxel_repair(const WorldDev &w, const VoxelDev &v, int32_t x0, int32_t y0, i
 int launch_voxel_trace(const RenderParams &p, const VoxelDev &v, const VoxelParams &q,
                        uint32_t n_cams, uint32_t max_tiles, void *stream);  // tiles of 8 x 4 pixels
 
-// Launch wrappers (hf_trace.cu)
-// How the trace kernels follow rays: warps of rays in beams; one ray at a time
-// (a step limit set by the caller: p.max_steps); the same with fetch counters.
 // Whether the rays of a warp's 32 pixels stay close enough for beams (hf_api.cpp).
 bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw);
+// How the trace kernels follow rays: warps of rays in beams; one ray at a time
+// (a step limit set by the caller: p.max_steps); the same with fetch counters.
 enum TraceKind { kTraceBeams = 0, kTraceGeneral = 1, kTraceStats = 2, kTraceKinds = 3 };
+// Threads of a trace block (hf_trace.cu and hf_single.cu say why).
+constexpr int trace_threads(int kind) { return kind == kTraceBeams ? 128 : 256; }
+
+// Launch wrappers (hf_trace.cu)
 // The trace kernels are instantiated per level-0 storage; p.world.pair picks one.
 int launch_trace_batched(const RenderParams &p, bool shadows, int kind, int blocks, void *stream);
 // (the plain kernel takes its camera record as a launch parameter)
 int launch_trace_plain(const RenderParams &p, bool shadows, int kind, const CamDev &cam,
                        uint32_t n_tiles, void *stream);
 const void *trace_batched_fn(bool shadows, int kind, bool pair);
+// The kernels of the other two kinds (hf_single.cu).
+const void *single_batched_fn(bool shadows, bool stats, bool pair);
+int launch_single_plain(const RenderParams &p, bool shadows, bool stats, const CamDev &cam,
+                        uint32_t n_tiles, void *stream);
 int trace_batched_occupancy(bool shadows, int kind, bool pair, int *blocks_per_sm);
 
 // What the allocation-free render needs to know about a context (hf_api.cpp).

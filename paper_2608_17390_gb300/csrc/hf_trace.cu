@@ -1,4 +1,5 @@
-// hf_trace.cu -- per-pixel exact ray casting through a two-interval height field.
+// hf_trace.cu -- per-pixel exact ray casting through a two-interval height field, a
+// warp's rays together; the allocation-free render.
 //
 // One warp owns one tile of tile_w x tile_h pixels; lane l takes the tile's
 // pixels l, l + 32, ...  The hit cell, layer and face of every ray equal the
@@ -10,8 +11,8 @@
 //     known-empty space, Section 3.2 of the paper), and what they leave open is
 //     decided in exact integer arithmetic (hf_cast.h): the SOLID predicate of
 //     Section 3.1, closed ends, floor unbounded below;
-//   * renders with a step limit of the caller's, or with fetch counters, follow
-//     each ray by itself (cast_general);
+//   * renders with a step limit of the caller's, or with fetch counters, or whose
+//     rays lie far apart, follow each ray by itself (hf_single.cu);
 //   * a shadow ray starts at the floor of the hit point (an exact floor
 //     division: a float estimate and one integer correction), one fixed-point
 //     unit outward along the face normal.
@@ -24,6 +25,7 @@
 #include "hf.h"
 #include "hf_beam.h"
 #include "hf_internal.h"
+#include "hf_trace.h"
 
 namespace hf {
 namespace {
@@ -34,57 +36,7 @@ namespace {
 // without: four blocks 10.62 ms / -, five 9.66 / -, six 9.39 / 8.15, seven (up to
 // 4 % more instructions) 9.43 / 8.57.
 constexpr int kTraceMinBlocks = 6;
-
-__constant__ float c_albedo[8][3] = HF_ALBEDO_TABLE;
-constexpr float kKa = kAmbient, kKd = kDiffuse;
-constexpr uint32_t kSky = kSkyColour;
-
-// int64 -> float through two 32-bit conversions (64-bit integer conversions
-// run on the FP64 pipe, which is narrow on this GPU).  |v| < 2^52.
-__device__ __forceinline__ float i64_to_f32(int64_t v) {
-    return fmaf((float)(int32_t)(v >> 32), 4294967296.0f, (float)(uint32_t)v);
-}
-
-// floor(a / b) for |a| < 2^52, 0 < b < 2^21 and |a / b| < 2^30: a float
-// estimate, a second estimate from the remainder, then one exact correction.
-__device__ __forceinline__ int32_t floor_div_small(int64_t a, int32_t b, float rcp_b) {
-    int32_t q = (int32_t)floorf(i64_to_f32(a) * rcp_b);        // within ~2^9 of the quotient
-    const int32_t r1 = (int32_t)(a - (int64_t)q * b);          // |r1| < 2^31
-    q += (int32_t)floorf((float)r1 * rcp_b);                   // within 1
-    const int64_t r = a - (int64_t)q * b;
-    if (r < 0) q -= 1;
-    else if (r >= b) q += 1;
-    return q;
-}
-
-__device__ __forceinline__ uint32_t load_word(const WorldDev &w, int level, int32_t x, int32_t y) {
-    return __ldg(w.base + w.off[level] + (uint32_t)y * w.stride[level] + (uint32_t)x);
-}
-
-// Node-form word of level-0 cell (x, y) for the storage the kernel was
-// instantiated for (the choice is made at compile time).
-template <bool PAIR>
-__device__ __forceinline__ uint32_t level0_word(const WorldDev &w, int32_t x, int32_t y) {
-    if (PAIR)
-        return pair_node(__ldg(w.base + (uint32_t)y * ((uint32_t)w.W >> 1) + ((uint32_t)x >> 1)),
-                         (uint32_t)x & 1);
-    return load_word(w, 0, x, y);
-}
-
-__device__ __forceinline__ uint32_t shade(uint32_t m, uint8_t face, bool visible,
-                                          const float *ln) {
-    // the normal's axis is face / 2, its sign face's lowest bit
-    const float n = face < kFaceNY ? ln[0] : face < kFaceNZ ? ln[1] : ln[2];
-    const float ndl = face == kFaceInside ? 0.0f : face & 1 ? n : -n;
-    const float k = kKa + kKd * fmaxf(ndl, 0.0f) * (visible ? 1.0f : 0.0f);
-    uint32_t out = 0xFF000000u;
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-        const float v = fminf(fmaxf(c_albedo[m][ch] * k, 0.0f), 1.0f);
-        out |= ((uint32_t)(255.0f * v + 0.5f)) << (8 * ch);
-    }
-    return out;
-}
+constexpr int kThreads = trace_threads(kTraceBeams);
 
 // Casts one ray per active lane; every lane of the warp calls.  only: of a hit
 // nothing matters but that there is one.
@@ -183,27 +135,16 @@ __device__ __forceinline__ void tile_pixel(const RenderParams &p, const TileDev 
     py = t.y0 + (i >> p.tile_w_log2);
 }
 
-// The ray of a camera's pixel.
-__device__ __forceinline__ Ray primary_ray(const CamDev &c, int32_t px, int32_t py) {
-    const int32_t a = 2 * px + 1 - (int32_t)c.w;
-    const int32_t b = (int32_t)c.h - 1 - 2 * py;
-    return Ray{c.o[0], c.o[1], c.o[2], c.F[0] + a * c.R[0] + b * c.U[0],
-               c.F[1] + a * c.R[1] + b * c.U[1], c.F[2] + a * c.R[2] + b * c.U[2]};
-}
-
 // One pixel per lane: its primary ray, then (with shadows) the shadow ray, in
 // a second pass of the same traversal code.  Every lane of the warp calls;
-// `inside` says whether the lane has a pixel.
-template <bool SHADOWS, int KIND, bool PAIR>
+// 
+template <bool SHADOWS, bool PAIR>
 __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelDev *lvt,
-                                             const TileDev &t, int start, int i, bool &inside,
-                                             const BeamDir &sun, Counters &cnt, Counters &scnt,
-                                             uint32_t &nshadow, bool &err) {
-    constexpr bool STATS = KIND == kTraceStats;
+                                             const TileDev &t, int i, const BeamDir &sun) {
     const CamDev &c = t.cam;
     int32_t px, py;
     tile_pixel(p, t, i, px, py);
-    inside = px < (int32_t)c.w && py < (int32_t)c.h;
+    bool inside = px < (int32_t)c.w && py < (int32_t)c.h;
     Ray r = primary_ray(c, px, py);
     uint32_t tag = kFaceMiss;  // of the primary hit: face and material (bits 8..10)
     bool visible = true;
@@ -212,24 +153,9 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
     for (int pass = 0;; ++pass) {
         const bool sp = SHADOWS && pass;
         Hit h;
-        Counters pc{0, 0};
-        if (KIND == kTraceBeams) {
-            const BeamDir d = sp ? sun : beam_dir(r.dx, r.dy, r.dz);
-            cast_beams<PAIR>(p, lvt, d, beam_ray(d, r), r.oz, r.dz, cast,
-                             sp ? p.shadow_mip : p.mip_start, sp, h);
-        } else {
-            h.face = kFaceMiss;
-            h.layer = 255;
-            if (cast)
-                cast_general<STATS, PAIR>(lvt, r, sp ? min(kShadowStart, p.shadow_mip) : start,
-                                          sp ? p.shadow_mip : p.mip_start, p.max_steps, h, pc);
-        }
-        if (STATS) {
-            Counters &dst = sp ? scnt : cnt;
-            dst.nodes += pc.nodes;
-            dst.cells += pc.cells;
-        }
-        if (KIND != kTraceBeams && cast && h.face == kFaceError) err = true;
+        const BeamDir d = sp ? sun : beam_dir(r.dx, r.dy, r.dz);
+        cast_beams<PAIR>(p, lvt, d, beam_ray(d, r), r.oz, r.dz, cast,
+                         sp ? p.shadow_mip : p.mip_start, sp, h);
         if (sp) {
             if (cast) visible = h.face == kFaceMiss;
             break;
@@ -280,7 +206,6 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
             const int32_t sxp = r.ox + (on_x ? qn : qa);
             const int32_t syp = r.oy + (on_x ? qa : on_z ? qb : qn);
             const int32_t szp = r.oz + (on_z ? qn : qb);
-            if (STATS) nshadow++;
             cast = true;
             if (p.sun_bounds) {
                 // the start cell's proven bounds decide most shadow rays at once:
@@ -291,7 +216,6 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
                 if ((uint32_t)bx < (uint32_t)p.world.W && (uint32_t)by < (uint32_t)p.world.H) {
                     const uint32_t fg =
                         __ldg(p.sun_bounds + (uint32_t)by * (uint32_t)p.world.W + (uint32_t)bx);
-                    if (STATS) scnt.cells++;
                     if (szp <= (int32_t)((fg & 0xFFFFu) << 8)) {
                         visible = false;
                         cast = false;
@@ -316,84 +240,18 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
     if (c.rgba) __stcs(c.rgba + pix, face < kFaceError ? shade(tag >> 8, face, visible, p.sun_n) : kSky);
 }
 
-// Start level of a camera's primary rays: the largest level l <= mip_start
-// whose node around the camera cell has every top below the camera, but not
-// below level min(2, mip_start) (a measured floor: climbing out of levels 0
-// and 1 costs more steps than the two descents it saves).  Node tops only
-// grow with the level, so the levels under the camera are 0..l; lane k tests
-// level k.  A camera outside the grid starts at mip_start.  The traversal is
-// exact from any start level (a ray climbs as it crosses parent boundaries);
-// the rule only saves descents through nodes around the camera that cannot
-// be empty.
-template <bool PAIR>
-__device__ __forceinline__ int primary_start(const RenderParams &p, const CamDev &c, int lane) {
-    const WorldDev &w = p.world;
-    const int32_t cx = c.o[0] >> kShift, cy = c.o[1] >> kShift;
-    if ((uint32_t)cx >= (uint32_t)w.W || (uint32_t)cy >= (uint32_t)w.H) return p.mip_start;
-    bool above = false;
-    if (lane <= p.mip_start) {
-        const uint32_t word =
-            lane ? load_word(w, lane, cx >> lane, cy >> lane) : level0_word<PAIR>(w, cx, cy);
-        const int32_t top = (word >> 16) & 0xFF;  // every level in node form
-        above = c.o[2] > (top << kShift);
-    }
-    const uint32_t mask = __ballot_sync(kFull, above);
-    return max(min(2, p.mip_start), __ffs(~mask) - 2);
-}
-
 // One warp renders one tile: lane l traces the tile's pixels l, l+32, ...
-template <bool SHADOWS, int KIND, bool PAIR>
+template <bool SHADOWS, bool PAIR>
 __device__ __forceinline__ void trace_tile(const RenderParams &p, const LevelDev *lvt,
                                            const BeamDir &sun, TileDev &t, uint32_t local_tile,
                                            int lane) {
-    const CamDev &c = t.cam;
     if (lane == 0) {
-        t.x0 = (int32_t)(local_tile % c.tiles_x) << p.tile_w_log2;
-        t.y0 = (int32_t)(local_tile / c.tiles_x) << p.tile_h_log2;
+        t.x0 = (int32_t)(local_tile % t.cam.tiles_x) << p.tile_w_log2;
+        t.y0 = (int32_t)(local_tile / t.cam.tiles_x) << p.tile_h_log2;
     }
     __syncwarp();
-    Counters cnt{0, 0}, scnt{0, 0};
-    uint32_t nshadow = 0, nrays = 0;
-    bool err = false;
-    constexpr bool STATS = KIND == kTraceStats;
-    const int start = KIND == kTraceBeams ? 0 : primary_start<PAIR>(p, c, lane);
-    for (int i = lane; i < 1 << (p.tile_w_log2 + p.tile_h_log2); i += 32) {
-        bool inside;
-        trace_pixels<SHADOWS, KIND, PAIR>(p, lvt, t, start, i, inside, sun, cnt, scnt, nshadow, err);
-        if (STATS && inside) nrays++;
-    }
-    if (KIND != kTraceBeams && __any_sync(kFull, err) && lane == 0) atomicOr(p.status, 1u);
-    if (STATS) {
-        const uint32_t vn = __reduce_add_sync(kFull, cnt.nodes);
-        const uint32_t vc = __reduce_add_sync(kFull, cnt.cells);
-        const uint32_t vr = __reduce_add_sync(kFull, nrays);
-        const uint32_t vs = __reduce_add_sync(kFull, nshadow);
-        const uint32_t vf = __reduce_add_sync(kFull, scnt.nodes + scnt.cells);
-        if (lane == 0) {
-            atomicAdd(p.stats + 0, (unsigned long long)vn);
-            atomicAdd(p.stats + 1, (unsigned long long)vc);
-            atomicAdd(p.stats + 2, (unsigned long long)vr);
-            atomicAdd(p.stats + 3, (unsigned long long)vs);
-            atomicAdd(p.stats + 4, (unsigned long long)vf);
-        }
-    }
-}
-
-// Asks L2 for the world's coarse levels (all of a small world) as a launch
-// starts, spread over all its threads.  A ray's fetches form one dependent
-// chain, so a short render of a world that is not in L2 would otherwise wait
-// on DRAM at every step of every ray.
-__device__ __forceinline__ void prefetch_world(const RenderParams &p) {
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < p.prefetch_lines; i += stride)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p.prefetch + (size_t)i * 32));
-}
-
-// stride of level 0 is its width in cells also for paired texels (whose rows
-// then hold stride / 2 words)
-__device__ __forceinline__ void fill_levels(LevelDev *s_lv, const WorldDev &w) {
-    const int k = threadIdx.x;
-    if (k <= w.L) s_lv[k] = LevelDev{w.base + w.off[k], (uint32_t)w.stride[k], (uint32_t)w.rows[k]};
+    for (int i = lane; i < 1 << (p.tile_w_log2 + p.tile_h_log2); i += 32)
+        trace_pixels<SHADOWS, PAIR>(p, lvt, t, i, sun);
 }
 
 // Copy camera i into this warp's shared slot.
@@ -410,7 +268,7 @@ __device__ __forceinline__ TileDev &stage_cam(TileDev *slot, const CamDev *cams,
 
 // Persistent batched kernel: warps pop (camera, tile) items from one atomic
 // counter until the batch is drained.  One launch renders every camera.
-template <bool SHADOWS, int KIND, bool PAIR>
+template <bool SHADOWS, bool PAIR>
 __global__ void __launch_bounds__(kThreads, kTraceMinBlocks) k_trace_batched(const RenderParams p) {
     __shared__ uint32_t s_base[kMaxCams + 1];
     __shared__ TileDev s_tile[kThreads / 32];
@@ -437,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks) k_trace_batched(con
             else hi = mid;
         }
         TileDev &tile = stage_cam(&s_tile[threadIdx.x >> 5], p.cams, lo, lane);
-        trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, tile, t - s_base[lo], lane);
+        trace_tile<SHADOWS, PAIR>(p, s_lv, s_sun, tile, t - s_base[lo], lane);
     }
 }
 
@@ -446,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks) k_trace_batched(con
 // it to the device; each warp stages it in shared memory like the batched
 // kernel (reading the fields from parameter space instead changes the
 // traversal's register allocation, measured 3-8 % slower on large images).
-template <bool SHADOWS, int KIND, bool PAIR>
+template <bool SHADOWS, bool PAIR>
 __global__ void __launch_bounds__(kThreads, kTraceMinBlocks)
     k_trace_plain(const __grid_constant__ RenderParams p, const __grid_constant__ CamDev cam,
                   uint32_t n_tiles) {
@@ -461,37 +319,25 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks)
     if (t >= n_tiles) return;
     const int lane = threadIdx.x & 31;
     TileDev &tile = stage_cam(&s_tile[threadIdx.x >> 5], &cam, 0, lane);
-    trace_tile<SHADOWS, KIND, PAIR>(p, s_lv, s_sun, tile, t, lane);
-}
-
-template <bool SH, int KIND, bool PA>
-const void *batched_ptr() {
-    return reinterpret_cast<const void *>(&k_trace_batched<SH, KIND, PA>);
+    trace_tile<SHADOWS, PAIR>(p, s_lv, s_sun, tile, t, lane);
 }
 
 template <bool SH, bool PA>
-const void *batched_fn(int kind) {
-    return kind == kTraceBeams     ? batched_ptr<SH, kTraceBeams, PA>()
-           : kind == kTraceGeneral ? batched_ptr<SH, kTraceGeneral, PA>()
-                                   : batched_ptr<SH, kTraceStats, PA>();
-}
-
-template <bool SH, int KIND, bool PA>
-void plain_launch(const RenderParams &p, uint32_t blocks, cudaStream_t s, const CamDev &cam,
-                  uint32_t n_tiles) {
-    k_trace_plain<SH, KIND, PA><<<blocks, kThreads, 0, s>>>(p, cam, n_tiles);
+const void *batched_ptr() {
+    return reinterpret_cast<const void *>(&k_trace_batched<SH, PA>);
 }
 
 }  // namespace
 
 const void *trace_batched_fn(bool shadows, int kind, bool pair) {
-    if (shadows) return pair ? batched_fn<true, true>(kind) : batched_fn<true, false>(kind);
-    return pair ? batched_fn<false, true>(kind) : batched_fn<false, false>(kind);
+    if (kind != kTraceBeams) return single_batched_fn(shadows, kind == kTraceStats, pair);
+    if (shadows) return pair ? batched_ptr<true, true>() : batched_ptr<true, false>();
+    return pair ? batched_ptr<false, true>() : batched_ptr<false, false>();
 }
 
 int trace_batched_occupancy(bool shadows, int kind, bool pair, int *blocks_per_sm) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        blocks_per_sm, trace_batched_fn(shadows, kind, pair), kThreads, 0);
+        blocks_per_sm, trace_batched_fn(shadows, kind, pair), trace_threads(kind), 0);
     return e == cudaSuccess ? 0 : -1;
 }
 
@@ -499,25 +345,21 @@ int launch_trace_batched(const RenderParams &p, bool shadows, int kind, int bloc
     void *args[] = {const_cast<RenderParams *>(&p)};
     const cudaError_t e =
         cudaLaunchKernel(trace_batched_fn(shadows, kind, p.world.pair != 0), dim3(blocks),
-                         dim3(kThreads), args, 0, (cudaStream_t)stream);
+                         dim3(trace_threads(kind)), args, 0, (cudaStream_t)stream);
     return e == cudaSuccess ? 0 : -1;
 }
 
 int launch_trace_plain(const RenderParams &p, bool shadows, int kind, const CamDev &cam,
                        uint32_t n_tiles, void *stream) {
     if (n_tiles == 0) return 0;
+    if (kind != kTraceBeams)
+        return launch_single_plain(p, shadows, kind == kTraceStats, cam, n_tiles, stream);
     cudaStream_t s = (cudaStream_t)stream;
-    const uint32_t warps = kThreads / 32;
-    const uint32_t blocks = (n_tiles + warps - 1) / warps;
-    using Fn = void (*)(const RenderParams &, uint32_t, cudaStream_t, const CamDev &, uint32_t);
-    static const Fn table[12] = {
-        plain_launch<false, kTraceBeams, false>,   plain_launch<false, kTraceBeams, true>,
-        plain_launch<false, kTraceGeneral, false>, plain_launch<false, kTraceGeneral, true>,
-        plain_launch<false, kTraceStats, false>,   plain_launch<false, kTraceStats, true>,
-        plain_launch<true, kTraceBeams, false>,    plain_launch<true, kTraceBeams, true>,
-        plain_launch<true, kTraceGeneral, false>,  plain_launch<true, kTraceGeneral, true>,
-        plain_launch<true, kTraceStats, false>,    plain_launch<true, kTraceStats, true>};
-    table[(shadows ? 6 : 0) + 2 * kind + (p.world.pair ? 1 : 0)](p, blocks, s, cam, n_tiles);
+    const uint32_t warps = kThreads / 32, blocks = (n_tiles + warps - 1) / warps;
+    if (shadows && p.world.pair) k_trace_plain<true, true><<<blocks, kThreads, 0, s>>>(p, cam, n_tiles);
+    else if (shadows) k_trace_plain<true, false><<<blocks, kThreads, 0, s>>>(p, cam, n_tiles);
+    else if (p.world.pair) k_trace_plain<false, true><<<blocks, kThreads, 0, s>>>(p, cam, n_tiles);
+    else k_trace_plain<false, false><<<blocks, kThreads, 0, s>>>(p, cam, n_tiles);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
