@@ -35,6 +35,14 @@ struct Ray {
     int32_t ox, oy, oz, dx, dy, dz;
 };
 
+// The ray of a camera's pixel.
+HF_HD Ray primary_ray(const CamDev &c, int32_t px, int32_t py) {
+    const int32_t a = 2 * px + 1 - (int32_t)c.w;
+    const int32_t b = (int32_t)c.h - 1 - 2 * py;
+    return Ray{c.o[0], c.o[1], c.o[2], c.F[0] + a * c.R[0] + b * c.U[0],
+               c.F[1] + a * c.R[1] + b * c.U[1], c.F[2] + a * c.R[2] + b * c.U[2]};
+}
+
 // One pyramid level as the traversal reads it (a per-block shared table, so
 // lanes at different levels read it in one shared-memory access).
 struct LevelDev {

@@ -17,7 +17,7 @@
 // in a stretch that the beam does not prove empty, at a height that its cells
 // reach, are looked up (hf_march.h: the bounds of their rounding).
 // Bound by instruction issue: 12 views of 1280 x 800 over 2048 x 16384 cells, 128
-// samples a ray, 1.229 -> 0.627 ms.
+// samples a ray, 1.229 -> 0.617 ms.
 #include <cuda_runtime.h>
 
 #include "hf_beam.h"
@@ -36,10 +36,10 @@ constexpr int kMarchMinBlocks = 9;
 // / beams: 12 views of 1280 x 800 over 2048 x 16384 cells, 32 samples 630 / 609
 // us, 128 1517 / 596; but 16 views of 640 x 360 near the ground of a 2048 x 2048
 // world, 48 samples 0.70, 96 1.03, 128 1.26 times as fast with beams.  The kernel
-// without beams needs 40 registers, so that 48 warps fit an SM; in blocks of 128
-// threads it is 3 % slower.
+// without beams needs 40 registers, so that six blocks fit an SM (asked for, they
+// cost it 0.6 %); in blocks of 128 threads it is 3 % slower.
 constexpr int kMarchBeamSteps = 96;
-constexpr int kMarchAllMinBlocks = 6, kMarchAllThreads = 256;
+constexpr int kMarchAllBlocks = 6, kMarchAllThreads = 256;
 
 struct MarchPoint {
     bool solid;
@@ -119,16 +119,9 @@ __device__ __forceinline__ int32_t march_beams(const RenderParams &p, const Marc
     return found;
 }
 
-// One pixel per lane; every lane of the warp calls.
-template <bool BEAMS>
-__device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchParams &mp,
-                                             const LevelDev *lvt, const CamDev &c, int32_t px,
-                                             int32_t py, bool inside) {
-    const int32_t a = 2 * px + 1 - (int32_t)c.w;
-    const int32_t b = (int32_t)c.h - 1 - 2 * py;
+// The ray of a pixel, its samples and its length.
+__device__ __forceinline__ MarchRay march_ray(const MarchParams &mp, const Ray &r, float &len) {
     const float inv_s = 1.0f / 65536.0f;
-    const Ray r{c.o[0], c.o[1], c.o[2], c.F[0] + a * c.R[0] + b * c.U[0],
-                c.F[1] + a * c.R[1] + b * c.U[1], c.F[2] + a * c.R[2] + b * c.U[2]};
     MarchRay m;
     m.ox = __fmul_rn(__int2float_rn(r.ox), inv_s);
     m.oy = __fmul_rn(__int2float_rn(r.oy), inv_s);
@@ -139,29 +132,26 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
     float sq = __fmul_rn(m.dx, m.dx);
     sq = __fadd_rn(sq, __fmul_rn(m.dy, m.dy));
     sq = __fadd_rn(sq, __fmul_rn(m.dz, m.dz));
-    const float len = __fsqrt_rn(sq);
+    len = __fsqrt_rn(sq);
     float t_end = __fdiv_rn(mp.far_dist, len);
     if (m.dz < 0.0f) {
         const float tz = __fdiv_rn(-m.oz, m.dz);
         if (tz < t_end) t_end = tz;
     }
     m.dt = __fdiv_rn(t_end, (float)(mp.steps + 1));
+    return m;
+}
 
-    int32_t found = 0;
-    if (!BEAMS && inside)
-        for (int32_t i = 1; i <= mp.steps; ++i)
-            if (march_at(p.world, m, __fmul_rn((float)i, m.dt)).solid) {
-                found = i;
-                break;
-            }
-    if (BEAMS) found = march_beams(p, mp, lvt, r, m, inside);
-
-    if (!inside) return;
+// A pixel's outputs: found says whether the sample at tb is its first solid one;
+// ta: the sample before.
+__device__ __forceinline__ void march_store(const RenderParams &p, const MarchParams &mp,
+                                            const CamDev &c, int32_t px, int32_t py,
+                                            const MarchRay &m, float len, bool found, float ta,
+                                            float tb) {
     uint32_t cell = 0xFFFFFFFFu;
     uint8_t layer = 255;
     float depth = __int_as_float(0x7f800000);
     if (found) {
-        float ta = __fmul_rn((float)(found - 1), m.dt), tb = __fmul_rn((float)found, m.dt);
         for (int k = 0; k < mp.bisections; ++k) {
             const float tm = __fmul_rn(__fadd_rn(ta, tb), 0.5f);
             if (march_at(p.world, m, tm).solid) tb = tm;
@@ -178,6 +168,40 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
     if (c.depth) __stcs(c.depth + pix, depth);
 }
 
+// One pixel per lane; every lane of the warp calls.
+__device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchParams &mp,
+                                             const LevelDev *lvt, const CamDev &c, int32_t px,
+                                             int32_t py) {
+    const bool inside = px < (int32_t)c.w && py < (int32_t)c.h;
+    const Ray r = primary_ray(c, px, py);
+    float len;
+    const MarchRay m = march_ray(mp, r, len);
+    const int32_t i = march_beams(p, mp, lvt, r, m, inside);
+    if (inside)
+        march_store(p, mp, c, px, py, m, len, i != 0, __fmul_rn((float)(i - 1), m.dt),
+                    __fmul_rn((float)i, m.dt));
+}
+
+// One pixel of a lane that takes every sample.
+__device__ __forceinline__ void march_pixel(const RenderParams &p, const MarchParams &mp,
+                                            const CamDev &c, int32_t px, int32_t py) {
+    if (px >= (int32_t)c.w || py >= (int32_t)c.h) return;
+    float len;
+    const MarchRay m = march_ray(mp, primary_ray(c, px, py), len);
+    bool found = false;
+    float ta = 0.0f, tb = 0.0f;
+    for (int i = 1; i <= mp.steps; ++i) {
+        const float t = __fmul_rn((float)i, m.dt);
+        if (march_at(p.world, m, t).solid) {
+            found = true;
+            tb = t;
+            ta = __fmul_rn((float)(i - 1), m.dt);
+            break;
+        }
+    }
+    march_store(p, mp, c, px, py, m, len, found, ta, tb);
+}
+
 __device__ __forceinline__ const CamDev &stage(CamDev *slot, const CamDev *cams, uint32_t i,
                                                int lane) {
     const uint32_t *src = reinterpret_cast<const uint32_t *>(cams + i);
@@ -191,7 +215,7 @@ __device__ __forceinline__ const CamDev &stage(CamDev *slot, const CamDev *cams,
 // Persistent: warps pop (camera, tile) items from the batch's atomic counter.
 template <bool BEAMS>
 __global__ void __launch_bounds__(BEAMS ? kMarchThreads : kMarchAllThreads,
-                                  BEAMS ? kMarchMinBlocks : kMarchAllMinBlocks)
+                                  BEAMS ? kMarchMinBlocks : 1)
     k_march_batched(const RenderParams p, const MarchParams m) {
     __shared__ LevelDev s_lv[kMaxLevels + 1];
     __shared__ uint32_t s_base[kMaxCams + 1];
@@ -224,7 +248,8 @@ __global__ void __launch_bounds__(BEAMS ? kMarchThreads : kMarchAllThreads,
         for (int i = lane; i < npix; i += 32) {
             const int32_t px = x0 + (i & ((1 << p.tile_w_log2) - 1));
             const int32_t py = y0 + (i >> p.tile_w_log2);
-            march_pixels<BEAMS>(p, m, s_lv, c, px, py, px < (int32_t)c.w && py < (int32_t)c.h);
+            if (BEAMS) march_pixels(p, m, s_lv, c, px, py);
+            else march_pixel(p, m, c, px, py);
         }
     }
 }
@@ -238,7 +263,7 @@ int launch_march_batched(const RenderParams &p, const MarchParams &m, bool beams
     if (beams && m.steps >= kMarchBeamSteps) {
         k_march_batched<true><<<blocks, kMarchThreads, 0, s>>>(p, m);
     } else {
-        const int all = (blocks * kMarchAllMinBlocks + kMarchMinBlocks - 1) / kMarchMinBlocks;
+        const int all = (blocks * kMarchAllBlocks + kMarchMinBlocks - 1) / kMarchMinBlocks;
         k_march_batched<false><<<all, kMarchAllThreads, 0, s>>>(p, m);
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;

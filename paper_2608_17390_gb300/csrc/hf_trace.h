@@ -45,14 +45,6 @@ __device__ __forceinline__ uint32_t shade(uint32_t m, uint8_t face, bool visible
     return out;
 }
 
-// The ray of a camera's pixel.
-__device__ __forceinline__ Ray primary_ray(const CamDev &c, int32_t px, int32_t py) {
-    const int32_t a = 2 * px + 1 - (int32_t)c.w;
-    const int32_t b = (int32_t)c.h - 1 - 2 * py;
-    return Ray{c.o[0], c.o[1], c.o[2], c.F[0] + a * c.R[0] + b * c.U[0],
-               c.F[1] + a * c.R[1] + b * c.U[1], c.F[2] + a * c.R[2] + b * c.U[2]};
-}
-
 // Asks L2 for the world's coarse levels (all of a small world) as a launch
 // starts, spread over all its threads.  A ray's fetches form one dependent
 // chain, so a short render of a world that is not in L2 would otherwise wait
