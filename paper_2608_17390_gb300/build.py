@@ -41,7 +41,8 @@ def build(verbose=False, extra=()):
     os.makedirs(OUT, exist_ok=True)
     headers = [os.path.join(ROOT, "include", "hf.h"), os.path.join(CSRC, "hf_internal.h"),
                os.path.join(CSRC, "hf_cast.h"), os.path.join(CSRC, "hf_beam.h"),
-               os.path.join(CSRC, "hf_march.h"), os.path.join(CSRC, "hf_trace.h")]
+               os.path.join(CSRC, "hf_march.h"), os.path.join(CSRC, "hf_trace.h"),
+               os.path.join(CSRC, "hf_rules.h")]
     jobs = []
     objs = []
     for src in SOURCES:

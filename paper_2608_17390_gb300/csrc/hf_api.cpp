@@ -20,6 +20,7 @@
 
 #include "hf.h"
 #include "hf_internal.h"
+#include "hf_rules.h"
 
 namespace {
 
@@ -212,38 +213,6 @@ int ctx_view(const hf_ctx *c, CtxView *out) {
     return 0;
 }
 
-}  // namespace hf
-
-// A beam pays where the rays of a warp go through the same cells.  The angle that
-// the warp's group of 32 pixels spans (8 x 4, or a row of a wide tile), times the
-// length of the world, says how far they fall apart.  Rays each by itself over
-// beams, single views and batches of 16, with and without shadows, 8 x 4 tiles:
-//   span (rad)   0.017        0.025       0.033       0.05        0.067       0.1
-//   256^2        1.29 - 1.85  1.28 - 1.8  1.07 - 1.7  1.01 - 1.65 0.91 - 1.43 0.77 - 1.48
-//   2048^2       1.47 - 1.80  1.28 - 1.8  1.11 - 1.4  0.90 - 1.73 0.78 - 1.60 0.66 - 1.73
-//   2048 x 8192  1.49 - 2.03  1.16 - 1.9  0.73 - 2.0  0.21 - 1.54 0.17 - 1.48 0.12 - 1.39
-// So spans up to 0.04 get beams, up to 0.06 in worlds of up to 512 cells, and up to
-// 0.028 in worlds of more than 4096.  In a batch the pixels of cameras beyond that
-// may make up one in 32: they cost up to ten times as much.
-namespace hf {
-bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw) {
-    const int32_t size = W > H ? W : H;
-    const double most = size <= 512 ? 0.06 : size <= 4096 ? 0.04 : 0.028;
-    const double gw = tw < 32 ? tw : 32, gh = 32 / gw;
-    uint64_t all = 0, wide = 0;
-    for (uint32_t i = 0; i < n; ++i) {
-        const hf_camera &k = cams[i];
-        auto norm2 = [](const int32_t *v) {
-            return (double)v[0] * v[0] + (double)v[1] * v[1] + (double)v[2] * v[2];
-        };
-        // neighbouring pixels are 2 |right|, 2 |up| apart at distance |fwd|
-        const double across = 4.0 * gw * gw * norm2(k.right), along = 4.0 * gh * gh * norm2(k.up);
-        const uint64_t px = (uint64_t)k.w * k.h;
-        all += px;
-        if ((across > along ? across : along) > most * most * norm2(k.fwd)) wide += px;
-    }
-    return wide * 32 <= all;
-}
 }  // namespace hf
 
 extern "C" {
@@ -1126,33 +1095,6 @@ static int render_host_staged(hf_ctx *c, const hf_camera *cams, uint32_t n, cons
     return HF_OK;
 }
 
-// The warp tile of a render that leaves its sides at 0.  8 x 4 is one pixel per
-// lane, the most warps: right while a render fills the GPU but a few times over,
-// as its slowest warps decide its end.  Beyond that narrow and tall tiles win:
-// 32 pixels of 4 x 8 go through nearly the same columns of the grid, and longer
-// tiles share one fetch of the tile and of its camera.  Measured over 2048 x 2048
-// and 2048 x 16384 cells (us, 8 x 4 against the choice):
-//   groups of 32 pixels per resident warp   8 x 4    choice
-//   1280 x 720 with shadows       8           81      76  (4 x 8;  4 x 16: 77)
-//   960 x 540 with shadows        4           59      61  (4 x 8, so still 8 x 4)
-//   1920 x 1080                  15          119     113  (4 x 16; 4 x 8: 118)
-//   1920 x 1080 with shadows     18          149     140  (4 x 16; 4 x 32: 142)
-//   4K with shadows              71          517     477  (4 x 32; 4 x 16: 487)
-//   20 views of 1920 x 1080     355         2142    1952  (4 x 32; 4 x 16: 1997)
-// Stores to host memory want wide rows, and the traversal of single rays was
-// tuned on 8 x 4: both keep it.
-static void default_tile(const hf_camera *cams, uint32_t n, bool beams, uint64_t warps,
-                         uint32_t flags, uint32_t &tw, uint32_t &th) {
-    tw = 8;
-    th = 4;
-    if (!beams || (flags & HF_HOST_OUTPUTS)) return;
-    uint64_t groups = 0;
-    for (uint32_t i = 0; i < n; ++i) groups += ((uint64_t)cams[i].w * cams[i].h + 31) / 32;
-    if (groups < 6 * warps) return;
-    tw = 4;
-    th = groups < 12 * warps ? 8 : groups < 64 * warps ? 16 : 32;
-}
-
 int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *outs,
               const hf_render_opts *opts) {
     if (!c) return HF_E_INVALID_ARG;
@@ -1184,9 +1126,9 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
     for (uint32_t i = 0; i < n; ++i)  // before anything is built or enqueued
         if (hf_validate_camera(c->W, c->H, &cams[i]) != HF_OK) return HF_E_INVALID_ARG;
     if (!o.tile_w && !o.tile_h)
-        default_tile(cams, n, kind == hf::kTraceBeams,
-                     (uint64_t)c->sm_count * c->occ[shadows][kind] * (hf::trace_threads(kind) / 32), o.flags, tw,
-                     th);
+        hf::default_tile(cams, n, kind == hf::kTraceBeams,
+                         (uint64_t)c->sm_count * c->occ[shadows][kind] * (hf::trace_threads(kind) / 32),
+                         o.flags, tw, th);
     const uint32_t *bounds = nullptr;
     if (shadows) {
         const int brc = ensure_sun_bounds(c, sun, &bounds);

@@ -183,8 +183,6 @@ int voxel_repair(const WorldDev &w, const VoxelDev &v, int32_t x0, int32_t y0, i
 int launch_voxel_trace(const RenderParams &p, const VoxelDev &v, const VoxelParams &q,
                        uint32_t n_cams, uint32_t max_tiles, void *stream);  // tiles of 8 x 4 pixels
 
-// Whether the rays of a warp's 32 pixels stay close enough for beams (hf_api.cpp).
-bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw);
 // How the trace kernels follow rays: warps of rays in beams; one ray at a time
 // (a step limit set by the caller: p.max_steps); the same with fetch counters.
 enum TraceKind { kTraceBeams = 0, kTraceGeneral = 1, kTraceStats = 2, kTraceKinds = 3 };

@@ -1,6 +1,6 @@
 // hf_single.cu -- the trace kernels that follow each ray by itself: renders with a
 // step limit of the caller's or with fetch counters, and views whose rays lie too
-// far apart for beams (beams_fit in hf_api.cpp).
+// far apart for beams (beams_fit in hf_rules.h).
 //
 // One warp owns one tile of tile_w x tile_h pixels; each lane traces the tile's
 // pixels lane, lane + 32, ... by hierarchical DDA over the min/max pyramid

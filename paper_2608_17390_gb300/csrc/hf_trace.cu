@@ -25,6 +25,7 @@
 #include "hf.h"
 #include "hf_beam.h"
 #include "hf_internal.h"
+#include "hf_rules.h"
 #include "hf_trace.h"
 
 namespace hf {

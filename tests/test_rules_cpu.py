@@ -1,0 +1,72 @@
+"""The rules that pick a render's launch from its cameras (csrc/hf_rules.h), on
+the CPU."""
+
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import synth
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SHIM = r"""
+#include "hf_rules.h"
+extern "C" void tile(const hf_camera *c, uint32_t n, int beams, uint64_t warps, uint32_t flags, uint32_t *t) {
+    hf::default_tile(c, n, beams, warps, flags, t[0], t[1]);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    (d / "shim.cpp").write_text(SHIM)
+    so = str(d / "rules.so")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"),
+                           "-I", os.path.join(ROOT, "paper_2608_17390_gb300", "csrc"),
+                           str(d / "shim.cpp"), "-o", so])
+    return ctypes.CDLL(so)
+
+
+def _cams(w, h, n):
+    return np.repeat(synth.camera_array([((0, 0, 0), (1 << 19, 0, 0), (0, 9, 0), (0, 0, 9), w, h)]), n)
+
+
+def _tile(lib, cams, warps=3648, beams=True, flags=0):
+    t = (ctypes.c_uint32 * 2)()
+    lib.tile(ctypes.c_void_p(cams.ctypes.data), len(cams), int(beams), ctypes.c_uint64(warps), flags, t)
+    return tuple(t)
+
+
+@pytest.mark.parametrize("w,h,n,want", [
+    (320, 240, 1, (8, 4)), (1280, 720, 1, (4, 8)), (1920, 1080, 1, (4, 16)), (3840, 2160, 1, (4, 32)),
+    (1920, 1080, 100, (4, 32)), (640, 360, 100, (4, 32)), (16384, 16384, 1, (4, 32)),
+    # images lower than the tiles, or a little higher than a number of them
+    (2048, 1, 4096, (8, 4)), (2048, 2, 4000, (8, 4)), (3840, 9, 100, (8, 4)), (3840, 9, 4000, (8, 4)),
+    (3840, 8, 4000, (4, 8)), (1024, 17, 4000, (8, 4)), (1024, 40, 4000, (4, 8)), (1024, 32, 4000, (4, 32)),
+    (1, 1, 4096, (8, 4)), (2, 512, 4096, (4, 16))])
+def test_default_tile(lib, w, h, n, want):
+    assert _tile(lib, _cams(w, h, n)) == want
+    assert _tile(lib, _cams(w, h, n), beams=False) == (8, 4)
+    assert _tile(lib, _cams(w, h, n), flags=64 | 128 | 256) == (8, 4)
+
+
+def test_default_tile_makes_no_more_groups(lib):
+    rng = np.random.default_rng(2)
+    for _ in range(300):
+        cams = np.concatenate([_cams(*(int(2.0 ** rng.uniform(0, 13)) for _ in range(2)), int(rng.integers(1, 40)))
+                               for _ in range(3)])
+        tw, th = _tile(lib, cams)
+        w, h = cams["w"].astype(np.int64), cams["h"].astype(np.int64)
+        wide = (-(-w // 8) * -(-h // 4)).sum()
+        if tw == 4:
+            assert (-(-w // 4) * -(-h // 8)).sum() <= wide * 33 / 32
+            assert (-(-w // 4) * -(-h // th)).sum() * (th // 8) <= (-(-w // 4) * -(-h // 8)).sum() * 9 / 8
+
+
+def test_a_batch_refused_in_8_by_4_tiles_stays_refused(lib):
+    """2^32 tiles of 8 x 4 are one too many; taller tiles would make them fewer."""
+    assert _tile(lib, _cams(16384, 16384, 512)) == (8, 4)
+    assert _tile(lib, _cams(16384, 16384, 511)) == (4, 32)
