@@ -750,7 +750,8 @@ static int launch_graph(hf_ctx *c, Slot &s, const GraphKey &key, const hf::Rende
     return HF_OK;
 }
 
-// Validates the cameras, takes a render slot and fills its camera table.
+// Validates the cameras, takes a render slot and fills its camera table.  beam_tw:
+// the tile width that wide views are told by, 0 where no beams are cast.
 struct Batch {
     int slot;
     size_t bytes, bucket;
@@ -774,8 +775,8 @@ static void *device_alias(void *ptr) {
 }
 
 static int prepare_batch(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *outs,
-                         uint32_t tw, uint32_t th, bool nowait, void *user_stream, Batch &b,
-                         bool host_outputs = false, size_t extra_bytes = 0) {
+                         uint32_t tw, uint32_t th, uint32_t beam_tw, bool nowait, void *user_stream,
+                         Batch &b, bool host_outputs = false, size_t extra_bytes = 0) {
     const int twl = ilog2_exact(tw), thl = ilog2_exact(th);
     if (twl < 0 || thl < 0 || tw * th < 32 || tw * th > 256 || tw > 256 || th > 256)
         return HF_E_INVALID_ARG;
@@ -801,10 +802,10 @@ static int prepare_batch(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_
     hdr->total_tiles = (uint32_t)total_tiles;
     auto *cd = (hf::CamDev *)((char *)s.h_staging + sizeof(hf::BatchHeader));
     b.tiles.assign(n, 0);
-    uint32_t base = 0;
-    for (uint32_t i = 0; i < n; ++i) {
+    uint32_t base = 0, at = 0;
+    auto put = [&](uint32_t i, bool single) {
         const hf_camera &k = cams[i];
-        hf::CamDev &v = cd[i];
+        hf::CamDev &v = cd[at];
         for (int a = 0; a < 3; ++a) {
             v.o[a] = (int32_t)k.origin[a];
             v.F[a] = k.fwd[a];
@@ -814,15 +815,16 @@ static int prepare_batch(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_
         v.w = k.w;
         v.h = k.h;
         v.tiles_x = (k.w + tw - 1) / tw;
-        b.tiles[i] = v.tiles_x * ((k.h + th - 1) / th);
+        b.tiles[at] = v.tiles_x * ((k.h + th - 1) / th);
         v.tile_base = base;
-        base += b.tiles[i];
+        base += b.tiles[at++];
         v.hit_cell = outs[i].hit_cell;
         v.layer = outs[i].layer;
         v.face = outs[i].face;
         v.depth = outs[i].depth;
         v.rgba = outs[i].rgba;
         v.shadow = outs[i].shadow;
+        v.single = single;
         if (host_outputs) {
             const hf_outputs &u = outs[i];
             v.hit_cell = static_cast<uint32_t *>(device_alias(u.hit_cell));
@@ -833,9 +835,17 @@ static int prepare_batch(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_
             v.shadow = static_cast<uint8_t *>(device_alias(u.shadow));
             if ((u.hit_cell && !v.hit_cell) || (u.layer && !v.layer) || (u.face && !v.face) ||
                 (u.depth && !v.depth) || (u.rgba && !v.rgba) || (u.shadow && !v.shadow))
-                return HF_E_INVALID_ARG;  // the slot was not yet marked in flight
+                return false;  // the slot was not yet marked in flight
         }
-    }
+        return true;
+    };
+    // wide views first: their warps take longest, and would be a batch's tail
+    auto wide = [&](uint32_t i) {
+        return beam_tw && hf::view_wide((int32_t)c->W, (int32_t)c->H, cams[i], beam_tw);
+    };
+    for (const bool single : {true, false})
+        for (uint32_t i = 0; i < n; ++i)
+            if (wide(i) == single && !put(i, single)) return HF_E_INVALID_ARG;
     std::memset(&b.p, 0, sizeof(b.p));
     b.p.world = c->wd;
     {  // the levels the trace kernels warm in L2: from the finest level whose
@@ -1115,9 +1125,12 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         if (iabs64(sun[i]) >= kLimit21) return HF_E_INVALID_ARG;
     const bool shadows = (o.flags & HF_SHADOWS) != 0;
     const int kind = (o.flags & HF_STATS) ? hf::kTraceStats
-                     : o.max_steps || !hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw)
+                     : o.max_steps || !hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kTraceShare)
                          ? hf::kTraceGeneral
                          : hf::kTraceBeams;
+    // (plain launches pick their kernel one by one)
+    const bool plain = (o.flags & HF_PLAIN) != 0;
+    const uint32_t fit_tw = tw, beam_tw = kind == hf::kTraceBeams && !plain ? tw : 0;
     const uint32_t mip = o.mip_start == HF_MIP_AUTO ? hf::kDefaultMipStart : o.mip_start;
     const uint32_t mip_c = mip > c->L ? c->L : mip;
     const uint64_t guard = 4ull * (c->W + c->H) + 64;
@@ -1135,8 +1148,8 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         if (brc != HF_OK) return brc;
     }
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, tw, th, (o.flags & HF_NOWAIT) != 0, o.cuda_stream, b,
-                           (o.flags & HF_HOST_OUTPUTS) != 0);
+    int rc = prepare_batch(c, cams, n, outs, tw, th, beam_tw, (o.flags & HF_NOWAIT) != 0,
+                           o.cuda_stream, b, (o.flags & HF_HOST_OUTPUTS) != 0);
     if (rc != HF_OK) return rc;
     b.p.sun_bounds = bounds;
     Slot &s = c->slots[b.slot];
@@ -1155,9 +1168,14 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
     if ((o.flags & HF_PLAIN) || (n == 1 && !(o.flags & HF_NOGRAPH))) {
         // each launch takes its camera record as a parameter: no copy to the device
         const auto *cd = (const hf::CamDev *)((const char *)s.h_staging + sizeof(hf::BatchHeader));
-        for (uint32_t i = 0; i < n; ++i)
-            if (hf::launch_trace_plain(p, shadows, kind, cd[i], b.tiles[i], b.stream))
+        for (uint32_t i = 0; i < n; ++i) {
+            const int one = kind == hf::kTraceStats || o.max_steps ? kind
+                            : hf::view_wide((int32_t)c->W, (int32_t)c->H, cams[i], fit_tw)
+                                ? hf::kTraceGeneral
+                                : hf::kTraceBeams;
+            if (hf::launch_trace_plain(p, shadows, one, cd[i], b.tiles[i], b.stream))
                 return HF_E_CUDA;
+        }
     } else if (o.flags & HF_NOGRAPH) {
         CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));
         if (hf::launch_trace_batched(p, shadows, kind, c->sm_count * c->occ[shadows][kind],
@@ -1194,11 +1212,11 @@ int hf_render_march(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outpu
     const uint32_t tw = o.tile_w ? o.tile_w : 8, th = o.tile_h ? o.tile_h : 4;
     if (c->occ_march < 1) return HF_E_CUDA;
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, tw, th, false, o.cuda_stream, b);
+    int rc = prepare_batch(c, cams, n, outs, tw, th, tw, false, o.cuda_stream, b);
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
     CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));
-    const bool beams = hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw);
+    const bool beams = hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kMarchShare);
     if (hf::launch_march_batched(b.p, m, beams, c->sm_count * c->occ_march, b.stream)) return HF_E_CUDA;
     return finish_batch(c, b, (o.flags & HF_SYNC) != 0);
 }
@@ -1301,7 +1319,7 @@ int hf_render_scatter(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_foo
     }
     sp.max_pixels = maxpix;
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, 8, 4, false, o.cuda_stream, b, false,
+    int rc = prepare_batch(c, cams, n, outs, 8, 4, 0, false, o.cuda_stream, b, false,
                            (size_t)n * sizeof(hf_footprint));
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
@@ -1394,7 +1412,7 @@ int hf_render_voxel(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outpu
     q.far_dist = o.far_dist != 0.0f ? o.far_dist : 600.0f;
     if (o.outer > 1u << 20 || o.inner > 4096 || !(q.far_dist > 0.0f)) return HF_E_INVALID_ARG;
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, 8, 4, false, o.cuda_stream, b);
+    int rc = prepare_batch(c, cams, n, outs, 8, 4, 0, false, o.cuda_stream, b);
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
     CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));

@@ -103,7 +103,9 @@ struct CamDev {
     int32_t o[3];
     int32_t F[3], R[3], U[3];
     uint32_t w, h;
-    uint32_t tiles_x, tile_base;  // tiles per image row, first global tile of this camera
+    uint32_t tiles_x : 31;        // tiles per image row
+    uint32_t single : 1;          // its rays lie too far apart for beams (hf_rules.h)
+    uint32_t tile_base;           // first global tile of this camera
     uint32_t *hit_cell;
     uint8_t *layer;
     uint8_t *face;
@@ -111,6 +113,8 @@ struct CamDev {
     uint32_t *rgba;
     uint8_t *shadow;
 };
+// (what follows a table of them is read by 16 bytes)
+static_assert(sizeof(CamDev) == 112, "camera record");
 
 struct BatchHeader {
     uint32_t counter;      // next global tile (atomic, zero at launch)

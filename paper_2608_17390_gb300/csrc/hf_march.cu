@@ -79,15 +79,16 @@ __device__ __forceinline__ int32_t march_samples(const WorldDev &w, const MarchR
 // The first solid sample of each lane's ray, or 0; every lane of the warp calls.
 __device__ __forceinline__ int32_t march_beams(const RenderParams &p, const MarchParams &mp,
                                                const LevelDev *lvt, const Ray &r, const MarchRay &m,
-                                               bool inside) {
+                                               bool inside, bool single) {
     int32_t found = 0;
     const int lane = threadIdx.x & 31;
     const BeamDir d = beam_dir(r.dx, r.dy, r.dz);
     BeamRay q = beam_ray(d, r);
     const MarchRate rate = march_rate(m, d);
     const float steps = (float)mp.steps;
-    // every sample of a ray that is vertical or whose spacing is no ordinary number
-    const bool plain = d.du == 0 || !(m.dt > 1e-9f && m.dt < 1e9f);
+    // every sample of a wide view's rays, and of a ray that is vertical or whose
+    // spacing is no ordinary number
+    const bool plain = single || d.du == 0 || !(m.dt > 1e-9f && m.dt < 1e9f);
     uint32_t todo = __ballot_sync(kFull, inside && !plain);
     while (todo) {
         const int lead = __ffs(todo) - 1;
@@ -176,7 +177,7 @@ __device__ __forceinline__ void march_pixels(const RenderParams &p, const MarchP
     const Ray r = primary_ray(c, px, py);
     float len;
     const MarchRay m = march_ray(mp, r, len);
-    const int32_t i = march_beams(p, mp, lvt, r, m, inside);
+    const int32_t i = march_beams(p, mp, lvt, r, m, inside, c.single != 0);
     if (inside)
         march_store(p, mp, c, px, py, m, len, i != 0, __fmul_rn((float)(i - 1), m.dt),
                     __fmul_rn((float)i, m.dt));

@@ -16,25 +16,43 @@ namespace hf {
 //   2048^2       1.47 - 1.80  1.28 - 1.8  1.11 - 1.4  0.90 - 1.73 0.78 - 1.60 0.66 - 1.73
 //   2048 x 8192  1.49 - 2.03  1.16 - 1.9  0.73 - 2.0  0.21 - 1.54 0.17 - 1.48 0.12 - 1.39
 // So spans up to 0.04 get beams, up to 0.06 in worlds of up to 512 cells, and up to
-// 0.028 in worlds of more than 4096.  In a batch the pixels of cameras beyond that
-// may make up one in 32: they cost up to ten times as much.
-inline bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw) {
+// 0.028 in worlds of more than 4096.
+inline bool view_wide(int32_t W, int32_t H, const hf_camera &k, uint32_t tw) {
     const int32_t size = W > H ? W : H;
     const double most = size <= 512 ? 0.06 : size <= 4096 ? 0.04 : 0.028;
     const double gw = tw < 32 ? tw : 32, gh = 32 / gw;
+    auto norm2 = [](const int32_t *v) {
+        return (double)v[0] * v[0] + (double)v[1] * v[1] + (double)v[2] * v[2];
+    };
+    // neighbouring pixels are 2 |right|, 2 |up| apart at distance |fwd|
+    const double across = 4.0 * gw * gw * norm2(k.right), along = 4.0 * gh * gh * norm2(k.up);
+    return (across > along ? across : along) > most * most * norm2(k.fwd);
+}
+
+// Whether a batch takes the kernel with beams: if of `share` pixels at most one is a
+// wide view's.  In a batch that does, the rays of its wide views go each by itself
+// too (CamDev::single; in beams, batches over 2048 x 16384 cells with 3 % of their
+// pixels in views of 64 x 48 took up to seven times as long), but in a kernel whose
+// registers are the beams'.  All rays by themselves over beams for the views that
+// fit, by the share of the wide views' pixels:
+//   share           0.08         0.13         0.21         0.37         0.57         0.84
+//   traced, 2048^2  0.99 - 1.59  1.17 - 1.49  1.23 - 1.55  1.09 - 1.42  0.91 - 1.22  0.95 - 1.20
+//   2048 x 16384    1.34 - 1.71  1.33 - 1.51  1.33 - 1.63  1.13 - 1.27  0.91 - 1.14  0.86 - 1.00
+//   (32 views of 320 x 200 and 64 of 200 x 150, a quarter to half of them wide, the six
+//   that lose most: 0.84 - 0.95; so the line is at a quarter)
+//   share           0.04         0.07         0.17         0.20         0.44         0.55
+//   marched, 100    0.86 - 1.78  0.98 - 1.30  0.85 - 1.32  1.00 - 1.25  0.81 - 1.06  0.94 - 1.00
+//   samples; 256    1.26 - 2.97  0.76 - 1.64  1.00 - 2.04  0.77 - 1.58  1.00 - 1.48  1.00 - 1.37
+constexpr uint32_t kTraceShare = 4, kMarchShare = 32;
+inline bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw,
+                      uint32_t share) {
     uint64_t all = 0, wide = 0;
     for (uint32_t i = 0; i < n; ++i) {
-        const hf_camera &k = cams[i];
-        auto norm2 = [](const int32_t *v) {
-            return (double)v[0] * v[0] + (double)v[1] * v[1] + (double)v[2] * v[2];
-        };
-        // neighbouring pixels are 2 |right|, 2 |up| apart at distance |fwd|
-        const double across = 4.0 * gw * gw * norm2(k.right), along = 4.0 * gh * gh * norm2(k.up);
-        const uint64_t px = (uint64_t)k.w * k.h;
+        const uint64_t px = (uint64_t)cams[i].w * cams[i].h;
         all += px;
-        if ((across > along ? across : along) > most * most * norm2(k.fwd)) wide += px;
+        if (view_wide(W, H, cams[i], tw)) wide += px;
     }
-    return wide * 32 <= all;
+    return wide * share <= all;
 }
 
 // The warp tile of a render that leaves its sides at 0.  8 x 4 is one pixel per

@@ -39,8 +39,8 @@ namespace {
 constexpr int kTraceMinBlocks = 6;
 constexpr int kThreads = trace_threads(kTraceBeams);
 
-// Casts one ray per active lane; every lane of the warp calls.  only: of a hit
-// nothing matters but that there is one.
+// Casts one ray per active lane; every lane of the warp calls.  single: each by
+// itself; only: of a hit nothing matters but that there is one.
 //
 // The rays that go the same way and start side by side form a beam (hf_beam.h);
 // they are walked, all together, through the runs of columns that it does not
@@ -55,14 +55,14 @@ constexpr int kThreads = trace_threads(kTraceBeams);
 template <bool PAIR>
 __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev *lvt,
                                            const BeamDir &d, BeamRay q, int32_t oz, int32_t dz,
-                                           bool active, int mip, bool only, Hit &h) {
+                                           bool active, bool single, int mip, bool only, Hit &h) {
     BeamHit b;
     b.kind = -1;
     const uint32_t W = (uint32_t)p.world.W, H = (uint32_t)p.world.H;
     const uint32_t *cells = p.world.base;
     const int lane = threadIdx.x & 31;
-    // rays that no beam takes: vertical ones, and (below) through corners
-    bool alone = active && d.du == 0;
+    // rays that no beam takes: vertical ones, a wide view's, and (below) through corners
+    bool alone = active && (single || d.du == 0);
     active = active && !alone && (uint32_t)(d.key & 2 ? ~q.fu : q.fu) < (d.key & 4 ? W : H) &&
              (uint32_t)(d.key & 1 ? ~q.fv : q.fv) < (d.key & 4 ? H : W);
     uint32_t todo = __ballot_sync(kFull, active);
@@ -139,7 +139,8 @@ __device__ __forceinline__ void tile_pixel(const RenderParams &p, const TileDev 
 // One pixel per lane: its primary ray, then (with shadows) the shadow ray, in
 // a second pass of the same traversal code.  Every lane of the warp calls;
 // 
-template <bool SHADOWS, bool PAIR>
+// WIDE: the view may be a wide one (a launch of one view is not).
+template <bool SHADOWS, bool PAIR, bool WIDE>
 __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelDev *lvt,
                                              const TileDev &t, int i, const BeamDir &sun) {
     const CamDev &c = t.cam;
@@ -155,7 +156,7 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
         const bool sp = SHADOWS && pass;
         Hit h;
         const BeamDir d = sp ? sun : beam_dir(r.dx, r.dy, r.dz);
-        cast_beams<PAIR>(p, lvt, d, beam_ray(d, r), r.oz, r.dz, cast,
+        cast_beams<PAIR>(p, lvt, d, beam_ray(d, r), r.oz, r.dz, cast, WIDE && c.single,
                          sp ? p.shadow_mip : p.mip_start, sp, h);
         if (sp) {
             if (cast) visible = h.face == kFaceMiss;
@@ -242,7 +243,7 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
 }
 
 // One warp renders one tile: lane l traces the tile's pixels l, l+32, ...
-template <bool SHADOWS, bool PAIR>
+template <bool SHADOWS, bool PAIR, bool WIDE>
 __device__ __forceinline__ void trace_tile(const RenderParams &p, const LevelDev *lvt,
                                            const BeamDir &sun, TileDev &t, uint32_t local_tile,
                                            int lane) {
@@ -252,7 +253,7 @@ __device__ __forceinline__ void trace_tile(const RenderParams &p, const LevelDev
     }
     __syncwarp();
     for (int i = lane; i < 1 << (p.tile_w_log2 + p.tile_h_log2); i += 32)
-        trace_pixels<SHADOWS, PAIR>(p, lvt, t, i, sun);
+        trace_pixels<SHADOWS, PAIR, WIDE>(p, lvt, t, i, sun);
 }
 
 // Copy camera i into this warp's shared slot.
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks) k_trace_batched(con
             else hi = mid;
         }
         TileDev &tile = stage_cam(&s_tile[threadIdx.x >> 5], p.cams, lo, lane);
-        trace_tile<SHADOWS, PAIR>(p, s_lv, s_sun, tile, t - s_base[lo], lane);
+        trace_tile<SHADOWS, PAIR, true>(p, s_lv, s_sun, tile, t - s_base[lo], lane);
     }
 }
 
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, kTraceMinBlocks)
     if (t >= n_tiles) return;
     const int lane = threadIdx.x & 31;
     TileDev &tile = stage_cam(&s_tile[threadIdx.x >> 5], &cam, 0, lane);
-    trace_tile<SHADOWS, PAIR>(p, s_lv, s_sun, tile, t, lane);
+    trace_tile<SHADOWS, PAIR, false>(p, s_lv, s_sun, tile, t, lane);
 }
 
 template <bool SH, bool PA>
@@ -457,31 +458,36 @@ extern "C" int hf_render_noalloc(hf_ctx *ctx, const hf_camera *cams, uint32_t n,
     auto *hdr = reinterpret_cast<BatchHeader *>(buf);
     std::memset(hdr, 0, sizeof(*hdr));
     auto *cd = reinterpret_cast<CamDev *>(buf + kNoallocCamOff);
-    uint64_t base = 0;
-    for (uint32_t i = 0; i < n; ++i) {
-        const hf_camera &k = cams[i];
-        if (hf_validate_camera((uint32_t)v.world.W, (uint32_t)v.world.H, &k) != HF_OK)
+    for (uint32_t i = 0; i < n; ++i)
+        if (hf_validate_camera((uint32_t)v.world.W, (uint32_t)v.world.H, &cams[i]) != HF_OK)
             return HF_E_INVALID_ARG;
-        CamDev &c = cd[i];
-        for (int a = 0; a < 3; ++a) {
-            c.o[a] = (int32_t)k.origin[a];
-            c.F[a] = k.fwd[a];
-            c.R[a] = k.right[a];
-            c.U[a] = k.up[a];
+    uint64_t base = 0;
+    uint32_t at = 0;
+    for (const bool single : {true, false})  // wide views first, as in hf_render
+        for (uint32_t i = 0; i < n; ++i) {
+            const hf_camera &k = cams[i];
+            if (view_wide(v.world.W, v.world.H, k, tw) != single) continue;
+            CamDev &c = cd[at++];
+            for (int a = 0; a < 3; ++a) {
+                c.o[a] = (int32_t)k.origin[a];
+                c.F[a] = k.fwd[a];
+                c.R[a] = k.right[a];
+                c.U[a] = k.up[a];
+            }
+            c.w = k.w;
+            c.h = k.h;
+            c.tiles_x = (k.w + tw - 1) / tw;
+            c.single = single;
+            c.tile_base = (uint32_t)base;
+            base += (uint64_t)c.tiles_x * ((k.h + th - 1) / th);
+            if (base >= 0xFFFFFFFFull) return HF_E_INVALID_ARG;
+            c.hit_cell = outs[i].hit_cell;
+            c.layer = outs[i].layer;
+            c.face = outs[i].face;
+            c.depth = outs[i].depth;
+            c.rgba = outs[i].rgba;
+            c.shadow = outs[i].shadow;
         }
-        c.w = k.w;
-        c.h = k.h;
-        c.tiles_x = (k.w + tw - 1) / tw;
-        c.tile_base = (uint32_t)base;
-        base += (uint64_t)c.tiles_x * ((k.h + th - 1) / th);
-        if (base >= 0xFFFFFFFFull) return HF_E_INVALID_ARG;
-        c.hit_cell = outs[i].hit_cell;
-        c.layer = outs[i].layer;
-        c.face = outs[i].face;
-        c.depth = outs[i].depth;
-        c.rgba = outs[i].rgba;
-        c.shadow = outs[i].shadow;
-    }
     hdr->n_cams = n;
     hdr->total_tiles = (uint32_t)base;
 
@@ -525,7 +531,7 @@ extern "C" int hf_render_noalloc(hf_ctx *ctx, const hf_camera *cams, uint32_t n,
         p.sun[i] = sun[i];
         p.sun_n[i] = (float)(sun[i] / sn);
     }
-    const int kind = o.max_steps || !beams_fit(v.world.W, v.world.H, cams, n, tw)
+    const int kind = o.max_steps || !beams_fit(v.world.W, v.world.H, cams, n, tw, kTraceShare)
                          ? kTraceGeneral
                          : kTraceBeams;
     const int blocks = v.sm_count * v.occ[shadows ? 1 : 0][kind];

@@ -1,0 +1,20 @@
+"""The rule that tells wide views from those whose rays go in beams
+(csrc/hf_rules.h), for tests that have to know which way a view goes."""
+
+import numpy as np
+
+
+def wide_views(W, H, cams, tile_w=8):
+    """Per camera: whether a group of 32 of its pixels spans too much for a beam."""
+    size = max(W, H)
+    most = 0.06 if size <= 512 else 0.04 if size <= 4096 else 0.028
+    gw = min(tile_w, 32)
+    gh = 32 // gw
+    f, r, u = (np.sqrt((cams[k].astype(float) ** 2).sum(1)) for k in "fru")
+    return np.maximum(2 * gw * r, 2 * gh * u) > most * f
+
+
+def share_of_wide(W, H, cams, tile_w=8):
+    """The share of the batch's pixels that are in wide views."""
+    px = cams["w"].astype(np.int64) * cams["h"]
+    return px[wide_views(W, H, cams, tile_w)].sum() / px.sum()

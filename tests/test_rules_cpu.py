@@ -16,6 +16,10 @@ SHIM = r"""
 extern "C" void tile(const hf_camera *c, uint32_t n, int beams, uint64_t warps, uint32_t flags, uint32_t *t) {
     hf::default_tile(c, n, beams, warps, flags, t[0], t[1]);
 }
+extern "C" int wide(int32_t W, int32_t H, const hf_camera *c, uint32_t tw) { return hf::view_wide(W, H, *c, tw); }
+extern "C" int fit(int32_t W, int32_t H, const hf_camera *c, uint32_t n, uint32_t tw, uint32_t share) {
+    return hf::beams_fit(W, H, c, n, tw, share);
+}
 """
 
 
@@ -70,3 +74,27 @@ def test_a_batch_refused_in_8_by_4_tiles_stays_refused(lib):
     """2^32 tiles of 8 x 4 are one too many; taller tiles would make them fewer."""
     assert _tile(lib, _cams(16384, 16384, 512)) == (8, 4)
     assert _tile(lib, _cams(16384, 16384, 511)) == (4, 32)
+
+
+@pytest.mark.parametrize("W,H,most", [(512, 200, 0.06), (513, 4, 0.04), (30, 4096, 0.04), (4097, 2, 0.028)])
+@pytest.mark.parametrize("tw", [1, 4, 8, 32, 256])
+def test_view_wide(lib, W, H, most, tw):
+    """A group of 32 pixels that spans more than `most` radians; pixels of 2 / f."""
+    gw = min(tw, 32)
+    long = max(gw, 32 // gw)
+    for span, want in ((0.98 * most, False), (1.02 * most, True)):
+        f = int(round(2 * long * 999 / span))
+        cams = synth.camera_array([((0, 0, 0), (0, f, 0), (999, 0, 0), (0, 0, 999), 64, 48)])
+        assert bool(lib.wide(W, H, ctypes.c_void_p(cams.ctypes.data), tw)) == want
+
+
+def test_share_of_wide_views(lib):
+    """Wide pixels: up to a quarter of a traced batch, one in 32 of a marched one."""
+    f = 2 * 8 * 999
+    narrow = synth.camera_array([((0, 0, 0), (0, f * 100, 0), (999, 0, 0), (0, 0, 999), 64, 32)])
+    wide = synth.camera_array([((0, 0, 0), (0, f, 0), (999, 0, 0), (0, 0, 999), 64, 32)])
+    for share in (4, 32):
+        for k, want in ((share - 1, True), (share - 2, False)):
+            cams = np.concatenate([wide, np.repeat(narrow, k)])
+            fit = lib.fit(300, 300, ctypes.c_void_p(cams.ctypes.data), len(cams), 8, share)
+            assert bool(fit) == want, (share, k)
