@@ -159,7 +159,8 @@ typedef struct {
                                 larger values are clamped to the pyramid's top level */
     uint32_t flags;          /* HF_SHADOWS | HF_PLAIN | HF_SYNC | HF_STATS | HF_NOGRAPH | HF_NOWAIT
                                 | HF_HOST_OUTPUTS | HF_HOST_STAGED */
-    uint32_t max_steps;      /* traversal iterations allowed per ray; 0 = default guard */
+    uint32_t max_steps;      /* traversal iterations allowed per ray; 0 = a default guard,
+                                4 (width + height) + 64, which no ray reaches */
     int32_t sun[3];          /* direction toward the sun; all zero = (321060, -321060, 262144),
                                 elevation 30 deg, azimuth 135 deg; each |sun_i| < 2^21.
                                 With HF_SHADOWS and a sun that rises (sun[2] > 0), is not

@@ -76,7 +76,7 @@ __device__ __forceinline__ void trace_pixel(const RenderParams &p, const LevelDe
         Counters pc{0, 0};
         cast_single<STATS, PAIR, SHADOWS, false>(
             p.world.W, p.world.H, p.world.base, lvt, r, sp ? min(kShadowStart, p.shadow_mip) : start,
-            sp ? p.shadow_mip : p.mip_start, p.max_steps, h, pc);
+            sp ? p.shadow_mip : p.mip_start, p.max_steps, nullptr, h, pc);
         if (STATS) {
             Counters &dst = sp ? scnt : cnt;
             dst.nodes += pc.nodes;

@@ -113,7 +113,8 @@ __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev
     if (alone) {
         Counters none{0, 0};
         const int level = min(kBeamLevel, mip);
-        cast_general<false, PAIR>(lvt, beam_unray(d, q, oz, dz), level, mip, 0x7FFFFFFF, h, none);
+        cast_general<false, PAIR>(lvt, beam_unray(d, q, oz, dz), level, mip, p.max_steps, h, none,
+                                  p.status);
     } else if (only) {
         h.face = b.kind < 0 ? kFaceMiss : kFaceInside;
     } else if (b.kind >= 0) {
