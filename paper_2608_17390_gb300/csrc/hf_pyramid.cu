@@ -19,7 +19,11 @@ namespace hf {
 namespace {
 
 constexpr uint32_t kIdentity = 0x0000FF00u;  // max h0 0, min h1 255, max top 0
-constexpr int64_t kTailNodes = 2048;  // up to this many, finish in one block
+// Levels of up to kTailNodes nodes finish in one block, which also makes the one
+// below them if that has up to kTailFirst.  (With a launch of its own for the one
+// below, edits of 92 to 128 cells a side took up to 15 % longer: 96 x 96 cells of a
+// 256 x 256 world, call to end, 18.4 -> 21.1 us.)
+constexpr int64_t kTailNodes = 2048, kTailFirst = 4096;
 constexpr int kTailWords = 8352;  // nodes of its levels with siblings: at most 8344 (1024 x 2, straddling)
 constexpr int kTailThreads = 512;
 
@@ -93,18 +97,35 @@ __device__ __forceinline__ TailRect tail_rect(int32_t k, int32_t x0, int32_t y0,
     return r;
 }
 
-// Levels k_from..L of a small rectangle (at most kTailNodes nodes on level
-// k_from) in one block.  Bound by latency: a level is a few instructions but
+// Levels k_from..L of a small rectangle in one block (first: level k_from has more
+// than kTailNodes nodes, the next one does not).  Bound by latency: a level is a few instructions but
 // waits for the one below.  So the levels pass their nodes on in shared memory,
 // and the siblings outside the rectangle, which do not change, are read before
 // the first level is made: 61 x 57 cells of a 1999 x 1501 world 17.9 -> 11.8 us
 // with cold caches, against levels that read each other's nodes back from global
 // memory.
 __global__ void __launch_bounds__(kTailThreads) k_pyr_tail(uint32_t *world, const WorldDev w,
-                                                           int32_t k_from, int32_t x0,
+                                                           int32_t k_from, bool first, int32_t x0,
                                                            int32_t y0, int32_t x1, int32_t y1) {
     __shared__ uint32_t s_node[kTailWords];  // the levels' rectangles, one after the other
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // a node of level k from the level below it in global memory
+    auto from_below = [&](int32_t k, int32_t i, int32_t j) {
+        return reduce_children(world + w.off[k - 1], w.stride[k - 1],
+                               k == 1 ? w.W : (int32_t)w.stride[k - 1],
+                               k == 1 ? w.H : (int32_t)w.rows[k - 1], k == 1 ? 1 + w.pair : 0, i, j);
+    };
+    if (first) {  // read back from global memory by the next level, after the barrier
+        const TailRect r = tail_rect(k_from, x0, y0, x1, y1);
+        const int32_t ni = r.i1 - r.i0 + 1, nj = r.j1 - r.j0 + 1;
+        uint32_t *dst = world + w.off[k_from];
+        for (int32_t n = threadIdx.x; n < ni * nj; n += blockDim.x) {
+            const int32_t i = r.i0 + n % ni, j = r.j0 + n / ni;
+            dst[(uint32_t)j * w.stride[k_from] + (uint32_t)i] = from_below(k_from, i, j);
+        }
+        __syncthreads();
+        ++k_from;
+    }
     for (int k = k_from, at = 0; k < w.L; ++k) {
         const TailRect r = tail_rect(k, x0, y0, x1, y1);
         if ((k - k_from) % (kTailThreads / 32) == warp)
@@ -133,10 +154,7 @@ __global__ void __launch_bounds__(kTailThreads) k_pyr_tail(uint32_t *world, cons
             const int32_t b = (int32_t)(((float)n + 0.5f) * per), a = n - b * ni;
             uint32_t v;
             if (k == k_from) {
-                v = reduce_children(world + w.off[k - 1], w.stride[k - 1],
-                                    k == 1 ? w.W : (int32_t)w.stride[k - 1],
-                                    k == 1 ? w.H : (int32_t)w.rows[k - 1],
-                                    k == 1 ? 1 + w.pair : 0, r.i0 + a, r.j0 + b);
+                v = from_below(k, r.i0 + a, r.j0 + b);
             } else {
                 const uint32_t *c = s_node + from + 2 * b * (2 * ni) + 2 * a;
                 v = combine(combine(c[0], c[1]), combine(c[2 * ni], c[2 * ni + 1]));
@@ -283,12 +301,16 @@ int pyramid_repair_from(uint32_t *world, const WorldDev &w, int k_from, int32_t 
                         int32_t x1, int32_t y1, void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
     if (x1 <= x0 || y1 <= y0 || w.L == 0 || k_from > w.L) return 0;
+    auto nodes = [&](int k) {
+        return (int64_t)(((x1 - 1) >> k) - (x0 >> k) + 1) * (((y1 - 1) >> k) - (y0 >> k) + 1);
+    };
     int k = k_from;
+    bool first = false;
     for (; k <= w.L; ++k) {
-        const int32_t i0 = x0 >> k, i1 = (x1 - 1) >> k, j0 = y0 >> k, j1 = (y1 - 1) >> k;
-        const int64_t ni = i1 - i0 + 1, nj = j1 - j0 + 1;
-        const int64_t count = ni * nj;
-        if (count <= kTailNodes) break;
+        const int32_t i0 = x0 >> k, i1 = (x1 - 1) >> k, j0 = y0 >> k;
+        const int64_t ni = i1 - i0 + 1, count = nodes(k);
+        first = count > kTailNodes;
+        if (!first || (count <= kTailFirst && k < w.L && nodes(k + 1) <= kTailNodes)) break;
         const int32_t sw = (w.W + (1 << (k - 1)) - 1) >> (k - 1);
         const int32_t sh = (w.H + (1 << (k - 1)) - 1) >> (k - 1);
         const int threads = 256;
@@ -300,7 +322,7 @@ int pyramid_repair_from(uint32_t *world, const WorldDev &w, int k_from, int32_t 
         if (cudaGetLastError() != cudaSuccess) return -1;
     }
     if (k <= w.L) {
-        k_pyr_tail<<<1, kTailThreads, 0, s>>>(world, w, k, x0, y0, x1, y1);
+        k_pyr_tail<<<1, kTailThreads, 0, s>>>(world, w, k, first, x0, y0, x1, y1);
         if (cudaGetLastError() != cudaSuccess) return -1;
     }
     return 0;
