@@ -1326,7 +1326,7 @@ int hf_render_scatter(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_foo
     std::memcpy((char *)s.h_staging + sizeof(hf::BatchHeader) + (size_t)n * sizeof(hf::CamDev),
                 fp.data(), (size_t)n * sizeof(hf_footprint));
     CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));
-    if (hf::launch_scatter(b.p, sp, n, b.stream)) return HF_E_CUDA;
+    if (hf::launch_scatter(b.p, sp, n, c->sm_count, b.stream)) return HF_E_CUDA;
     return finish_batch(c, b, (o.flags & HF_SYNC) != 0);
 }
 

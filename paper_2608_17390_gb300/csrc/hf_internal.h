@@ -161,7 +161,8 @@ struct ScatterParams {
     uint32_t colour[8];      // resolved colour per material (an up-facing, lit surface)
     int32_t raw;             // 1: leave the packed words in hit_cell, no resolve
 };
-int launch_scatter(const RenderParams &p, const ScatterParams &s, uint32_t n_cams, void *stream);
+int launch_scatter(const RenderParams &p, const ScatterParams &s, uint32_t n_cams, int sm_count,
+                   void *stream);
 
 // The voxel occupancy pyramid of the RayVoxel comparison renderer
 // (hf_voxel.cu): level l of nx x ny x nz voxels in Morton-coded 8^3 tiles of

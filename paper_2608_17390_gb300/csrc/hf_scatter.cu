@@ -211,7 +211,16 @@ __global__ void k_scatter_clear(const RenderParams p) {
 //
 // Bound by instruction issue: 280 warp instructions to place a column and clip
 // it, 72 a point.  12 views of 1280 x 800, 1024 x 1024 samples of 16 points:
-// 484 us; 693 us with every point projected, by two rounded divisions.
+// about 480 us; 693 us with every point projected, by two rounded divisions.  (The first
+// thread of a warp of its own makes the camera's terms: with the first thread of
+// the table's, renders took 1.6 % longer on the average.)
+//
+// FEW: a launch that leaves most of the GPU idle is bound by the latency of a
+// thread's points instead.  Floor and slab take their points in one loop then, so
+// that one's work goes on while the other's waits: 64 x 64 samples of 1000 points
+// 634 -> 530 us, 256 x 256 of 32 over paired texels 41 -> 37.  Where warps abound
+// the loop of both costs 3 to 5 % (a slab's lanes hold up the others' floors).
+template <bool FEW>
 __global__ void __launch_bounds__(kScatterThreads) k_scatter(const RenderParams p,
                                                              const ScatterParams s) {
     __shared__ float s_tm[kScatterMaxPoints];  // column fractions m / (nz - 1)
@@ -221,7 +230,7 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter(const RenderParams 
     const CamDev &c = p.cams[cam];
     for (uint32_t m = threadIdx.x; m < s.nz; m += blockDim.x)
         s_tm[m] = __fdiv_rn((float)m, zden);
-    if (threadIdx.x == 0) s_cam = scatter_cam(c);
+    if (threadIdx.x == 32) s_cam = scatter_cam(c);
     __syncthreads();
     const float4 fp = reinterpret_cast<const float4 *>(p.cams + p.hdr->n_cams)[cam];
     const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -251,17 +260,29 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter(const RenderParams 
     const float h0 = (float)b0, h1 = (float)b1, h2 = (float)b2;
     const float qscale = s.qscale;
     uint32_t *buf = c.hit_cell;
-    uint32_t m0, m1, pix, q;
+    uint32_t m0, m1, s0 = 0, s1 = 0, pix, q;
     visible_points(h0, 0.0f, za, zb, s.nz, m0, m1);
-    for (uint32_t m = m0; m < m1; ++m)
+    auto floor_point = [&](uint32_t m) {
         if (project(k, wf, hf, w, qscale, cp, __fsub_rn(h0, __fmul_rn(h0, s_tm[m])), pix, q))
             atomicMin(buf + pix, (q << 8) | mat);
-    if (!slab) return;
-    visible_points(h2, h1, za, zb, s.nz, m0, m1);
-    for (uint32_t m = m0; m < m1; ++m)
+    };
+    auto slab_point = [&](uint32_t m) {
         if (project(k, wf, hf, w, qscale, cp,
                     __fadd_rn(h2, __fmul_rn(__fsub_rn(h1, h2), s_tm[m])), pix, q))
             atomicMin(buf + pix, (q << 8) | mat | 8u);
+    };
+    if (FEW) {
+        if (slab) visible_points(h2, h1, za, zb, s.nz, s0, s1);
+        for (uint32_t m = m1 ? (s1 ? min(m0, s0) : m0) : s0; m < max(m1, s1); ++m) {
+            if (m >= m0 && m < m1) floor_point(m);
+            if (m >= s0 && m < s1) slab_point(m);
+        }
+        return;
+    }
+    for (uint32_t m = m0; m < m1; ++m) floor_point(m);
+    if (!slab) return;
+    visible_points(h2, h1, za, zb, s.nz, s0, s1);
+    for (uint32_t m = s0; m < s1; ++m) slab_point(m);
 }
 
 __global__ void k_scatter_resolve(const RenderParams p, const ScatterParams s) {
@@ -299,13 +320,18 @@ __global__ void k_scatter_resolve(const RenderParams p, const ScatterParams s) {
 
 }  // namespace
 
-int launch_scatter(const RenderParams &p, const ScatterParams &s, uint32_t n_cams, void *stream) {
+int launch_scatter(const RenderParams &p, const ScatterParams &s, uint32_t n_cams, int sm_count,
+                   void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
     const uint32_t px_blocks = (s.max_pixels + kScatterThreads - 1) / kScatterThreads;
     k_scatter_clear<<<dim3(px_blocks < 1024 ? px_blocks : 1024, n_cams), kScatterThreads, 0, st>>>(p);
-    const uint32_t samples = s.nu * s.nv;
-    k_scatter<<<dim3((samples + kScatterThreads - 1) / kScatterThreads, n_cams), kScatterThreads, 0,
-                st>>>(p, s);
+    const dim3 grid((s.nu * s.nv + kScatterThreads - 1) / kScatterThreads, n_cams);
+    // four of the eight blocks that an SM holds: 256 x 256 samples of one view are
+    // 1.7 (FEW 10 % faster with 32 points), 512 x 512 6.7 (1 % slower)
+    if (grid.x * n_cams <= 4 * (uint32_t)sm_count)
+        k_scatter<true><<<grid, kScatterThreads, 0, st>>>(p, s);
+    else
+        k_scatter<false><<<grid, kScatterThreads, 0, st>>>(p, s);
     if (!s.raw)
         k_scatter_resolve<<<dim3(px_blocks, n_cams), kScatterThreads, 0, st>>>(p, s);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
