@@ -60,8 +60,6 @@ namespace {
 //       rise in the bounds' units (2^-8 world units), saturated at kRiseSat
 //       (every quantity it is compared with is below 2^17, so saturation
 //       changes no outcome).
-// A bound reads columns up to K + 63 (K <= kSunMaxReach): always in range.
-constexpr int kRowTable = (int)kSunMaxReach + 128;
 constexpr int32_t kRiseSat = 1 << 21;
 
 constexpr int kSunThreads = 128;
@@ -81,6 +79,16 @@ constexpr int kSunSplit = 8;
 // 1080p views 1331 -> 1254 us (parts of 8: 1282; of 16 over 16 x 16 nodes: 1.5 % more).
 constexpr int kSunPart = 16, kSunPartLevel = 3;
 constexpr uint32_t kSunSplitBelow = 16384;
+
+// The table's entries.  No column past K + 1, K = kSunMaxReach, can raise a bound
+// (sun_bounds_eligible), so none is looked into: the last round that is ends at
+// column K + 32 and asks for the rows after K + 33, entry K + 34; a split warp's next
+// part starts up to kSunPart * kSunSplit columns further on, and is looked up, entry
+// k + 2, before it is left out.
+constexpr int kRowTable = (int)kSunMaxReach + kSunPart * kSunSplit + 64;
+static_assert(kRowTable > (int)kSunMaxReach + 1 + kSunPart * kSunSplit + 2 &&
+                  kRowTable > (int)kSunMaxReach + 1 + 32 + 1,
+              "every column that a bound may ask for has its entry");
 
 __global__ void k_sun_rows(int4 *tab, int64_t lmin, int64_t lmaj, int64_t lz) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
