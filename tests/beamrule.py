@@ -18,3 +18,15 @@ def share_of_wide(W, H, cams, tile_w=8):
     """The share of the batch's pixels that are in wide views."""
     px = cams["w"].astype(np.int64) * cams["h"]
     return px[wide_views(W, H, cams, tile_w)].sum() / px.sum()
+
+
+def close_views(W, H, cams, tile_w=8):
+    """The same cameras with their pixels brought together until none is wide."""
+    cams = cams.copy()
+    for i in range(len(cams)):
+        one = cams[i:i + 1]
+        while wide_views(W, H, one, tile_w)[0]:
+            for k in "ru":
+                one[k] = one[k] * 9 // 10
+    assert not wide_views(W, H, cams, tile_w).any()
+    return cams
