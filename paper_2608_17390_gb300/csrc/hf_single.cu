@@ -41,6 +41,20 @@ __device__ __forceinline__ uint32_t level0_word(const WorldDev &w, int32_t x, in
     return load_word(w, 0, x, y);
 }
 
+// The cosine of a face with the sun's direction (by a switch: as selects, it cost
+// renders with shadows 2 %, by their registers).
+__device__ __forceinline__ float face_cosine(uint8_t face, const float *ln) {
+    switch (face) {
+        case kFaceNX: return -ln[0];
+        case kFacePX: return ln[0];
+        case kFaceNY: return -ln[1];
+        case kFacePY: return ln[1];
+        case kFaceNZ: return -ln[2];
+        case kFacePZ: return ln[2];
+        default: return 0.0f;
+    }
+}
+
 // Writes one pixel's outputs.
 __device__ __forceinline__ void store_pixel(const RenderParams &p, const CamDev &c, uint32_t pix,
                                             const Hit &ph, float depth, bool visible,
@@ -53,7 +67,9 @@ __device__ __forceinline__ void store_pixel(const RenderParams &p, const CamDev 
     if (c.layer) __stcs(c.layer + pix, hit ? ph.layer : (uint8_t)255);
     if (c.face) __stcs(c.face + pix, ph.face);
     if (c.depth) __stcs(c.depth + pix, depth);
-    if (c.rgba) __stcs(c.rgba + pix, hit ? shade(ph.word >> 24 & 7, ph.face, visible, p.sun_n) : kSky);
+    if (c.rgba)
+        __stcs(c.rgba + pix,
+               hit ? shade(ph.word >> 24 & 7, face_cosine(ph.face, p.sun_n), visible) : kSky);
 }
 
 // One pixel: its primary ray, then (with shadows) the shadow ray, which

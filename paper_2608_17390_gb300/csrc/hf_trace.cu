@@ -122,6 +122,13 @@ __device__ __forceinline__ void cast_beams(const RenderParams &p, const LevelDev
     }
 }
 
+// The cosine of a face with the sun's direction ln: the normal's axis is face / 2,
+// its sign face's lowest bit.
+__device__ __forceinline__ float face_cosine(uint8_t face, const float *ln) {
+    const float n = face < kFaceNY ? ln[0] : face < kFaceNZ ? ln[1] : ln[2];
+    return face == kFaceInside ? 0.0f : face & 1 ? n : -n;
+}
+
 // What a warp works on, in shared memory: its camera's record and its tile's
 // first pixel.  Fields are read when they are needed instead of being held in
 // registers through a cast, where registers decide how many warps fit.
@@ -240,7 +247,8 @@ __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelD
     const uint32_t pix = (uint32_t)py * c.w + (uint32_t)px;
     const uint8_t face = tag & 0xFF;
     if (SHADOWS && c.shadow) __stcs(c.shadow + pix, (uint8_t)(visible ? 0 : 1));
-    if (c.rgba) __stcs(c.rgba + pix, face < kFaceError ? shade(tag >> 8, face, visible, p.sun_n) : kSky);
+    if (c.rgba)
+        __stcs(c.rgba + pix, face < kFaceError ? shade(tag >> 8, face_cosine(face, p.sun_n), visible) : kSky);
 }
 
 // One warp renders one tile: lane l traces the tile's pixels l, l+32, ...

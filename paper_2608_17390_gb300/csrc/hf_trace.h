@@ -30,11 +30,8 @@ __device__ __forceinline__ int32_t floor_div_small(int64_t a, int32_t b, float r
     return q;
 }
 
-__device__ __forceinline__ uint32_t shade(uint32_t m, uint8_t face, bool visible,
-                                          const float *ln) {
-    // the normal's axis is face / 2, its sign face's lowest bit
-    const float n = face < kFaceNY ? ln[0] : face < kFaceNZ ? ln[1] : ln[2];
-    const float ndl = face == kFaceInside ? 0.0f : face & 1 ? n : -n;
+// The colour of material m under the cosine ndl of the sun's angle.
+__device__ __forceinline__ uint32_t shade(uint32_t m, float ndl, bool visible) {
     const float k = kKa + kKd * fmaxf(ndl, 0.0f) * (visible ? 1.0f : 0.0f);
     uint32_t out = 0xFF000000u;
 #pragma unroll
