@@ -59,7 +59,7 @@ def _dist():
 # ------------------------------------------------------------- ncu traffic
 
 TRACE_SOURCES = tuple("paper_2608_17390_gb300/csrc/" + f
-                      for f in ("hf_trace.cu", "hf_beam.h", "hf_cast.h", "hf_internal.h"))
+                      for f in ("hf_trace.cu", "hf_trace.h", "hf_beam.h", "hf_cast.h", "hf_internal.h"))
 
 
 def trace_source_hash():
@@ -351,8 +351,8 @@ def run_hf(args):
     else:
         opts = hf.make_opts(flags=flags, mip_start=args.mip, tile_w=args.tile_w,
                             tile_h=args.tile_h)
-    opts.tile_w, opts.tile_h = opts.tile_w or 8, opts.tile_h or 4  # (what the line reports)
     tile_w, tile_h, mip_start = opts.tile_w, opts.tile_h, opts.mip_start
+    tile = "%dx%d" % (tile_w, tile_h) if tile_w and tile_h else "default"  # (the library's choice)
     rng = np.random.default_rng(1234)
     H, W = cells.shape
 
@@ -559,7 +559,7 @@ def run_hf(args):
     alg_bytes = fetch_b + out_b
     r_ms = float(np.mean(render_ms))
     achieved = alg_bytes / (r_ms / 1e3) / 1e9
-    traffic = _profiled_traffic(args.workload, rays, "%dx%d" % (tile_w, tile_h), mip_start)
+    traffic = _profiled_traffic(args.workload, rays, tile, mip_start)
     line = {
         "metric": "primary rays/s (batched, exact two-interval height-field ray cast)",
         "value": value, "unit": "primary rays/s", "n_gpus": ws, "steps": args.steps,
@@ -569,11 +569,11 @@ def run_hf(args):
         "config": {"workload": wl["name"], "rays_per_step": int(rays_step),
                    "grid": "%dx%d" % (W, H), "l2": "flushed between steps (256 MiB write)",
                    "mip_start": "library default" if mip_start == 0xFFFFFFFF else mip_start,
-                   "tile": "%dx%d" % (tile_w, tile_h),
+                   "tile": tile,
                    "autotuned": tuned,
                    "world_bytes": info["cell_bytes"] + info["pyramid_bytes"]},
         "plain_rays_per_s": plain,
-        "plain_tile": ("%dx%d" % plain_tile) if plain_tile else None,
+        "plain_tile": plain_tile and ("%dx%d" % plain_tile if all(plain_tile) else "default"),
         "batched_over_plain": (value / ws / plain) if plain else None,
         "render_ms": r_ms,
         "pyramid_build_ms": build_ms,
@@ -588,7 +588,7 @@ def run_hf(args):
                              "with HF_STATS) + %d B output per ray; the timed kernels test nodes "
                              "for 32 rays at a time and fetch fewer, mostly from L1 and L2"
                              % (14 + (1 if wl["shadows"] else 0))},
-        "alu_roofline": _alu_roofline(args.workload, rays, r_ms, "%dx%d" % (tile_w, tile_h),
+        "alu_roofline": _alu_roofline(args.workload, rays, r_ms, tile,
                                       mip_start, info["sm_count"],
                                       (ck or {}).get("sm_mhz") or _peak_sm_mhz()),
         "fetches_per_ray": (st["node_fetches"] + st["cell_fetches"]) / max(rays, 1),

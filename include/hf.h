@@ -247,7 +247,8 @@ int hf_render(hf_ctx *ctx, const hf_camera *cams, uint32_t n, const hf_outputs *
  * It renders n <= HF_NOALLOC_MAX_CAMERAS cameras with the same kernel and the
  * same results as hf_render, always as one batched launch on the context's
  * own stream (opts->cuda_stream must be NULL or that stream), so edits and
- * renders stay ordered.  Accepted flags: HF_SHADOWS and HF_SYNC (with HF_SYNC
+ * renders stay ordered.  Tile sides of 0 mean 8 x 4 whatever the batch.
+ * Accepted flags: HF_SHADOWS and HF_SYNC (with HF_SYNC
  * the step-guard status is returned; without it this entry point reports no
  * step-guard status, and hf_sync does not see it).  Any other flag is refused
  * with HF_E_INVALID_ARG before anything is enqueued.
