@@ -1211,7 +1211,8 @@ int hf_render_march(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outpu
     if (o.steps > 65536 || o.bisections > 65536 || !(m.far_dist > 0.0f)) return HF_E_INVALID_ARG;
     const uint32_t tw = o.tile_w ? o.tile_w : 8, th = o.tile_h ? o.tile_h : 4;
     if (c->occ_march < 1) return HF_E_CUDA;
-    const bool beams = hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kMarchShare);
+    const bool beams = hf::march_beams_pay((int32_t)c->W, (int32_t)c->H, m.steps, m.far_dist) &&
+                       hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kMarchShare);
     Batch b;
     int rc = prepare_batch(c, cams, n, outs, tw, th, beams ? tw : 0, false, o.cuda_stream, b);
     if (rc != HF_OK) return rc;

@@ -86,7 +86,7 @@ __device__ __forceinline__ bool beam_next(BeamScan &s, const LevelDev *lvt, cons
             s.u = (s.j + 32) * (1 << s.level);
             s.level = min(s.level + 2, s.top_level);
         } else {
-            s.open = open;
+            s.open = SAMPLES ? beam_joined(open) : open;
         }
     }
     const int i = __ffs(s.open) - 1, run = beam_run(s.open, i);

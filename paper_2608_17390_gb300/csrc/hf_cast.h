@@ -757,6 +757,11 @@ HF_HD int beam_run(uint32_t open, int i) {
 #endif
 }
 
+// The open stretches, with single closed ones between two of them: a march's run
+// over such a gap costs less than two runs beside it (1.5 % over 384 renders;
+// gaps of three stretches: no better than none, of seven or all: worse).
+HF_HD uint32_t beam_joined(uint32_t open) { return open | (open << 1 & open >> 1); }
+
 // The shortest stretches worth testing from u on: at least an eighth as long
 // as the beam is wide there, so that one covers few nodes.
 HF_HD int beam_least(const Beam &m, int32_t u, int base, int top) {

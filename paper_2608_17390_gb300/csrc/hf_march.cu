@@ -17,7 +17,7 @@
 // in a stretch that the beam does not prove empty, at a height that its cells
 // reach, are looked up (hf_march.h: the bounds of their rounding).
 // Bound by instruction issue: 12 views of 1280 x 800 over 2048 x 16384 cells, 128
-// samples a ray, 1.229 -> 0.617 ms.
+// samples a ray, 1.229 -> 0.608 ms.
 #include <cuda_runtime.h>
 
 #include "hf_beam.h"
@@ -31,14 +31,9 @@ constexpr int kMarchThreads = 128;
 // Nine blocks leave each thread 56 registers.  12 views of 1280 x 800 with 128
 // samples a ray: seven blocks 638 us, nine 622, eleven (46 registers) 692.
 constexpr int kMarchMinBlocks = 9;
-// From this many samples a ray on, and where the rays of a warp stay close (as
-// for the exact cast), beams are cheaper than taking every sample.  Every sample
-// / beams: 12 views of 1280 x 800 over 2048 x 16384 cells, 32 samples 630 / 609
-// us, 128 1517 / 596; but 16 views of 640 x 360 near the ground of a 2048 x 2048
-// world, 48 samples 0.70, 96 1.03, 128 1.26 times as fast with beams.  The kernel
-// without beams needs 40 registers, so that six blocks fit an SM (asked for, they
-// cost it 0.6 %); in blocks of 128 threads it is 3 % slower.
-constexpr int kMarchBeamSteps = 96;
+// The kernel that takes every sample (hf_rules.h says when) needs 40 registers, so
+// that six blocks fit an SM (asked for, they cost it 0.6 %); in blocks of 128 threads
+// it is 3 % slower.
 constexpr int kMarchAllBlocks = 6, kMarchAllThreads = 256;
 
 struct MarchPoint {
@@ -261,7 +256,7 @@ __global__ void __launch_bounds__(BEAMS ? kMarchThreads : kMarchAllThreads,
 int launch_march_batched(const RenderParams &p, const MarchParams &m, bool beams, int blocks,
                          void *stream) {
     cudaStream_t s = (cudaStream_t)stream;
-    if (beams && m.steps >= kMarchBeamSteps) {
+    if (beams) {
         k_march_batched<true><<<blocks, kMarchThreads, 0, s>>>(p, m);
     } else {
         const int all = (blocks * kMarchAllBlocks + kMarchMinBlocks - 1) / kMarchMinBlocks;

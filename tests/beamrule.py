@@ -20,6 +20,11 @@ def share_of_wide(W, H, cams, tile_w=8):
     return px[wide_views(W, H, cams, tile_w)].sum() / px.sum()
 
 
+def march_in_beams(W, H, steps, far):
+    """Whether a march of close views takes beams."""
+    return steps * min(1.0, max(W, H) / far) >= 112
+
+
 def close_views(W, H, cams, tile_w=8):
     """The same cameras with their pixels brought together until none is wide."""
     cams = cams.copy()

@@ -1,12 +1,13 @@
 """The march in beams against the oracle, bit for bit (GPU only): views whose
-rays lie close enough for the rule that picks beams (which is checked), from 96
-samples a ray on: over odd, one-cell and paired grids in every direction, and
+rays lie close enough, with enough samples in the grid, for the rules that pick
+beams (which is checked): over odd, one-cell and paired grids in every direction, and
 over the widest grids beside high columns, where a sample's rounding shows."""
 
 import numpy as np
 import pytest
 
 import synth
+from beamrule import march_in_beams, wide_views
 from test_gpu_march import _gpu, hf  # noqa: F401
 from test_gpu_march_edges import _check
 from oracle import march
@@ -15,20 +16,10 @@ pytestmark = pytest.mark.gpu
 S = 65536
 
 
-def _close(W, H, cams, tile_w):
-    """Whether every view's groups of 32 pixels pass the rule for beams."""
-    size = max(W, H)
-    most = 0.06 if size <= 512 else 0.04 if size <= 4096 else 0.028
-    gw = min(tile_w, 32)
-    gh = 32 // gw
-    f, r, u = (np.sqrt((cams[k].astype(float) ** 2).sum(1)) for k in "fru")
-    return (np.maximum(2 * gw * r, 2 * gh * u) <= most * f).all()
-
-
 def _compare(hf, cells, cams, steps, far, tile, texels=None):
     cams = synth.camera_array(cams)
     H, W = cells.shape
-    assert _close(W, H, cams, tile[0]) and steps >= 96
+    assert not wide_views(W, H, cams, tile[0]).any() and march_in_beams(W, H, steps, far)
     ctx = hf.hf_create(cells) if texels is None else hf.hf_create_pairs(texels)
     try:
         got = _gpu(hf, ctx, cams, hf.make_march_opts(steps=steps, far_dist=far, tile_w=tile[0],
@@ -41,9 +32,10 @@ def _compare(hf, cells, cams, steps, far, tile, texels=None):
 
 @pytest.mark.parametrize("W,H,pairs", [(1, 1, False), (37, 53, False), (300, 9, False), (130, 97, True),
                                        (700, 613, False)])
-@pytest.mark.parametrize("steps,far,tile", [(128, 600.0, (8, 4)), (1000, 90.0, (4, 32)),
-                                            (96, 5000.0, (32, 1)), (300, 0.05, (16, 8))])
-def test_close_rays(hf, W, H, pairs, steps, far, tile):  # noqa: F811
+@pytest.mark.parametrize("steps,part,tile", [(128, 1.0, (8, 4)), (1000, 3.0, (4, 32)), (113, 1.0, (32, 1)),
+                                             (2000, 0.2, (8, 4)), (300, 0.0005, (16, 8))])
+def test_close_rays(hf, W, H, pairs, steps, part, tile):  # noqa: F811
+    far = part * max(W, H)
     rng = np.random.default_rng(W * H + steps)
     cells, _ = synth.make_grid(W, H, seed=W + H, slab_frac=0.4, n_walls=max(1, W // 10))
     if pairs:

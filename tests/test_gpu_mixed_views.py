@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 import synth
-from beamrule import share_of_wide, wide_views
+from beamrule import march_in_beams, share_of_wide, wide_views
 from hfcheck import compare, gpu_render
 from oracle import march
 from test_gpu_march import _gpu, hf  # noqa: F401
@@ -69,8 +69,10 @@ def test_marched(hf, W, H, order):  # noqa: F811
     assert 0 < share_of_wide(W, H, cams) <= 1 / 32
     ctx = hf.hf_create(cells)
     try:
-        got = _gpu(hf, ctx, cams, hf.make_march_opts(steps=128))
+        far = float(max(W, H))
+        assert march_in_beams(W, H, 128, far)
+        got = _gpu(hf, ctx, cams, hf.make_march_opts(steps=128, far_dist=far))
         for i, c in enumerate(cams):
-            _check(got[i], march.march_camera(cells, c, steps=128), i)
+            _check(got[i], march.march_camera(cells, c, steps=128, far=far), i)
     finally:
         hf.hf_destroy(ctx)

@@ -100,6 +100,7 @@ static void march_warp(const World &w, const Ray *r, const MarchRay *m, int n, i
                 continue;
             }
             const bool met = open != 0;
+            open = beam_joined(open);
             while (open) {
                 const int i = __builtin_ctz(open), run = beam_run(open, i);
                 open &= i + run < 32 ? 0xFFFFFFFFu << (i + run) : 0u;

@@ -16,6 +16,7 @@ SHIM = r"""
 extern "C" void tile(const hf_camera *c, uint32_t n, int beams, uint64_t warps, uint32_t flags, uint32_t *t) {
     hf::default_tile(c, n, beams, warps, flags, t[0], t[1]);
 }
+extern "C" int pay(int32_t W, int32_t H, int32_t steps, float far_dist) { return hf::march_beams_pay(W, H, steps, far_dist); }
 extern "C" int wide(int32_t W, int32_t H, const hf_camera *c, uint32_t tw) { return hf::view_wide(W, H, *c, tw); }
 extern "C" int fit(int32_t W, int32_t H, const hf_camera *c, uint32_t n, uint32_t tw, uint32_t share) {
     return hf::beams_fit(W, H, c, n, tw, share);
@@ -98,3 +99,11 @@ def test_share_of_wide_views(lib):
             cams = np.concatenate([wide, np.repeat(narrow, k)])
             fit = lib.fit(300, 300, ctypes.c_void_p(cams.ctypes.data), len(cams), 8, share)
             assert bool(fit) == want, (share, k)
+
+
+@pytest.mark.parametrize("W,H,steps,far,want", [
+    (2048, 16384, 112, 600.0, True), (2048, 16384, 111, 600.0, False), (300, 2, 128, 300.0, True),
+    (300, 200, 223, 600.0, False), (300, 200, 224, 600.0, True), (1, 1, 65536, 600.0, False),
+    (1, 1, 112, 0.5, True), (16384, 16384, 1, 1e30, False)])
+def test_march_beams_pay(lib, W, H, steps, far, want):
+    assert bool(lib.pay(W, H, steps, ctypes.c_float(far))) == want
