@@ -750,8 +750,8 @@ static int launch_graph(hf_ctx *c, Slot &s, const GraphKey &key, const hf::Rende
     return HF_OK;
 }
 
-// Validates the cameras, takes a render slot and fills its camera table.  beam_tw:
-// the tile width that wide views are told by, 0 where no beams are cast.
+// Validates the cameras, takes a render slot and fills its camera table.  wide: which
+// views are, for a batch that casts beams (else null).
 struct Batch {
     int slot;
     size_t bytes, bucket;
@@ -775,8 +775,8 @@ static void *device_alias(void *ptr) {
 }
 
 static int prepare_batch(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *outs,
-                         uint32_t tw, uint32_t th, uint32_t beam_tw, bool nowait, void *user_stream,
-                         Batch &b, bool host_outputs = false, size_t extra_bytes = 0) {
+                         uint32_t tw, uint32_t th, const uint8_t *wide, bool nowait,
+                         void *user_stream, Batch &b, bool host_outputs = false, size_t extra_bytes = 0) {
     const int twl = ilog2_exact(tw), thl = ilog2_exact(th);
     if (twl < 0 || thl < 0 || tw * th < 32 || tw * th > 256 || tw > 256 || th > 256)
         return HF_E_INVALID_ARG;
@@ -840,12 +840,9 @@ static int prepare_batch(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_
         return true;
     };
     // wide views first: their warps take longest, and would be a batch's tail
-    auto wide = [&](uint32_t i) {
-        return beam_tw && hf::view_wide((int32_t)c->W, (int32_t)c->H, cams[i], beam_tw);
-    };
     for (const bool single : {true, false})
         for (uint32_t i = 0; i < n; ++i)
-            if (wide(i) == single && !put(i, single)) return HF_E_INVALID_ARG;
+            if ((wide && wide[i]) == single && !put(i, single)) return HF_E_INVALID_ARG;
     std::memset(&b.p, 0, sizeof(b.p));
     b.p.world = c->wd;
     {  // the levels the trace kernels warm in L2: from the finest level whose
@@ -1124,13 +1121,12 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
     for (int i = 0; i < 3; ++i)
         if (iabs64(sun[i]) >= kLimit21) return HF_E_INVALID_ARG;
     const bool shadows = (o.flags & HF_SHADOWS) != 0;
+    std::vector<uint8_t> wide(n);
+    const bool fit = hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kTraceShare,
+                                   wide.data());
     const int kind = (o.flags & HF_STATS) ? hf::kTraceStats
-                     : o.max_steps || !hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kTraceShare)
-                         ? hf::kTraceGeneral
-                         : hf::kTraceBeams;
-    // (plain launches pick their kernel one by one)
-    const bool plain = (o.flags & HF_PLAIN) != 0;
-    const uint32_t fit_tw = tw, beam_tw = kind == hf::kTraceBeams && !plain ? tw : 0;
+                     : o.max_steps || !fit ? hf::kTraceGeneral
+                                           : hf::kTraceBeams;
     const uint32_t mip = o.mip_start == HF_MIP_AUTO ? hf::kDefaultMipStart : o.mip_start;
     const uint32_t mip_c = mip > c->L ? c->L : mip;
     const uint64_t guard = 4ull * (c->W + c->H) + 64;
@@ -1148,8 +1144,11 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         if (brc != HF_OK) return brc;
     }
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, tw, th, beam_tw, (o.flags & HF_NOWAIT) != 0,
-                           o.cuda_stream, b, (o.flags & HF_HOST_OUTPUTS) != 0);
+    // (plain launches keep their order and pick their kernels one by one)
+    const bool sort = kind == hf::kTraceBeams && !(o.flags & HF_PLAIN);
+    int rc = prepare_batch(c, cams, n, outs, tw, th, sort ? wide.data() : nullptr,
+                           (o.flags & HF_NOWAIT) != 0, o.cuda_stream, b,
+                           (o.flags & HF_HOST_OUTPUTS) != 0);
     if (rc != HF_OK) return rc;
     b.p.sun_bounds = bounds;
     Slot &s = c->slots[b.slot];
@@ -1170,9 +1169,8 @@ int hf_render(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outputs *ou
         const auto *cd = (const hf::CamDev *)((const char *)s.h_staging + sizeof(hf::BatchHeader));
         for (uint32_t i = 0; i < n; ++i) {
             const int one = kind == hf::kTraceStats || o.max_steps ? kind
-                            : hf::view_wide((int32_t)c->W, (int32_t)c->H, cams[i], fit_tw)
-                                ? hf::kTraceGeneral
-                                : hf::kTraceBeams;
+                            : wide[i]                              ? hf::kTraceGeneral
+                                                                   : hf::kTraceBeams;
             if (hf::launch_trace_plain(p, shadows, one, cd[i], b.tiles[i], b.stream))
                 return HF_E_CUDA;
         }
@@ -1211,10 +1209,13 @@ int hf_render_march(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outpu
     if (o.steps > 65536 || o.bisections > 65536 || !(m.far_dist > 0.0f)) return HF_E_INVALID_ARG;
     const uint32_t tw = o.tile_w ? o.tile_w : 8, th = o.tile_h ? o.tile_h : 4;
     if (c->occ_march < 1) return HF_E_CUDA;
+    std::vector<uint8_t> wide(n);
     const bool beams = hf::march_beams_pay((int32_t)c->W, (int32_t)c->H, m.steps, m.far_dist) &&
-                       hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kMarchShare);
+                       hf::beams_fit((int32_t)c->W, (int32_t)c->H, cams, n, tw, hf::kMarchShare,
+                                     wide.data());
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, tw, th, beams ? tw : 0, false, o.cuda_stream, b);
+    int rc = prepare_batch(c, cams, n, outs, tw, th, beams ? wide.data() : nullptr, false,
+                           o.cuda_stream, b);
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
     CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));
@@ -1320,7 +1321,7 @@ int hf_render_scatter(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_foo
     }
     sp.max_pixels = maxpix;
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, 8, 4, 0, false, o.cuda_stream, b, false,
+    int rc = prepare_batch(c, cams, n, outs, 8, 4, nullptr, false, o.cuda_stream, b, false,
                            (size_t)n * sizeof(hf_footprint));
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
@@ -1413,7 +1414,7 @@ int hf_render_voxel(hf_ctx *c, const hf_camera *cams, uint32_t n, const hf_outpu
     q.far_dist = o.far_dist != 0.0f ? o.far_dist : 600.0f;
     if (o.outer > 1u << 20 || o.inner > 4096 || !(q.far_dist > 0.0f)) return HF_E_INVALID_ARG;
     Batch b;
-    int rc = prepare_batch(c, cams, n, outs, 8, 4, 0, false, o.cuda_stream, b);
+    int rc = prepare_batch(c, cams, n, outs, 8, 4, nullptr, false, o.cuda_stream, b);
     if (rc != HF_OK) return rc;
     Slot &s = c->slots[b.slot];
     CK(cudaMemcpyAsync(s.d_scratch, s.h_staging, b.bytes, cudaMemcpyHostToDevice, b.stream));

@@ -30,7 +30,7 @@ inline bool view_wide(int32_t W, int32_t H, const hf_camera &k, uint32_t tw) {
 }
 
 // Whether a batch takes the kernel with beams: if of `share` pixels at most one is a
-// wide view's.  In a batch that does, the rays of its wide views go each by itself
+// wide view's (wide: where to say which views are).  In a batch that does, the rays of its wide views go each by itself
 // too (CamDev::single; in beams, batches over 2048 x 16384 cells with 3 % of their
 // pixels in views of 64 x 48 took up to seven times as long), but in a kernel whose
 // registers are the beams'.  All rays by themselves over beams for the views that
@@ -45,14 +45,15 @@ inline bool view_wide(int32_t W, int32_t H, const hf_camera &k, uint32_t tw) {
 //   samples; 256    1.26 - 2.97  0.76 - 1.64  1.00 - 2.04  0.77 - 1.58  1.00 - 1.48  1.00 - 1.37
 constexpr uint32_t kTraceShare = 4, kMarchShare = 32;
 inline bool beams_fit(int32_t W, int32_t H, const hf_camera *cams, uint32_t n, uint32_t tw,
-                      uint32_t share) {
-    uint64_t all = 0, wide = 0;
+                      uint32_t share, uint8_t *wide) {
+    uint64_t all = 0, some = 0;
     for (uint32_t i = 0; i < n; ++i) {
         const uint64_t px = (uint64_t)cams[i].w * cams[i].h;
+        wide[i] = view_wide(W, H, cams[i], tw);
         all += px;
-        if (view_wide(W, H, cams[i], tw)) wide += px;
+        if (wide[i]) some += px;
     }
-    return wide * share <= all;
+    return some * share <= all;
 }
 
 // Whether a march whose views fit takes beams: from so many samples a ray on that

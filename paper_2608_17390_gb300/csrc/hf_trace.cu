@@ -145,8 +145,7 @@ __device__ __forceinline__ void tile_pixel(const RenderParams &p, const TileDev 
 }
 
 // One pixel per lane: its primary ray, then (with shadows) the shadow ray, in
-// a second pass of the same traversal code.  Every lane of the warp calls;
-// 
+// a second pass of the same traversal code.  Every lane of the warp calls.
 // WIDE: the view may be a wide one (a launch of one view is not).
 template <bool SHADOWS, bool PAIR, bool WIDE>
 __device__ __forceinline__ void trace_pixels(const RenderParams &p, const LevelDev *lvt,
@@ -470,12 +469,14 @@ extern "C" int hf_render_noalloc(hf_ctx *ctx, const hf_camera *cams, uint32_t n,
     for (uint32_t i = 0; i < n; ++i)
         if (hf_validate_camera((uint32_t)v.world.W, (uint32_t)v.world.H, &cams[i]) != HF_OK)
             return HF_E_INVALID_ARG;
+    uint8_t wide[HF_NOALLOC_MAX_CAMERAS];
+    const bool fit = beams_fit(v.world.W, v.world.H, cams, n, tw, kTraceShare, wide);
     uint64_t base = 0;
     uint32_t at = 0;
     for (const bool single : {true, false})  // wide views first, as in hf_render
         for (uint32_t i = 0; i < n; ++i) {
             const hf_camera &k = cams[i];
-            if (view_wide(v.world.W, v.world.H, k, tw) != single) continue;
+            if ((wide[i] != 0) != single) continue;
             CamDev &c = cd[at++];
             for (int a = 0; a < 3; ++a) {
                 c.o[a] = (int32_t)k.origin[a];
@@ -540,9 +541,7 @@ extern "C" int hf_render_noalloc(hf_ctx *ctx, const hf_camera *cams, uint32_t n,
         p.sun[i] = sun[i];
         p.sun_n[i] = (float)(sun[i] / sn);
     }
-    const int kind = o.max_steps || !beams_fit(v.world.W, v.world.H, cams, n, tw, kTraceShare)
-                         ? kTraceGeneral
-                         : kTraceBeams;
+    const int kind = o.max_steps || !fit ? kTraceGeneral : kTraceBeams;
     const int blocks = v.sm_count * v.occ[shadows ? 1 : 0][kind];
     if (launch_trace_batched(p, shadows, kind, blocks, stream)) return HF_E_CUDA;
     if (o.flags & HF_SYNC) {

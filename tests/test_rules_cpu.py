@@ -19,7 +19,8 @@ extern "C" void tile(const hf_camera *c, uint32_t n, int beams, uint64_t warps, 
 extern "C" int pay(int32_t W, int32_t H, int32_t steps, float far_dist) { return hf::march_beams_pay(W, H, steps, far_dist); }
 extern "C" int wide(int32_t W, int32_t H, const hf_camera *c, uint32_t tw) { return hf::view_wide(W, H, *c, tw); }
 extern "C" int fit(int32_t W, int32_t H, const hf_camera *c, uint32_t n, uint32_t tw, uint32_t share) {
-    return hf::beams_fit(W, H, c, n, tw, share);
+    uint8_t wide[64];
+    return hf::beams_fit(W, H, c, n, tw, share, wide);
 }
 """
 
