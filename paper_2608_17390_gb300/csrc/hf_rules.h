@@ -30,11 +30,11 @@ inline bool view_wide(int32_t W, int32_t H, const hf_camera &k, uint32_t tw) {
 }
 
 // Whether a batch takes the kernel with beams: if of `share` pixels at most one is a
-// wide view's (wide: where to say which views are).  In a batch that does, the rays of its wide views go each by itself
-// too (CamDev::single; in beams, batches over 2048 x 16384 cells with 3 % of their
-// pixels in views of 64 x 48 took up to seven times as long), but in a kernel whose
-// registers are the beams'.  All rays by themselves over beams for the views that
-// fit, by the share of the wide views' pixels:
+// wide view's (wide: where to say which views are).  In a batch that does, the rays of
+// its wide views go each by itself too (CamDev::single; in beams, batches over 2048 x
+// 16384 cells with 3 % of their pixels in views of 64 x 48 took up to seven times as
+// long), but in a kernel whose registers are the beams'.  All rays by themselves over
+// beams for the views that fit, by the share of the wide views' pixels:
 //   share           0.08         0.13         0.21         0.37         0.57         0.84
 //   traced, 2048^2  0.99 - 1.59  1.17 - 1.49  1.23 - 1.55  1.09 - 1.42  0.91 - 1.22  0.95 - 1.20
 //   2048 x 16384    1.34 - 1.71  1.33 - 1.51  1.33 - 1.63  1.13 - 1.27  0.91 - 1.14  0.86 - 1.00
